@@ -102,6 +102,61 @@ static void byte_tables(const int16_t *v, uint32_t n_loci, int32_t *lut) {
         }
 }
 
+// v * 2^s as f16, v of at most 11 significant bits, the result in the normal range.
+static uint32_t f16_scaled(int32_t v, int s) {
+    if (v == 0) return 0u;
+    const uint32_t m = (uint32_t)(v < 0 ? -v : v);
+    int e = 0;
+    while ((m >> e) > 1u) ++e;  // 2^e <= m < 2^(e+1)
+    const uint32_t frac = e > 10 ? (m >> (e - 10)) & 0x3FFu : (m << (10 - e)) & 0x3FFu;
+    return (v < 0 ? 0x8000u : 0u) | (uint32_t)(e + s + 15) << 10 | frac;
+}
+
+// The B fragments of the generation kernel's products (generations.cuh): lane
+// 4n + q holds column n of the element pairs that lane q of a row's group
+// makes.  Pair r of a lane: element position p (its bit in the half words,
+// after the kernel's shifts) and the loci in its low and high half.  Even
+// columns: the value (its low digit), odd columns: the allele count of the
+// element (its high digit of radix 2048), each scaled by 2^(4 - p).
+void value_fragments(const int16_t *effects, const int16_t *dominance, uint32_t n_loci, ValueFragments &vf,
+                     uint32_t &two_digits) {
+    const uint32_t W = n_loci / 32, regs = W >= 4 ? 16u : 4u * W, room = std::max(regs, 8u);
+    auto value = [&](uint32_t t, uint32_t l) {  // additive; heterozygous, homozygous
+        return !dominance ? (int32_t)effects[l] : t == 0 ? effects[l] + (int32_t)dominance[l] : 2 * (int32_t)effects[l];
+    };
+    two_digits = 0;
+    for (uint32_t t = 0; t < (dominance ? 2u : 1u); ++t)
+        for (uint32_t l = 0; l < n_loci; ++l)
+            if (value(t, l) > 2048 || value(t, l) < -2048) two_digits = 1;
+    std::memset(&vf, 0, sizeof vf);
+    for (uint32_t t = 0; t < (dominance ? 2u : 1u); ++t)
+        for (uint32_t set = 0; set < (W == 8 ? 2u : 1u); ++set)
+            for (uint32_t r = 0; r < regs; ++r)
+                for (uint32_t lane = 0; lane < 32; ++lane) {
+                    const uint32_t q = lane & 3u, odd = (lane >> 2) & 1u;
+                    const uint32_t word = W >= 4 ? 4u * set + q : W == 2 ? q & 1u : 0u;
+                    const uint32_t part = W >= 4 ? 0u : W == 2 ? 8u * (q >> 1) : 4u * q;  // first bit of the lane's part
+                    uint32_t bit, p;
+                    if (dominance) {  // one bit per locus
+                        bit = r;
+                        p = r <= 10 ? r : r - 5;
+                    } else {          // two bits per locus: even loci, then odd ones
+                        const uint32_t i = r % (regs / 2);
+                        bit = 2 * i + r / (regs / 2);
+                        p = i <= 5 ? 2 * i : 2 * i - 4;
+                    }
+                    uint32_t pair = 0;
+                    for (uint32_t h = 0; h < 2; ++h) {
+                        const int32_t v = value(t, 32u * word + part + bit + 16u * h);
+                        const int32_t d0 = two_digits ? ((v + 1024) & 2047) - 1024 : v;
+                        const int32_t x = !odd ? d0 : two_digits ? (v - d0) / 2048 : dominance && t == 1 ? 2 : 1;
+                        pair |= f16_scaled(x, 4 - (int)p) << (16 * h);
+                    }
+                    const uint32_t at = dominance ? r : r % (regs / 2) + r / (regs / 2) * (room / 2);
+                    vf.table[t][set * room * 32u + (at / 4u) * 128u + lane * 4u + at % 4u] = pair;
+                }
+}
+
 // Resource factor of the ecology, same arithmetic as the device finalizer.
 uint32_t factor_q32_host(double R, double R_half) {
     const double den = R + R_half;
@@ -296,6 +351,46 @@ PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap
         L.weights = take(sizeof(WeightParams));
         L.obin = take((size_t)n * 2);
         L.survw = take((size_t)n * 16);
+    }
+    L.total = off;
+    return L;
+}
+
+// Slots of a single population: at most kMaxSlots of whole groups of 32.
+uint32_t slot_length(uint32_t n) { return (uint32_t)(((uint64_t)n + 32ull * kMaxSlots - 1) / (32ull * kMaxSlots)); }
+uint32_t slot_count(uint32_t n) {
+    const uint32_t len = 32u * slot_length(n);
+    return (uint32_t)(((uint64_t)n + len - 1) / len);
+}
+
+// The arena of a single biallelic population (generations.cuh): one buffer
+// of full records, two of packed survivors.
+PopLayout solo_layout_for(uint32_t n, uint32_t words, uint32_t cap, bool weighted) {
+    PopLayout L{};
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off = align_up(off + bytes, 256);
+        return at;
+    };
+    L.solo = true;
+    L.params = take(sizeof(PopParams));
+    L.state = take(sizeof(DevState));
+    L.acc = take(sizeof(StatAcc) * kAccCopies);
+    L.geno0 = L.geno1 = take((size_t)n * 2 * words * 4);
+    for (size_t &x : L.packed) x = take((size_t)n * 2 * words * 4);
+    L.surv0 = L.surv1 = take((size_t)n * 4);
+    L.alive = take(((size_t)n + 31) / 32 * 4);
+    for (size_t &x : L.counts) x = take((size_t)slot_count(n) * 4);
+    L.block_stats = take(sizeof(BlockStats) * 2 * kSoloMaxBlocks);
+    L.barrier = take(sizeof(unsigned long long));
+    L.ring = take((size_t)cap * sizeof(spg_stats));
+    L.frag = take(sizeof(ValueFragments));
+    L.link = take(sizeof(LinkParams));
+    L.weighted = weighted;
+    if (weighted) {
+        L.weights = take(sizeof(WeightParams));
+        for (size_t &x : L.mate) x = take((size_t)n * 8);
     }
     L.total = off;
     return L;
@@ -671,11 +766,24 @@ int view_set_state(const PopView &v, uint32_t gen, uint32_t S, uint32_t f, doubl
                             reinterpret_cast<StatAcc *>(v.base + v.L.acc), gen, S, f, R, status, target, v.stream);
 }
 
+// The slot layout of generation `gen` of a single population from its full
+// records and survivor list (null: everyone).
+int view_pack(const PopView &v, uint32_t gen, const uint32_t *surv, uint32_t S) {
+    const uint32_t par = gen & 1u;
+    return launch_pack(reinterpret_cast<const PopParams *>(v.base + v.L.params), v.words,
+                       reinterpret_cast<const uint32_t *>(v.base + v.L.geno0), surv, S, v.n, slot_length(v.n),
+                       slot_count(v.n), reinterpret_cast<uint32_t *>(v.base + v.L.alive),
+                       reinterpret_cast<uint32_t *>(v.base + v.L.packed[par]),
+                       reinterpret_cast<uint32_t *>(v.base + v.L.counts[par]),
+                       v.L.weighted ? reinterpret_cast<uint2 *>(v.base + v.L.mate[par]) : nullptr, v.stream);
+}
+
 // Enqueue the generation-0 set-up of one population: parameters, counters,
 // founders and state.  `prm` and `init_genotypes` must stay valid until the
 // stream has run the copies (callers synchronise before returning).
 int view_init(const PopView &v, const PopParams &prm, const uint32_t *init_genotypes, uint32_t p0_q32) {
-    cudaError_t e = cudaMemsetAsync(v.base + v.L.buckets, 0, (size_t)2 * v.nbuckets * 4, v.stream);
+    cudaError_t e = v.L.solo ? cudaMemsetAsync(v.base + v.L.barrier, 0, sizeof(unsigned long long), v.stream)
+                             : cudaMemsetAsync(v.base + v.L.buckets, 0, (size_t)2 * v.nbuckets * 4, v.stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(v.base + v.L.ring, 0, (size_t)v.cap * sizeof(spg_stats), v.stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(v.base + v.L.params, &prm, sizeof(PopParams), cudaMemcpyHostToDevice, v.stream);
@@ -699,7 +807,10 @@ int view_init(const PopView &v, const PopParams &prm, const uint32_t *init_genot
                                  v.stream);
         if (rc != SPG_OK) return fail(rc, "dense-parent launch failed");
     }
-    if (v.L.weighted) {  // every founder is a potential parent, in index order
+    if (v.L.solo) {
+        rc = view_pack(v, 0, nullptr, v.n);
+        if (rc != SPG_OK) return fail(rc, "founder packing failed");
+    } else if (v.L.weighted) {  // every founder is a potential parent, in index order
         rc = launch_survivor_bins(reinterpret_cast<const PopParams *>(v.base + v.L.params), v.words, geno0, nullptr,
                                   v.n, v.n, reinterpret_cast<unsigned long long *>(v.base + v.L.survw), v.stream);
         if (rc != SPG_OK) return fail(rc, "survivor-bin launch failed");

@@ -1,0 +1,867 @@
+// The generation kernel of a single population (sm_103a): any number of
+// generations of Fig. 1 A-F in one cooperative launch.
+//
+// Blocks stay for the whole call, so the tables (thresholds, attack rates,
+// effect digits, linkage map) reach shared memory once per call instead of
+// once per launch and generation, and a generation costs one grid barrier.
+//
+// Slots.  The population's groups of 32 offspring are cut into at most
+// kMaxSlots slots of equal length, one per resident warp at large N.  A warp
+// forms its slot's groups in order and packs the survivors' records at the
+// start of the slot's own range, counting them; no other pass touches a
+// record.  Between generations every block turns the slots' counts into a
+// directory in its shared memory: slot s holds the survivors of ranks
+// P[s] .. P[s+1]-1 (index order, as slots are contiguous), at record
+// s * 32 * slot_len + (rank - P[s]).  A parent's rank finds its slot through a
+// guide by the draw's top bits and about a quarter of a step forward.  This replaces
+// a compaction launch that read every child and rewrote the survivors.
+//
+// Full records, the survivor bitmap and the ordered survivor list are only
+// visible between calls, so they are written in a call's last generation
+// (and in one that leaves no survivors: it is formed a second time for them).
+// The per-locus counts read full records, so those are written every
+// generation while counting.
+//
+// Genetic value.  A child's value is a counts x effects product: the warp's 32
+// records go through shared memory into mma.m16n8k16 fragments, each locus as
+// an f16 element.  The two haplotypes' bits of a locus are brought side by
+// side as a 2-bit count (carry-save: x = h0 ^ h1, 2 (h0 & h1)), and a count at
+// bits p, p+1 of a half word IS the f16 number count * 2^(p-24) for p <= 10
+// (subnormals and the first two binades are linear), so a mask makes two
+// elements: no conversion.  The effects (exact f16, |e| <= 2048) are scaled to
+// undo 2^p; every product is a multiple of 2^-20 and the sums stay below 2^22
+// of them: exact in the fp32 accumulators.  Even columns hold the effects for
+// every q, odd columns ones (the allele count), so each lane finds its own
+// offspring's sums without a shuffle; larger effects are two digits of radix
+// 2048 in the even and odd columns.  With dominance the elements are x (value
+// e + d) and h0 & h1 (value 2e) apart.  (e4m3 elements, four to a word, are
+// taken apart into f16 by this target: 2.4 times the instructions.)
+#pragma once
+
+#include "device_common.cuh"
+#include "ecology.cuh"
+
+namespace spg {
+namespace {
+
+// ------------------------------------------------------- shared memory
+constexpr int kGuideBits = 13;  // the parent draw's top bits that index the guide
+constexpr uint32_t kGuide = 1u << kGuideBits;
+
+template <int W, bool LINKED, int BLOCK>
+struct GenSmem {
+    static constexpr uint32_t NW = BLOCK / 32;
+    static constexpr uint32_t kPlanes = W <= 2 ? 1u : (uint32_t)W / 2u;  // 16-byte planes of a staged record
+    static constexpr uint32_t kSets = W == 8 ? 2u : 1u;                  // word sets of the value fragments
+    static constexpr uint32_t kRegs = W >= 4 ? 16u : 4u * W;             // element pairs of a lane, row and set
+    static constexpr uint32_t kRegRoom = kRegs < 8u ? 8u : kRegs;        // places for them (even loci, odd loci)
+    static constexpr uint32_t kThr = 0u, kAtt = kThr + kBins * 4u, kDir = kAtt + kBins * 4u;
+    static constexpr uint32_t kGuideOff = kDir + kMaxSlots * 8u;
+    static constexpr uint32_t kFrag = kGuideOff + kGuide * 2u;           // [table][set][kRegRoom / 4][32][4]
+    static constexpr uint32_t kSetBytes = kRegRoom * 128u, kTabBytes = kSets * kSetBytes;
+    static constexpr uint32_t kStage = kFrag + 2u * kTabBytes;
+    static constexpr uint32_t kRecStage = kPlanes * 512u;
+    static constexpr uint32_t kTog = LINKED ? 2u * 32u * ((uint32_t)W + 3u) * 4u : 0u;
+    static constexpr uint32_t kPerWarp = kRecStage > kTog ? kRecStage : (kTog + 15u) / 16u * 16u;
+    static constexpr uint32_t kLinkOff = kStage + NW * kPerWarp;
+    // linkage map: cdf, cum, guide, chrom, first, clast
+    static constexpr uint32_t kLinkBytes = LINKED ? kMaxKmax * 4u + kMaxLoci * 4u + kLinkGuide * 4u + kMaxLoci + kMaxChrom * 4u : 0u;
+    static constexpr uint32_t kThreads = BLOCK;
+    static constexpr uint32_t kStats = (kLinkOff + kLinkBytes + 15u) / 16u * 16u;  // lanes' statistics, 48 bytes each
+    static constexpr uint32_t kBytes = kStats + 48u * BLOCK;
+};
+
+extern __shared__ __align__(128) unsigned char g_smem[];
+
+__device__ __forceinline__ uint32_t sm_u32(uint32_t off) { return *reinterpret_cast<const uint32_t *>(g_smem + off); }
+
+// ------------------------------------------------------- grid barrier
+// All blocks of the (cooperative) grid arrive and wait; false when the wait
+// ran out.  The counter only grows, by gridDim.x per barrier.  (Every block
+// polling a word of every other took 5 us instead of 2 with 152 blocks.)
+constexpr uint32_t kBarrierTries = 1u << 23;  // polls of about half a microsecond before a wait gives up
+
+__device__ __forceinline__ bool grid_barrier(unsigned long long *ctr) {
+    __syncthreads();
+    int ok = 1;
+    if (threadIdx.x == 0) {
+        const unsigned long long G = gridDim.x;
+        unsigned long long old, v = 0;
+        asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;" : "=l"(old) : "l"(ctr) : "memory");
+        const unsigned long long want = (old / G + 1ull) * G;
+        for (uint32_t i = 0; i < kBarrierTries && v < want; ++i)
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        ok = v >= want ? 1 : 0;
+    }
+    return __syncthreads_and(threadIdx.x == 0 ? ok : 1) != 0;
+}
+
+// ------------------------------------------------------- record access
+// Parents are read through L2: their buffers change during the launch.
+template <int W>
+__device__ __forceinline__ void load_packed(const uint32_t *p, uint32_t (&r)[2 * W]) {
+    if constexpr (W == 1) {
+        asm volatile("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "l"(p) : "memory");
+    } else if constexpr (W == 2) {
+        asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "l"(p) : "memory");
+    } else {
+#pragma unroll
+        for (int q = 0; q < W / 4; ++q)
+            asm volatile("ld.global.cg.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(r[8 * q]), "=r"(r[8 * q + 1]), "=r"(r[8 * q + 2]), "=r"(r[8 * q + 3]),
+                           "=r"(r[8 * q + 4]), "=r"(r[8 * q + 5]), "=r"(r[8 * q + 6]), "=r"(r[8 * q + 7])
+                         : "l"(p + 8 * q) : "memory");
+    }
+}
+
+// ------------------------------------------------------- genetic value
+// A warp's staged records: lane l = 4g + q holds row 8q + g, at position
+// 8q + (g + 2q) % 8 of each 16-byte plane, so both the lanes' stores (any
+// eight consecutive lanes) and ldmatrix (the eight rows of a matrix) touch
+// all banks once.
+__device__ __forceinline__ uint32_t stage_row(uint32_t lane) {
+    const uint32_t g = lane >> 2, q = lane & 3u;
+    return 16u * (8u * q + ((g + 2u * q) & 7u));
+}
+__device__ __forceinline__ uint32_t matrix_row(uint32_t lane) {  // ldmatrix: the row lane supplies the address of
+    const uint32_t i = lane & 7u, q = lane >> 3;
+    return 16u * (8u * q + ((i + 2u * q) & 7u));
+}
+
+template <int W>
+__device__ __forceinline__ void stage_record(uint32_t addr, const uint32_t (&c)[2 * W]) {
+    if constexpr (W == 1) {  // twice: every lane of a row's four finds one haplotype
+        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %1, %2};" ::"r"(addr), "r"(c[0]), "r"(c[1]) : "memory");
+    } else {
+#pragma unroll
+        for (int p = 0; p < W / 2; ++p)
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr + 512u * p), "r"(c[4 * p]),
+                         "r"(c[4 * p + 1]), "r"(c[4 * p + 2]), "r"(c[4 * p + 3]) : "memory");
+    }
+}
+template <int W>
+__device__ __forceinline__ void unstage_record(uint32_t addr, uint32_t (&c)[2 * W]) {
+    if constexpr (W == 1) {
+        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(c[0]), "=r"(c[1]) : "r"(addr) : "memory");
+    } else {
+#pragma unroll
+        for (int p = 0; p < W / 2; ++p)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(c[4 * p]), "=r"(c[4 * p + 1]), "=r"(c[4 * p + 2]), "=r"(c[4 * p + 3])
+                         : "r"(addr + 512u * p) : "memory");
+    }
+}
+
+// Words of a plane in fragment order: x[i] is word q of row 8i + g.
+__device__ __forceinline__ void load_plane(uint32_t addr, uint32_t (&x)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(addr) : "memory");
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                        uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// N element pairs of every row (x: the four rows' words) from bit positions
+// 0, STEP, 2 STEP, ... of both half words times their fragments.  Positions
+// past the linear range come down by shifting the word (STEP 2: the seventh
+// and eighth by 4, STEP 1: from the twelfth on by 5).
+template <int N, int STEP>
+__device__ __forceinline__ void add_elements(float (&c0)[4], float (&c1)[4], const uint32_t (&x)[4], uint32_t frag) {
+    constexpr int LIN = STEP == 2 ? 6 : 11, SHIFT = STEP == 2 ? 4 : 5;
+    constexpr uint32_t ONE = STEP == 2 ? 0x00030003u : 0x00010001u;
+    uint32_t b[4];
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+        if (i % 4 == 0)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]) : "r"(frag + 128u * i) : "memory");
+        uint32_t e[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = i + h;
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                e[h][r] = (k < LIN ? x[r] : x[r] >> SHIFT) & (ONE << (k < LIN ? STEP * k : STEP * k - SHIFT));
+        }
+        mma_f16(c0, e[0][0], e[0][1], e[1][0], e[1][1], b[i % 4], b[i % 4 + 1]);
+        mma_f16(c1, e[0][2], e[0][3], e[1][2], e[1][3], b[i % 4], b[i % 4 + 1]);
+    }
+}
+
+// Genetic value and allele count of the lane's own staged record.  frag: the
+// shared address of the value fragments.
+template <int W, class SM>
+__device__ __forceinline__ void staged_value(uint32_t planes, uint32_t lane, uint32_t frag, bool dom, bool two_digits,
+                                             int32_t &raw, uint32_t &allele) {
+    const uint32_t at = planes + matrix_row(lane);
+    const uint32_t sh = W >= 4 ? 0u : W == 2 ? 8u * ((lane >> 1) & 1u) : 4u * (lane & 3u);  // the lane's part of a word
+    float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int s = 0; s < (int)SM::kSets; ++s) {
+        uint32_t x[4], y[4];
+        load_plane(at + 512u * s, x);
+        if constexpr (W <= 2) {  // the other haplotype's word sits in the lane W away
+#pragma unroll
+            for (int i = 0; i < 4; ++i) y[i] = __shfl_xor_sync(0xFFFFFFFFu, x[i], W);
+        } else {
+            load_plane(at + 512u * (s + (int)SM::kSets), y);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {  // x: heterozygous loci, y: homozygous for allele 1
+            const uint32_t t = x[i] ^ y[i];
+            y[i] &= x[i];
+            x[i] = t;
+        }
+        const uint32_t f0 = frag + s * SM::kSetBytes + 16u * lane;
+        if (!dom) {
+            constexpr uint32_t EVEN = 0x55555555u;
+            constexpr int N = (int)SM::kRegs / 2;
+            uint32_t z[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) z[i] = ((x[i] & EVEN) | ((y[i] << 1) & ~EVEN)) >> sh;
+            add_elements<N, 2>(c0, c1, z, f0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) z[i] = (((x[i] >> 1) & EVEN) | (y[i] & ~EVEN)) >> sh;
+            add_elements<N, 2>(c0, c1, z, f0 + SM::kSetBytes / 2u);
+        } else {
+            if constexpr (W < 4) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    x[i] >>= sh;
+                    y[i] >>= sh;
+                }
+            }
+            add_elements<(int)SM::kRegs, 1>(c0, c1, x, f0);
+            add_elements<(int)SM::kRegs, 1>(c0, c1, y, f0 + SM::kTabBytes);
+        }
+    }
+    // this lane's row: 8q + g is row g or g + 8 of tile q / 2
+    const bool up = (lane & 1u) != 0u, second = (lane & 2u) != 0u;
+    const float lo = second ? (up ? c1[2] : c1[0]) : (up ? c0[2] : c0[0]);
+    const float hi = second ? (up ? c1[3] : c1[1]) : (up ? c0[3] : c0[1]);
+    // a sum * 2^20 is a whole number below 2^22: read it off the mantissa
+    constexpr float kScale = 1048576.f, kMagic = 12582912.f;
+    raw = __float_as_int(fmaf(lo, kScale, kMagic)) - 0x4B400000;
+    const int32_t odd = __float_as_int(fmaf(hi, kScale, kMagic)) - 0x4B400000;
+    allele = (uint32_t)odd;
+    if (two_digits) raw += odd * 2048;
+}
+
+// Flip K distinct uniformly drawn positions of the lane's staged record
+// (per-locus mutation; the draws of mutate()).  Rare, so kept out of line: it
+// would cost every offspring the registers of its bookkeeping.
+__device__ __noinline__ void mutate_staged(uint32_t row, uint32_t copies, uint32_t k, uint32_t j, uint32_t g,
+                                           uint32_t rep, uint32_t k0, uint32_t k1) {
+    uint16_t taken[kMaxKmax];
+    uint32_t chosen = 0;
+    k = min(k, (uint32_t)kMaxKmax);
+    for (uint32_t a4 = 0; a4 < kMutDraws / 4 && chosen < k; ++a4) {
+        const uint4 d = philox(make_uint4(j, g, rep, (kMutPos << 24) | a4), k0, k1);
+        for (int l = 0; l < 4 && chosen < k; ++l) {
+            const uint32_t pos = __umulhi(lane_of(d, l), copies);  // [0, 2L)
+            bool dup = false;
+            for (uint32_t i = 0; i < chosen; ++i) dup |= taken[i] == pos;
+            if (!dup) {
+                taken[chosen++] = (uint16_t)pos;
+                const uint32_t w = pos >> 5, at = row + 512u * (w >> 2) + 4u * (w & 3u);
+                uint32_t v;
+                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(at), "r"(v ^ (1u << (pos & 31u))) : "memory");
+            }
+        }
+    }
+}
+
+// ------------------------------------------------------- Philox
+// Philox4x32-10 (see device_common.cuh) at counters (j, g, rep, word): the
+// round keys come from the kernel's parameters, and what the first two rounds
+// share is made once -- A * j per offspring, the rest (g, rep) per generation.
+struct GenRng {
+    uint32_t hx, lx;  // product of A and word 0 after round 0 (hx with round 1's key)
+};
+constexpr uint32_t kPhA = 0xD2511F53u, kPhB = 0xCD9E8D57u;
+__device__ __forceinline__ GenRng gen_rng(const SoloArgs &a, uint32_t g) {
+    const uint32_t x1 = (uint32_t)(((unsigned long long)kPhB * a.rep) >> 32) ^ g ^ a.keys[0];
+    const unsigned long long p = (unsigned long long)kPhA * x1;
+    return GenRng{(uint32_t)(p >> 32) ^ a.keys[3], (uint32_t)p};
+}
+__device__ __forceinline__ uint4 philox_at(const SoloArgs &a, const GenRng &r, unsigned long long aj, uint32_t word) {
+    unsigned long long p1 = (unsigned long long)kPhB * ((uint32_t)(aj >> 32) ^ word ^ a.keys[1]), p0;
+    uint4 c = make_uint4((uint32_t)(p1 >> 32) ^ (kPhB * a.rep) ^ a.keys[2], (uint32_t)p1, r.hx ^ (uint32_t)aj, r.lx);
+#pragma unroll
+    for (int i = 2; i < 10; ++i) {
+        p0 = (unsigned long long)kPhA * c.x;
+        p1 = (unsigned long long)kPhB * c.z;
+        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ a.keys[2 * i], (uint32_t)p1,
+                       (uint32_t)(p0 >> 32) ^ c.w ^ a.keys[2 * i + 1], (uint32_t)p0);
+    }
+    return c;
+}
+
+// ------------------------------------------------------- parents
+// Record of the survivor drawn by u (rank u * S / 2^32) in the slot layout.
+// one_step: no guide entry is more than one slot behind (build_directory), so
+// the search is a select.
+template <class SM>
+__device__ __forceinline__ uint32_t locate(uint32_t u, uint32_t S, bool one_step, uint32_t rec_slot) {
+    const uint32_t r = __umulhi(u, S);
+    uint32_t s = *reinterpret_cast<const uint16_t *>(g_smem + SM::kGuideOff + 2u * (u >> (32 - kGuideBits)));
+    uint2 e = *reinterpret_cast<const uint2 *>(g_smem + SM::kDir + 8u * s);
+    if (one_step) return r < e.x ? r + e.y : r - e.x + (s + 1u) * rec_slot;
+    while (e.x <= r) {  // the last slot's end is S > r
+        ++s;
+        e = *reinterpret_cast<const uint2 *>(g_smem + SM::kDir + 8u * s);
+    }
+    return r + e.y;
+}
+
+// Weighted parents (bounded rejection, see offspring.cuh): proposals in
+// pairs, both roles together; thr holds each survivor's thresholds as mother
+// and as father at its record's place.
+template <class SM>
+__device__ __forceinline__ void weighted_records(const SoloArgs &a, const uint2 *thr, const GenRng &rng,
+                                                 unsigned long long aj, uint32_t S, bool one_step,
+                                                 uint32_t rec_slot, uint32_t &mom,
+                                                 uint32_t &dad) {
+    bool open_m = true, open_f = true;
+    for (uint32_t k = 0; k < kMateAttempts && (open_m || open_f); k += 2) {
+        const uint32_t sub = (kMateW << 24) | (k >> 1);
+        uint4 dm = make_uint4(0u, 0u, 0u, 0u), df = dm;
+        uint32_t rm0 = 0, rm1 = 0, rf0 = 0, rf1 = 0, tm0 = 0, tm1 = 0, tf0 = 0, tf1 = 0;
+        if (open_m) {
+            dm = philox_at(a, rng, aj, sub);
+            rm0 = locate<SM>(dm.x, S, one_step, rec_slot);
+            rm1 = locate<SM>(dm.z, S, one_step, rec_slot);
+            tm0 = __ldcg(&thr[rm0].x);
+            tm1 = __ldcg(&thr[rm1].x);
+        }
+        if (open_f) {
+            df = philox_at(a, rng, aj, sub | (1u << 8));
+            rf0 = locate<SM>(df.x, S, one_step, rec_slot);
+            rf1 = locate<SM>(df.z, S, one_step, rec_slot);
+            tf0 = __ldcg(&thr[rf0].y);
+            tf1 = __ldcg(&thr[rf1].y);
+        }
+        if (open_m) {
+            const bool a0 = tm0 == kCertain || dm.y < tm0, a1 = tm1 == kCertain || dm.w < tm1;
+            mom = a0 ? rm0 : rm1;
+            open_m = !(a0 || a1);
+        }
+        if (open_f) {
+            const bool a0 = tf0 == kCertain || df.y < tf0, a1 = tf1 == kCertain || df.w < tf1;
+            dad = a0 ? rf0 : rf1;
+            open_f = !(a0 || a1);
+        }
+    }
+}
+
+// ------------------------------------------------------- the directory
+// Exclusive scan of the slots' survivor counts into the block's directory and
+// guide (all threads; returns the total, the same in every thread).  Slot s
+// holds ranks P[s] .. P[s+1]-1; entry s is {P[s+1], s * slot_records - P[s]}.
+// Guide entry h is a slot at or just before the one of the smallest rank drawn
+// by a u whose top bits are h, rank floor(h S / kGuide): slot s enters the
+// guide at the first h surely past kGuide P[s] / S.  Every block does this
+// every generation, so it takes a handful of instructions a slot (exact
+// entries by 64-bit products took a sixth of a generation at N = 10^6).
+// With no survivors the tables stay as they are.
+// one_step: whether every slot holds more ranks than a guide entry spans, so
+// that a rank lies in its entry's slot or the next.
+// The counts are loaded apart (load_counts), so that a caller can have them on
+// their way while it does something else.
+template <int BLOCK>
+struct SlotCounts {
+    static constexpr uint32_t PER = (kMaxSlots + BLOCK - 1) / BLOCK;
+    uint32_t c[PER];  // slots tid * per .. tid * per + per - 1, per = nslots / BLOCK rounded up
+};
+template <int BLOCK>
+__device__ __forceinline__ void load_counts(const uint32_t *counts, uint32_t nslots, SlotCounts<BLOCK> &sc) {
+    const uint32_t per = (nslots + BLOCK - 1) / BLOCK, s0 = threadIdx.x * per;
+#pragma unroll
+    for (uint32_t i = 0; i < SlotCounts<BLOCK>::PER; ++i)
+        sc.c[i] = i < per && s0 + i < nslots ? __ldcg(counts + s0 + i) : 0u;
+}
+template <class SM, int BLOCK>
+__device__ __forceinline__ uint32_t build_directory(const SlotCounts<BLOCK> &sc, uint32_t nslots, uint32_t slot_records,
+                                                    uint32_t *s_warp, bool &one_step) {
+    constexpr uint32_t NW = BLOCK / 32, PER = SlotCounts<BLOCK>::PER;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t per = (nslots + BLOCK - 1) / BLOCK, s0 = tid * per;
+    const uint32_t(&c)[PER] = sc.c;
+    uint32_t own = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < PER; ++i) own += c[i];
+    uint32_t incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if ((int)lane >= o) incl += y;
+    }
+    __syncthreads();  // s_warp is free, and the previous directory no longer read
+    if (lane == 31u) s_warp[warp] = incl;
+    __syncthreads();
+    const uint32_t w = lane < NW ? s_warp[lane] : 0u;
+    const uint32_t S = __reduce_add_sync(0xFFFFFFFFu, w);
+    if (S == 0u) return 0u;
+    uint32_t P = incl - own + __reduce_add_sync(0xFFFFFFFFu, lane < warp ? w : 0u);
+    // the first h with floor(h S / kGuide) >= P, or one later when the float
+    // quotient (off by less than 0.004) is too close to tell
+    const float inv = (float)kGuide / (float)S;
+    const uint32_t span = 2u * (S >> kGuideBits) + 2u;  // ranks of two entries, at most
+    bool wide = true;
+    auto entry_of = [&](uint32_t p) { return p ? min((uint32_t)fmaf((float)p, inv, 1.005f), kGuide) : 0u; };
+    uint32_t h = entry_of(P);
+#pragma unroll
+    for (uint32_t i = 0; i < PER; ++i) {
+        const uint32_t s = s0 + i, end = P + c[i];
+        if (i < per && s < nslots) {
+            *reinterpret_cast<uint2 *>(g_smem + SM::kDir + 8u * s) = make_uint2(end, s * slot_records - P);
+            for (const uint32_t hn = entry_of(end); h < hn; ++h)
+                *reinterpret_cast<uint16_t *>(g_smem + SM::kGuideOff + 2u * h) = (uint16_t)s;
+            wide = wide && c[i] > span;
+            P = end;
+        }
+    }
+    one_step = __syncthreads_and(wide) != 0;
+    return S;
+}
+
+// ------------------------------------------------------- per-locus counts
+// Allele copies of the block's own records [j0, j1), added to the generation's
+// row: bit-sliced counters per lane (plane k holds bit k of every locus's count
+// among the lane's records), transposed across the warp before they could
+// overflow (see k_locus_counts).  Four record words at a time.
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, uint32_t lane) {
+    constexpr uint32_t M[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const uint32_t s = 16u >> k;
+        const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, (int)s);
+        x = (lane & s) ? (((y >> s) & M[k]) | (x & ~M[k])) : ((x & M[k]) | ((y << s) & ~M[k]));
+    }
+    return x;
+}
+template <int W, int BLOCK>
+__device__ __forceinline__ void count_loci(const uint32_t *geno, uint32_t j0, uint32_t j1, uint32_t *s_cnt,
+                                           uint32_t *row) {
+    constexpr uint32_t L = 32u * W, NW = BLOCK / 32;
+    constexpr int C = W == 1 ? 2 : 4, K = kLocusPlanes;  // words of one pass
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    for (uint32_t i = tid; i < L; i += BLOCK) s_cnt[i] = 0u;
+    __syncthreads();  // and the block's records are written
+#pragma unroll 1
+    for (int p = 0; p < 2 * W / C; ++p) {
+        uint32_t v[C][K], held = 0;
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+#pragma unroll
+            for (int k = 0; k < K; ++k) v[c][k] = 0u;
+        auto flush = [&]() {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                uint32_t sum = 0;
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    sum += (uint32_t)__popc(transpose32(v[c][k], lane)) << k;
+                    v[c][k] = 0u;
+                }
+                atomicAdd(&s_cnt[32u * (uint32_t)((p * C + c) % W) + lane], sum);
+            }
+            held = 0;
+        };
+        for (uint32_t j = j0 + 32u * warp; j < j1; j += 32u * NW) {
+            uint32_t x[C];
+            const uint32_t *src = geno + (size_t)(j + lane) * (2 * W) + C * p;
+            if (j + lane < j1) {
+                if constexpr (C == 2) {
+                    const uint2 u = __ldcg(reinterpret_cast<const uint2 *>(src));
+                    x[0] = u.x;
+                    x[1] = u.y;
+                } else {
+                    const uint4 u = __ldcg(reinterpret_cast<const uint4 *>(src));
+                    x[0] = u.x;
+                    x[1] = u.y;
+                    x[2] = u.z;
+                    x[3] = u.w;
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < C; ++c) x[c] = 0u;
+            }
+#pragma unroll
+            for (int c = 0; c < C; ++c) {  // ripple-carry add of one bit per locus
+                uint32_t carry = x[c];
+#pragma unroll
+                for (int k = 0; k < K - 1; ++k) {
+                    const uint32_t t = v[c][k] & carry;
+                    v[c][k] ^= carry;
+                    carry = t;
+                }
+                v[c][K - 1] ^= carry;
+            }
+            if (++held == (1u << K) - 1u) flush();
+        }
+        if (held) flush();
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < L; i += BLOCK)
+        if (s_cnt[i]) atomicAdd(row + i, s_cnt[i]);
+}
+
+// ------------------------------------------------------- the kernel
+// A lane's statistics of one generation, and their exact sums over the block:
+// every lane leaves its own in shared memory, and after a block barrier warp k
+// takes field k (a reduction in every warp took three times as long).
+struct LaneStats {
+    long long sum_raw = 0, sum_raw_s = 0;
+    unsigned long long sum_raw2 = 0, cons = 0;
+    uint32_t het = 0, allele = 0;
+    int mn = INT_MAX, mx = INT_MIN;
+};
+template <class SM>
+__device__ __forceinline__ void put_stats(const LaneStats &ts, uint32_t tid) {
+    unsigned long long *s64 = reinterpret_cast<unsigned long long *>(g_smem + SM::kStats) + tid;
+    s64[0] = (unsigned long long)ts.sum_raw;
+    s64[SM::kThreads] = (unsigned long long)ts.sum_raw_s;
+    s64[2 * SM::kThreads] = ts.sum_raw2;
+    s64[3 * SM::kThreads] = ts.cons;
+    uint32_t *s32 = reinterpret_cast<uint32_t *>(g_smem + SM::kStats + 32u * SM::kThreads) + tid;
+    s32[0] = ts.het;
+    s32[SM::kThreads] = ts.allele;
+    s32[2 * SM::kThreads] = (uint32_t)ts.mn;
+    s32[3 * SM::kThreads] = (uint32_t)ts.mx;
+}
+template <class SM>
+__device__ __forceinline__ void block_stats(BlockStats *out, uint32_t warp, uint32_t lane) {
+    if (warp >= 8u) return;
+    if (warp < 6u) {
+        unsigned long long x = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < SM::NW; ++i)
+            x += warp < 4u ? *reinterpret_cast<const unsigned long long *>(g_smem + SM::kStats +
+                                                                           8u * (warp * SM::kThreads + 32u * i + lane))
+                           : sm_u32(SM::kStats + 32u * SM::kThreads + 4u * ((warp - 4u) * SM::kThreads + 32u * i + lane));
+        x = warp_sum_u64(x);  // modulo 2^64: signed sums too
+        if (lane == 0u) out->sum[warp] = x;
+    } else {
+        int x = warp == 6u ? INT_MAX : INT_MIN;
+#pragma unroll
+        for (uint32_t i = 0; i < SM::NW; ++i) {
+            const int y = (int)sm_u32(SM::kStats + 32u * SM::kThreads + 4u * ((warp - 4u) * SM::kThreads + 32u * i + lane));
+            x = warp == 6u ? min(x, y) : max(x, y);
+        }
+        x = warp == 6u ? __reduce_min_sync(0xFFFFFFFFu, x) : __reduce_max_sync(0xFFFFFFFFu, x);
+        if (lane == 0u) (warp == 6u ? out->mn : out->mx) = x;
+    }
+}
+
+template <int W, bool LINKED, bool WEIGHTED>
+__global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_constant__ SoloArgs a) {
+    constexpr int BLOCK = kSoloThreads;
+    using SM = GenSmem<W, LINKED, BLOCK>;
+    constexpr uint32_t NW = BLOCK / 32;
+    __shared__ uint32_t s_cdf[kMaxKmax];
+    __shared__ uint32_t s_scan[32];
+    __shared__ unsigned long long s_sum[6];  // block 0: sum_raw, sum_raw_s, sum_raw2, cons, het, allele
+    __shared__ int s_mm[2];
+    __shared__ uint32_t s_cnt[32 * W];
+    __shared__ double s_R;
+    __shared__ uint32_t s_f;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(g_smem);
+    const PopParams *P = a.prm;
+    DevState *st = a.state;
+
+    // the call's starting state (written by earlier launches)
+    uint32_t gen = ld_relaxed_u32(&st->gen), f = ld_relaxed_u32(&st->f);
+    const uint32_t target = ld_relaxed_u32(&st->target);
+    int32_t status = (int32_t)ld_relaxed_u32(reinterpret_cast<const uint32_t *>(&st->status));
+    double R = ld_relaxed_f64(&st->R);
+    if (status != SPG_OK || ld_relaxed_u32(&st->S) == 0u) return;
+
+    // tables
+    const bool eco = a.has_eco != 0u, dom = a.dom != 0u;
+    for (uint32_t i = tid; i < (uint32_t)kBins / 4u; i += BLOCK) {
+        cp_async_16(smem0 + SM::kThr + 16u * i, P->table + 4u * i);
+        if (eco) cp_async_16(smem0 + SM::kAtt + 16u * i, P->attack + 4u * i);
+    }
+    for (uint32_t i = tid; i < SM::kTabBytes / 16u; i += BLOCK) {
+        cp_async_16(smem0 + SM::kFrag + 16u * i, a.frag->table[0] + 4u * i);
+        if (dom) cp_async_16(smem0 + SM::kFrag + SM::kTabBytes + 16u * i, a.frag->table[1] + 4u * i);
+    }
+    cp_async_commit();
+    if (tid < (uint32_t)kMaxKmax) s_cdf[tid] = tid < a.kmax ? P->cdf[tid] : 0xFFFFFFFFu;
+    LinkSmem lk{};
+    if constexpr (LINKED) {
+        const LinkParams *lp = P->link;
+        uint32_t *cdf = reinterpret_cast<uint32_t *>(g_smem + SM::kLinkOff), *cum = cdf + kMaxKmax, *gd = cum + kMaxLoci;
+        uint16_t *first = reinterpret_cast<uint16_t *>(gd + kLinkGuide), *clast = first + kMaxChrom;
+        uint8_t *chrom = reinterpret_cast<uint8_t *>(clast + kMaxChrom);
+        if (tid < (uint32_t)kMaxKmax) cdf[tid] = lp->cdf[tid];
+        for (uint32_t i = tid; i < 32u * W; i += BLOCK) {
+            cum[i] = lp->cum[i];
+            chrom[i] = lp->chrom[i];
+        }
+        for (uint32_t i = tid; i < (uint32_t)kLinkGuide; i += BLOCK) gd[i] = lp->guide[i];
+        if (tid < (uint32_t)kMaxChrom) {
+            first[tid] = lp->first[tid];
+            clast[tid] = lp->clast[tid];
+        }
+        lk = LinkSmem{cdf, cum, chrom, first, clast, gd, lp->kmax, lp->nchrom, nullptr};
+    }
+    const uint32_t rep = a.rep, k0 = a.keys[0], k1 = a.keys[1];
+    const uint32_t rec_slot = a.slot_len * 32u;
+    const uint32_t stage = smem0 + SM::kStage + warp * SM::kPerWarp, my_row = stage + stage_row(lane);
+    if constexpr (LINKED) lk.tog = reinterpret_cast<uint32_t *>(g_smem + SM::kStage + warp * SM::kPerWarp) -
+                                   warp * (2u * 32u * ((uint32_t)W + 3u));  // the helper adds its warp's offset
+    const uint32_t slot0 = (uint32_t)(((unsigned long long)a.nslots * blockIdx.x) / gridDim.x);
+    const uint32_t slot1 = (uint32_t)(((unsigned long long)a.nslots * (blockIdx.x + 1u)) / gridDim.x);
+    cp_async_wait<0>();
+    bool one_step = false;
+    SlotCounts<BLOCK> sc;
+    load_counts<BLOCK>(a.counts[gen & 1u], a.nslots, sc);
+    uint32_t S = build_directory<SM, BLOCK>(sc, a.nslots, rec_slot, s_scan, one_step);
+
+    bool again = false;  // a generation without survivors formed once more for its full records
+    for (uint32_t done = 0; done < a.n_gen && (gen < target || again);) {
+        const uint32_t g = again ? gen : gen + 1u;
+        const bool list = again || (a.keep_last && done + 1u == a.n_gen) || g == target;
+        const bool full = list || a.locus_row[0] != nullptr;
+        const uint32_t *par = a.packed[(g + 1u) & 1u];
+        uint32_t *out = a.packed[g & 1u];
+        const GenRng rng = gen_rng(a, g);
+        if (eco && tid == BLOCK - 32u)  // the resource before consumption, while the generation is formed
+            s_R = a.eco_model == 1u
+                      ? resource_grown_bh(R, growth_rate(a.eco_r, a.eco_r_sd, g, rep, k0, k1), a.eco_K)
+                      : resource_grown(R, a.eco_r, a.eco_K);
+        LaneStats ts;
+        for (uint32_t slot = slot0 + warp; slot < slot1; slot += NW) {
+            const uint32_t base = slot * rec_slot, end = min(base + rec_slot, a.n);
+            uint32_t at0 = base;  // where the next survivor goes
+            // (A) a group's mate draw and parents; the next group's records are
+            // on their way while a group is formed
+            auto draw = [&](uint32_t j, uint4 &r, uint32_t (&pm)[2 * W], uint32_t (&pf)[2 * W]) {
+                const unsigned long long aj = (unsigned long long)kPhA * j;
+                r = philox_at(a, rng, aj, kMate << 24);
+                uint32_t mom, dad;
+                if constexpr (WEIGHTED) {
+                    weighted_records<SM>(a, a.mate[(g + 1u) & 1u], rng, aj, S, one_step, rec_slot, mom, dad);
+                } else {
+                    mom = locate<SM>(r.x, S, one_step, rec_slot);
+                    dad = locate<SM>(r.y, S, one_step, rec_slot);
+                }
+                load_packed<W>(par + (size_t)mom * (2 * W), pm);
+                load_packed<W>(par + (size_t)dad * (2 * W), pf);
+            };
+            uint4 r_next;
+            uint32_t pm_next[2 * W], pf_next[2 * W];
+            draw(base + lane, r_next, pm_next, pf_next);
+#pragma unroll 1
+            for (uint32_t j0 = base; j0 < end; j0 += 32u) {
+                const uint32_t j = j0 + lane;
+                const bool valid = j < a.n;
+                const uint4 r = r_next;
+                // (B) gametes: the mask streams, or the linkage map's masks
+                uint32_t ch[2 * W];
+                if constexpr (LINKED) {
+                    uint32_t mm[W], mf[W];
+                    linked_masks_warp<W>(lk, j, valid, g, rep, k0, k1, mm, mf);
+                    __syncwarp();  // the toggles' memory holds the staged records next
+#pragma unroll
+                    for (int w = 0; w < W; ++w) {
+                        ch[w] = (pm_next[w] & ~mm[w]) | (pm_next[W + w] & mm[w]);
+                        ch[W + w] = (pf_next[w] & ~mf[w]) | (pf_next[W + w] & mf[w]);
+                    }
+                } else {
+                    const unsigned long long aj = (unsigned long long)kPhA * j;
+#pragma unroll
+                    for (int q4 = 0; q4 < (2 * W + 3) / 4; ++q4) {
+                        const uint4 d = philox_at(a, rng, aj, (kRecomb << 24) | (uint32_t)q4);
+                        const int w = 2 * q4;
+                        ch[w] = (pm_next[w] & ~d.x) | (pm_next[W + w] & d.x);
+                        ch[W + w] = (pf_next[w] & ~d.y) | (pf_next[W + w] & d.y);
+                        if constexpr (W > 1) {
+                            ch[w + 1] = (pm_next[w + 1] & ~d.z) | (pm_next[W + w + 1] & d.z);
+                            ch[W + w + 1] = (pf_next[w + 1] & ~d.w) | (pf_next[W + w + 1] & d.w);
+                        }
+                    }
+                }
+                if (j0 + 32u < end) draw(j + 32u, r_next, pm_next, pf_next);
+                stage_record<W>(my_row, ch);
+                if (r.w >= a.mut_from) {  // (B) mutations, on the staged record
+                    uint32_t k = 0;
+                    for (uint32_t i = 0; i < a.kmax; ++i) k += (r.w >= s_cdf[i]) ? 1u : 0u;
+                    mutate_staged(my_row, 64u * W, k, j, g, rep, k0, k1);
+                    unstage_record<W>(my_row, ch);
+                    if constexpr (W == 1) stage_record<W>(my_row, ch);
+                }
+                __syncwarp();
+                // (C) genetic value
+                int32_t raw;
+                uint32_t allele, het = 0;
+                staged_value<W, SM>(stage, lane, smem0 + SM::kFrag, dom, a.two_digits != 0u, raw, allele);
+#pragma unroll
+                for (int w = 0; w < W; ++w) het += __popc(ch[w] ^ ch[W + w]);
+                if (a.two_digits) {
+                    allele = 0;
+#pragma unroll
+                    for (int w = 0; w < 2 * W; ++w) allele += __popc(ch[w]);
+                }
+                // (D) survival: the bin's threshold scaled by the resource factor
+                uint32_t bin;
+                if (a.narrow_bias) {  // raw + bias stays inside 32 bits
+                    bin = (uint32_t)min(max((raw + a.bias) >> a.shift, 0), kBins - 1);
+                } else {
+                    const long long v = (long long)raw + (long long)a.bias;
+                    bin = v < 0 ? 0u : (uint32_t)min(v >> a.shift, (long long)(kBins - 1));
+                }
+                uint32_t thr = sm_u32(SM::kThr + bin * 4u);
+                if (f != kCertain) thr = __umulhi(thr, f);
+                const bool alive = valid && min(r.z, kCertain - 1u) < thr;  // kCertain: whatever the draw
+                const uint32_t bits = __ballot_sync(0xFFFFFFFFu, alive);
+                // (E) the survivor's record at its place in the slot
+                const uint32_t at = at0 + __popc(bits & ((1u << lane) - 1u));
+                at0 += __popc(bits);
+                if (alive) {
+                    store_record<W>(out + (size_t)at * (2 * W), ch);
+                    if constexpr (WEIGHTED) {
+                        const WeightParams *wt = P->weights;
+                        a.mate[g & 1u][at] = make_uint2(__ldg(&wt->acc[0][bin]), __ldg(&wt->acc[1][bin]));
+                    }
+                    ts.sum_raw_s += raw;
+                    if (eco) ts.cons += sm_u32(SM::kAtt + bin * 4u);
+                }
+                if (valid) {
+                    ts.het += het;
+                    ts.allele += allele;
+                    ts.sum_raw += raw;
+                    ts.sum_raw2 += (unsigned long long)((long long)raw * (long long)raw);
+                    ts.mn = min(ts.mn, raw);
+                    ts.mx = max(ts.mx, raw);
+                    if (full) store_record<W>(a.geno + (size_t)j * (2 * W), ch);
+                }
+                if (full && lane == 0u) a.alive[j0 >> 5] = bits;
+            }
+            if (lane == 0u && !again) a.counts[g & 1u][slot] = at0 - base;
+        }
+        if (again) break;
+        put_stats<SM>(ts, tid);
+        if (a.locus_row[0])
+            count_loci<W, BLOCK>(a.geno, min(slot0 * rec_slot, a.n),
+                                 (uint32_t)min((unsigned long long)slot1 * rec_slot, (unsigned long long)a.n), s_cnt,
+                                 a.locus_row[g & 1u]);
+        __syncthreads();
+        BlockStats *bs = a.block_stats + (size_t)(g & 1u) * gridDim.x;
+        block_stats<SM>(bs + blockIdx.x, warp, lane);
+        if (!grid_barrier(a.barrier)) {  // the generation fails: every block gives up
+            if (tid == 0u) atomicExch(reinterpret_cast<int *>(&st->status), SPG_ERR_TIMEOUT);
+            return;
+        }
+        // close the generation: every block builds the directory and, with an
+        // ecology, the resource and factor (the same arithmetic in each);
+        // block 0 writes the statistics record and the state
+        load_counts<BLOCK>(a.counts[g & 1u], a.nslots, sc);
+        if (eco && warp == NW - 1u) {
+            unsigned long long x = 0;
+            for (uint32_t b = lane; b < gridDim.x; b += 32u) x += __ldcg(&bs[b].sum[3]);
+            x = warp_sum_u64(x);
+            if (lane == 0u) {
+                s_R = resource_eaten(s_R, x);
+                s_f = factor_q32(s_R, a.eco_R_half);
+            }
+        }
+        if (blockIdx.x == 0u && warp < 8u) {
+            if (warp < 6u) {
+                unsigned long long x = 0;
+                for (uint32_t b = lane; b < gridDim.x; b += 32u) x += __ldcg(&bs[b].sum[warp]);
+                x = warp_sum_u64(x);
+                if (lane == 0u) s_sum[warp] = x;
+            } else {
+                int x = warp == 6u ? INT_MAX : INT_MIN;
+                for (uint32_t b = lane; b < gridDim.x; b += 32u)
+                    x = warp == 6u ? min(x, __ldcg(&bs[b].mn)) : max(x, __ldcg(&bs[b].mx));
+                x = warp == 6u ? __reduce_min_sync(0xFFFFFFFFu, x) : __reduce_max_sync(0xFFFFFFFFu, x);
+                if (lane == 0u) s_mm[warp - 6u] = x;
+            }
+        }
+        const uint32_t S_new = build_directory<SM, BLOCK>(sc, a.nslots, rec_slot, s_scan, one_step);
+        if (S_new == 0u) __syncthreads();  // the sums above are visible (the directory was left alone)
+        const uint32_t f_new = eco ? s_f : f;
+        const double R_new = eco ? s_R : R;
+        status = S_new == 0u ? SPG_EXTINCT : SPG_OK;
+        if (blockIdx.x == 0u) {
+            if (tid == 0u) {
+                spg_stats *rec = a.ring + (g - 1u) % a.stats_cap;
+                rec->gen = g;
+                rec->n = a.n;
+                rec->s = S_new;
+                rec->status = (uint32_t)status;
+                rec->sum_raw = (long long)s_sum[0];
+                rec->sum_raw_surv = (long long)s_sum[1];
+                rec->sum_raw2 = s_sum[2];
+                rec->consumption = eco ? s_sum[3] : 0ull;
+                rec->het = s_sum[4];
+                rec->allele = s_sum[5];
+                rec->min_raw = s_mm[0];
+                rec->max_raw = s_mm[1];
+                rec->R = eco ? R_new : 0.0;
+                rec->f = f_new;
+                rec->pad = 0;
+                st->gen = g;
+                st->S = S_new;
+                st->f = f_new;
+                st->R = R_new;
+                st->status = status;
+            }
+            if (a.locus_row[0]) {  // the counted row to its place; clear for the generation after next
+                uint32_t *row = a.locus_row[g & 1u], *dst = a.locus_ring + (size_t)((g - 1u) % a.locus_cap) * (32u * W);
+                for (uint32_t i = tid; i < 32u * W; i += BLOCK) {
+                    dst[i] = __ldcg(row + i);
+                    row[i] = 0u;
+                }
+            }
+        }
+        if (list && S_new != 0u) {  // the ordered survivor list from the bitmap
+            for (uint32_t slot = blockIdx.x * NW + warp; slot < a.nslots; slot += gridDim.x * NW) {
+                uint32_t rank = slot * rec_slot - *reinterpret_cast<const uint32_t *>(g_smem + SM::kDir + 8u * slot + 4u);
+                for (uint32_t gi = 0; gi < a.slot_len && slot * rec_slot + 32u * gi < a.n; ++gi) {
+                    const uint32_t j = slot * rec_slot + 32u * gi, bits = __ldcg(a.alive + (j >> 5));
+                    if ((bits >> lane) & 1u) a.surv[rank + __popc(bits & ((1u << lane) - 1u))] = j + lane;
+                    rank += __popc(bits);
+                }
+            }
+        }
+        gen = g;
+        ++done;
+        if (S_new == 0u) {
+            if (list) break;  // its full records are written
+            again = true;     // form it once more for them (its parents and directory are still there)
+            --done;
+            __syncthreads();
+            continue;
+        }
+        S = S_new;
+        f = f_new;
+        R = R_new;
+        __syncthreads();  // s_R, s_f and the sums are read
+    }
+}
+
+template <int W, bool LINKED, bool WEIGHTED>
+SoloKernel solo_instance() {
+    SoloKernel k;
+    k.fn = &k_generations<W, LINKED, WEIGHTED>;
+    k.block = kSoloThreads;
+    k.smem = GenSmem<W, LINKED, kSoloThreads>::kBytes;
+    return k;
+}
+
+}  // namespace
+}  // namespace spg

@@ -27,59 +27,11 @@
 #include <cstdint>
 
 #include "device_common.cuh"
+#include "ecology.cuh"
 #include "spegg_internal.h"
 
 namespace spg {
 namespace {
-
-// ------------------------------------------------------ ecology (Fig. 1F)
-__device__ double resource_update(double R, double r, double K, unsigned long long C) {
-    const double ratio = __ddiv_rn(R, K);
-    const double room = __dsub_rn(1.0, ratio);
-    const double rR = __dmul_rn(r, R);
-    const double growth = __dmul_rn(rR, room);
-    const double grown = __dadd_rn(R, growth);
-    const double eaten = __dmul_rn(__ull2double_rn(C), 1.0 / 65536.0);
-    double next = __dsub_rn(grown, eaten);
-    if (!(next > 0.0)) next = 0.0;
-    return next;
-}
-
-// Beverton-Holt variant: R' = (r' R) / (1 + R/K) - C 2^-16, clamped at 0.
-__device__ double resource_update_bh(double R, double rg, double K, unsigned long long C) {
-    const double grown_num = __dmul_rn(rg, R);
-    const double ratio = __ddiv_rn(R, K);
-    const double den = __dadd_rn(1.0, ratio);
-    const double grown = __ddiv_rn(grown_num, den);
-    const double eaten = __dmul_rn(__ull2double_rn(C), 1.0 / 65536.0);
-    double next = __dsub_rn(grown, eaten);
-    if (!(next > 0.0)) next = 0.0;
-    return next;
-}
-
-// Growth rate of generation g: r + r_sd * z, z the Irwin-Hall(12) normal
-// (sum of twelve Philox lanes of counter (0, g, rep, 7<<24 | k/4)) * 2^-32 - 6.
-__device__ double growth_rate(const PopParams *P, uint32_t g) {
-    if (P->r_sd == 0.0) return P->r;
-    unsigned long long sum = 0;
-#pragma unroll
-    for (uint32_t k = 0; k < 3; ++k) {
-        const uint4 d = philox(make_uint4(0u, g, P->rep, (kGrowth << 24) | k), P->key0, P->key1);
-        sum += (unsigned long long)d.x + d.y + d.z + d.w;
-    }
-    const double u = __dmul_rn(__ull2double_rn(sum), 1.0 / 4294967296.0);
-    const double z = __dsub_rn(u, 6.0);
-    return __dadd_rn(P->r, __dmul_rn(P->r_sd, z));
-}
-
-__device__ uint32_t factor_q32(double R, double R_half) {
-    const double den = __dadd_rn(R, R_half);
-    const double q = __ddiv_rn(R, den);
-    const double scaled = __dmul_rn(q, 4294967296.0);
-    if (scaled >= 4294967294.0) return 0xFFFFFFFEu;
-    if (!(scaled > 0.0)) return 0u;
-    return __double2uint_rz(scaled);
-}
 
 __device__ __forceinline__ void clear_acc(StatAcc *a) {
     a->s = 0;
@@ -133,8 +85,10 @@ __device__ void finalize_warp(const Segment &sg, const PopParams *P, uint32_t g,
         uint32_t f_next = f_used;
         double R = 0.0;
         if (P->has_eco) {
-            R = P->eco_model == 1u ? resource_update_bh(R_prev, growth_rate(P, g), P->K, cons)
-                                   : resource_update(R_prev, P->r, P->K, cons);
+            R = resource_eaten(P->eco_model == 1u ? resource_grown_bh(R_prev, growth_rate(P->r, P->r_sd, g, P->rep, P->key0, P->key1),
+                                                                     P->K)
+                                                  : resource_grown(R_prev, P->r, P->K),
+                               cons);
             f_next = factor_q32(R, P->R_half);
         }
         const int32_t status = (S_new == 0ull) ? SPG_EXTINCT : SPG_OK;
@@ -740,18 +694,9 @@ __global__ void k_iota(uint32_t *__restrict__ surv, uint32_t n) {
     if (i < n) surv[i] = i;
 }
 
-// survw[pi * n + r] = surv[r] | (role pi's threshold for the survivor's bin)
-// << 32 for the current survivors, each bin from its record's genetic value
-// (planes read from the parameters).
+// Phenotype bin of a record, its genetic value from the effect planes.
 template <int W>
-__global__ void k_survivor_bins(const PopParams *__restrict__ P, const uint32_t *__restrict__ geno,
-                                const uint32_t *__restrict__ surv, uint32_t S, uint32_t n,
-                                unsigned long long *__restrict__ survw) {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= S) return;
-    const uint32_t idx = surv ? surv[r] : r;
-    uint32_t rec[2 * W];
-    load_record<W>(geno + (size_t)idx * (2 * W), rec);
+__device__ __forceinline__ uint32_t record_bin(const PopParams *__restrict__ P, const uint32_t (&rec)[2 * W]) {
     uint32_t total = 0, het = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
@@ -775,9 +720,62 @@ __global__ void k_survivor_bins(const PopParams *__restrict__ P, const uint32_t 
         raw += cnt << b;
     }
     const long long v = (long long)raw + (long long)P->bias;
-    const uint32_t bin = v < 0 ? 0u : (uint32_t)min(v >> P->shift, (long long)(kBins - 1));
+    return v < 0 ? 0u : (uint32_t)min(v >> P->shift, (long long)(kBins - 1));
+}
+
+// survw[pi * n + r] = surv[r] | (role pi's threshold for the survivor's bin)
+// << 32 for the current survivors, each bin from its record's genetic value
+// (planes read from the parameters).
+template <int W>
+__global__ void k_survivor_bins(const PopParams *__restrict__ P, const uint32_t *__restrict__ geno,
+                                const uint32_t *__restrict__ surv, uint32_t S, uint32_t n,
+                                unsigned long long *__restrict__ survw) {
+    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= S) return;
+    const uint32_t idx = surv ? surv[r] : r;
+    uint32_t rec[2 * W];
+    load_record<W>(geno + (size_t)idx * (2 * W), rec);
+    const uint32_t bin = record_bin<W>(P, rec);
     survw[r] = (unsigned long long)idx | ((unsigned long long)P->weights->acc[0][bin] << 32);
     survw[(size_t)n + r] = (unsigned long long)idx | ((unsigned long long)P->weights->acc[1][bin] << 32);
+}
+
+// The last bitmap word of a population whose size is not a multiple of 32.
+__global__ void k_mark_tail(uint32_t *word, uint32_t count) {
+    if (threadIdx.x == 0) *word = (1u << count) - 1u;
+}
+
+// Bitmap of a survivor list (the bitmap cleared before).
+__global__ void k_mark_alive(const uint32_t *__restrict__ surv, uint32_t S, uint32_t *__restrict__ alive) {
+    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < S) atomicOr(alive + (surv[r] >> 5), 1u << (surv[r] & 31u));
+}
+
+// The slot layout of a generation (generations.cuh) from its full records and
+// bitmap, one warp per slot; mate: the survivors' thresholds as mother and
+// father, each bin from its record's genetic value.
+template <int W>
+__global__ void k_pack(const PopParams *__restrict__ P, const uint32_t *__restrict__ geno,
+                       const uint32_t *__restrict__ alive, uint32_t n, uint32_t slot_len, uint32_t nslots,
+                       uint32_t *__restrict__ packed, uint32_t *__restrict__ counts, uint2 *__restrict__ mate) {
+    const uint32_t lane = threadIdx.x & 31u, slot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (slot >= nslots) return;
+    const uint32_t base = slot * slot_len * 32u;
+    uint32_t held = 0;
+    for (uint32_t gi = 0; gi < slot_len && base + 32u * gi < n; ++gi) {
+        const uint32_t j = base + 32u * gi + lane, bits = alive[(base >> 5) + gi];
+        const uint32_t at = base + held + __popc(bits & ((1u << lane) - 1u));
+        held += __popc(bits);
+        if (!((bits >> lane) & 1u)) continue;
+        uint32_t rec[2 * W];
+        load_record<W>(geno + (size_t)j * (2 * W), rec);
+        store_record<W>(packed + (size_t)at * (2 * W), rec);
+        if (mate) {
+            const uint32_t bin = record_bin<W>(P, rec);
+            mate[at] = make_uint2(P->weights->acc[0][bin], P->weights->acc[1][bin]);
+        }
+    }
+    if (lane == 0u) counts[slot] = held;
 }
 
 __global__ void k_set_state(DevState *st, StatAcc *acc, uint32_t gen, uint32_t S, uint32_t f, double R,
@@ -1103,6 +1101,54 @@ int launch_survivor_bins(const PopParams *prm, uint32_t words, const uint32_t *g
         default: return SPG_ERR_INVALID;
     }
     return cudaGetLastError() == cudaSuccess ? SPG_OK : SPG_ERR_CUDA;
+}
+
+int launch_pack(const PopParams *prm, uint32_t words, const uint32_t *geno, const uint32_t *surv, uint32_t S, uint32_t n,
+                uint32_t slot_len, uint32_t nslots, uint32_t *alive, uint32_t *packed, uint32_t *counts, uint2 *mate,
+                void *stream) {
+    cudaStream_t s = (cudaStream_t)stream;
+    const size_t words32 = ((size_t)n + 31) / 32;
+    cudaError_t e = cudaMemsetAsync(alive, surv ? 0 : 0xFF, words32 * 4, s);
+    if (e != cudaSuccess) return SPG_ERR_CUDA;
+    if (surv && S) k_mark_alive<<<(S + 255) / 256, 256, 0, s>>>(surv, S, alive);
+    if (!surv && (n & 31u)) k_mark_tail<<<1, 32, 0, s>>>(alive + words32 - 1, n & 31u);
+    const dim3 grid((nslots + 7) / 8), block(256);
+    switch (words) {
+        case 1: k_pack<1><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate); break;
+        case 2: k_pack<2><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate); break;
+        case 4: k_pack<4><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate); break;
+        case 8: k_pack<8><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate); break;
+        default: return SPG_ERR_INVALID;
+    }
+    return cudaGetLastError() == cudaSuccess ? SPG_OK : SPG_ERR_CUDA;
+}
+
+SoloKernel solo_kernel_w1(bool linked, bool weighted);
+SoloKernel solo_kernel_w2(bool linked, bool weighted);
+SoloKernel solo_kernel_w4(bool linked, bool weighted);
+SoloKernel solo_kernel_w8(bool linked, bool weighted);
+
+SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted) {
+    switch (words) {
+        case 1: return solo_kernel_w1(linked, weighted);
+        case 2: return solo_kernel_w2(linked, weighted);
+        case 4: return solo_kernel_w4(linked, weighted);
+        case 8: return solo_kernel_w8(linked, weighted);
+        default: return SoloKernel{};
+    }
+}
+
+int prepare_solo(SoloKernel &k) {
+    if (!k.fn) return SPG_ERR_INVALID;
+    const void *fn = reinterpret_cast<const void *>(k.fn);
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, (int)k.block, k.smem);
+    if (e != cudaSuccess || per_sm <= 0) return SPG_ERR_CUDA;
+    k.resident = (uint32_t)per_sm * (uint32_t)sms;
+    return SPG_OK;
 }
 
 int launch_set_state(DevState *st, StatAcc *acc, uint32_t gen, uint32_t S, uint32_t f, double R, int32_t status,

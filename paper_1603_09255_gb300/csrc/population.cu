@@ -29,9 +29,13 @@ struct spg_pop {
     char *arena = nullptr;
     PopLayout L{};
     PopParams *host_prm = nullptr;  // host copy of the parameters
+    ValueFragments frag{};          // fragments of the genetic value (biallelic records)
     LinkParams link{};              // linkage-map tables (when host_prm->linked)
     WeightParams *weights = nullptr;  // parent acceptance thresholds (when host_prm->weighted)
-    GenLaunch gl;
+    SoloKernel solo;   // biallelic records: the generation kernel, its grid and arguments
+    SoloArgs sa{};
+    uint32_t solo_blocks = 0;
+    GenLaunch gl;      // continuous allelic values: generation and compaction launches
     GraphChain chain;
     // per-locus allele counts (off until spg_set_locus_counts): ring, partial
     // rows and counter in one allocation; readable from generation locus_from
@@ -55,24 +59,96 @@ struct spg_pop {
 
 namespace {
 
-// The per-locus count kernel after each compaction, or none.
+// The rows the generation kernel adds its per-locus counts to, or none.
 void attach_locus(spg_pop *p) {
-    p->gl.locus = p->locus_on ? locus_kernel(p->words) : nullptr;
-    p->gl.la = p->locus;
-    p->chain.reset();
+    for (uint32_t i = 0; i < 2; ++i) p->sa.locus_row[i] = p->locus_on ? p->locus.acc + (size_t)i * p->n_loci : nullptr;
+    p->sa.locus_ring = p->locus.ring;
+    p->sa.locus_cap = p->locus.cap;
+}
+
+// The ecology as the generation kernel's arguments.
+void set_solo_ecology(spg_pop *p) {
+    const PopParams &prm = *p->host_prm;
+    p->sa.has_eco = prm.has_eco;
+    p->sa.eco_model = prm.eco_model;
+    p->sa.eco_r = prm.r;
+    p->sa.eco_r_sd = prm.r_sd;
+    p->sa.eco_K = prm.K;
+    p->sa.eco_R_half = prm.R_half;
+}
+
+// Least warps of work per block: a small population takes as few SMs as give
+// every one of them this many warps.
+constexpr uint32_t kSoloMinWarps = 4;
+constexpr uint32_t kSoloLaunchGens = 512;  // generations of one launch, at most
+
+// The generation kernel, its grid and its arguments.  The launch shape is
+// accepted and reported; the kernel has one shape of its own (results never
+// depend on it).
+int configure_solo(spg_pop *p, const Shape &shape) {
+    const PopParams &prm = *p->host_prm;
+    SoloKernel k = solo_kernel(p->words, prm.linked != 0u, prm.weighted != 0u);
+    const int rc = prepare_solo(k);
+    if (rc != SPG_OK) return fail(rc, "generation kernel setup failed");
+    p->solo = k;
+    p->shape = shape;
+    const uint32_t nslots = slot_count(p->n);
+    p->solo_blocks = std::max(1u, std::min(std::min(k.resident, kSoloMaxBlocks), nslots / kSoloMinWarps));
+    SoloArgs &a = p->sa;
+    a.prm = reinterpret_cast<const PopParams *>(p->arena + p->L.params);
+    a.frag = reinterpret_cast<const ValueFragments *>(p->arena + p->L.frag);
+    for (uint32_t i = 0; i < 2; ++i) {
+        a.packed[i] = reinterpret_cast<uint32_t *>(p->arena + p->L.packed[i]);
+        a.counts[i] = reinterpret_cast<uint32_t *>(p->arena + p->L.counts[i]);
+        a.mate[i] = p->L.weighted ? reinterpret_cast<uint2 *>(p->arena + p->L.mate[i]) : nullptr;
+    }
+    a.geno = reinterpret_cast<uint32_t *>(p->arena + p->L.geno0);
+    a.alive = reinterpret_cast<uint32_t *>(p->arena + p->L.alive);
+    a.surv = reinterpret_cast<uint32_t *>(p->arena + p->L.surv0);
+    a.state = reinterpret_cast<DevState *>(p->arena + p->L.state);
+    a.block_stats = reinterpret_cast<BlockStats *>(p->arena + p->L.block_stats);
+    a.barrier = reinterpret_cast<unsigned long long *>(p->arena + p->L.barrier);
+    a.ring = reinterpret_cast<spg_stats *>(p->arena + p->L.ring);
+    for (uint32_t i = 0; i < 10; ++i) {
+        a.keys[2 * i] = prm.key0 + i * 0x9E3779B9u;
+        a.keys[2 * i + 1] = prm.key1 + i * 0xBB67AE85u;
+    }
+    a.rep = prm.rep;
+    a.kmax = prm.kmax;
+    a.stats_cap = p->cap;
+    set_solo_ecology(p);
+    a.mut_from = prm.kmax ? prm.cdf[0] : 0xFFFFFFFFu;
+    a.shift = prm.shift;
+    a.bias = prm.bias;
+    a.narrow_bias = prm.bias < (1 << 30) && prm.bias > -(1 << 30) ? 1u : 0u;  // |genetic value| < 2^26
+    a.n = p->n;
+    a.slot_len = slot_length(p->n);
+    a.nslots = nslots;
+    attach_locus(p);
+    return SPG_OK;
+}
+
+// n_gen generations: one cooperative launch per kSoloLaunchGens of them (the
+// blocks meet at a grid barrier, so all must be resident).
+int enqueue_solo(spg_pop *p, uint32_t n_gen) {
+    for (uint32_t done = 0; done < n_gen;) {
+        SoloArgs a = p->sa;
+        a.n_gen = std::min(n_gen - done, kSoloLaunchGens);
+        done += a.n_gen;
+        a.keep_last = done == n_gen ? 1u : 0u;
+        void *params[] = {&a};
+        const cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(p->solo.fn), dim3(p->solo_blocks),
+                                                          dim3(p->solo.block), params, p->solo.smem, p->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "generation launch");
+    }
+    return SPG_OK;
 }
 
 // Point the launch at the population's single segment with a launch shape
 // (uploads the device copy of the segment; synchronous).
 int configure_launch(spg_pop *p, const Shape &shape) {
     const PopParams &prm = *p->host_prm;
-    const bool continuous = prm.continuous != 0u;
-    OffspringKernel k;
-    if (continuous) {
-        if (shape.block != (uint32_t)kBlock || shape.items != 1u)
-            return fail(SPG_ERR_INVALID, "continuous allelic values run 256 threads, one offspring each");
-        k = continuous_kernel(p->n_loci);
-    } else {
+    if (!prm.continuous) {
         if (!supported_shape(p->words, shape))
             return fail(SPG_ERR_INVALID,
                         "unsupported launch shape (%u threads, %u offspring per thread, %u lanes per offspring) for %u loci",
@@ -80,13 +156,15 @@ int configure_launch(spg_pop *p, const Shape &shape) {
         if ((prm.linked || prm.weighted) && (shape.block != 256u || shape.items != 1u || shape.lanes != 1u))
             return fail(SPG_ERR_INVALID,
                         "a population with a linkage map or parent weights runs 256 threads, one offspring each");
-        k = offspring_kernel(p->words, shape, prm.linked != 0u, prm.weighted != 0u, prm.has_eco != 0u,
-                             prm.has_dom != 0u, prm.weighted != 0u || (size_t)p->n * 8u * p->words > kStageParentBytes);
+        return configure_solo(p, shape);
     }
+    if (shape.block != (uint32_t)kBlock || shape.items != 1u)
+        return fail(SPG_ERR_INVALID, "continuous allelic values run 256 threads, one offspring each");
+    OffspringKernel k = continuous_kernel(p->n_loci);
     int rc = prepare_offspring(k);
     if (rc != SPG_OK) return fail(rc, "offspring kernel setup failed");
     p->shape = shape;
-    p->ntiles = continuous ? (p->n + kBlock - 1) / kBlock : tiles_for(p->n, shape);
+    p->ntiles = (p->n + kBlock - 1) / kBlock;
     const Segment seg = segment_at(p->arena, p->L, p->n, p->ntiles, 0, p->nbuckets, 0);
     cudaError_t e = cudaMemcpyAsync(p->arena + p->L.segment, &seg, sizeof seg, cudaMemcpyHostToDevice, p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "upload segment");
@@ -100,10 +178,9 @@ int configure_launch(spg_pop *p, const Shape &shape) {
     p->gl.args.nsegs = 1;
     p->gl.args.total_tiles = p->ntiles;
     p->gl.args.total_buckets = p->nbuckets;
-    if (!continuous) apply_kernel(k, p->gl.args);
-    p->gl.blocks = continuous ? p->ntiles : std::min(p->ntiles, k.resident);  // continuous: not persistent
+    p->gl.blocks = p->ntiles;  // not persistent
     p->gl.buckets = p->nbuckets;
-    attach_locus(p);  // also drops the cached graph
+    p->chain.reset();
     return SPG_OK;
 }
 
@@ -164,12 +241,22 @@ int spg_create_population(const spg_pop_desc *desc, const spg_allocator *alloc, 
         }
         p->own_stream = true;
     }
-    p->L = layout_for(p->n, p->words, p->nbuckets, p->cap, p->host_prm->weighted != 0u,
-                      p->host_prm->continuous == 0u);
+    p->L = p->host_prm->continuous ? layout_for(p->n, p->words, p->nbuckets, p->cap, false, false)
+                                   : solo_layout_for(p->n, p->words, p->cap, p->host_prm->weighted != 0u);
     p->arena = static_cast<char *>(p->alloc.alloc(p->L.total, p->stream));
     if (!p->arena) {
         spg_destroy(p);
         return fail(SPG_ERR_OOM, "device allocation of %zu bytes failed", p->L.total);
+    }
+    if (p->L.solo) {
+        p->sa.dom = p->host_prm->has_dom;
+        value_fragments(desc->effects, p->sa.dom ? desc->dominance : nullptr, p->n_loci, p->frag, p->sa.two_digits);
+        const cudaError_t e =
+            cudaMemcpyAsync(p->arena + p->L.frag, &p->frag, sizeof(ValueFragments), cudaMemcpyHostToDevice, p->stream);
+        if (e != cudaSuccess) {
+            spg_destroy(p);
+            return cuda_fail(e, "upload value fragments");
+        }
     }
     if (p->host_prm->linked) {
         p->host_prm->link = reinterpret_cast<const LinkParams *>(p->arena + p->L.link);
@@ -206,15 +293,13 @@ int spg_create_population(const spg_pop_desc *desc, const spg_allocator *alloc, 
 int spg_set_ecology(spg_pop *p, const spg_ecology *eco) {
     if (!p) return fail(SPG_ERR_INVALID, "population is NULL");
     const int rc = view_set_ecology(p->view(), *p->host_prm, eco);
-    if (rc != SPG_OK) return rc;
-    // the survival table of the offspring kernel now carries attack rates
-    if (!p->host_prm->continuous && !p->gl.offspring.eco_table) return configure_launch(p, p->shape);
-    return SPG_OK;
+    if (rc == SPG_OK) set_solo_ecology(p);
+    return rc;
 }
 
 int spg_step_generations(spg_pop *p, uint32_t n_gen) {
     if (!p) return fail(SPG_ERR_INVALID, "population is NULL");
-    return enqueue_generations(p->gl, n_gen, p->chain, p->stream);
+    return p->host_prm->continuous ? enqueue_generations(p->gl, n_gen, p->chain, p->stream) : enqueue_solo(p, n_gen);
 }
 
 int spg_read_stats(spg_pop *p, uint32_t first_gen, uint32_t count, spg_stats *out) {
@@ -229,21 +314,14 @@ int spg_set_locus_counts(spg_pop *p, int enable) {
     int rc = view_state(p->view(), st);  // synchronises: no generation in flight
     if (rc != SPG_OK) return rc;
     if (enable && !p->locus_mem) {
-        const uint32_t L = p->n_loci, blocks = locus_blocks(p->n);
-        const size_t ring = align_up((size_t)p->cap * L * 4u, 256), row = align_up((size_t)L * 4u, 256);
-        p->locus_mem = static_cast<char *>(p->alloc.alloc(ring + row + 256u, p->stream));
-        if (!p->locus_mem) return fail(SPG_ERR_OOM, "device allocation of %zu bytes failed", ring + row + 256u);
+        const uint32_t L = p->n_loci;
+        const size_t ring = align_up((size_t)p->cap * L * 4u, 256), rows = (size_t)2 * L * 4u;
+        p->locus_mem = static_cast<char *>(p->alloc.alloc(ring + rows, p->stream));
+        if (!p->locus_mem) return fail(SPG_ERR_OOM, "device allocation of %zu bytes failed", ring + rows);
         p->locus.ring = reinterpret_cast<uint32_t *>(p->locus_mem);
-        p->locus.acc = reinterpret_cast<uint32_t *>(p->locus_mem + ring);
-        p->locus.done = reinterpret_cast<uint32_t *>(p->locus_mem + ring + row);
-        p->locus.last = p->locus.done + 1;
+        p->locus.acc = reinterpret_cast<uint32_t *>(p->locus_mem + ring);  // two rows, zero between launches
         p->locus.cap = p->cap;
-        p->locus.blocks = blocks;
-        const cudaError_t e = cudaMemsetAsync(p->locus.acc, 0, row + 8u, p->stream);  // row, counter, last
-        if (e != cudaSuccess) return cuda_fail(e, "clear per-locus counts");
-    }
-    if (enable && !p->locus_on && p->locus_mem) {  // the next generation is counted whatever was counted before
-        const cudaError_t e = cudaMemsetAsync(p->locus.last, 0, 4, p->stream);
+        const cudaError_t e = cudaMemsetAsync(p->locus.acc, 0, rows, p->stream);
         if (e != cudaSuccess) return cuda_fail(e, "clear per-locus counts");
     }
     if (enable) {
@@ -353,31 +431,17 @@ int spg_restore(spg_pop *p, const void *host, size_t bytes) {
                        (size_t)h.S * 4, cudaMemcpyHostToDevice);
     // per-bucket survivor counts of the replaced run must not leak into the
     // generations about to be replayed
-    if (e == cudaSuccess) e = cudaMemset(p->arena + p->L.buckets, 0, (size_t)2 * p->nbuckets * 4);
+    if (e == cudaSuccess && p->L.solo) e = cudaMemset(p->arena + p->L.barrier, 0, sizeof(unsigned long long));
+    if (e == cudaSuccess && !p->L.solo) e = cudaMemset(p->arena + p->L.buckets, 0, (size_t)2 * p->nbuckets * 4);
     if (e != cudaSuccess) return cuda_fail(e, "restore copy");
-    if (p->L.dense) {  // the restored survivors' records in rank order: the next generation's parents
-        const uint32_t par = h.gen & 1u;
-        rc = launch_dense_gather(p->words, reinterpret_cast<const uint32_t *>(p->arena + (par ? p->L.geno1 : p->L.geno0)),
-                                 reinterpret_cast<const uint32_t *>(p->arena + (par ? p->L.surv1 : p->L.surv0)), h.S,
-                                 reinterpret_cast<uint32_t *>(p->arena + p->L.dense), p->stream);
-        if (rc != SPG_OK) return fail(rc, "dense-parent launch failed");
-    }
-    if (p->host_prm->weighted) {  // the restored survivors' bins, from their records
-        const uint32_t par = h.gen & 1u;
-        rc = launch_survivor_bins(reinterpret_cast<const PopParams *>(p->arena + p->L.params), p->words,
-                                  reinterpret_cast<const uint32_t *>(p->arena + (par ? p->L.geno1 : p->L.geno0)),
-                                  reinterpret_cast<const uint32_t *>(p->arena + (par ? p->L.surv1 : p->L.surv0)), h.S,
-                                  p->n, reinterpret_cast<unsigned long long *>(p->arena + p->L.survw), p->stream);
-        if (rc != SPG_OK) return fail(rc, "survivor-bin launch failed");
+    if (p->L.solo) {  // the restored survivors in the slot layout: the next generation's parents
+        rc = view_pack(p->view(), h.gen, reinterpret_cast<const uint32_t *>(p->arena + p->L.surv0), h.S);
+        if (rc != SPG_OK) return fail(rc, "survivor packing failed");
     }
     rc = view_set_state(p->view(), h.gen, h.S, h.f, h.R, h.status, 0xFFFFFFFFu);
     if (rc != SPG_OK) return rc;
     p->locus_from = h.gen + 1u;  // counts of the restored run start with its next generation
     p->locus_until = h.gen;
-    if (p->locus_mem) {  // that generation is counted even if a generation of that number was before
-        const cudaError_t e = cudaMemsetAsync(p->locus.last, 0, 4, p->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "clear per-locus counts");
-    }
     return view_sync(p->view());
 }
 
@@ -404,9 +468,9 @@ int spg_set_launch_shape(spg_pop *p, const spg_launch_shape *shape) {
 
 int spg_get_launch_shape(spg_pop *p, spg_launch_shape *out) {
     if (!p || !out) return fail(SPG_ERR_INVALID, "NULL argument");
-    out->threads_per_block = p->gl.offspring.block;
-    out->items_per_thread = p->gl.offspring.items;
-    out->lanes_per_offspring = p->gl.offspring.lanes;
+    out->threads_per_block = p->shape.block;
+    out->items_per_thread = p->shape.items;
+    out->lanes_per_offspring = p->shape.lanes;
     return SPG_OK;
 }
 

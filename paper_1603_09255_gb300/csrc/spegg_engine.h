@@ -38,6 +38,10 @@ struct PopLayout {
     size_t params, state, acc, geno0, geno1, dense, surv0, surv1, alive, buckets, ring, segment, link;
     size_t weights, obin, survw;  // weighted parents only (0 otherwise)
     bool weighted;
+    // a single biallelic population (solo_layout_for): geno0 = geno1 and
+    // surv0 = surv1, no dense buffer, buckets, bins or segment
+    bool solo;
+    size_t packed[2], counts[2], mate[2], block_stats, barrier, frag;
     size_t total;
 };
 
@@ -77,6 +81,10 @@ uint32_t mutation_cdf(double mu, uint32_t n_copies, uint32_t *cdf);
 void effect_planes(const int16_t *effects, uint32_t n_loci, PopParams &prm);
 uint32_t factor_q32_host(double R, double R_half);
 size_t align_up(size_t x, size_t a);
+// Value fragments of the effects and dominance deviations (null: none);
+// two_digits: some value is beyond 2048 in magnitude.
+void value_fragments(const int16_t *effects, const int16_t *dominance, uint32_t n_loci, ValueFragments &vf,
+                     uint32_t &two_digits);
 int validate_desc(const spg_pop_desc *d);
 int build_params(const spg_pop_desc *d, PopParams &prm);
 // Linkage-map tables from map_morgans[L] (validated; see spegg.h).
@@ -90,6 +98,10 @@ PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap
 Segment segment_at(char *base, const PopLayout &L, uint32_t n, uint32_t ntiles, uint32_t tile_begin,
                    uint32_t nbuckets, uint32_t bucket_begin);
 uint32_t bucket_count(uint32_t n);
+uint32_t slot_length(uint32_t n);
+uint32_t slot_count(uint32_t n);
+PopLayout solo_layout_for(uint32_t n, uint32_t words, uint32_t cap, bool weighted);
+int view_pack(const PopView &v, uint32_t gen, const uint32_t *surv, uint32_t S);
 Shape default_shape(uint32_t words);
 constexpr uint32_t kAutotuneCandidates = SPG_AUTOTUNE_CANDIDATES;  // launch shapes timed per group
 Shape autotune_candidate(uint32_t words, uint32_t c);

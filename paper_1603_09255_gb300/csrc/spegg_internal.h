@@ -5,6 +5,8 @@
 #include <cstddef>
 #include <cstdint>
 
+#include <cuda_runtime.h>
+
 #include "spegg.h"
 
 namespace spg {
@@ -183,6 +185,64 @@ struct GenArgs {
 };
 
 using GenKernel = void (*)(GenArgs);
+
+// A single population's generations (generations.cuh).  Its groups of 32
+// offspring are cut into slots of slot_len groups; a generation's survivors
+// are packed slot by slot in packed[generation & 1], counts[generation & 1]
+// holding their number per slot.
+constexpr uint32_t kSoloThreads = 512;
+constexpr uint32_t kMaxSlots = 152 * (kSoloThreads / 32);  // one per resident warp on 152 SMs
+// The per-locus values as f16 elements, laid out as the matrix fragments of
+// the generation kernel (value_fragments): the additive values, or with
+// dominance those of heterozygous and of homozygous loci.
+struct alignas(16) ValueFragments {
+    uint32_t table[2][1024];
+};
+struct BlockStats {
+    unsigned long long sum[6];  // raw, raw over survivors, raw^2, consumption, heterozygosity, alleles
+    int mn, mx;
+};
+struct SoloArgs {
+    const PopParams *prm;
+    const ValueFragments *frag;
+    uint32_t *packed[2];               // survivors' records by generation parity [N * 2W]
+    uint2 *mate[2];                    // weighted parents: their thresholds as mother and father, same places
+    uint32_t *counts[2];               // survivors per slot [nslots]
+    uint32_t *geno;                    // full records of the last generation of a call [N * 2W]
+    uint32_t *alive;                   // its survivor bitmap
+    uint32_t *surv;                    // its ordered survivor list [N]
+    DevState *state;
+    BlockStats *block_stats;           // [2][kSoloMaxBlocks]
+    unsigned long long *barrier;       // grid barrier arrivals, a multiple of the grid between launches
+    spg_stats *ring;
+    uint32_t *locus_row[2];            // per-locus counts of the generation being formed, by parity (null: off)
+    uint32_t *locus_ring;              // [locus_cap][L]
+    uint32_t locus_cap;
+    uint32_t n, slot_len, nslots;
+    uint32_t keys[20];                 // Philox round keys (word 0, word 1 of each round)
+    uint32_t rep, kmax, shift;
+    uint32_t mut_from;                 // mutation draws from here on count a mutation (kmax 0: none do)
+    int32_t bias;
+    uint32_t narrow_bias;              // genetic value + bias fits 32 bits
+    uint32_t has_eco, eco_model, stats_cap;
+    double eco_r, eco_r_sd, eco_K, eco_R_half;
+    uint32_t dom, two_digits;          // fragments: dominance, values beyond 2048 in magnitude
+    uint32_t n_gen;                    // generations of this launch
+    uint32_t keep_last;                // the last of them is the call's last
+};
+constexpr uint32_t kSoloMaxBlocks = 256;
+struct SoloKernel {
+    void (*fn)(SoloArgs) = nullptr;
+    uint32_t block = 0, smem = 0, resident = 0;  // resident: blocks on the device at a time
+};
+SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted);
+int prepare_solo(SoloKernel &k);  // sets the shared-memory limit, fills `resident`
+// Enqueue the slot layout of a generation: bitmap words and per-slot counts
+// of the survivors (surv: their ordered list of S, null for all n), their
+// records packed[slot ...] and, when mate is given, their parent thresholds.
+int launch_pack(const PopParams *prm, uint32_t words, const uint32_t *geno, const uint32_t *surv, uint32_t S, uint32_t n,
+                uint32_t slot_len, uint32_t nslots, uint32_t *alive, uint32_t *packed, uint32_t *counts, uint2 *mate,
+                void *stream);
 
 // Launch shape of the offspring kernel: threads per block, offspring per
 // thread (per lane pair when lanes = 2) and lanes per offspring (1, or 2 for
