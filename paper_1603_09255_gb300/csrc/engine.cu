@@ -356,8 +356,12 @@ PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap
     return L;
 }
 
-// Slots of a single population: at most kMaxSlots of whole groups of 32.
-uint32_t slot_length(uint32_t n) { return (uint32_t)(((uint64_t)n + 32ull * kMaxSlots - 1) / (32ull * kMaxSlots)); }
+// Slots of a single population: at most kMaxSlots of whole groups of 32, or
+// one per warp of a block for a population that one block forms.
+uint32_t slot_length(uint32_t n) {
+    const uint64_t slots = n <= 32u * kOneBlockGroups ? kSoloThreads / 32u : kMaxSlots;
+    return (uint32_t)(((uint64_t)n + 32ull * slots - 1) / (32ull * slots));
+}
 uint32_t slot_count(uint32_t n) {
     const uint32_t len = 32u * slot_length(n);
     return (uint32_t)(((uint64_t)n + len - 1) / len);
@@ -382,7 +386,7 @@ PopLayout solo_layout_for(uint32_t n, uint32_t words, uint32_t cap, bool weighte
     L.surv0 = L.surv1 = take((size_t)n * 4);
     L.alive = take(((size_t)n + 31) / 32 * 4);
     for (size_t &x : L.counts) x = take((size_t)slot_count(n) * 4);
-    L.block_stats = take(sizeof(BlockStats) * 2 * kSoloMaxBlocks);
+    L.gen_acc = take(sizeof(GenAcc) * 3 * kGenAccCopies);
     L.barrier = take(sizeof(unsigned long long));
     L.ring = take((size_t)cap * sizeof(spg_stats));
     L.frag = take(sizeof(ValueFragments));
@@ -775,15 +779,17 @@ int view_pack(const PopView &v, uint32_t gen, const uint32_t *surv, uint32_t S) 
                        slot_count(v.n), reinterpret_cast<uint32_t *>(v.base + v.L.alive),
                        reinterpret_cast<uint32_t *>(v.base + v.L.packed[par]),
                        reinterpret_cast<uint32_t *>(v.base + v.L.counts[par]),
-                       v.L.weighted ? reinterpret_cast<uint2 *>(v.base + v.L.mate[par]) : nullptr, v.stream);
+                       v.L.weighted ? reinterpret_cast<uint2 *>(v.base + v.L.mate[par]) : nullptr,
+                       reinterpret_cast<GenAcc *>(v.base + v.L.gen_acc),
+                       reinterpret_cast<unsigned long long *>(v.base + v.L.barrier), v.stream);
 }
 
 // Enqueue the generation-0 set-up of one population: parameters, counters,
 // founders and state.  `prm` and `init_genotypes` must stay valid until the
 // stream has run the copies (callers synchronise before returning).
 int view_init(const PopView &v, const PopParams &prm, const uint32_t *init_genotypes, uint32_t p0_q32) {
-    cudaError_t e = v.L.solo ? cudaMemsetAsync(v.base + v.L.barrier, 0, sizeof(unsigned long long), v.stream)
-                             : cudaMemsetAsync(v.base + v.L.buckets, 0, (size_t)2 * v.nbuckets * 4, v.stream);
+    cudaError_t e = cudaSuccess;
+    if (!v.L.solo) e = cudaMemsetAsync(v.base + v.L.buckets, 0, (size_t)2 * v.nbuckets * 4, v.stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(v.base + v.L.ring, 0, (size_t)v.cap * sizeof(spg_stats), v.stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(v.base + v.L.params, &prm, sizeof(PopParams), cudaMemcpyHostToDevice, v.stream);

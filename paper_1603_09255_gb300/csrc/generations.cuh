@@ -45,8 +45,7 @@ namespace spg {
 namespace {
 
 // ------------------------------------------------------- shared memory
-constexpr int kGuideBits = 13;  // the parent draw's top bits that index the guide
-constexpr uint32_t kGuide = 1u << kGuideBits;
+constexpr uint32_t kGuide = 1u << kMaxGuideBits;  // most entries of the guide
 
 template <int W, bool LINKED, int BLOCK>
 struct GenSmem {
@@ -83,6 +82,7 @@ constexpr uint32_t kBarrierTries = 1u << 23;  // polls of about half a microseco
 
 __device__ __forceinline__ bool grid_barrier(unsigned long long *ctr) {
     __syncthreads();
+    if (gridDim.x == 1u) return true;
     int ok = 1;
     if (threadIdx.x == 0) {
         const unsigned long long G = gridDim.x;
@@ -306,20 +306,29 @@ __device__ __forceinline__ uint4 philox_at(const SoloArgs &a, const GenRng &r, u
 }
 
 // ------------------------------------------------------- parents
-// Record of the survivor drawn by u (rank u * S / 2^32) in the slot layout.
-// one_step: no guide entry is more than one slot behind (build_directory), so
-// the search is a select.
+// Records of the survivors drawn by u0 and u1 (rank u * S / 2^32) in the slot
+// layout.  one_step: no guide entry is more than one slot behind
+// (build_directory), so the search is a select.
 template <class SM>
-__device__ __forceinline__ uint32_t locate(uint32_t u, uint32_t S, bool one_step, uint32_t rec_slot) {
-    const uint32_t r = __umulhi(u, S);
-    uint32_t s = *reinterpret_cast<const uint16_t *>(g_smem + SM::kGuideOff + 2u * (u >> (32 - kGuideBits)));
-    uint2 e = *reinterpret_cast<const uint2 *>(g_smem + SM::kDir + 8u * s);
-    if (one_step) return r < e.x ? r + e.y : r - e.x + (s + 1u) * rec_slot;
-    while (e.x <= r) {  // the last slot's end is S > r
-        ++s;
-        e = *reinterpret_cast<const uint2 *>(g_smem + SM::kDir + 8u * s);
+__device__ __forceinline__ void locate(const SoloArgs &a, uint32_t u0, uint32_t u1, uint32_t S, bool one_step,
+                                       uint32_t &i0, uint32_t &i1) {
+    auto guide = [&](uint32_t u) {
+        return (uint32_t)*reinterpret_cast<const uint16_t *>(g_smem + SM::kGuideOff + 2u * (u >> (32u - a.guide_bits)));
+    };
+    auto slot = [&](uint32_t s) { return *reinterpret_cast<const uint2 *>(g_smem + SM::kDir + 8u * s); };
+    const uint32_t r0 = __umulhi(u0, S), r1 = __umulhi(u1, S);
+    uint32_t s0 = guide(u0), s1 = guide(u1);
+    uint2 e0 = slot(s0), e1 = slot(s1);
+    if (one_step) {
+        const uint32_t rec = a.slot_len * 32u;
+        i0 = r0 < e0.x ? r0 + e0.y : r0 - e0.x + (s0 + 1u) * rec;
+        i1 = r1 < e1.x ? r1 + e1.y : r1 - e1.x + (s1 + 1u) * rec;
+        return;
     }
-    return r + e.y;
+    while (e0.x <= r0) e0 = slot(++s0);  // the last slot's end is S > r
+    while (e1.x <= r1) e1 = slot(++s1);
+    i0 = r0 + e0.y;
+    i1 = r1 + e1.y;
 }
 
 // Weighted parents (bounded rejection, see offspring.cuh): proposals in
@@ -328,7 +337,7 @@ __device__ __forceinline__ uint32_t locate(uint32_t u, uint32_t S, bool one_step
 template <class SM>
 __device__ __forceinline__ void weighted_records(const SoloArgs &a, const uint2 *thr, const GenRng &rng,
                                                  unsigned long long aj, uint32_t S, bool one_step,
-                                                 uint32_t rec_slot, uint32_t &mom,
+                                                 uint32_t &mom,
                                                  uint32_t &dad) {
     bool open_m = true, open_f = true;
     for (uint32_t k = 0; k < kMateAttempts && (open_m || open_f); k += 2) {
@@ -337,15 +346,13 @@ __device__ __forceinline__ void weighted_records(const SoloArgs &a, const uint2 
         uint32_t rm0 = 0, rm1 = 0, rf0 = 0, rf1 = 0, tm0 = 0, tm1 = 0, tf0 = 0, tf1 = 0;
         if (open_m) {
             dm = philox_at(a, rng, aj, sub);
-            rm0 = locate<SM>(dm.x, S, one_step, rec_slot);
-            rm1 = locate<SM>(dm.z, S, one_step, rec_slot);
+            locate<SM>(a, dm.x, dm.z, S, one_step, rm0, rm1);
             tm0 = __ldcg(&thr[rm0].x);
             tm1 = __ldcg(&thr[rm1].x);
         }
         if (open_f) {
             df = philox_at(a, rng, aj, sub | (1u << 8));
-            rf0 = locate<SM>(df.x, S, one_step, rec_slot);
-            rf1 = locate<SM>(df.z, S, one_step, rec_slot);
+            locate<SM>(a, df.x, df.z, S, one_step, rf0, rf1);
             tf0 = __ldcg(&thr[rf0].y);
             tf1 = __ldcg(&thr[rf1].y);
         }
@@ -364,73 +371,86 @@ __device__ __forceinline__ void weighted_records(const SoloArgs &a, const uint2 
 
 // ------------------------------------------------------- the directory
 // Exclusive scan of the slots' survivor counts into the block's directory and
-// guide (all threads; returns the total, the same in every thread).  Slot s
-// holds ranks P[s] .. P[s+1]-1; entry s is {P[s+1], s * slot_records - P[s]}.
-// Guide entry h is a slot at or just before the one of the smallest rank drawn
-// by a u whose top bits are h, rank floor(h S / kGuide): slot s enters the
-// guide at the first h surely past kGuide P[s] / S.  Every block does this
-// every generation, so it takes a handful of instructions a slot (exact
-// entries by 64-bit products took a sixth of a generation at N = 10^6).
-// With no survivors the tables stay as they are.
-// one_step: whether every slot holds more ranks than a guide entry spans, so
-// that a rank lies in its entry's slot or the next.
-// The counts are loaded apart (load_counts), so that a caller can have them on
-// their way while it does something else.
-template <int BLOCK>
-struct SlotCounts {
-    static constexpr uint32_t PER = (kMaxSlots + BLOCK - 1) / BLOCK;
-    uint32_t c[PER];  // slots tid * per .. tid * per + per - 1, per = nslots / BLOCK rounded up
-};
-template <int BLOCK>
-__device__ __forceinline__ void load_counts(const uint32_t *counts, uint32_t nslots, SlotCounts<BLOCK> &sc) {
-    const uint32_t per = (nslots + BLOCK - 1) / BLOCK, s0 = threadIdx.x * per;
-#pragma unroll
-    for (uint32_t i = 0; i < SlotCounts<BLOCK>::PER; ++i)
-        sc.c[i] = i < per && s0 + i < nslots ? __ldcg(counts + s0 + i) : 0u;
-}
-template <class SM, int BLOCK>
-__device__ __forceinline__ uint32_t build_directory(const SlotCounts<BLOCK> &sc, uint32_t nslots, uint32_t slot_records,
-                                                    uint32_t *s_warp, bool &one_step) {
-    constexpr uint32_t NW = BLOCK / 32, PER = SlotCounts<BLOCK>::PER;
+// guide, by all warps but the block's last (which has the resource to close).
+// Slot s holds ranks P[s] .. P[s+1]-1; entry s is {P[s+1], s * slot_records -
+// P[s]}.  Guide entry h is a slot at or just before the one of the smallest
+// rank drawn by a u whose top bits are h, rank floor(h S / entries): slot s
+// enters the guide at the first h surely past entries * P[s] / S.  Every block
+// does this every generation, so it takes a handful of instructions a slot
+// (exact entries by 64-bit products took a sixth of a generation at N = 10^6)
+// and the guide grows with the slots (four to eight entries each, 3.4 at the
+// most slots).  Writes the total to *total; with no survivors the tables stay
+// as they are.  Returns whether every slot of the thread holds more ranks than
+// two guide entries span, so that a rank lies in its entry's slot or the next.
+// PER: runs of 32 slots a warp takes, at most.
+template <class SM, uint32_t PER>
+__device__ __forceinline__ bool directory_of(const uint32_t *counts, uint32_t nslots, uint32_t slot_records,
+                                                uint32_t guide_bits, uint32_t *s_warp, uint32_t *total) {
+    constexpr uint32_t T = SM::kThreads - 32u, NW = T / 32u;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    const uint32_t per = (nslots + BLOCK - 1) / BLOCK, s0 = tid * per;
-    const uint32_t(&c)[PER] = sc.c;
-    uint32_t own = 0;
-#pragma unroll
-    for (uint32_t i = 0; i < PER; ++i) own += c[i];
-    uint32_t incl = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if ((int)lane >= o) incl += y;
-    }
-    __syncthreads();  // s_warp is free, and the previous directory no longer read
-    if (lane == 31u) s_warp[warp] = incl;
-    __syncthreads();
-    const uint32_t w = lane < NW ? s_warp[lane] : 0u;
-    const uint32_t S = __reduce_add_sync(0xFFFFFFFFu, w);
-    if (S == 0u) return 0u;
-    uint32_t P = incl - own + __reduce_add_sync(0xFFFFFFFFu, lane < warp ? w : 0u);
-    // the first h with floor(h S / kGuide) >= P, or one later when the float
-    // quotient (off by less than 0.004) is too close to tell
-    const float inv = (float)kGuide / (float)S;
-    const uint32_t span = 2u * (S >> kGuideBits) + 2u;  // ranks of two entries, at most
-    bool wide = true;
-    auto entry_of = [&](uint32_t p) { return p ? min((uint32_t)fmaf((float)p, inv, 1.005f), kGuide) : 0u; };
-    uint32_t h = entry_of(P);
+    // warp w takes per runs of 32 consecutive slots from s0, lane l slot l of each
+    const uint32_t per = (nslots + T - 1) / T, s0 = warp * 32u * per + lane;
+    uint32_t c[PER], own = 0;
 #pragma unroll
     for (uint32_t i = 0; i < PER; ++i) {
-        const uint32_t s = s0 + i, end = P + c[i];
-        if (i < per && s < nslots) {
-            *reinterpret_cast<uint2 *>(g_smem + SM::kDir + 8u * s) = make_uint2(end, s * slot_records - P);
-            for (const uint32_t hn = entry_of(end); h < hn; ++h)
-                *reinterpret_cast<uint16_t *>(g_smem + SM::kGuideOff + 2u * h) = (uint16_t)s;
-            wide = wide && c[i] > span;
-            P = end;
-        }
+        c[i] = i < per && s0 + 32u * i < nslots ? __ldcg(counts + s0 + 32u * i) : 0u;
+        own += c[i];
     }
-    one_step = __syncthreads_and(wide) != 0;
-    return S;
+    own = __reduce_add_sync(0xFFFFFFFFu, own);
+    if (lane == 0u) s_warp[warp] = own;
+    asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory");
+    const uint32_t w = lane < NW ? s_warp[lane] : 0u;
+    const uint32_t S = __reduce_add_sync(0xFFFFFFFFu, w);
+    if (tid == 0u) *total = S;
+    if (S == 0u) return true;
+    uint32_t P = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? w : 0u);
+    // the first h with floor(h S / entries) >= P, or one later when the float
+    // quotient (off by less than 0.004) is too close to tell
+    const uint32_t entries = 1u << guide_bits, span = 2u * (S >> guide_bits) + 2u;
+    const float inv = (float)entries / (float)S;
+    auto entry_of = [&](uint32_t p) { return p ? min((uint32_t)fmaf((float)p, inv, 1.005f), entries) : 0u; };
+    // all runs stage by stage, so that their latencies overlap
+    uint32_t end[PER], h[PER];
+#pragma unroll
+    for (uint32_t i = 0; i < PER; ++i) end[i] = c[i];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (uint32_t i = 0; i < PER; ++i) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, end[i], o);
+            if ((int)lane >= o) end[i] += y;
+        }
+    bool wide = true;
+    uint32_t run = entry_of(P), left = 0;  // the run's first guide entry, the most entries a slot has
+#pragma unroll
+    for (uint32_t i = 0; i < PER; ++i) {
+        const uint32_t s = s0 + 32u * i;
+        end[i] += P;
+        P = __shfl_sync(0xFFFFFFFFu, end[i], 31);
+        const bool mine = i < per && s < nslots;
+        if (mine)
+            *reinterpret_cast<uint2 *>(g_smem + SM::kDir + 8u * s) = make_uint2(end[i], s * slot_records - (end[i] - c[i]));
+        wide = wide && (c[i] > span || !mine);
+        end[i] = entry_of(end[i]);  // from here on the slot's last entry
+        const uint32_t before = __shfl_up_sync(0xFFFFFFFFu, end[i], 1);
+        h[i] = lane ? before : run;
+        run = __shfl_sync(0xFFFFFFFFu, end[i], 31);
+        left = max(left, end[i] - h[i]);
+    }
+    for (uint32_t k = 0; k < left; ++k) {
+#pragma unroll
+        for (uint32_t i = 0; i < PER; ++i)
+            if (h[i] + k < end[i])
+                *reinterpret_cast<uint16_t *>(g_smem + SM::kGuideOff + 2u * (h[i] + k)) = (uint16_t)(s0 + 32u * i);
+    }
+    return wide;
+}
+template <class SM>
+__device__ __forceinline__ bool build_directory(const uint32_t *counts, uint32_t nslots, uint32_t slot_records,
+                                                uint32_t guide_bits, uint32_t *s_warp, uint32_t *total) {
+    constexpr uint32_t T = SM::kThreads - 32u;
+    if (nslots <= T) return directory_of<SM, 1>(counts, nslots, slot_records, guide_bits, s_warp, total);
+    return directory_of<SM, (kMaxSlots + T - 1) / T>(counts, nslots, slot_records, guide_bits, s_warp, total);
 }
 
 // ------------------------------------------------------- per-locus counts
@@ -539,7 +559,7 @@ __device__ __forceinline__ void put_stats(const LaneStats &ts, uint32_t tid) {
     s32[3 * SM::kThreads] = (uint32_t)ts.mx;
 }
 template <class SM>
-__device__ __forceinline__ void block_stats(BlockStats *out, uint32_t warp, uint32_t lane) {
+__device__ __forceinline__ void add_stats(GenAcc *acc, uint32_t warp, uint32_t lane) {
     if (warp >= 8u) return;
     if (warp < 6u) {
         unsigned long long x = 0;
@@ -549,7 +569,7 @@ __device__ __forceinline__ void block_stats(BlockStats *out, uint32_t warp, uint
                                                                            8u * (warp * SM::kThreads + 32u * i + lane))
                            : sm_u32(SM::kStats + 32u * SM::kThreads + 4u * ((warp - 4u) * SM::kThreads + 32u * i + lane));
         x = warp_sum_u64(x);  // modulo 2^64: signed sums too
-        if (lane == 0u) out->sum[warp] = x;
+        if (lane == 0u) atomicAdd(&acc->sum[warp], x);
     } else {
         int x = warp == 6u ? INT_MAX : INT_MIN;
 #pragma unroll
@@ -558,22 +578,41 @@ __device__ __forceinline__ void block_stats(BlockStats *out, uint32_t warp, uint
             x = warp == 6u ? min(x, y) : max(x, y);
         }
         x = warp == 6u ? __reduce_min_sync(0xFFFFFFFFu, x) : __reduce_max_sync(0xFFFFFFFFu, x);
-        if (lane == 0u) (warp == 6u ? out->mn : out->mx) = x;
+        if (lane == 0u) {
+            if (warp == 6u) atomicMin(&acc->mn, x);
+            else atomicMax(&acc->mx, x);
+        }
     }
 }
 
-template <int W, bool LINKED, bool WEIGHTED>
+// The generation's totals over the accumulator's copies, by one warp: lane l
+// reads word l % 8 of copy l / 8 and returns the total of that word (words 0-5
+// sums, 6 the minimum below the maximum).
+__device__ __forceinline__ unsigned long long total_stats(const GenAcc *acc, uint32_t lane) {
+    static_assert(sizeof(GenAcc) == 64 && kGenAccCopies == 4, "a lane per word");
+    unsigned long long x = __ldcg(reinterpret_cast<const unsigned long long *>(acc) + lane);
+#pragma unroll
+    for (int o = 8; o <= 16; o <<= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, x, o);
+        if ((lane & 7u) == 6u)
+            x = (unsigned long long)(uint32_t)min((int)(uint32_t)x, (int)(uint32_t)y) |
+                (unsigned long long)(uint32_t)max((int)(x >> 32), (int)(y >> 32)) << 32;
+        else x += y;
+    }
+    return x;
+}
+
+// GENERAL: dominance, values beyond 2048 in magnitude or a bias beyond 2^30
+// (the others' instance has none of these branches in its loop).
+template <int W, bool LINKED, bool WEIGHTED, bool GENERAL>
 __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_constant__ SoloArgs a) {
     constexpr int BLOCK = kSoloThreads;
     using SM = GenSmem<W, LINKED, BLOCK>;
     constexpr uint32_t NW = BLOCK / 32;
     __shared__ uint32_t s_cdf[kMaxKmax];
     __shared__ uint32_t s_scan[32];
-    __shared__ unsigned long long s_sum[6];  // block 0: sum_raw, sum_raw_s, sum_raw2, cons, het, allele
-    __shared__ int s_mm[2];
     __shared__ uint32_t s_cnt[32 * W];
-    __shared__ double s_R;
-    __shared__ uint32_t s_f;
+    __shared__ uint32_t s_total, s_f[2];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(g_smem);
     const PopParams *P = a.prm;
@@ -587,7 +626,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
     if (status != SPG_OK || ld_relaxed_u32(&st->S) == 0u) return;
 
     // tables
-    const bool eco = a.has_eco != 0u, dom = a.dom != 0u;
+    const bool eco = a.has_eco != 0u, dom = GENERAL && a.dom != 0u;
     for (uint32_t i = tid; i < (uint32_t)kBins / 4u; i += BLOCK) {
         cp_async_16(smem0 + SM::kThr + 16u * i, P->table + 4u * i);
         if (eco) cp_async_16(smem0 + SM::kAtt + 16u * i, P->attack + 4u * i);
@@ -623,11 +662,12 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
                                    warp * (2u * 32u * ((uint32_t)W + 3u));  // the helper adds its warp's offset
     const uint32_t slot0 = (uint32_t)(((unsigned long long)a.nslots * blockIdx.x) / gridDim.x);
     const uint32_t slot1 = (uint32_t)(((unsigned long long)a.nslots * (blockIdx.x + 1u)) / gridDim.x);
-    cp_async_wait<0>();
-    bool one_step = false;
-    SlotCounts<BLOCK> sc;
-    load_counts<BLOCK>(a.counts[gen & 1u], a.nslots, sc);
-    uint32_t S = build_directory<SM, BLOCK>(sc, a.nslots, rec_slot, s_scan, one_step);
+    bool one_step = true;
+    if (warp + 1u < NW)
+        one_step = build_directory<SM>(a.counts[gen & 1u], a.nslots, rec_slot, a.guide_bits, s_scan, &s_total);
+    cp_async_wait<0>();  // the tables have landed meanwhile
+    one_step = __syncthreads_and(one_step) != 0;
+    uint32_t S = s_total;
 
     bool again = false;  // a generation without survivors formed once more for its full records
     for (uint32_t done = 0; done < a.n_gen && (gen < target || again);) {
@@ -637,10 +677,11 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
         const uint32_t *par = a.packed[(g + 1u) & 1u];
         uint32_t *out = a.packed[g & 1u];
         const GenRng rng = gen_rng(a, g);
-        if (eco && tid == BLOCK - 32u)  // the resource before consumption, while the generation is formed
-            s_R = a.eco_model == 1u
-                      ? resource_grown_bh(R, growth_rate(a.eco_r, a.eco_r_sd, g, rep, k0, k1), a.eco_K)
-                      : resource_grown(R, a.eco_r, a.eco_K);
+        double grown = 0.0;  // the resource before consumption (the block's last warp), while the generation is formed
+        if (eco && tid == BLOCK - 32u)
+            grown = a.eco_model == 1u
+                        ? resource_grown_bh(R, growth_rate(a.eco_r, a.eco_r_sd, g, rep, k0, k1), a.eco_K)
+                        : resource_grown(R, a.eco_r, a.eco_K);
         LaneStats ts;
         for (uint32_t slot = slot0 + warp; slot < slot1; slot += NW) {
             const uint32_t base = slot * rec_slot, end = min(base + rec_slot, a.n);
@@ -652,10 +693,9 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
                 r = philox_at(a, rng, aj, kMate << 24);
                 uint32_t mom, dad;
                 if constexpr (WEIGHTED) {
-                    weighted_records<SM>(a, a.mate[(g + 1u) & 1u], rng, aj, S, one_step, rec_slot, mom, dad);
+                    weighted_records<SM>(a, a.mate[(g + 1u) & 1u], rng, aj, S, one_step, mom, dad);
                 } else {
-                    mom = locate<SM>(r.x, S, one_step, rec_slot);
-                    dad = locate<SM>(r.y, S, one_step, rec_slot);
+                    locate<SM>(a, r.x, r.y, S, one_step, mom, dad);
                 }
                 load_packed<W>(par + (size_t)mom * (2 * W), pm);
                 load_packed<W>(par + (size_t)dad * (2 * W), pf);
@@ -706,24 +746,24 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
                 // (C) genetic value
                 int32_t raw;
                 uint32_t allele, het = 0;
-                staged_value<W, SM>(stage, lane, smem0 + SM::kFrag, dom, a.two_digits != 0u, raw, allele);
+                staged_value<W, SM>(stage, lane, smem0 + SM::kFrag, dom, GENERAL && a.two_digits != 0u, raw, allele);
 #pragma unroll
                 for (int w = 0; w < W; ++w) het += __popc(ch[w] ^ ch[W + w]);
-                if (a.two_digits) {
+                if (GENERAL && a.two_digits) {
                     allele = 0;
 #pragma unroll
                     for (int w = 0; w < 2 * W; ++w) allele += __popc(ch[w]);
                 }
                 // (D) survival: the bin's threshold scaled by the resource factor
                 uint32_t bin;
-                if (a.narrow_bias) {  // raw + bias stays inside 32 bits
+                if (!GENERAL || a.narrow_bias) {  // raw + bias stays inside 32 bits
                     bin = (uint32_t)min(max((raw + a.bias) >> a.shift, 0), kBins - 1);
                 } else {
                     const long long v = (long long)raw + (long long)a.bias;
                     bin = v < 0 ? 0u : (uint32_t)min(v >> a.shift, (long long)(kBins - 1));
                 }
                 uint32_t thr = sm_u32(SM::kThr + bin * 4u);
-                if (f != kCertain) thr = __umulhi(thr, f);
+                thr = f != kCertain ? __umulhi(thr, f) : thr;
                 const bool alive = valid && min(r.z, kCertain - 1u) < thr;  // kCertain: whatever the draw
                 const uint32_t bits = __ballot_sync(0xFFFFFFFFu, alive);
                 // (E) the survivor's record at its place in the slot
@@ -758,67 +798,62 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
                                  (uint32_t)min((unsigned long long)slot1 * rec_slot, (unsigned long long)a.n), s_cnt,
                                  a.locus_row[g & 1u]);
         __syncthreads();
-        BlockStats *bs = a.block_stats + (size_t)(g & 1u) * gridDim.x;
-        block_stats<SM>(bs + blockIdx.x, warp, lane);
+        GenAcc *acc = a.acc + (size_t)(g % 3u) * kGenAccCopies;
+        add_stats<SM>(acc + blockIdx.x % kGenAccCopies, warp, lane);
         if (!grid_barrier(a.barrier)) {  // the generation fails: every block gives up
             if (tid == 0u) atomicExch(reinterpret_cast<int *>(&st->status), SPG_ERR_TIMEOUT);
             return;
         }
-        // close the generation: every block builds the directory and, with an
-        // ecology, the resource and factor (the same arithmetic in each);
-        // block 0 writes the statistics record and the state
-        load_counts<BLOCK>(a.counts[g & 1u], a.nslots, sc);
-        if (eco && warp == NW - 1u) {
-            unsigned long long x = 0;
-            for (uint32_t b = lane; b < gridDim.x; b += 32u) x += __ldcg(&bs[b].sum[3]);
-            x = warp_sum_u64(x);
-            if (lane == 0u) {
-                s_R = resource_eaten(s_R, x);
-                s_f = factor_q32(s_R, a.eco_R_half);
+        // close the generation: every block builds the directory while its last
+        // warp finishes the resource and factor (the same arithmetic in each);
+        // block 0's last warp writes the statistics record and the state
+        bool wide = true;
+        unsigned long long sum = 0;
+        if (warp + 1u < NW) {
+            wide = build_directory<SM>(a.counts[g & 1u], a.nslots, rec_slot, a.guide_bits, s_scan, &s_total);
+        } else if (eco || blockIdx.x == 0u) {
+            sum = total_stats(acc, lane);
+            const unsigned long long cons = __shfl_sync(0xFFFFFFFFu, sum, 3);
+            if (lane == 0u && eco) {
+                R = resource_eaten(grown, cons);
+                s_f[g & 1u] = factor_q32(R, a.eco_R_half);
             }
         }
-        if (blockIdx.x == 0u && warp < 8u) {
-            if (warp < 6u) {
-                unsigned long long x = 0;
-                for (uint32_t b = lane; b < gridDim.x; b += 32u) x += __ldcg(&bs[b].sum[warp]);
-                x = warp_sum_u64(x);
-                if (lane == 0u) s_sum[warp] = x;
-            } else {
-                int x = warp == 6u ? INT_MAX : INT_MIN;
-                for (uint32_t b = lane; b < gridDim.x; b += 32u)
-                    x = warp == 6u ? min(x, __ldcg(&bs[b].mn)) : max(x, __ldcg(&bs[b].mx));
-                x = warp == 6u ? __reduce_min_sync(0xFFFFFFFFu, x) : __reduce_max_sync(0xFFFFFFFFu, x);
-                if (lane == 0u) s_mm[warp - 6u] = x;
-            }
-        }
-        const uint32_t S_new = build_directory<SM, BLOCK>(sc, a.nslots, rec_slot, s_scan, one_step);
-        if (S_new == 0u) __syncthreads();  // the sums above are visible (the directory was left alone)
-        const uint32_t f_new = eco ? s_f : f;
-        const double R_new = eco ? s_R : R;
+        wide = __syncthreads_and(wide) != 0;
+        const uint32_t S_new = s_total, f_new = eco ? s_f[g & 1u] : f;
         status = S_new == 0u ? SPG_EXTINCT : SPG_OK;
         if (blockIdx.x == 0u) {
-            if (tid == 0u) {
+            if (warp == NW - 1u) {
                 spg_stats *rec = a.ring + (g - 1u) % a.stats_cap;
-                rec->gen = g;
-                rec->n = a.n;
-                rec->s = S_new;
-                rec->status = (uint32_t)status;
-                rec->sum_raw = (long long)s_sum[0];
-                rec->sum_raw_surv = (long long)s_sum[1];
-                rec->sum_raw2 = s_sum[2];
-                rec->consumption = eco ? s_sum[3] : 0ull;
-                rec->het = s_sum[4];
-                rec->allele = s_sum[5];
-                rec->min_raw = s_mm[0];
-                rec->max_raw = s_mm[1];
-                rec->R = eco ? R_new : 0.0;
-                rec->f = f_new;
-                rec->pad = 0;
-                st->gen = g;
-                st->S = S_new;
-                st->f = f_new;
-                st->R = R_new;
-                st->status = status;
+                if (lane == 0u) {
+                    rec->gen = g;
+                    rec->n = a.n;
+                    rec->s = S_new;
+                    rec->status = (uint32_t)status;
+                    rec->R = eco ? R : 0.0;
+                    rec->f = f_new;
+                    rec->pad = 0;
+                    rec->sum_raw = (long long)sum;
+                    st->gen = g;
+                    st->S = S_new;
+                    st->f = f_new;
+                    st->R = R;
+                    st->status = status;
+                } else if (lane < 7u) {
+                    if (lane == 1u) rec->sum_raw_surv = (long long)sum;
+                    if (lane == 2u) rec->sum_raw2 = sum;
+                    if (lane == 3u) rec->consumption = eco ? sum : 0ull;
+                    if (lane == 4u) rec->het = sum;
+                    if (lane == 5u) rec->allele = sum;
+                    if (lane == 6u) {
+                        rec->min_raw = (int)(uint32_t)sum;
+                        rec->max_raw = (int)(sum >> 32);
+                    }
+                }
+                // empty sums for the generation after next: every block has read
+                // what they held, and none adds before the next barrier
+                reinterpret_cast<unsigned long long *>(a.acc + (size_t)((g + 2u) % 3u) * kGenAccCopies)[lane] =
+                    (lane & 7u) == 6u ? kEmptyMinMax : 0ull;
             }
             if (a.locus_row[0]) {  // the counted row to its place; clear for the generation after next
                 uint32_t *row = a.locus_row[g & 1u], *dst = a.locus_ring + (size_t)((g - 1u) % a.locus_cap) * (32u * W);
@@ -844,20 +879,18 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
             if (list) break;  // its full records are written
             again = true;     // form it once more for them (its parents and directory are still there)
             --done;
-            __syncthreads();
             continue;
         }
+        one_step = wide;
         S = S_new;
         f = f_new;
-        R = R_new;
-        __syncthreads();  // s_R, s_f and the sums are read
     }
 }
 
 template <int W, bool LINKED, bool WEIGHTED>
-SoloKernel solo_instance() {
+SoloKernel solo_instance(bool general) {
     SoloKernel k;
-    k.fn = &k_generations<W, LINKED, WEIGHTED>;
+    k.fn = general ? &k_generations<W, LINKED, WEIGHTED, true> : &k_generations<W, LINKED, WEIGHTED, false>;
     k.block = kSoloThreads;
     k.smem = GenSmem<W, LINKED, kSoloThreads>::kBytes;
     return k;

@@ -3,9 +3,9 @@
 
 namespace spg {
 
-SoloKernel solo_kernel_w1(bool linked, bool weighted) {
-    if (linked) return weighted ? solo_instance<1, true, true>() : solo_instance<1, true, false>();
-    return weighted ? solo_instance<1, false, true>() : solo_instance<1, false, false>();
+SoloKernel solo_kernel_w1(bool linked, bool weighted, bool general) {
+    if (linked) return weighted ? solo_instance<1, true, true>(general) : solo_instance<1, true, false>(general);
+    return weighted ? solo_instance<1, false, true>(general) : solo_instance<1, false, false>(general);
 }
 
 }  // namespace spg

@@ -3,9 +3,9 @@
 
 namespace spg {
 
-SoloKernel solo_kernel_w2(bool linked, bool weighted) {
-    if (linked) return weighted ? solo_instance<2, true, true>() : solo_instance<2, true, false>();
-    return weighted ? solo_instance<2, false, true>() : solo_instance<2, false, false>();
+SoloKernel solo_kernel_w2(bool linked, bool weighted, bool general) {
+    if (linked) return weighted ? solo_instance<2, true, true>(general) : solo_instance<2, true, false>(general);
+    return weighted ? solo_instance<2, false, true>(general) : solo_instance<2, false, false>(general);
 }
 
 }  // namespace spg

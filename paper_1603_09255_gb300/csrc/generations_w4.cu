@@ -3,9 +3,9 @@
 
 namespace spg {
 
-SoloKernel solo_kernel_w4(bool linked, bool weighted) {
-    if (linked) return weighted ? solo_instance<4, true, true>() : solo_instance<4, true, false>();
-    return weighted ? solo_instance<4, false, true>() : solo_instance<4, false, false>();
+SoloKernel solo_kernel_w4(bool linked, bool weighted, bool general) {
+    if (linked) return weighted ? solo_instance<4, true, true>(general) : solo_instance<4, true, false>(general);
+    return weighted ? solo_instance<4, false, true>(general) : solo_instance<4, false, false>(general);
 }
 
 }  // namespace spg

@@ -3,9 +3,9 @@
 
 namespace spg {
 
-SoloKernel solo_kernel_w8(bool linked, bool weighted) {
-    if (linked) return weighted ? solo_instance<8, true, true>() : solo_instance<8, true, false>();
-    return weighted ? solo_instance<8, false, true>() : solo_instance<8, false, false>();
+SoloKernel solo_kernel_w8(bool linked, bool weighted, bool general) {
+    if (linked) return weighted ? solo_instance<8, true, true>(general) : solo_instance<8, true, false>(general);
+    return weighted ? solo_instance<8, false, true>(general) : solo_instance<8, false, false>(general);
 }
 
 }  // namespace spg

@@ -757,8 +757,13 @@ __global__ void k_mark_alive(const uint32_t *__restrict__ surv, uint32_t S, uint
 template <int W>
 __global__ void k_pack(const PopParams *__restrict__ P, const uint32_t *__restrict__ geno,
                        const uint32_t *__restrict__ alive, uint32_t n, uint32_t slot_len, uint32_t nslots,
-                       uint32_t *__restrict__ packed, uint32_t *__restrict__ counts, uint2 *__restrict__ mate) {
-    const uint32_t lane = threadIdx.x & 31u, slot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+                       uint32_t *__restrict__ packed, uint32_t *__restrict__ counts, uint2 *__restrict__ mate,
+                       GenAcc *__restrict__ acc, unsigned long long *__restrict__ barrier) {
+    const uint32_t gid = blockIdx.x * blockDim.x + threadIdx.x;
+    if (gid < 3u * kGenAccCopies * 8u)
+        reinterpret_cast<unsigned long long *>(acc)[gid] = (gid & 7u) == 6u ? kEmptyMinMax : 0ull;
+    if (gid == 0u) *barrier = 0ull;
+    const uint32_t lane = threadIdx.x & 31u, slot = gid >> 5;
     if (slot >= nslots) return;
     const uint32_t base = slot * slot_len * 32u;
     uint32_t held = 0;
@@ -1105,7 +1110,7 @@ int launch_survivor_bins(const PopParams *prm, uint32_t words, const uint32_t *g
 
 int launch_pack(const PopParams *prm, uint32_t words, const uint32_t *geno, const uint32_t *surv, uint32_t S, uint32_t n,
                 uint32_t slot_len, uint32_t nslots, uint32_t *alive, uint32_t *packed, uint32_t *counts, uint2 *mate,
-                void *stream) {
+                GenAcc *acc, unsigned long long *barrier, void *stream) {
     cudaStream_t s = (cudaStream_t)stream;
     const size_t words32 = ((size_t)n + 31) / 32;
     cudaError_t e = cudaMemsetAsync(alive, surv ? 0 : 0xFF, words32 * 4, s);
@@ -1114,26 +1119,26 @@ int launch_pack(const PopParams *prm, uint32_t words, const uint32_t *geno, cons
     if (!surv && (n & 31u)) k_mark_tail<<<1, 32, 0, s>>>(alive + words32 - 1, n & 31u);
     const dim3 grid((nslots + 7) / 8), block(256);
     switch (words) {
-        case 1: k_pack<1><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate); break;
-        case 2: k_pack<2><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate); break;
-        case 4: k_pack<4><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate); break;
-        case 8: k_pack<8><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate); break;
+        case 1: k_pack<1><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate, acc, barrier); break;
+        case 2: k_pack<2><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate, acc, barrier); break;
+        case 4: k_pack<4><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate, acc, barrier); break;
+        case 8: k_pack<8><<<grid, block, 0, s>>>(prm, geno, alive, n, slot_len, nslots, packed, counts, mate, acc, barrier); break;
         default: return SPG_ERR_INVALID;
     }
     return cudaGetLastError() == cudaSuccess ? SPG_OK : SPG_ERR_CUDA;
 }
 
-SoloKernel solo_kernel_w1(bool linked, bool weighted);
-SoloKernel solo_kernel_w2(bool linked, bool weighted);
-SoloKernel solo_kernel_w4(bool linked, bool weighted);
-SoloKernel solo_kernel_w8(bool linked, bool weighted);
+SoloKernel solo_kernel_w1(bool linked, bool weighted, bool general);
+SoloKernel solo_kernel_w2(bool linked, bool weighted, bool general);
+SoloKernel solo_kernel_w4(bool linked, bool weighted, bool general);
+SoloKernel solo_kernel_w8(bool linked, bool weighted, bool general);
 
-SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted) {
+SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted, bool general) {
     switch (words) {
-        case 1: return solo_kernel_w1(linked, weighted);
-        case 2: return solo_kernel_w2(linked, weighted);
-        case 4: return solo_kernel_w4(linked, weighted);
-        case 8: return solo_kernel_w8(linked, weighted);
+        case 1: return solo_kernel_w1(linked, weighted, general);
+        case 2: return solo_kernel_w2(linked, weighted, general);
+        case 4: return solo_kernel_w4(linked, weighted, general);
+        case 8: return solo_kernel_w8(linked, weighted, general);
         default: return SoloKernel{};
     }
 }

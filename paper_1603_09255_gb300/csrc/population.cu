@@ -87,14 +87,16 @@ constexpr uint32_t kSoloLaunchGens = 512;  // generations of one launch, at most
 // depend on it).
 int configure_solo(spg_pop *p, const Shape &shape) {
     const PopParams &prm = *p->host_prm;
-    SoloKernel k = solo_kernel(p->words, prm.linked != 0u, prm.weighted != 0u);
+    SoloArgs &a = p->sa;
+    a.narrow_bias = prm.bias < (1 << 30) && prm.bias > -(1 << 30) ? 1u : 0u;  // |genetic value| < 2^26
+    SoloKernel k = solo_kernel(p->words, prm.linked != 0u, prm.weighted != 0u, a.dom || a.two_digits || !a.narrow_bias);
     const int rc = prepare_solo(k);
     if (rc != SPG_OK) return fail(rc, "generation kernel setup failed");
     p->solo = k;
     p->shape = shape;
     const uint32_t nslots = slot_count(p->n);
-    p->solo_blocks = std::max(1u, std::min(std::min(k.resident, kSoloMaxBlocks), nslots / kSoloMinWarps));
-    SoloArgs &a = p->sa;
+    p->solo_blocks =
+        p->n <= 32u * kOneBlockGroups ? 1u : std::max(1u, std::min(k.resident, nslots / kSoloMinWarps));
     a.prm = reinterpret_cast<const PopParams *>(p->arena + p->L.params);
     a.frag = reinterpret_cast<const ValueFragments *>(p->arena + p->L.frag);
     for (uint32_t i = 0; i < 2; ++i) {
@@ -106,7 +108,7 @@ int configure_solo(spg_pop *p, const Shape &shape) {
     a.alive = reinterpret_cast<uint32_t *>(p->arena + p->L.alive);
     a.surv = reinterpret_cast<uint32_t *>(p->arena + p->L.surv0);
     a.state = reinterpret_cast<DevState *>(p->arena + p->L.state);
-    a.block_stats = reinterpret_cast<BlockStats *>(p->arena + p->L.block_stats);
+    a.acc = reinterpret_cast<GenAcc *>(p->arena + p->L.gen_acc);
     a.barrier = reinterpret_cast<unsigned long long *>(p->arena + p->L.barrier);
     a.ring = reinterpret_cast<spg_stats *>(p->arena + p->L.ring);
     for (uint32_t i = 0; i < 10; ++i) {
@@ -120,10 +122,11 @@ int configure_solo(spg_pop *p, const Shape &shape) {
     a.mut_from = prm.kmax ? prm.cdf[0] : 0xFFFFFFFFu;
     a.shift = prm.shift;
     a.bias = prm.bias;
-    a.narrow_bias = prm.bias < (1 << 30) && prm.bias > -(1 << 30) ? 1u : 0u;  // |genetic value| < 2^26
     a.n = p->n;
     a.slot_len = slot_length(p->n);
     a.nslots = nslots;
+    a.guide_bits = 2;  // four to eight entries per slot
+    while ((nslots >> (a.guide_bits - 2)) != 0u && a.guide_bits < (uint32_t)kMaxGuideBits) ++a.guide_bits;
     attach_locus(p);
     return SPG_OK;
 }
@@ -137,8 +140,11 @@ int enqueue_solo(spg_pop *p, uint32_t n_gen) {
         done += a.n_gen;
         a.keep_last = done == n_gen ? 1u : 0u;
         void *params[] = {&a};
-        const cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(p->solo.fn), dim3(p->solo_blocks),
-                                                          dim3(p->solo.block), params, p->solo.smem, p->stream);
+        const void *fn = reinterpret_cast<const void *>(p->solo.fn);
+        const cudaError_t e =
+            p->solo_blocks == 1u
+                ? cudaLaunchKernel(fn, dim3(1), dim3(p->solo.block), params, p->solo.smem, p->stream)
+                : cudaLaunchCooperativeKernel(fn, dim3(p->solo_blocks), dim3(p->solo.block), params, p->solo.smem, p->stream);
         if (e != cudaSuccess) return cuda_fail(e, "generation launch");
     }
     return SPG_OK;
@@ -431,7 +437,6 @@ int spg_restore(spg_pop *p, const void *host, size_t bytes) {
                        (size_t)h.S * 4, cudaMemcpyHostToDevice);
     // per-bucket survivor counts of the replaced run must not leak into the
     // generations about to be replayed
-    if (e == cudaSuccess && p->L.solo) e = cudaMemset(p->arena + p->L.barrier, 0, sizeof(unsigned long long));
     if (e == cudaSuccess && !p->L.solo) e = cudaMemset(p->arena + p->L.buckets, 0, (size_t)2 * p->nbuckets * 4);
     if (e != cudaSuccess) return cuda_fail(e, "restore copy");
     if (p->L.solo) {  // the restored survivors in the slot layout: the next generation's parents

@@ -41,7 +41,7 @@ struct PopLayout {
     // a single biallelic population (solo_layout_for): geno0 = geno1 and
     // surv0 = surv1, no dense buffer, buckets, bins or segment
     bool solo;
-    size_t packed[2], counts[2], mate[2], block_stats, barrier, frag;
+    size_t packed[2], counts[2], mate[2], gen_acc, barrier, frag;
     size_t total;
 };
 

@@ -192,16 +192,23 @@ using GenKernel = void (*)(GenArgs);
 // holding their number per slot.
 constexpr uint32_t kSoloThreads = 512;
 constexpr uint32_t kMaxSlots = 152 * (kSoloThreads / 32);  // one per resident warp on 152 SMs
+constexpr uint32_t kOneBlockGroups = 16;  // groups up to which one block is no slower than several and a grid barrier
 // The per-locus values as f16 elements, laid out as the matrix fragments of
 // the generation kernel (value_fragments): the additive values, or with
 // dominance those of heterozygous and of homozygous loci.
 struct alignas(16) ValueFragments {
     uint32_t table[2][1024];
 };
-struct BlockStats {
+// Statistics of the generation being formed, in kGenAccCopies copies (block b
+// adds to copy b % kGenAccCopies); three generations' worth, by generation % 3.
+struct alignas(64) GenAcc {
     unsigned long long sum[6];  // raw, raw over survivors, raw^2, consumption, heterozygosity, alleles
     int mn, mx;
+    unsigned long long pad;
 };
+constexpr uint32_t kGenAccCopies = 4;
+constexpr unsigned long long kEmptyMinMax = 0x800000007FFFFFFFull;  // mx INT_MIN over mn INT_MAX
+constexpr int kMaxGuideBits = 13;  // the parent draw's top bits that index the directory's guide, at most
 struct SoloArgs {
     const PopParams *prm;
     const ValueFragments *frag;
@@ -212,13 +219,13 @@ struct SoloArgs {
     uint32_t *alive;                   // its survivor bitmap
     uint32_t *surv;                    // its ordered survivor list [N]
     DevState *state;
-    BlockStats *block_stats;           // [2][kSoloMaxBlocks]
+    GenAcc *acc;                       // [3][kGenAccCopies], by generation % 3
     unsigned long long *barrier;       // grid barrier arrivals, a multiple of the grid between launches
     spg_stats *ring;
     uint32_t *locus_row[2];            // per-locus counts of the generation being formed, by parity (null: off)
     uint32_t *locus_ring;              // [locus_cap][L]
     uint32_t locus_cap;
-    uint32_t n, slot_len, nslots;
+    uint32_t n, slot_len, nslots, guide_bits;
     uint32_t keys[20];                 // Philox round keys (word 0, word 1 of each round)
     uint32_t rep, kmax, shift;
     uint32_t mut_from;                 // mutation draws from here on count a mutation (kmax 0: none do)
@@ -230,19 +237,19 @@ struct SoloArgs {
     uint32_t n_gen;                    // generations of this launch
     uint32_t keep_last;                // the last of them is the call's last
 };
-constexpr uint32_t kSoloMaxBlocks = 256;
 struct SoloKernel {
     void (*fn)(SoloArgs) = nullptr;
     uint32_t block = 0, smem = 0, resident = 0;  // resident: blocks on the device at a time
 };
-SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted);
+SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted, bool general);
 int prepare_solo(SoloKernel &k);  // sets the shared-memory limit, fills `resident`
 // Enqueue the slot layout of a generation: bitmap words and per-slot counts
 // of the survivors (surv: their ordered list of S, null for all n), their
-// records packed[slot ...] and, when mate is given, their parent thresholds.
+// records packed[slot ...] and, when mate is given, their parent thresholds;
+// the accumulators and the barrier counter start empty.
 int launch_pack(const PopParams *prm, uint32_t words, const uint32_t *geno, const uint32_t *surv, uint32_t S, uint32_t n,
                 uint32_t slot_len, uint32_t nslots, uint32_t *alive, uint32_t *packed, uint32_t *counts, uint2 *mate,
-                void *stream);
+                GenAcc *acc, unsigned long long *barrier, void *stream);
 
 // Launch shape of the offspring kernel: threads per block, offspring per
 // thread (per lane pair when lanes = 2) and lanes per offspring (1, or 2 for
