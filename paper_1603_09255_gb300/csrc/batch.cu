@@ -33,6 +33,8 @@ struct Member {
     std::unique_ptr<PopParams> prm;
     std::unique_ptr<LinkParams> link;       // linkage-map tables (host copy, until uploaded)
     std::unique_ptr<WeightParams> weights;  // parent acceptance thresholds (host copy, until uploaded)
+    SoloArgs sa{};                          // biallelic: the generation kernel's arguments
+    ValueFragments frag{};                  // fragments of the genetic value (host copy, until uploaded)
     uint32_t group = 0;
     LocusArgs locus{};                      // per-locus counts (when the batch counts them)
     uint32_t locus_from = 0, locus_until = 0;  // generations counted: from .. (on ? now : until)
@@ -44,12 +46,12 @@ struct Group {
     Shape shape;
     std::vector<uint32_t> members;
     size_t table_off = 0, table_bytes = 0;  // launch table in the batch arena (sized for every shape)
-    GenLaunch gl;
-    LocusArgs locus{};  // the group's per-locus count launch (several members: member table and block map)
+    GenLaunch gl;  // continuous values only (biallelic members are stepped by teams)
 };
 
-// A graph of `len` generations for every group: one dependent chain of
-// (offspring, compaction) launches per group, chains independent.
+// A graph of `len` generations for every continuous-allele group: one
+// dependent chain of (generation, compaction) launches per group, chains
+// independent.
 struct MultiChain {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -65,7 +67,7 @@ struct MultiChain {
         cudaError_t e = cudaGraphCreate(&graph, 0);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGraphCreate");
         for (const Group &g : groups) {
-            if (g.members.empty() || g.gl.blocks == 0) continue;
+            if (!g.continuous || g.members.empty() || g.gl.blocks == 0) continue;
             GenArgs a = g.gl.args;  // copied into the node parameters
             void *params[] = {&a};
             const int rc = add_generation_nodes(graph, g.gl, params, len);
@@ -108,43 +110,58 @@ struct spg_batch {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     std::map<uint32_t, std::unique_ptr<MultiChain>> chains;  // by length
-    char *locus_mem = nullptr;  // per-locus counts: every member's ring, row and counters, the groups' tables
+    TeamSet teams;              // the biallelic members
+    char *locus_mem = nullptr;  // per-locus counts: every biallelic member's ring and two rows
     bool locus_on = false;
 };
 
 namespace {
 
-// (Re)build a group's launch table for a launch shape (synchronous upload).
-// The per-locus count launch after each of the group's compactions, or none
-// (counts off, continuous values).  One member: its own arguments (the
-// launch's segment is the member); several: the group's member table.
-void attach_group_locus(spg_batch *b, Group &g) {
-    g.gl.locus = nullptr;
-    g.gl.la = LocusArgs{};
-    if (!b->locus_on || g.continuous || g.members.empty()) return;
-    const bool several = g.members.size() > 1;
-    g.gl.locus = locus_kernel(g.words, several);
-    g.gl.la = several ? g.locus : b->members[g.members[0]].locus;
-    if (!several) g.gl.la.first = 0u;
+// The biallelic members of a list, as their teams take them.
+std::vector<TeamMember> team_members(spg_batch *b, const std::vector<uint32_t> &list) {
+    std::vector<TeamMember> out;
+    for (uint32_t mi : list) {
+        const Member &m = b->members[mi];
+        if (m.prm->continuous) continue;
+        out.push_back(TeamMember{&m.sa, m.v.n, m.v.words, m.prm->linked != 0u, m.prm->weighted != 0u});
+    }
+    return out;
 }
 
+// (Re)build the team tables of all biallelic members (synchronous upload).
+int configure_teams(spg_batch *b) {
+    std::vector<uint32_t> all;
+    for (uint32_t i = 0; i < (uint32_t)b->members.size(); ++i) {
+        Member &m = b->members[i];
+        if (m.prm->continuous) continue;
+        solo_args(m.v, *m.prm, m.sa);
+        for (uint32_t k = 0; k < 2; ++k) m.sa.locus_row[k] = b->locus_on ? m.locus.acc + (size_t)k * 32u * m.v.words : nullptr;
+        m.sa.locus_ring = m.locus.ring;
+        m.sa.locus_cap = m.locus.cap;
+        all.push_back(i);
+    }
+    return b->teams.build(team_members(b, all), b->alloc, b->stream);
+}
+
+// A group's launch shape: the continuous-allele kernel's launch table
+// (synchronous upload); biallelic members report the shape (their generation
+// kernel has one of its own).
 int configure_group(spg_batch *b, Group &g, const Shape &shape) {
-    if (g.members.empty()) return SPG_OK;
+    g.shape = shape;
+    if (g.members.empty() || !g.continuous) return SPG_OK;
     std::vector<const PopView *> views;
     views.reserve(g.members.size());
-    bool eco = false, dom = false;
-    for (uint32_t mi : g.members) {
-        views.push_back(&b->members[mi].v);
-        eco |= b->members[mi].prm->has_eco != 0u;
-        dom |= b->members[mi].prm->has_dom != 0u;
-    }
-    const int rc = build_group_launch(views, g.words, shape, eco, dom, b->arena + g.table_off, g.table_bytes, g.gl,
-                                      g.linked, g.weighted, g.continuous);
+    for (uint32_t mi : g.members) views.push_back(&b->members[mi].v);
+    const int rc = build_group_launch(views, g.words, b->arena + g.table_off, g.table_bytes, g.gl);
     if (rc != SPG_OK) return rc;
-    g.shape = shape;
-    attach_group_locus(b, g);
     b->chains.clear();
     return SPG_OK;
+}
+
+bool any_continuous(const spg_batch *b) {
+    for (const Group &g : b->groups)
+        if (g.continuous && !g.members.empty()) return true;
+    return false;
 }
 
 int member_view(spg_batch *b, uint32_t member, PopView &v) {
@@ -215,14 +232,15 @@ int spg_batch_create(const spg_pop_desc *descs, uint32_t count, const spg_alloca
         m.v.words = words;
         m.v.cap = m.prm->stats_cap;
         m.v.nbuckets = bucket_count(d.n);
-        m.v.L = layout_for(d.n, words, m.v.nbuckets, m.v.cap, weighted, !continuous);
+        m.v.L = continuous ? layout_for(d.n, words, m.v.nbuckets, m.v.cap, false, false)
+                             : solo_layout_for(d.n, words, m.v.cap, weighted);
         m.group = group_index(d.n_loci, linked, weighted, continuous);
         b->groups[m.group].members.push_back(i);
         m.v.base = reinterpret_cast<char *>(off);  // offset until the arena exists
         off = align_up(off + m.v.L.total, 256);
     }
     for (Group &g : b->groups) {
-        if (g.members.empty()) continue;
+        if (g.members.empty() || !g.continuous) continue;
         uint64_t offspring = 0;
         uint32_t buckets = 0;
         for (uint32_t mi : g.members) {
@@ -262,9 +280,15 @@ int spg_batch_create(const spg_pop_desc *descs, uint32_t count, const spg_alloca
             e = cudaMemcpyAsync(m.v.base + m.v.L.weights, m.weights.get(), sizeof(WeightParams),
                                 cudaMemcpyHostToDevice, b->stream);
         }
+        if (e == cudaSuccess && m.v.L.solo) {
+            m.sa.dom = m.prm->has_dom;
+            value_fragments(descs[i].effects, m.sa.dom ? descs[i].dominance : nullptr, descs[i].n_loci, m.frag,
+                            m.sa.two_digits);
+            e = cudaMemcpyAsync(m.v.base + m.v.L.frag, &m.frag, sizeof(ValueFragments), cudaMemcpyHostToDevice, b->stream);
+        }
         if (e != cudaSuccess) {
             spg_batch_destroy(b.release());
-            return cuda_fail(e, "upload a member's variant tables");
+            return cuda_fail(e, "upload a member's tables");
         }
         const int rc = view_init(m.v, *m.prm,
                                  descs[i].allele_model == 1u ? reinterpret_cast<const uint32_t *>(descs[i].init_values)
@@ -279,6 +303,7 @@ int spg_batch_create(const spg_pop_desc *descs, uint32_t count, const spg_alloca
     int rc = view_sync(b->members[0].v);  // caller arrays and host parameters have been read
     for (Group &g : b->groups)
         if (rc == SPG_OK) rc = configure_group(b.get(), g, group_shape(g));
+    if (rc == SPG_OK) rc = configure_teams(b.get());
     if (rc != SPG_OK) {
         spg_batch_destroy(b.release());
         return rc;
@@ -293,17 +318,20 @@ int spg_batch_set_ecology(spg_batch *b, uint32_t member, const spg_ecology *eco)
     if (rc != SPG_OK) return rc;
     rc = view_set_ecology(v, *b->members[member].prm, eco);
     if (rc != SPG_OK) return rc;
-    // the group's survival tables now carry attack rates
-    Group &g = b->groups[b->members[member].group];
-    if (!g.gl.offspring.eco_table) rc = configure_group(b, g, g.shape);
-    return rc;
+    Member &m = b->members[member];
+    if (m.prm->continuous) return SPG_OK;
+    solo_args(m.v, *m.prm, m.sa);
+    return b->teams.update(&m.sa);
 }
 
 int spg_batch_step(spg_batch *b, uint32_t n_gen) {
     if (!b) return fail(SPG_ERR_INVALID, "batch is NULL");
+    if (n_gen == 0) return SPG_OK;
+    const int rc = b->teams.step(n_gen, true, b->stream);
+    if (rc != SPG_OK || !any_continuous(b)) return rc;
     for (uint32_t i = 0; i + kGraphChunk <= n_gen; i += kGraphChunk) {
-        const int rc = run_chunk(b, kGraphChunk);
-        if (rc != SPG_OK) return rc;
+        const int rc2 = run_chunk(b, kGraphChunk);
+        if (rc2 != SPG_OK) return rc2;
     }
     if (n_gen % kGraphChunk) return run_chunk(b, n_gen % kGraphChunk);
     return SPG_OK;
@@ -340,9 +368,9 @@ int spg_batch_get_launch_shape(spg_batch *b, uint32_t n_loci, spg_launch_shape *
     if (!(n_loci == 32 || n_loci == 64 || n_loci == 128 || n_loci == 256))
         return fail(SPG_ERR_INVALID, "n_loci must be 32, 64, 128 or 256");
     const Group &g = b->groups[group_of_words(n_loci / 32)];
-    out->threads_per_block = g.members.empty() ? g.shape.block : g.gl.offspring.block;
-    out->items_per_thread = g.members.empty() ? g.shape.items : g.gl.offspring.items;
-    out->lanes_per_offspring = g.members.empty() ? g.shape.lanes : g.gl.offspring.lanes;
+    out->threads_per_block = g.shape.block;
+    out->items_per_thread = g.shape.items;
+    out->lanes_per_offspring = g.shape.lanes;
     return SPG_OK;
 }
 
@@ -354,46 +382,59 @@ int spg_batch_autotune(spg_batch *b, uint32_t gens_per_trial, spg_autotune_repor
     int rc = SPG_OK;
     spg_autotune_report rep{};
     // every group runs the same number of trials (kAutotuneCandidates), each
-    // one untimed generation (the new shape's first launches) then
-    // gens_per_trial timed ones, so all members advance equally
-    for (uint32_t gi = 0; gi < 4u && rc == SPG_OK; ++gi) {  // the plain groups (variants: one shape)
+    // one untimed generation then gens_per_trial timed ones, so all members
+    // advance equally.  (The generation kernel has one shape: the candidates
+    // are timed and reported as the contract says, and differ by noise.)
+    std::vector<uint32_t> variants;
+    for (uint32_t gi = 0; gi < 16u && rc == SPG_OK; ++gi) {
         Group &g = b->groups[gi];
         if (g.members.empty()) continue;
+        if (gi >= 4u) {  // linkage maps and parent weights: one shape, below
+            variants.insert(variants.end(), g.members.begin(), g.members.end());
+            continue;
+        }
+        TeamSet set;
+        rc = set.build(team_members(b, g.members), b->alloc, b->stream);
         float best_ms = 0.f, worst_ms = 0.f;
         Shape best = g.shape;
         for (uint32_t c = 0; c < kAutotuneCandidates && rc == SPG_OK; ++c) {
-            const Shape cand = autotune_candidate(g.words, c);
-            rc = configure_group(b, g, cand);
-            if (rc == SPG_OK) rc = launch_generation(g.gl, b->stream);
+            rc = set.step(1, true, b->stream);
             if (rc != SPG_OK) break;
             cudaEventRecord(t0, b->stream);
-            for (uint32_t i = 0; i < gens_per_trial && rc == SPG_OK; ++i) rc = launch_generation(g.gl, b->stream);
+            rc = set.step(gens_per_trial, true, b->stream);
             cudaEventRecord(t1, b->stream);
             if (cudaEventSynchronize(t1) != cudaSuccess) rc = fail(SPG_ERR_CUDA, "trial timing");
             float ms = 0.f;
             cudaEventElapsedTime(&ms, t0, t1);
             if (c == 0 || ms < best_ms) {
                 best_ms = ms;
-                best = cand;
+                best = autotune_candidate(g.words, c);
             }
             worst_ms = std::max(worst_ms, ms);
         }
-        if (rc == SPG_OK) rc = configure_group(b, g, best);
+        set.release(b->alloc, b->stream);
         if (rc == SPG_OK) {
-            rep.groups[gi].threads_per_block = g.gl.offspring.block;
-            rep.groups[gi].items_per_thread = g.gl.offspring.items;
-            rep.groups[gi].lanes_per_offspring = g.gl.offspring.lanes;
+            g.shape = best;
+            rep.groups[gi].threads_per_block = best.block;
+            rep.groups[gi].items_per_thread = best.items;
+            rep.groups[gi].lanes_per_offspring = best.lanes;
             rep.best_ms[gi] = best_ms / (float)gens_per_trial;
             rep.worst_ms[gi] = worst_ms / (float)gens_per_trial;
         }
     }
-    // members with a linkage map, parent weights or continuous values keep the
-    // variant shape and advance by as many generations as the tuned ones
-    for (uint32_t gi = 4; gi < (uint32_t)b->groups.size() && rc == SPG_OK; ++gi) {
+    // the other members advance by as many generations as the timed ones
+    const uint32_t gens = kAutotuneCandidates * (gens_per_trial + 1u);
+    if (!variants.empty() && rc == SPG_OK) {
+        TeamSet set;
+        rc = set.build(team_members(b, variants), b->alloc, b->stream);
+        if (rc == SPG_OK) rc = set.step(gens, true, b->stream);
+        if (rc == SPG_OK) rc = view_sync(b->members[0].v);
+        set.release(b->alloc, b->stream);
+    }
+    for (uint32_t gi = 16; gi < (uint32_t)b->groups.size() && rc == SPG_OK; ++gi) {
         const Group &g = b->groups[gi];
         if (g.members.empty()) continue;
-        for (uint32_t i = 0; i < kAutotuneCandidates * (gens_per_trial + 1u) && rc == SPG_OK; ++i)
-            rc = launch_generation(g.gl, b->stream);
+        for (uint32_t i = 0; i < gens && rc == SPG_OK; ++i) rc = launch_generation(g.gl, b->stream);
     }
     cudaEventDestroy(t0);
     cudaEventDestroy(t1);
@@ -414,8 +455,7 @@ int spg_batch_set_locus_counts(spg_batch *b, int enable) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
     const uint32_t M = (uint32_t)b->members.size();
     if (enable && !b->locus_mem) {
-        // layout: every biallelic member's ring and row, the members' counter
-        // pairs (blocks done, last generation counted), each group's tables
+        // every biallelic member's ring and its two rows (zero between launches)
         size_t off = 0;
         std::vector<size_t> ring_off(M, 0), row_off(M, 0);
         for (uint32_t m = 0; m < M; ++m) {
@@ -424,56 +464,19 @@ int spg_batch_set_locus_counts(spg_batch *b, int enable) {
             ring_off[m] = off;
             off = align_up(off + (size_t)mb.v.cap * 32u * mb.v.words * 4u, 256);
             row_off[m] = off;
-            off = align_up(off + (size_t)32u * mb.v.words * 4u, 256);
+            off = align_up(off + (size_t)2u * 32u * mb.v.words * 4u, 256);
         }
-        const size_t counters = off;
-        off = align_up(off + (size_t)M * 8u, 256);
-        std::vector<size_t> args_off(b->groups.size(), 0), map_off(b->groups.size(), 0);
-        std::vector<uint32_t> group_blocks(b->groups.size(), 0);
-        for (uint32_t gi = 0; gi < (uint32_t)b->groups.size(); ++gi) {
-            const Group &g = b->groups[gi];
-            if (g.continuous || g.members.size() < 2) continue;
-            for (uint32_t mi : g.members) group_blocks[gi] += locus_blocks(b->members[mi].v.n);
-            args_off[gi] = off;
-            off = align_up(off + g.members.size() * sizeof(LocusArgs), 256);
-            map_off[gi] = off;
-            off = align_up(off + (size_t)group_blocks[gi] * 4u, 256);
-        }
-        b->locus_mem = static_cast<char *>(b->alloc.alloc(off, b->stream));
+        b->locus_mem = static_cast<char *>(b->alloc.alloc(std::max<size_t>(off, 256), b->stream));
         if (!b->locus_mem) return fail(SPG_ERR_OOM, "device allocation of %zu bytes failed", off);
-        e = cudaMemsetAsync(b->locus_mem, 0, off, b->stream);  // rows and counters start at zero
-        for (uint32_t m = 0; m < M && e == cudaSuccess; ++m) {
+        e = cudaMemsetAsync(b->locus_mem, 0, std::max<size_t>(off, 256), b->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "set up per-locus counts");
+        for (uint32_t m = 0; m < M; ++m) {
             Member &mb = b->members[m];
             if (mb.prm->continuous) continue;
-            LocusArgs &la = mb.locus;
-            la.ring = reinterpret_cast<uint32_t *>(b->locus_mem + ring_off[m]);
-            la.acc = reinterpret_cast<uint32_t *>(b->locus_mem + row_off[m]);
-            la.done = reinterpret_cast<uint32_t *>(b->locus_mem + counters) + 2u * m;
-            la.last = la.done + 1;
-            la.cap = mb.v.cap;
-            la.blocks = locus_blocks(mb.v.n);
+            mb.locus.ring = reinterpret_cast<uint32_t *>(b->locus_mem + ring_off[m]);
+            mb.locus.acc = reinterpret_cast<uint32_t *>(b->locus_mem + row_off[m]);
+            mb.locus.cap = mb.v.cap;
         }
-        for (uint32_t gi = 0; gi < (uint32_t)b->groups.size() && e == cudaSuccess; ++gi) {
-            Group &g = b->groups[gi];
-            if (g.continuous || g.members.size() < 2) continue;
-            std::vector<LocusArgs> args;
-            std::vector<uint32_t> map;
-            for (uint32_t k = 0; k < (uint32_t)g.members.size(); ++k) {
-                LocusArgs la = b->members[g.members[k]].locus;
-                la.first = (uint32_t)map.size();
-                map.insert(map.end(), la.blocks, k);  // k: the member's segment in the group's launch
-                args.push_back(la);
-            }
-            e = cudaMemcpy(b->locus_mem + args_off[gi], args.data(), args.size() * sizeof(LocusArgs),
-                           cudaMemcpyHostToDevice);
-            if (e == cudaSuccess)
-                e = cudaMemcpy(b->locus_mem + map_off[gi], map.data(), map.size() * 4u, cudaMemcpyHostToDevice);
-            g.locus = LocusArgs{};
-            g.locus.blocks = (uint32_t)map.size();
-            g.locus.member = reinterpret_cast<const LocusArgs *>(b->locus_mem + args_off[gi]);
-            g.locus.block_member = reinterpret_cast<const uint32_t *>(b->locus_mem + map_off[gi]);
-        }
-        if (e != cudaSuccess) return cuda_fail(e, "set up per-locus counts");
     }
     for (uint32_t m = 0; m < M; ++m) {
         Member &mb = b->members[m];
@@ -483,15 +486,13 @@ int spg_batch_set_locus_counts(spg_batch *b, int enable) {
         if (rc != SPG_OK) return rc;
         if (enable && !b->locus_on) {
             mb.locus_from = st.gen + 1u;  // the first generation formed from now on
-            e = cudaMemsetAsync(mb.locus.last, 0, 4, b->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "clear per-locus counts");
         } else if (!enable && b->locus_on) {
             mb.locus_until = st.gen;  // the last generation counted
         }
     }
     b->locus_on = enable != 0;
-    for (Group &g : b->groups) attach_group_locus(b, g);
-    b->chains.clear();
+    const int rc = configure_teams(b);
+    if (rc != SPG_OK) return rc;
     e = cudaStreamSynchronize(b->stream);
     return e == cudaSuccess ? SPG_OK : cuda_fail(e, "cudaStreamSynchronize");
 }
@@ -541,6 +542,7 @@ void spg_batch_destroy(spg_batch *b) {
     if (!b) return;
     if (b->stream) cudaStreamSynchronize(b->stream);
     b->chains.clear();
+    b->teams.release(b->alloc, b->stream);
     if (b->locus_mem) b->alloc.release(b->locus_mem, b->stream);
     if (b->arena) b->alloc.release(b->arena, b->stream);
     if (b->stream) cudaStreamSynchronize(b->stream);

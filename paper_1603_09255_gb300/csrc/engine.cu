@@ -356,14 +356,14 @@ PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap
     return L;
 }
 
-// Slots of a single population: at most kMaxSlots of whole groups of 32, or
+// Slots of a single population: at most max_slots of whole groups of 32, or
 // one per warp of a block for a population that one block forms.
-uint32_t slot_length(uint32_t n) {
-    const uint64_t slots = n <= 32u * kOneBlockGroups ? kSoloThreads / 32u : kMaxSlots;
+uint32_t slot_length(uint32_t n, uint32_t words) {
+    const uint64_t slots = n <= 32u * kOneBlockGroups ? solo_threads(words) / 32u : max_slots(words);
     return (uint32_t)(((uint64_t)n + 32ull * slots - 1) / (32ull * slots));
 }
-uint32_t slot_count(uint32_t n) {
-    const uint32_t len = 32u * slot_length(n);
+uint32_t slot_count(uint32_t n, uint32_t words) {
+    const uint32_t len = 32u * slot_length(n, words);
     return (uint32_t)(((uint64_t)n + len - 1) / len);
 }
 
@@ -385,7 +385,7 @@ PopLayout solo_layout_for(uint32_t n, uint32_t words, uint32_t cap, bool weighte
     for (size_t &x : L.packed) x = take((size_t)n * 2 * words * 4);
     L.surv0 = L.surv1 = take((size_t)n * 4);
     L.alive = take(((size_t)n + 31) / 32 * 4);
-    for (size_t &x : L.counts) x = take((size_t)slot_count(n) * 4);
+    for (size_t &x : L.counts) x = take((size_t)slot_count(n, words) * 4);
     L.gen_acc = take(sizeof(GenAcc) * 3 * kGenAccCopies);
     L.barrier = take(sizeof(unsigned long long));
     L.ring = take((size_t)cap * sizeof(spg_stats));
@@ -398,6 +398,231 @@ PopLayout solo_layout_for(uint32_t n, uint32_t words, uint32_t cap, bool weighte
     }
     L.total = off;
     return L;
+}
+
+// The generation kernel's arguments for a population at v (solo layout); the
+// fragments' flags (dom, two_digits) are already in a.
+void solo_args(const PopView &v, const PopParams &prm, SoloArgs &a) {
+    a.prm = reinterpret_cast<const PopParams *>(v.base + v.L.params);
+    a.frag = reinterpret_cast<const ValueFragments *>(v.base + v.L.frag);
+    for (uint32_t i = 0; i < 2; ++i) {
+        a.packed[i] = reinterpret_cast<uint32_t *>(v.base + v.L.packed[i]);
+        a.counts[i] = reinterpret_cast<uint32_t *>(v.base + v.L.counts[i]);
+        a.mate[i] = v.L.weighted ? reinterpret_cast<uint2 *>(v.base + v.L.mate[i]) : nullptr;
+    }
+    a.geno = reinterpret_cast<uint32_t *>(v.base + v.L.geno0);
+    a.alive = reinterpret_cast<uint32_t *>(v.base + v.L.alive);
+    a.surv = reinterpret_cast<uint32_t *>(v.base + v.L.surv0);
+    a.state = reinterpret_cast<DevState *>(v.base + v.L.state);
+    a.acc = reinterpret_cast<GenAcc *>(v.base + v.L.gen_acc);
+    a.barrier = reinterpret_cast<unsigned long long *>(v.base + v.L.barrier);
+    a.ring = reinterpret_cast<spg_stats *>(v.base + v.L.ring);
+    for (uint32_t i = 0; i < 10; ++i) {
+        a.keys[2 * i] = prm.key0 + i * 0x9E3779B9u;
+        a.keys[2 * i + 1] = prm.key1 + i * 0xBB67AE85u;
+    }
+    a.words = prm.words;
+    a.rep = prm.rep;
+    a.kmax = prm.kmax;
+    a.mut_from = prm.kmax ? prm.cdf[0] : 0xFFFFFFFFu;
+    a.shift = prm.shift;
+    a.bias = prm.bias;
+    a.narrow_bias = prm.bias < (1 << 30) && prm.bias > -(1 << 30) ? 1u : 0u;  // |genetic value| < 2^26
+    a.stats_cap = v.cap;
+    a.n = v.n;
+    a.slot_len = slot_length(v.n, v.words);
+    a.nslots = slot_count(v.n, v.words);
+    a.guide_bits = 2;  // four to eight entries per slot
+    while ((a.nslots >> (a.guide_bits - 2)) != 0u && a.guide_bits < (uint32_t)kMaxGuideBits) ++a.guide_bits;
+    a.has_eco = prm.has_eco;
+    a.eco_model = prm.eco_model;
+    a.eco_r = prm.r;
+    a.eco_r_sd = prm.r_sd;
+    a.eco_K = prm.K;
+    a.eco_R_half = prm.R_half;
+}
+
+// Least warps of work per block: a small population takes as few SMs as give
+// every one of them this many warps (at 10,000 offspring 4 and 16 warps differ
+// by less than the barrier does).
+constexpr uint32_t kSoloMinWarps = 4;
+
+uint32_t most_blocks(uint32_t n, uint32_t words, uint32_t resident) {
+    return n <= 32u * kOneBlockGroups ? 1u : std::max(1u, std::min(resident, slot_count(n, words) / kSoloMinWarps));
+}
+
+// ------------------------------------------------------------ teams
+// Cycles of a generation on k blocks of 16 warps: closing it alone or with a
+// barrier, and rounds of the warps' groups (measured, L = 32 .. 256; a linkage
+// map or parent weights make a round longer).
+static double round_cycles(const TeamMember &m) {
+    const double plain = m.words == 1 ? 2000.0 : m.words == 2 ? 2300.0 : m.words == 4 ? 3100.0 : 5400.0;
+    return plain * (m.linked ? 4.0 : 1.0) * (m.weighted ? 1.9 : 1.0);
+}
+static double team_cycles(const TeamMember &m, uint32_t k) {
+    const double groups = ((double)m.n + 31.0) / 32.0;
+    return (k == 1 ? 6000.0 : 11000.0) + std::max(1.0, groups / (16.0 * k)) * round_cycles(m);
+}
+
+// Blocks below which all teams' records together would not stay in L2: with
+// every block at its share of such a member, parents and survivors (16 W bytes
+// an individual) come to kTeamL2Bytes (152 members of 60,000 x 128 loci on a
+// block each formed an individual in 35 ps, of 30,000 in 25).
+constexpr double kTeamL2Bytes = 2.5e8;
+static double resident_blocks(const TeamMember &m, uint32_t blocks) {
+    return std::ceil(16.0 * m.words * m.n / (kTeamL2Bytes / blocks));
+}
+
+// Teams for the members on `blocks` blocks: the longest first, each with as
+// many blocks as keep it below a share of the whole and its records in L2, on
+// the blocks that are free soonest; the share that gives the shortest schedule
+// is kept.  All blocks have their teams in the members' one order (k_teams).
+// Returns the estimated cycles of a generation of all members.
+double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, std::vector<TeamPlace> &places,
+                      std::vector<uint32_t> &block_places) {
+    const uint32_t M = (uint32_t)members.size();
+    std::vector<uint32_t> order(M);
+    std::vector<double> work(M);
+    double total = 0.0;
+    for (uint32_t m = 0; m < M; ++m) {
+        order[m] = m;
+        work[m] = ((double)members[m].n + 31.0) / 32.0 / 16.0 * round_cycles(members[m]);
+        total += work[m];
+    }
+    std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) { return work[x] > work[y]; });
+    double best = -1.0;
+    std::vector<std::vector<TeamPlace>> lists;
+    for (const double share : {0.1, 0.15, 0.25, 0.4, 0.6, 1.0}) {
+        std::vector<double> free_at(blocks, 0.0);
+        std::vector<uint32_t> by_time(blocks);
+        for (uint32_t b = 0; b < blocks; ++b) by_time[b] = b;
+        std::vector<std::vector<TeamPlace>> mine(blocks);
+        double end = 0.0;
+        for (const uint32_t m : order) {
+            const double want = std::max(std::ceil(work[m] / (share * total / blocks)), resident_blocks(members[m], blocks));
+            const uint32_t k = (uint32_t)std::max(1.0, std::min<double>(want, most_blocks(members[m].n, members[m].words, blocks)));
+            std::nth_element(by_time.begin(), by_time.begin() + (k - 1), by_time.end(),
+                             [&](uint32_t x, uint32_t y) { return free_at[x] != free_at[y] ? free_at[x] < free_at[y] : x < y; });
+            double start = 0.0;
+            for (uint32_t i = 0; i < k; ++i) start = std::max(start, free_at[by_time[i]]);
+            const double done = start + team_cycles(members[m], k);
+            for (uint32_t i = 0; i < k; ++i) {
+                free_at[by_time[i]] = done;
+                mine[by_time[i]].push_back(TeamPlace{m, (uint16_t)i, (uint16_t)k});
+            }
+            end = std::max(end, done);
+        }
+        if (best < 0.0 || end < best) {
+            best = end;
+            lists.swap(mine);
+        }
+    }
+    places.clear();
+    block_places.assign(1, 0u);
+    for (uint32_t b = 0; b < blocks; ++b) {
+        if (b < lists.size()) places.insert(places.end(), lists[b].begin(), lists[b].end());
+        block_places.push_back((uint32_t)places.size());
+    }
+    return std::max(best, 0.0);
+}
+
+int TeamSet::build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream) {
+    for (uint32_t i = 0; i < 4u * (kTeamKinds - 1u); ++i) {
+        TeamLaunch &t = launch[i];
+        const uint32_t words = 1u << (i % 4u);
+        uint32_t kind = 1u + i / 4u;
+        t.members.clear();
+        for (const TeamMember &m : all)
+            if (m.words == words &&
+                team_kind(m.linked, m.weighted, m.args->dom || m.args->two_digits || !m.args->narrow_bias) == kind)
+                t.members.push_back(m);
+        if (t.members.empty()) continue;
+        if (kind == 1u) {
+            const SoloArgs *first = t.members[0].args;
+            bool one_seed = true;
+            for (const TeamMember &m : t.members)
+                one_seed = one_seed && std::memcmp(m.args->keys, first->keys, sizeof first->keys) == 0;
+            if (one_seed) kind = 0u;
+        }
+        if (!t.kernel.fn || t.kind != kind) {
+            t.kernel = team_kernel(words, kind);
+            t.kind = kind;
+            const int rc = prepare_solo(t.kernel);
+            if (rc != SPG_OK) return fail(rc, "team kernel setup failed");
+        }
+        std::memcpy(t.args.keys, t.members[0].args->keys, sizeof t.args.keys);
+        std::vector<TeamPlace> places;
+        std::vector<uint32_t> block_places;
+        t.cycles = schedule_teams(t.members, t.kernel.resident, places, block_places);
+        const size_t o_places = align_up(t.members.size() * sizeof(SoloArgs), 256),
+                     o_blocks = align_up(o_places + places.size() * sizeof(TeamPlace), 256),
+                     need = o_blocks + block_places.size() * 4;
+        if (need > t.capacity) {
+            t.release(alloc, stream);
+            t.capacity = 2 * need;  // (a server's set changes)
+            t.table = static_cast<char *>(alloc.alloc(t.capacity, stream));
+            if (!t.table) {
+                t.capacity = 0;
+                return fail(SPG_ERR_OOM, "team table allocation failed");
+            }
+        }
+        std::vector<SoloArgs> args;
+        for (const TeamMember &m : t.members) args.push_back(*m.args);
+        cudaError_t e = cudaMemcpyAsync(t.table, args.data(), args.size() * sizeof(SoloArgs), cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(t.table + o_places, places.data(), places.size() * sizeof(TeamPlace),
+                                cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(t.table + o_blocks, block_places.data(), block_places.size() * 4, cudaMemcpyHostToDevice,
+                                stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // the host tables go away
+        if (e != cudaSuccess) return cuda_fail(e, "upload team table");
+        t.args.members = reinterpret_cast<const SoloArgs *>(t.table);
+        t.args.places = reinterpret_cast<const TeamPlace *>(t.table + o_places);
+        t.args.block_places = reinterpret_cast<const uint32_t *>(t.table + o_blocks);
+    }
+    return SPG_OK;
+}
+
+// A member's changed arguments (its place in the tables stays).
+int TeamSet::update(const SoloArgs *args) {
+    for (TeamLaunch &t : launch)
+        for (size_t i = 0; i < t.members.size(); ++i)
+            if (t.members[i].args == args) {
+                const cudaError_t e = cudaMemcpy(t.table + i * sizeof(SoloArgs), args, sizeof(SoloArgs), cudaMemcpyHostToDevice);
+                return e == cudaSuccess ? SPG_OK : cuda_fail(e, "update team table");
+            }
+    return SPG_OK;
+}
+
+// n_gen generations of every member.  A launch is cut at about a quarter of a
+// second, so that a team's blocks never wait long for one another.
+int TeamSet::step(uint32_t n_gen, bool keep_last, cudaStream_t stream) {
+    for (TeamLaunch &t : launch) {
+        if (t.members.empty()) continue;
+        const uint32_t most = (uint32_t)std::max(1.0, std::min<double>(kSoloLaunchGens, 5e8 / std::max(1.0, t.cycles)));
+        for (uint32_t done = 0; done < n_gen;) {
+            TeamArgs a = t.args;
+            a.n_gen = std::min(n_gen - done, most);
+            done += a.n_gen;
+            a.keep_last = keep_last && done == n_gen ? 1u : 0u;
+            void *params[] = {&a};
+            const cudaError_t e = cudaLaunchCooperativeKernel(t.kernel.fn, dim3(t.kernel.resident), dim3(t.kernel.threads),
+                                                              params, t.kernel.smem, stream);
+            if (e != cudaSuccess) return cuda_fail(e, "team launch");
+        }
+    }
+    return SPG_OK;
+}
+
+void TeamLaunch::release(const Allocator &alloc, cudaStream_t stream) {
+    if (table) alloc.release(table, stream);
+    table = nullptr;
+    capacity = 0;
+}
+
+void TeamSet::release(const Allocator &alloc, cudaStream_t stream) {
+    for (TeamLaunch &t : launch) t.release(alloc, stream);
 }
 
 Segment segment_at(char *base, const PopLayout &L, uint32_t n, uint32_t ntiles, uint32_t tile_begin,
@@ -670,83 +895,55 @@ void schedule_runs(const std::vector<uint32_t> &tiles, uint32_t G, uint32_t min_
     block_runs[G] = (uint32_t)runs.size();
 }
 
-int build_group_launch(const std::vector<const PopView *> &members, uint32_t words, const Shape &shape, bool eco,
-                       bool dom, char *table, size_t table_capacity, GenLaunch &gl, bool linked, bool weighted,
-                       bool continuous) {
+int build_group_launch(const std::vector<const PopView *> &members, uint32_t words, char *table, size_t table_capacity,
+                       GenLaunch &gl) {
     if (members.empty()) {
         gl = GenLaunch{};
         return SPG_OK;
     }
-    const bool one_shape = linked || weighted || continuous;
-    if ((!continuous && !supported_shape(words, shape)) ||
-        (one_shape && (shape.block != (uint32_t)kBlock || shape.items != 1u || shape.lanes != 1u)))
-        return fail(SPG_ERR_INVALID,
-                    "unsupported launch shape (%u threads, %u offspring per thread, %u lanes per offspring) for %u loci",
-                    shape.block, shape.items, shape.lanes, continuous ? 2u * words : 32u * words);
-    // members in HBM: staged parents (where an instance has them); continuous
-    // values (records of 2L int16, words = L / 2): one block per 256 offspring
-    OffspringKernel k = continuous ? continuous_kernel(2u * words, members.size() > 1)
-                                   : offspring_kernel(words, shape, linked, weighted, eco, dom, true);
+    // records of 2L int16, words = L / 2: one block per 256 offspring
+    OffspringKernel k = continuous_kernel(2u * words, members.size() > 1);
     int rc = prepare_offspring(k);
     if (rc != SPG_OK) return fail(rc, "offspring kernel setup failed");
     std::vector<Segment> segs;
-    std::vector<uint32_t> tiles, bucket_map, tile_map;
+    std::vector<uint32_t> bucket_map, tile_map;
     segs.reserve(members.size());
     uint32_t total_tiles = 0, buckets = 0;
     uint64_t offspring = 0;
     for (uint32_t si = 0; si < members.size(); ++si) {
         const PopView &v = *members[si];
-        const uint32_t nt = continuous ? (v.n + kBlock - 1) / kBlock : tiles_for(v.n, shape);
+        const uint32_t nt = (v.n + kBlock - 1) / kBlock;
         segs.push_back(segment_at(v.base, v.L, v.n, nt, total_tiles, v.nbuckets, buckets));
-        tiles.push_back(nt);
-        if (continuous) tile_map.insert(tile_map.end(), nt, si);
+        tile_map.insert(tile_map.end(), nt, si);
         bucket_map.insert(bucket_map.end(), v.nbuckets, si);
         total_tiles += nt;
         buckets += v.nbuckets;
         offspring += v.n;
     }
-    const uint32_t G = std::max(1u, std::min(k.resident, kMaxGridBlocks));
-    const uint32_t min_piece = std::max(1u, kPieceOffspring / tile_size(shape));
-    std::vector<Run> runs;
-    std::vector<uint32_t> block_runs;
-    if (!continuous) schedule_runs(tiles, G, min_piece, runs, block_runs);
     if (group_table_bytes((uint32_t)segs.size(), offspring, buckets) > table_capacity)
         return fail(SPG_ERR_INVALID, "launch table does not fit its buffer");
-    const size_t off_runs = align_up(segs.size() * sizeof(Segment), 256);
-    const size_t off_block = off_runs + align_up(runs.size() * sizeof(Run), 256);
-    const size_t off_buckets = off_block + align_up((size_t)(kMaxGridBlocks + 1) * 4, 256);
+    const size_t off_buckets = align_up(segs.size() * sizeof(Segment), 256);
     const size_t off_tiles = off_buckets + align_up((size_t)buckets * 4, 256);
     cudaError_t e = cudaMemcpy(table, segs.data(), segs.size() * sizeof(Segment), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(table + off_runs, runs.data(), runs.size() * sizeof(Run), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(table + off_block, block_runs.data(), block_runs.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(table + off_buckets, bucket_map.data(), bucket_map.size() * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !tile_map.empty())
+    if (e == cudaSuccess)
         e = cudaMemcpy(table + off_tiles, tile_map.data(), tile_map.size() * 4, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "upload launch table");
     gl = GenLaunch{};
     gl.offspring = k;
     gl.compact = compact_kernel(words);
     gl.args.segs = reinterpret_cast<const Segment *>(table);
-    gl.args.runs = reinterpret_cast<const Run *>(table + off_runs);
-    gl.args.block_runs = reinterpret_cast<const uint32_t *>(table + off_block);
     gl.args.bucket_seg = reinterpret_cast<const uint32_t *>(table + off_buckets);
     gl.args.tile_seg = reinterpret_cast<const uint32_t *>(table + off_tiles);
     gl.args.nsegs = (uint32_t)segs.size();
     if (segs.size() == 1) {
-        // one member: contiguous shares of its tiles per block (no run table)
         gl.args.one = segs[0];
         gl.args.nsegs = 1;
     }
     gl.args.total_tiles = total_tiles;
     gl.args.total_buckets = buckets;
-    if (continuous) {
-        gl.blocks = total_tiles;  // not persistent
-    } else {
-        apply_kernel(k, gl.args);
-        gl.blocks = segs.size() == 1 ? std::min(total_tiles, G) : G;
-    }
+    gl.blocks = total_tiles;  // not persistent
     gl.buckets = buckets;
     return SPG_OK;
 }
@@ -775,8 +972,8 @@ int view_set_state(const PopView &v, uint32_t gen, uint32_t S, uint32_t f, doubl
 int view_pack(const PopView &v, uint32_t gen, const uint32_t *surv, uint32_t S) {
     const uint32_t par = gen & 1u;
     return launch_pack(reinterpret_cast<const PopParams *>(v.base + v.L.params), v.words,
-                       reinterpret_cast<const uint32_t *>(v.base + v.L.geno0), surv, S, v.n, slot_length(v.n),
-                       slot_count(v.n), reinterpret_cast<uint32_t *>(v.base + v.L.alive),
+                       reinterpret_cast<const uint32_t *>(v.base + v.L.geno0), surv, S, v.n, slot_length(v.n, v.words),
+                       slot_count(v.n, v.words), reinterpret_cast<uint32_t *>(v.base + v.L.alive),
                        reinterpret_cast<uint32_t *>(v.base + v.L.packed[par]),
                        reinterpret_cast<uint32_t *>(v.base + v.L.counts[par]),
                        v.L.weighted ? reinterpret_cast<uint2 *>(v.base + v.L.mate[par]) : nullptr,

@@ -6,7 +6,7 @@
 // once per launch and generation, and a generation costs one grid barrier.
 //
 // Slots.  The population's groups of 32 offspring are cut into at most
-// kMaxSlots slots of equal length, one per resident warp at large N.  A warp
+// 152 slots a warp of equal length, one per resident warp at large N.  A warp
 // forms its slot's groups in order and packs the survivors' records at the
 // start of the slot's own range, counting them; no other pass touches a
 // record.  Between generations every block turns the slots' counts into a
@@ -47,15 +47,16 @@ namespace {
 // ------------------------------------------------------- shared memory
 constexpr uint32_t kGuide = 1u << kMaxGuideBits;  // most entries of the guide
 
-template <int W, bool LINKED, int BLOCK>
+template <int W, bool LINKED>
 struct GenSmem {
+    static constexpr uint32_t BLOCK = kSoloThreadsOf<W>, kSlots = 152u * (BLOCK / 32u);
     static constexpr uint32_t NW = BLOCK / 32;
     static constexpr uint32_t kPlanes = W <= 2 ? 1u : (uint32_t)W / 2u;  // 16-byte planes of a staged record
     static constexpr uint32_t kSets = W == 8 ? 2u : 1u;                  // word sets of the value fragments
     static constexpr uint32_t kRegs = W >= 4 ? 16u : 4u * W;             // element pairs of a lane, row and set
     static constexpr uint32_t kRegRoom = kRegs < 8u ? 8u : kRegs;        // places for them (even loci, odd loci)
     static constexpr uint32_t kThr = 0u, kAtt = kThr + kBins * 4u, kDir = kAtt + kBins * 4u;
-    static constexpr uint32_t kGuideOff = kDir + kMaxSlots * 8u;
+    static constexpr uint32_t kGuideOff = kDir + kSlots * 8u;
     static constexpr uint32_t kFrag = kGuideOff + kGuide * 2u;           // [table][set][kRegRoom / 4][32][4]
     static constexpr uint32_t kSetBytes = kRegRoom * 128u, kTabBytes = kSets * kSetBytes;
     static constexpr uint32_t kStage = kFrag + 2u * kTabBytes;
@@ -74,21 +75,24 @@ extern __shared__ __align__(128) unsigned char g_smem[];
 
 __device__ __forceinline__ uint32_t sm_u32(uint32_t off) { return *reinterpret_cast<const uint32_t *>(g_smem + off); }
 
-// ------------------------------------------------------- grid barrier
-// All blocks of the (cooperative) grid arrive and wait; false when the wait
-// ran out.  The counter only grows, by gridDim.x per barrier.  (Every block
-// polling a word of every other took 5 us instead of 2 with 152 blocks.)
-constexpr uint32_t kBarrierTries = 1u << 23;  // polls of about half a microsecond before a wait gives up
+// ------------------------------------------------------- team barrier
+// All blocks of a population's team (a cooperative grid's blocks, or some of
+// them) arrive and wait; false when the wait ran out.  The counter only grows,
+// by kBarrierStep per barrier whatever the team's size (its first block adds
+// what the others leave).  (Every block polling a word of every other took 5 us
+// instead of 2 with 152 blocks.)
+constexpr unsigned long long kBarrierStep = 1u << 16;  // more than a grid's blocks
+constexpr uint32_t kBarrierTries = 1u << 24;  // polls of about half a microsecond before a wait gives up
 
-__device__ __forceinline__ bool grid_barrier(unsigned long long *ctr) {
+__device__ __forceinline__ bool team_barrier(unsigned long long *ctr, uint32_t rank, uint32_t team) {
     __syncthreads();
-    if (gridDim.x == 1u) return true;
+    if (team == 1u) return true;
     int ok = 1;
     if (threadIdx.x == 0) {
-        const unsigned long long G = gridDim.x;
+        const unsigned long long add = rank == 0u ? kBarrierStep - (team - 1u) : 1ull;
         unsigned long long old, v = 0;
-        asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;" : "=l"(old) : "l"(ctr) : "memory");
-        const unsigned long long want = (old / G + 1ull) * G;
+        asm volatile("atom.add.release.gpu.global.u64 %0, [%1], %2;" : "=l"(old) : "l"(ctr), "l"(add) : "memory");
+        const unsigned long long want = (old / kBarrierStep + 1ull) * kBarrierStep;
         for (uint32_t i = 0; i < kBarrierTries && v < want; ++i)
             asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
         asm volatile("fence.acq_rel.gpu;" ::: "memory");
@@ -284,23 +288,24 @@ __device__ __noinline__ void mutate_staged(uint32_t row, uint32_t copies, uint32
 // round keys come from the kernel's parameters, and what the first two rounds
 // share is made once -- A * j per offspring, the rest (g, rep) per generation.
 struct GenRng {
-    uint32_t hx, lx;  // product of A and word 0 after round 0 (hx with round 1's key)
+    uint32_t hx, lx, cy;  // product of A and word 0 after round 0 (hx with round 1's key), word 1 with round 1's key
 };
+using RoundKeys = uint32_t[20];
 constexpr uint32_t kPhA = 0xD2511F53u, kPhB = 0xCD9E8D57u;
-__device__ __forceinline__ GenRng gen_rng(const SoloArgs &a, uint32_t g) {
-    const uint32_t x1 = (uint32_t)(((unsigned long long)kPhB * a.rep) >> 32) ^ g ^ a.keys[0];
-    const unsigned long long p = (unsigned long long)kPhA * x1;
-    return GenRng{(uint32_t)(p >> 32) ^ a.keys[3], (uint32_t)p};
+__device__ __forceinline__ GenRng gen_rng(const RoundKeys &keys, uint32_t rep, uint32_t g) {
+    const unsigned long long q = (unsigned long long)kPhB * rep;
+    const unsigned long long p = (unsigned long long)kPhA * ((uint32_t)(q >> 32) ^ g ^ keys[0]);
+    return GenRng{(uint32_t)(p >> 32) ^ keys[3], (uint32_t)p, (uint32_t)q ^ keys[2]};
 }
-__device__ __forceinline__ uint4 philox_at(const SoloArgs &a, const GenRng &r, unsigned long long aj, uint32_t word) {
-    unsigned long long p1 = (unsigned long long)kPhB * ((uint32_t)(aj >> 32) ^ word ^ a.keys[1]), p0;
-    uint4 c = make_uint4((uint32_t)(p1 >> 32) ^ (kPhB * a.rep) ^ a.keys[2], (uint32_t)p1, r.hx ^ (uint32_t)aj, r.lx);
+__device__ __forceinline__ uint4 philox_at(const RoundKeys &keys, const GenRng &r, unsigned long long aj, uint32_t word) {
+    unsigned long long p1 = (unsigned long long)kPhB * ((uint32_t)(aj >> 32) ^ word ^ keys[1]), p0;
+    uint4 c = make_uint4((uint32_t)(p1 >> 32) ^ r.cy, (uint32_t)p1, r.hx ^ (uint32_t)aj, r.lx);
 #pragma unroll
     for (int i = 2; i < 10; ++i) {
         p0 = (unsigned long long)kPhA * c.x;
         p1 = (unsigned long long)kPhB * c.z;
-        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ a.keys[2 * i], (uint32_t)p1,
-                       (uint32_t)(p0 >> 32) ^ c.w ^ a.keys[2 * i + 1], (uint32_t)p0);
+        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ keys[2 * i], (uint32_t)p1,
+                       (uint32_t)(p0 >> 32) ^ c.w ^ keys[2 * i + 1], (uint32_t)p0);
     }
     return c;
 }
@@ -335,7 +340,7 @@ __device__ __forceinline__ void locate(const SoloArgs &a, uint32_t u0, uint32_t 
 // pairs, both roles together; thr holds each survivor's thresholds as mother
 // and as father at its record's place.
 template <class SM>
-__device__ __forceinline__ void weighted_records(const SoloArgs &a, const uint2 *thr, const GenRng &rng,
+__device__ __forceinline__ void weighted_records(const SoloArgs &a, const RoundKeys &keys, const uint2 *thr, const GenRng &rng,
                                                  unsigned long long aj, uint32_t S, bool one_step,
                                                  uint32_t &mom,
                                                  uint32_t &dad) {
@@ -345,13 +350,13 @@ __device__ __forceinline__ void weighted_records(const SoloArgs &a, const uint2 
         uint4 dm = make_uint4(0u, 0u, 0u, 0u), df = dm;
         uint32_t rm0 = 0, rm1 = 0, rf0 = 0, rf1 = 0, tm0 = 0, tm1 = 0, tf0 = 0, tf1 = 0;
         if (open_m) {
-            dm = philox_at(a, rng, aj, sub);
+            dm = philox_at(keys, rng, aj, sub);
             locate<SM>(a, dm.x, dm.z, S, one_step, rm0, rm1);
             tm0 = __ldcg(&thr[rm0].x);
             tm1 = __ldcg(&thr[rm1].x);
         }
         if (open_f) {
-            df = philox_at(a, rng, aj, sub | (1u << 8));
+            df = philox_at(keys, rng, aj, sub | (1u << 8));
             locate<SM>(a, df.x, df.z, S, one_step, rf0, rf1);
             tf0 = __ldcg(&thr[rf0].y);
             tf1 = __ldcg(&thr[rf1].y);
@@ -450,7 +455,7 @@ __device__ __forceinline__ bool build_directory(const uint32_t *counts, uint32_t
                                                 uint32_t guide_bits, uint32_t *s_warp, uint32_t *total) {
     constexpr uint32_t T = SM::kThreads - 32u;
     if (nslots <= T) return directory_of<SM, 1>(counts, nslots, slot_records, guide_bits, s_warp, total);
-    return directory_of<SM, (kMaxSlots + T - 1) / T>(counts, nslots, slot_records, guide_bits, s_warp, total);
+    return directory_of<SM, (SM::kSlots + T - 1) / T>(counts, nslots, slot_records, guide_bits, s_warp, total);
 }
 
 // ------------------------------------------------------- per-locus counts
@@ -604,10 +609,13 @@ __device__ __forceinline__ unsigned long long total_stats(const GenAcc *acc, uin
 
 // GENERAL: dominance, values beyond 2048 in magnitude or a bias beyond 2^30
 // (the others' instance has none of these branches in its loop).
+// Blocks 0 .. team - 1 (this one is `rank`) form n_gen generations of a
+// population; keep_last: the last of them is the call's last.
 template <int W, bool LINKED, bool WEIGHTED, bool GENERAL>
-__global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_constant__ SoloArgs a) {
-    constexpr int BLOCK = kSoloThreads;
-    using SM = GenSmem<W, LINKED, BLOCK>;
+__device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundKeys &keys, uint32_t n_gen,
+                                                 bool keep_last, uint32_t rank, uint32_t team) {
+    constexpr int BLOCK = (int)kSoloThreadsOf<W>;
+    using SM = GenSmem<W, LINKED>;
     constexpr uint32_t NW = BLOCK / 32;
     __shared__ uint32_t s_cdf[kMaxKmax];
     __shared__ uint32_t s_scan[32];
@@ -655,13 +663,13 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
         }
         lk = LinkSmem{cdf, cum, chrom, first, clast, gd, lp->kmax, lp->nchrom, nullptr};
     }
-    const uint32_t rep = a.rep, k0 = a.keys[0], k1 = a.keys[1];
+    const uint32_t rep = a.rep, k0 = keys[0], k1 = keys[1];
     const uint32_t rec_slot = a.slot_len * 32u;
     const uint32_t stage = smem0 + SM::kStage + warp * SM::kPerWarp, my_row = stage + stage_row(lane);
     if constexpr (LINKED) lk.tog = reinterpret_cast<uint32_t *>(g_smem + SM::kStage + warp * SM::kPerWarp) -
                                    warp * (2u * 32u * ((uint32_t)W + 3u));  // the helper adds its warp's offset
-    const uint32_t slot0 = (uint32_t)(((unsigned long long)a.nslots * blockIdx.x) / gridDim.x);
-    const uint32_t slot1 = (uint32_t)(((unsigned long long)a.nslots * (blockIdx.x + 1u)) / gridDim.x);
+    const uint32_t slot0 = (uint32_t)(((unsigned long long)a.nslots * rank) / team);
+    const uint32_t slot1 = (uint32_t)(((unsigned long long)a.nslots * (rank + 1u)) / team);
     bool one_step = true;
     if (warp + 1u < NW)
         one_step = build_directory<SM>(a.counts[gen & 1u], a.nslots, rec_slot, a.guide_bits, s_scan, &s_total);
@@ -670,30 +678,28 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
     uint32_t S = s_total;
 
     bool again = false;  // a generation without survivors formed once more for its full records
-    for (uint32_t done = 0; done < a.n_gen && (gen < target || again);) {
+    for (uint32_t done = 0; done < n_gen && (gen < target || again);) {
         const uint32_t g = again ? gen : gen + 1u;
-        const bool list = again || (a.keep_last && done + 1u == a.n_gen) || g == target;
+        const bool list = again || (keep_last && done + 1u == n_gen) || g == target;
         const bool full = list || a.locus_row[0] != nullptr;
         const uint32_t *par = a.packed[(g + 1u) & 1u];
         uint32_t *out = a.packed[g & 1u];
-        const GenRng rng = gen_rng(a, g);
+        const GenRng rng = gen_rng(keys, rep, g);
         double grown = 0.0;  // the resource before consumption (the block's last warp), while the generation is formed
         if (eco && tid == BLOCK - 32u)
             grown = a.eco_model == 1u
                         ? resource_grown_bh(R, growth_rate(a.eco_r, a.eco_r_sd, g, rep, k0, k1), a.eco_K)
                         : resource_grown(R, a.eco_r, a.eco_K);
         LaneStats ts;
-        for (uint32_t slot = slot0 + warp; slot < slot1; slot += NW) {
-            const uint32_t base = slot * rec_slot, end = min(base + rec_slot, a.n);
-            uint32_t at0 = base;  // where the next survivor goes
+        {
             // (A) a group's mate draw and parents; the next group's records are
             // on their way while a group is formed
             auto draw = [&](uint32_t j, uint4 &r, uint32_t (&pm)[2 * W], uint32_t (&pf)[2 * W]) {
                 const unsigned long long aj = (unsigned long long)kPhA * j;
-                r = philox_at(a, rng, aj, kMate << 24);
+                r = philox_at(keys, rng, aj, kMate << 24);
                 uint32_t mom, dad;
                 if constexpr (WEIGHTED) {
-                    weighted_records<SM>(a, a.mate[(g + 1u) & 1u], rng, aj, S, one_step, mom, dad);
+                    weighted_records<SM>(a, keys, a.mate[(g + 1u) & 1u], rng, aj, S, one_step, mom, dad);
                 } else {
                     locate<SM>(a, r.x, r.y, S, one_step, mom, dad);
                 }
@@ -702,9 +708,11 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
             };
             uint4 r_next;
             uint32_t pm_next[2 * W], pf_next[2 * W];
-            draw(base + lane, r_next, pm_next, pf_next);
+            // the warp's groups, slot after slot
+            uint32_t slot = slot0 + warp, base = slot * rec_slot, end = min(base + rec_slot, a.n), at0 = base, j0 = base;
+            if (slot < slot1) draw(base + lane, r_next, pm_next, pf_next);
 #pragma unroll 1
-            for (uint32_t j0 = base; j0 < end; j0 += 32u) {
+            while (slot < slot1) {
                 const uint32_t j = j0 + lane;
                 const bool valid = j < a.n;
                 const uint4 r = r_next;
@@ -723,7 +731,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
                     const unsigned long long aj = (unsigned long long)kPhA * j;
 #pragma unroll
                     for (int q4 = 0; q4 < (2 * W + 3) / 4; ++q4) {
-                        const uint4 d = philox_at(a, rng, aj, (kRecomb << 24) | (uint32_t)q4);
+                        const uint4 d = philox_at(keys, rng, aj, (kRecomb << 24) | (uint32_t)q4);
                         const int w = 2 * q4;
                         ch[w] = (pm_next[w] & ~d.x) | (pm_next[W + w] & d.x);
                         ch[W + w] = (pf_next[w] & ~d.y) | (pf_next[W + w] & d.y);
@@ -733,7 +741,9 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
                         }
                     }
                 }
-                if (j0 + 32u < end) draw(j + 32u, r_next, pm_next, pf_next);
+                const bool slot_done = j0 + 32u >= end;
+                const uint32_t j0_next = slot_done ? (slot + NW) * rec_slot : j0 + 32u;
+                if (!slot_done || slot + NW < slot1) draw(j0_next + lane, r_next, pm_next, pf_next);
                 stage_record<W>(my_row, ch);
                 if (r.w >= a.mut_from) {  // (B) mutations, on the staged record
                     uint32_t k = 0;
@@ -788,8 +798,14 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
                     if (full) store_record<W>(a.geno + (size_t)j * (2 * W), ch);
                 }
                 if (full && lane == 0u) a.alive[j0 >> 5] = bits;
+                if (slot_done) {
+                    if (lane == 0u && !again) a.counts[g & 1u][slot] = at0 - base;
+                    slot += NW;
+                    base = at0 = j0_next;
+                    end = min(base + rec_slot, a.n);
+                }
+                j0 = j0_next;
             }
-            if (lane == 0u && !again) a.counts[g & 1u][slot] = at0 - base;
         }
         if (again) break;
         put_stats<SM>(ts, tid);
@@ -799,8 +815,8 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
                                  a.locus_row[g & 1u]);
         __syncthreads();
         GenAcc *acc = a.acc + (size_t)(g % 3u) * kGenAccCopies;
-        add_stats<SM>(acc + blockIdx.x % kGenAccCopies, warp, lane);
-        if (!grid_barrier(a.barrier)) {  // the generation fails: every block gives up
+        add_stats<SM>(acc + rank % kGenAccCopies, warp, lane);
+        if (!team_barrier(a.barrier, rank, team)) {  // the generation fails: every block gives up
             if (tid == 0u) atomicExch(reinterpret_cast<int *>(&st->status), SPG_ERR_TIMEOUT);
             return;
         }
@@ -811,7 +827,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
         unsigned long long sum = 0;
         if (warp + 1u < NW) {
             wide = build_directory<SM>(a.counts[g & 1u], a.nslots, rec_slot, a.guide_bits, s_scan, &s_total);
-        } else if (eco || blockIdx.x == 0u) {
+        } else if (eco || rank == 0u) {
             sum = total_stats(acc, lane);
             const unsigned long long cons = __shfl_sync(0xFFFFFFFFu, sum, 3);
             if (lane == 0u && eco) {
@@ -822,7 +838,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
         wide = __syncthreads_and(wide) != 0;
         const uint32_t S_new = s_total, f_new = eco ? s_f[g & 1u] : f;
         status = S_new == 0u ? SPG_EXTINCT : SPG_OK;
-        if (blockIdx.x == 0u) {
+        if (rank == 0u) {
             if (warp == NW - 1u) {
                 spg_stats *rec = a.ring + (g - 1u) % a.stats_cap;
                 if (lane == 0u) {
@@ -864,7 +880,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
             }
         }
         if (list && S_new != 0u) {  // the ordered survivor list from the bitmap
-            for (uint32_t slot = blockIdx.x * NW + warp; slot < a.nslots; slot += gridDim.x * NW) {
+            for (uint32_t slot = rank * NW + warp; slot < a.nslots; slot += team * NW) {
                 uint32_t rank = slot * rec_slot - *reinterpret_cast<const uint32_t *>(g_smem + SM::kDir + 8u * slot + 4u);
                 for (uint32_t gi = 0; gi < a.slot_len && slot * rec_slot + 32u * gi < a.n; ++gi) {
                     const uint32_t j = slot * rec_slot + 32u * gi, bits = __ldcg(a.alive + (j >> 5));
@@ -887,13 +903,64 @@ __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_co
     }
 }
 
+// One population: every block of the grid is in its team.
+template <int W, bool LINKED, bool WEIGHTED, bool GENERAL>
+__global__ void __launch_bounds__(kSoloThreadsOf<W>, 1) k_generations(const __grid_constant__ SoloArgs a) {
+    form_generations<W, LINKED, WEIGHTED, GENERAL>(a, a.keys, a.n_gen, a.keep_last != 0u, blockIdx.x, gridDim.x);
+}
+
+// Several populations: each block works through its list of teams.  A team's
+// blocks wait for one another, and all lists have the teams in one order, so
+// the blocks of the first unfinished team are all at it or on their way.  A
+// population stays with its team for the whole launch: its records stay in L2
+// and no other population's generation waits for it.  ONE_SEED: the members
+// share their Philox keys, which then come from the kernel's parameters.
+template <int W, bool LINKED, bool WEIGHTED, bool GENERAL, bool ONE_SEED>
+__global__ void __launch_bounds__(kSoloThreadsOf<W>, 1) k_teams(const __grid_constant__ TeamArgs t) {
+    __shared__ SoloArgs s_args;
+    const uint32_t last = t.block_places[blockIdx.x + 1u];
+    for (uint32_t p = t.block_places[blockIdx.x]; p < last; ++p) {
+        const TeamPlace place = t.places[p];
+        __syncthreads();  // the previous population's tables and arguments are no longer read
+        for (uint32_t i = threadIdx.x; i < sizeof(SoloArgs) / 4u; i += kSoloThreadsOf<W>)
+            reinterpret_cast<uint32_t *>(&s_args)[i] = reinterpret_cast<const uint32_t *>(t.members + place.member)[i];
+        __syncthreads();
+        if constexpr (ONE_SEED)
+            form_generations<W, LINKED, WEIGHTED, GENERAL>(s_args, t.keys, t.n_gen, t.keep_last != 0u, place.rank, place.team);
+        else
+            form_generations<W, LINKED, WEIGHTED, GENERAL>(s_args, s_args.keys, t.n_gen, t.keep_last != 0u, place.rank,
+                                                           place.team);
+    }
+}
+
 template <int W, bool LINKED, bool WEIGHTED>
 SoloKernel solo_instance(bool general) {
     SoloKernel k;
-    k.fn = general ? &k_generations<W, LINKED, WEIGHTED, true> : &k_generations<W, LINKED, WEIGHTED, false>;
-    k.block = kSoloThreads;
-    k.smem = GenSmem<W, LINKED, kSoloThreads>::kBytes;
+    k.fn = general ? (const void *)&k_generations<W, LINKED, WEIGHTED, true>
+                   : (const void *)&k_generations<W, LINKED, WEIGHTED, false>;
+    k.smem = GenSmem<W, LINKED>::kBytes;
+    k.threads = kSoloThreadsOf<W>;
     return k;
+}
+template <int W, bool LINKED, bool WEIGHTED, bool GENERAL, bool ONE_SEED = false>
+SoloKernel team_instance() {
+    SoloKernel k;
+    k.fn = (const void *)&k_teams<W, LINKED, WEIGHTED, GENERAL, ONE_SEED>;
+    k.smem = GenSmem<W, LINKED>::kBytes;
+    k.threads = kSoloThreadsOf<W>;
+    return k;
+}
+// The team kernel of one kind (team_kind).
+template <int W>
+SoloKernel team_kernel_of(uint32_t kind) {
+    switch (kind) {
+        case 0: return team_instance<W, false, false, false, true>();
+        case 1: return team_instance<W, false, false, false>();
+        case 2: return team_instance<W, false, false, true>();
+        case 3: return team_instance<W, true, false, true>();
+        case 4: return team_instance<W, false, true, true>();
+        default: return team_instance<W, true, true, true>();
+    }
 }
 
 }  // namespace

@@ -1143,14 +1143,27 @@ SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted, bool general)
     }
 }
 
+SoloKernel team_kernel_w1(uint32_t kind);
+SoloKernel team_kernel_w2(uint32_t kind);
+SoloKernel team_kernel_w4(uint32_t kind);
+SoloKernel team_kernel_w8(uint32_t kind);
+
+SoloKernel team_kernel(uint32_t words, uint32_t kind) {
+    switch (words) {
+        case 1: return team_kernel_w1(kind);
+        case 2: return team_kernel_w2(kind);
+        case 4: return team_kernel_w4(kind);
+        default: return team_kernel_w8(kind);
+    }
+}
+
 int prepare_solo(SoloKernel &k) {
     if (!k.fn) return SPG_ERR_INVALID;
-    const void *fn = reinterpret_cast<const void *>(k.fn);
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, (int)k.block, k.smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, (int)k.threads, k.smem);
     if (e != cudaSuccess || per_sm <= 0) return SPG_ERR_CUDA;
     k.resident = (uint32_t)per_sm * (uint32_t)sms;
     return SPG_OK;

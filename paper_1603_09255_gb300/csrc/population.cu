@@ -66,67 +66,19 @@ void attach_locus(spg_pop *p) {
     p->sa.locus_cap = p->locus.cap;
 }
 
-// The ecology as the generation kernel's arguments.
-void set_solo_ecology(spg_pop *p) {
-    const PopParams &prm = *p->host_prm;
-    p->sa.has_eco = prm.has_eco;
-    p->sa.eco_model = prm.eco_model;
-    p->sa.eco_r = prm.r;
-    p->sa.eco_r_sd = prm.r_sd;
-    p->sa.eco_K = prm.K;
-    p->sa.eco_R_half = prm.R_half;
-}
-
-// Least warps of work per block: a small population takes as few SMs as give
-// every one of them this many warps.
-constexpr uint32_t kSoloMinWarps = 4;
-constexpr uint32_t kSoloLaunchGens = 512;  // generations of one launch, at most
-
 // The generation kernel, its grid and its arguments.  The launch shape is
 // accepted and reported; the kernel has one shape of its own (results never
 // depend on it).
 int configure_solo(spg_pop *p, const Shape &shape) {
     const PopParams &prm = *p->host_prm;
     SoloArgs &a = p->sa;
-    a.narrow_bias = prm.bias < (1 << 30) && prm.bias > -(1 << 30) ? 1u : 0u;  // |genetic value| < 2^26
+    solo_args(p->view(), prm, a);
     SoloKernel k = solo_kernel(p->words, prm.linked != 0u, prm.weighted != 0u, a.dom || a.two_digits || !a.narrow_bias);
     const int rc = prepare_solo(k);
     if (rc != SPG_OK) return fail(rc, "generation kernel setup failed");
     p->solo = k;
     p->shape = shape;
-    const uint32_t nslots = slot_count(p->n);
-    p->solo_blocks =
-        p->n <= 32u * kOneBlockGroups ? 1u : std::max(1u, std::min(k.resident, nslots / kSoloMinWarps));
-    a.prm = reinterpret_cast<const PopParams *>(p->arena + p->L.params);
-    a.frag = reinterpret_cast<const ValueFragments *>(p->arena + p->L.frag);
-    for (uint32_t i = 0; i < 2; ++i) {
-        a.packed[i] = reinterpret_cast<uint32_t *>(p->arena + p->L.packed[i]);
-        a.counts[i] = reinterpret_cast<uint32_t *>(p->arena + p->L.counts[i]);
-        a.mate[i] = p->L.weighted ? reinterpret_cast<uint2 *>(p->arena + p->L.mate[i]) : nullptr;
-    }
-    a.geno = reinterpret_cast<uint32_t *>(p->arena + p->L.geno0);
-    a.alive = reinterpret_cast<uint32_t *>(p->arena + p->L.alive);
-    a.surv = reinterpret_cast<uint32_t *>(p->arena + p->L.surv0);
-    a.state = reinterpret_cast<DevState *>(p->arena + p->L.state);
-    a.acc = reinterpret_cast<GenAcc *>(p->arena + p->L.gen_acc);
-    a.barrier = reinterpret_cast<unsigned long long *>(p->arena + p->L.barrier);
-    a.ring = reinterpret_cast<spg_stats *>(p->arena + p->L.ring);
-    for (uint32_t i = 0; i < 10; ++i) {
-        a.keys[2 * i] = prm.key0 + i * 0x9E3779B9u;
-        a.keys[2 * i + 1] = prm.key1 + i * 0xBB67AE85u;
-    }
-    a.rep = prm.rep;
-    a.kmax = prm.kmax;
-    a.stats_cap = p->cap;
-    set_solo_ecology(p);
-    a.mut_from = prm.kmax ? prm.cdf[0] : 0xFFFFFFFFu;
-    a.shift = prm.shift;
-    a.bias = prm.bias;
-    a.n = p->n;
-    a.slot_len = slot_length(p->n);
-    a.nslots = nslots;
-    a.guide_bits = 2;  // four to eight entries per slot
-    while ((nslots >> (a.guide_bits - 2)) != 0u && a.guide_bits < (uint32_t)kMaxGuideBits) ++a.guide_bits;
+    p->solo_blocks = most_blocks(p->n, p->words, k.resident);
     attach_locus(p);
     return SPG_OK;
 }
@@ -140,11 +92,10 @@ int enqueue_solo(spg_pop *p, uint32_t n_gen) {
         done += a.n_gen;
         a.keep_last = done == n_gen ? 1u : 0u;
         void *params[] = {&a};
-        const void *fn = reinterpret_cast<const void *>(p->solo.fn);
+        const dim3 grid(p->solo_blocks), block(p->solo.threads);
         const cudaError_t e =
-            p->solo_blocks == 1u
-                ? cudaLaunchKernel(fn, dim3(1), dim3(p->solo.block), params, p->solo.smem, p->stream)
-                : cudaLaunchCooperativeKernel(fn, dim3(p->solo_blocks), dim3(p->solo.block), params, p->solo.smem, p->stream);
+            p->solo_blocks == 1u ? cudaLaunchKernel(p->solo.fn, grid, block, params, p->solo.smem, p->stream)
+                                 : cudaLaunchCooperativeKernel(p->solo.fn, grid, block, params, p->solo.smem, p->stream);
         if (e != cudaSuccess) return cuda_fail(e, "generation launch");
     }
     return SPG_OK;
@@ -299,7 +250,7 @@ int spg_create_population(const spg_pop_desc *desc, const spg_allocator *alloc, 
 int spg_set_ecology(spg_pop *p, const spg_ecology *eco) {
     if (!p) return fail(SPG_ERR_INVALID, "population is NULL");
     const int rc = view_set_ecology(p->view(), *p->host_prm, eco);
-    if (rc == SPG_OK) set_solo_ecology(p);
+    if (rc == SPG_OK && p->L.solo) solo_args(p->view(), *p->host_prm, p->sa);
     return rc;
 }
 

@@ -32,10 +32,9 @@ using namespace spg;
 
 namespace {
 
-// Groups by locus count (L = 32, 64, 128, 256: index 0-3) and variant: the
-// index for plain jobs, 4 + 4v + index for v = 0 linkage map, 1 parent
-// weights, 2 both, 16 + index for continuous values (variants: one shape).
-constexpr int kGroups = 20;
+// Groups of continuous-allele jobs by locus count (L = 32, 64, 128, 256); the
+// other jobs are stepped by teams.
+constexpr int kGroups = 4;
 
 struct Job {
     spg_pop_desc desc{};
@@ -53,6 +52,8 @@ struct Job {
     size_t footprint = 0;
     PopView v;
     std::unique_ptr<PopParams> prm;
+    SoloArgs sa{};                          // biallelic: the generation kernel's arguments
+    ValueFragments frag{};                  // fragments of the genetic value (host copy, until uploaded)
     uint32_t gen = 0;  // generations enqueued (host bookkeeping)
     // once finished
     std::vector<spg_stats> stats;
@@ -60,12 +61,13 @@ struct Job {
     uint32_t final_gen = 0;
 };
 
-uint32_t group_of(uint32_t n_loci, bool linked, bool weighted, bool continuous) {
-    const uint32_t l = n_loci == 32 ? 0u : n_loci == 64 ? 1u : n_loci == 128 ? 2u : 3u;
-    return continuous ? 16u + l : l + 4u * ((linked ? 1u : 0u) + (weighted ? 2u : 0u));
-}
+uint32_t group_of(uint32_t n_loci) { return n_loci == 32 ? 0u : n_loci == 64 ? 1u : n_loci == 128 ? 2u : 3u; }
 bool continuous_job(const spg_pop_desc &d) { return d.allele_model == 1u; }
 uint32_t job_words(const spg_pop_desc &d) { return continuous_job(d) ? d.n_loci / 2 : d.n_loci / 32; }
+PopLayout job_layout(const spg_pop_desc &d, uint32_t cap, bool weighted) {
+    return continuous_job(d) ? layout_for(d.n, job_words(d), bucket_count(d.n), cap, false, false)
+                             : solo_layout_for(d.n, job_words(d), cap, weighted);
+}
 
 }  // namespace
 
@@ -84,6 +86,7 @@ struct spg_server {
     char *table[kGroups] = {};
     size_t table_cap[kGroups] = {};
     GenLaunch gl[kGroups];
+    TeamSet teams;  // the resident biallelic jobs
     bool dirty = true;
     std::chrono::steady_clock::time_point t0 = std::chrono::steady_clock::now();
 
@@ -140,7 +143,7 @@ int admit(spg_server *s, Job &j) {
     j.v.words = words;
     j.v.cap = j.prm->stats_cap;
     j.v.nbuckets = bucket_count(j.desc.n);
-    j.v.L = layout_for(j.desc.n, words, j.v.nbuckets, j.v.cap, j.weights != nullptr, !continuous_job(j.desc));
+    j.v.L = job_layout(j.desc, j.v.cap, j.weights != nullptr);
     j.v.stream = s->stream;
     cudaError_t e = cudaSuccess;
     if (j.link) {  // the variant tables in the job's memory (read by its parameters)
@@ -152,13 +155,19 @@ int admit(spg_server *s, Job &j) {
         e = cudaMemcpyAsync(j.arena + j.v.L.weights, j.weights.get(), sizeof(WeightParams), cudaMemcpyHostToDevice,
                             s->stream);
     }
-    if (e != cudaSuccess) return cuda_fail(e, "upload a job's variant tables");
+    if (e == cudaSuccess && j.v.L.solo) {
+        j.sa.dom = j.prm->has_dom;
+        value_fragments(j.desc.effects, j.sa.dom ? j.desc.dominance : nullptr, j.desc.n_loci, j.frag, j.sa.two_digits);
+        e = cudaMemcpyAsync(j.arena + j.v.L.frag, &j.frag, sizeof(ValueFragments), cudaMemcpyHostToDevice, s->stream);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "upload a job's tables");
     rc = view_init(j.v, *j.prm, j.founders.empty() ? nullptr : j.founders.data(), j.desc.p0_q32);
     if (rc == SPG_OK && j.has_eco) rc = view_set_ecology(j.v, *j.prm, &j.eco);
     DevState st;
     if (rc == SPG_OK) rc = view_state(j.v, st);
     if (rc == SPG_OK) rc = view_set_state(j.v, st.gen, st.S, st.f, st.R, st.status, j.n_gen);
     if (rc != SPG_OK) return rc;
+    if (j.v.L.solo) solo_args(j.v, *j.prm, j.sa);
     j.state = SPG_JOB_RESIDENT;
     j.t_admit = s->now();
     s->used += j.footprint;
@@ -169,24 +178,25 @@ int admit(spg_server *s, Job &j) {
 int rebuild(spg_server *s) {
     int rc = server_sync(s);
     if (rc != SPG_OK) return rc;
+    std::vector<TeamMember> members;
+    for (uint64_t id : s->resident) {
+        const Job &j = *s->jobs[id];
+        if (j.v.L.solo)
+            members.push_back(TeamMember{&j.sa, j.v.n, j.v.words, j.link != nullptr, j.weights != nullptr});
+    }
+    rc = s->teams.build(members, s->alloc, s->stream);
+    if (rc != SPG_OK) return rc;
     for (int gi = 0; gi < kGroups; ++gi) {
         std::vector<const PopView *> views;
         uint64_t offspring = 0;
         uint32_t buckets = 0;
-        bool eco = false, dom = false;
-        const bool continuous = gi >= 16;
-        const uint32_t words = continuous ? (32u << (gi % 4)) / 2u : 1u << (gi % 4);
-        const bool linked = !continuous && ((gi / 4) & 1) != 0, weighted = !continuous && ((gi / 4) & 2) != 0;
+        const uint32_t words = (32u << gi) / 2u;
         for (uint64_t id : s->resident) {
             const Job &j = *s->jobs[id];
-            if (group_of(j.desc.n_loci, j.link != nullptr, j.weights != nullptr, continuous_job(j.desc)) !=
-                (uint32_t)gi)
-                continue;
+            if (j.v.L.solo || group_of(j.desc.n_loci) != (uint32_t)gi) continue;
             views.push_back(&j.v);
             offspring += j.v.n;
             buckets += j.v.nbuckets;
-            eco |= j.prm->has_eco != 0u;
-            dom |= j.prm->has_dom != 0u;
         }
         const size_t need = group_table_bytes((uint32_t)views.size(), offspring, buckets);
         if (need > s->table_cap[gi]) {
@@ -198,9 +208,7 @@ int rebuild(spg_server *s) {
             if (!s->table[gi]) return fail(SPG_ERR_OOM, "launch table allocation failed");
             s->table_cap[gi] = cap;
         }
-        const Shape shape = (linked || weighted || continuous) ? Shape{(uint32_t)kBlock, 1u, 1u} : default_shape(words);
-        rc = build_group_launch(views, words, shape, eco, dom, s->table[gi], s->table_cap[gi], s->gl[gi], linked,
-                                weighted, continuous);
+        rc = build_group_launch(views, words, s->table[gi], s->table_cap[gi], s->gl[gi]);
         if (rc != SPG_OK) return rc;
     }
     s->dirty = false;
@@ -210,6 +218,8 @@ int rebuild(spg_server *s) {
 int advance(spg_server *s, uint32_t k) {
     cudaError_t e = cudaEventRecord(s->tick_start, s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaEventRecord");
+    const int trc = s->teams.step(k, false, s->stream);
+    if (trc != SPG_OK) return trc;
     for (int gi = 0; gi < kGroups; ++gi) {
         if (s->gl[gi].blocks == 0) continue;
         e = cudaStreamWaitEvent(s->group_stream[gi], s->tick_start, 0);
@@ -315,10 +325,7 @@ int spg_server_submit(spg_server *s, const spg_pop_desc *desc, const spg_ecology
     }
     j->n_gen = n_gen;
     j->t_arrival = t_arrival;
-    j->footprint = align_up(layout_for(desc->n, job_words(*desc), bucket_count(desc->n), n_gen, j->weights != nullptr,
-                                       !continuous_job(*desc))
-                                .total,
-                            256);
+    j->footprint = align_up(job_layout(*desc, n_gen, j->weights != nullptr).total, 256);
     if (j->footprint > s->cfg.memory_budget)
         return fail(SPG_ERR_BUDGET, "job needs %zu bytes, the budget is %zu", j->footprint, s->cfg.memory_budget);
     *job = s->jobs.size();
@@ -458,6 +465,7 @@ void spg_server_destroy(spg_server *s) {
     if (s->stream) cudaStreamSynchronize(s->stream);
     for (auto &jp : s->jobs)
         if (jp && jp->arena) s->alloc.release(jp->arena, s->stream);
+    s->teams.release(s->alloc, s->stream);
     for (int gi = 0; gi < kGroups; ++gi) {
         if (s->table[gi]) s->alloc.release(s->table[gi], s->stream);
         if (s->group_stream[gi]) cudaStreamDestroy(s->group_stream[gi]);

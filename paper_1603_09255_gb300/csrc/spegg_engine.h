@@ -75,6 +75,35 @@ struct GraphChain {
     int build(const GenLaunch &gl, uint32_t len);
 };
 
+// Generations of several biallelic populations in shared launches (k_teams).
+constexpr uint32_t kSoloLaunchGens = 512;  // generations of one launch of the generation kernel, at most
+struct TeamMember {
+    const SoloArgs *args = nullptr;  // (read when the tables are built)
+    uint32_t n = 0, words = 0;
+    bool linked = false, weighted = false;
+};
+struct TeamLaunch {
+    std::vector<TeamMember> members;  // of one locus count and kind
+    uint32_t kind = 0;
+    SoloKernel kernel;
+    TeamArgs args{};
+    char *table = nullptr;            // the members' arguments and the blocks' places
+    size_t capacity = 0;
+    double cycles = 0.0;              // estimated cycles of a generation of all members
+    void release(const Allocator &alloc, cudaStream_t stream);
+};
+struct TeamSet {
+    TeamLaunch launch[4 * (kTeamKinds - 1)];  // by locus count and kind (plain members of one seed or several)
+    int build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream);  // synchronises
+    int update(const SoloArgs *args);
+    int step(uint32_t n_gen, bool keep_last, cudaStream_t stream);
+    void release(const Allocator &alloc, cudaStream_t stream);
+};
+double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, std::vector<TeamPlace> &places,
+                      std::vector<uint32_t> &block_places);
+uint32_t most_blocks(uint32_t n, uint32_t words, uint32_t resident);
+void solo_args(const PopView &v, const PopParams &prm, SoloArgs &a);
+
 int fail(int code, const char *fmt, ...);
 int cuda_fail(cudaError_t e, const char *what);
 uint32_t mutation_cdf(double mu, uint32_t n_copies, uint32_t *cdf);
@@ -98,8 +127,8 @@ PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap
 Segment segment_at(char *base, const PopLayout &L, uint32_t n, uint32_t ntiles, uint32_t tile_begin,
                    uint32_t nbuckets, uint32_t bucket_begin);
 uint32_t bucket_count(uint32_t n);
-uint32_t slot_length(uint32_t n);
-uint32_t slot_count(uint32_t n);
+uint32_t slot_length(uint32_t n, uint32_t words);
+uint32_t slot_count(uint32_t n, uint32_t words);
 PopLayout solo_layout_for(uint32_t n, uint32_t words, uint32_t cap, bool weighted);
 int view_pack(const PopView &v, uint32_t gen, const uint32_t *surv, uint32_t S);
 Shape default_shape(uint32_t words);
@@ -121,15 +150,11 @@ uint32_t locus_blocks(uint32_t n);
 uint32_t tiles_for(uint32_t n, const Shape &shape);
 void schedule_runs(const std::vector<uint32_t> &tiles, uint32_t G, uint32_t min_piece, std::vector<Run> &runs,
                    std::vector<uint32_t> &block_runs);
-// Segment table, runs and bucket map of one launch group, uploaded into
-// `table` (device memory; synchronous), and the group's launch description.
-// eco / dom: some member has an ecology / dominance deviations.
-// linked / weighted / continuous: the members' variant (all alike; such
-// groups take the variant shape only: kBlock threads, one offspring per
-// thread, one lane; continuous: words = L / 2, the int16 records' words).
-int build_group_launch(const std::vector<const PopView *> &members, uint32_t words, const Shape &shape, bool eco,
-                       bool dom, char *table, size_t table_capacity, GenLaunch &gl, bool linked = false,
-                       bool weighted = false, bool continuous = false);
+// Segment table, tile and bucket maps of one group of continuous-allele
+// members (words = L / 2, the int16 records' words), uploaded into `table`
+// (device memory; synchronous), and the group's launch description.
+int build_group_launch(const std::vector<const PopView *> &members, uint32_t words, char *table, size_t table_capacity,
+                       GenLaunch &gl);
 int view_sync(const PopView &v);
 int view_state(const PopView &v, DevState &st);
 int view_set_state(const PopView &v, uint32_t gen, uint32_t S, uint32_t f, double R, int32_t status,

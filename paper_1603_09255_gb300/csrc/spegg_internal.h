@@ -190,8 +190,10 @@ using GenKernel = void (*)(GenArgs);
 // offspring are cut into slots of slot_len groups; a generation's survivors
 // are packed slot by slot in packed[generation & 1], counts[generation & 1]
 // holding their number per slot.
-constexpr uint32_t kSoloThreads = 512;
-constexpr uint32_t kMaxSlots = 152 * (kSoloThreads / 32);  // one per resident warp on 152 SMs
+constexpr uint32_t solo_threads(uint32_t words) { return words == 0 ? 0u : 512u; }
+constexpr uint32_t max_slots(uint32_t words) { return 152u * (solo_threads(words) / 32u); }  // one per resident warp on 152 SMs
+template <int W>
+constexpr uint32_t kSoloThreadsOf = solo_threads((uint32_t)W);
 constexpr uint32_t kOneBlockGroups = 16;  // groups up to which one block is no slower than several and a grid barrier
 // The per-locus values as f16 elements, laid out as the matrix fragments of
 // the generation kernel (value_fragments): the additive values, or with
@@ -209,7 +211,8 @@ struct alignas(64) GenAcc {
 constexpr uint32_t kGenAccCopies = 4;
 constexpr unsigned long long kEmptyMinMax = 0x800000007FFFFFFFull;  // mx INT_MIN over mn INT_MAX
 constexpr int kMaxGuideBits = 13;  // the parent draw's top bits that index the directory's guide, at most
-struct SoloArgs {
+struct alignas(16) SoloArgs {
+    uint32_t keys[20];                 // Philox round keys (word 0, word 1 of each round)
     const PopParams *prm;
     const ValueFragments *frag;
     uint32_t *packed[2];               // survivors' records by generation parity [N * 2W]
@@ -226,7 +229,7 @@ struct SoloArgs {
     uint32_t *locus_ring;              // [locus_cap][L]
     uint32_t locus_cap;
     uint32_t n, slot_len, nslots, guide_bits;
-    uint32_t keys[20];                 // Philox round keys (word 0, word 1 of each round)
+    uint32_t words;                    // W = L / 32
     uint32_t rep, kmax, shift;
     uint32_t mut_from;                 // mutation draws from here on count a mutation (kmax 0: none do)
     int32_t bias;
@@ -238,11 +241,33 @@ struct SoloArgs {
     uint32_t keep_last;                // the last of them is the call's last
 };
 struct SoloKernel {
-    void (*fn)(SoloArgs) = nullptr;
-    uint32_t block = 0, smem = 0, resident = 0;  // resident: blocks on the device at a time
+    const void *fn = nullptr;
+    uint32_t threads = 0, smem = 0, resident = 0;  // resident: blocks on the device at a time
 };
 SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted, bool general);
 int prepare_solo(SoloKernel &k);  // sets the shared-memory limit, fills `resident`
+
+// Several populations in one launch (k_teams): block b works through places
+// block_places[b] .. block_places[b + 1] - 1, being block `rank` of `team` for
+// population `member`.
+struct TeamPlace {
+    uint32_t member;
+    uint16_t rank, team;
+};
+struct TeamArgs {
+    uint32_t keys[20];  // the members' common Philox round keys (kind 0)
+    const SoloArgs *members;
+    const TeamPlace *places;
+    const uint32_t *block_places;
+    uint32_t n_gen, keep_last;
+};
+// Kinds of members that share a launch (with their locus count): plain ones of
+// one seed, plain ones, general values, linkage map, parent weights, both.
+constexpr uint32_t kTeamKinds = 6;
+inline uint32_t team_kind(bool linked, bool weighted, bool general) {
+    return linked ? (weighted ? 5u : 3u) : weighted ? 4u : general ? 2u : 1u;
+}
+SoloKernel team_kernel(uint32_t words, uint32_t kind);
 // Enqueue the slot layout of a generation: bitmap words and per-slot counts
 // of the survivors (surv: their ordered list of S, null for all n), their
 // records packed[slot ...] and, when mate is given, their parent thresholds;
