@@ -356,14 +356,14 @@ PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap
     return L;
 }
 
-// Slots of a single population: at most max_slots of whole groups of 32, or
+// Slots of a single population: at most kMaxSlots of whole groups of 32, or
 // one per warp of a block for a population that one block forms.
-uint32_t slot_length(uint32_t n, uint32_t words) {
-    const uint64_t slots = n <= 32u * kOneBlockGroups ? solo_threads(words) / 32u : max_slots(words);
+uint32_t slot_length(uint32_t n) {
+    const uint64_t slots = n <= 32u * kOneBlockGroups ? kSoloThreads / 32u : kMaxSlots;
     return (uint32_t)(((uint64_t)n + 32ull * slots - 1) / (32ull * slots));
 }
-uint32_t slot_count(uint32_t n, uint32_t words) {
-    const uint32_t len = 32u * slot_length(n, words);
+uint32_t slot_count(uint32_t n) {
+    const uint32_t len = 32u * slot_length(n);
     return (uint32_t)(((uint64_t)n + len - 1) / len);
 }
 
@@ -385,7 +385,7 @@ PopLayout solo_layout_for(uint32_t n, uint32_t words, uint32_t cap, bool weighte
     for (size_t &x : L.packed) x = take((size_t)n * 2 * words * 4);
     L.surv0 = L.surv1 = take((size_t)n * 4);
     L.alive = take(((size_t)n + 31) / 32 * 4);
-    for (size_t &x : L.counts) x = take((size_t)slot_count(n, words) * 4);
+    for (size_t &x : L.counts) x = take((size_t)slot_count(n) * 4);
     L.gen_acc = take(sizeof(GenAcc) * 3 * kGenAccCopies);
     L.barrier = take(sizeof(unsigned long long));
     L.ring = take((size_t)cap * sizeof(spg_stats));
@@ -430,8 +430,8 @@ void solo_args(const PopView &v, const PopParams &prm, SoloArgs &a) {
     a.narrow_bias = prm.bias < (1 << 30) && prm.bias > -(1 << 30) ? 1u : 0u;  // |genetic value| < 2^26
     a.stats_cap = v.cap;
     a.n = v.n;
-    a.slot_len = slot_length(v.n, v.words);
-    a.nslots = slot_count(v.n, v.words);
+    a.slot_len = slot_length(v.n);
+    a.nslots = slot_count(v.n);
     a.guide_bits = 2;  // four to eight entries per slot
     while ((a.nslots >> (a.guide_bits - 2)) != 0u && a.guide_bits < (uint32_t)kMaxGuideBits) ++a.guide_bits;
     a.has_eco = prm.has_eco;
@@ -447,8 +447,8 @@ void solo_args(const PopView &v, const PopParams &prm, SoloArgs &a) {
 // by less than the barrier does).
 constexpr uint32_t kSoloMinWarps = 4;
 
-uint32_t most_blocks(uint32_t n, uint32_t words, uint32_t resident) {
-    return n <= 32u * kOneBlockGroups ? 1u : std::max(1u, std::min(resident, slot_count(n, words) / kSoloMinWarps));
+uint32_t most_blocks(uint32_t n, uint32_t resident) {
+    return n <= 32u * kOneBlockGroups ? 1u : std::max(1u, std::min(resident, slot_count(n) / kSoloMinWarps));
 }
 
 // ------------------------------------------------------------ teams
@@ -473,7 +473,8 @@ static double resident_blocks(const TeamMember &m, uint32_t blocks) {
     return std::ceil(16.0 * m.words * m.n / (kTeamL2Bytes / blocks));
 }
 
-// Teams for the members on `blocks` blocks: the longest first, each with as
+// Teams for the members on `blocks` blocks: by locus count (the order in which
+// k_teams takes them), the longest first, each with as
 // many blocks as keep it below a share of the whole and its records in L2, on
 // the blocks that are free soonest; the share that gives the shortest schedule
 // is kept.  All blocks have their teams in the members' one order (k_teams).
@@ -489,7 +490,9 @@ double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, s
         work[m] = ((double)members[m].n + 31.0) / 32.0 / 16.0 * round_cycles(members[m]);
         total += work[m];
     }
-    std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) { return work[x] > work[y]; });
+    std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
+        return members[x].words != members[y].words ? members[x].words > members[y].words : work[x] > work[y];
+    });
     double best = -1.0;
     std::vector<std::vector<TeamPlace>> lists;
     for (const double share : {0.1, 0.15, 0.25, 0.4, 0.6, 1.0}) {
@@ -500,7 +503,7 @@ double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, s
         double end = 0.0;
         for (const uint32_t m : order) {
             const double want = std::max(std::ceil(work[m] / (share * total / blocks)), resident_blocks(members[m], blocks));
-            const uint32_t k = (uint32_t)std::max(1.0, std::min<double>(want, most_blocks(members[m].n, members[m].words, blocks)));
+            const uint32_t k = (uint32_t)std::max(1.0, std::min<double>(want, most_blocks(members[m].n, blocks)));
             std::nth_element(by_time.begin(), by_time.begin() + (k - 1), by_time.end(),
                              [&](uint32_t x, uint32_t y) { return free_at[x] != free_at[y] ? free_at[x] < free_at[y] : x < y; });
             double start = 0.0;
@@ -527,30 +530,18 @@ double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, s
 }
 
 int TeamSet::build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream) {
-    for (uint32_t i = 0; i < 4u * (kTeamKinds - 1u); ++i) {
-        TeamLaunch &t = launch[i];
-        const uint32_t words = 1u << (i % 4u);
-        uint32_t kind = 1u + i / 4u;
+    for (uint32_t kind = 0; kind < kTeamKinds; ++kind) {
+        TeamLaunch &t = launch[kind];
         t.members.clear();
         for (const TeamMember &m : all)
-            if (m.words == words &&
-                team_kind(m.linked, m.weighted, m.args->dom || m.args->two_digits || !m.args->narrow_bias) == kind)
+            if (team_kind(m.linked, m.weighted, m.args->dom || m.args->two_digits || !m.args->narrow_bias) == kind)
                 t.members.push_back(m);
         if (t.members.empty()) continue;
-        if (kind == 1u) {
-            const SoloArgs *first = t.members[0].args;
-            bool one_seed = true;
-            for (const TeamMember &m : t.members)
-                one_seed = one_seed && std::memcmp(m.args->keys, first->keys, sizeof first->keys) == 0;
-            if (one_seed) kind = 0u;
-        }
-        if (!t.kernel.fn || t.kind != kind) {
-            t.kernel = team_kernel(words, kind);
-            t.kind = kind;
+        if (!t.kernel.fn) {
+            t.kernel = team_kernel(kind);
             const int rc = prepare_solo(t.kernel);
             if (rc != SPG_OK) return fail(rc, "team kernel setup failed");
         }
-        std::memcpy(t.args.keys, t.members[0].args->keys, sizeof t.args.keys);
         std::vector<TeamPlace> places;
         std::vector<uint32_t> block_places;
         t.cycles = schedule_teams(t.members, t.kernel.resident, places, block_places);
@@ -607,7 +598,7 @@ int TeamSet::step(uint32_t n_gen, bool keep_last, cudaStream_t stream) {
             done += a.n_gen;
             a.keep_last = keep_last && done == n_gen ? 1u : 0u;
             void *params[] = {&a};
-            const cudaError_t e = cudaLaunchCooperativeKernel(t.kernel.fn, dim3(t.kernel.resident), dim3(t.kernel.threads),
+            const cudaError_t e = cudaLaunchCooperativeKernel(t.kernel.fn, dim3(t.kernel.resident), dim3(kSoloThreads),
                                                               params, t.kernel.smem, stream);
             if (e != cudaSuccess) return cuda_fail(e, "team launch");
         }
@@ -972,8 +963,8 @@ int view_set_state(const PopView &v, uint32_t gen, uint32_t S, uint32_t f, doubl
 int view_pack(const PopView &v, uint32_t gen, const uint32_t *surv, uint32_t S) {
     const uint32_t par = gen & 1u;
     return launch_pack(reinterpret_cast<const PopParams *>(v.base + v.L.params), v.words,
-                       reinterpret_cast<const uint32_t *>(v.base + v.L.geno0), surv, S, v.n, slot_length(v.n, v.words),
-                       slot_count(v.n, v.words), reinterpret_cast<uint32_t *>(v.base + v.L.alive),
+                       reinterpret_cast<const uint32_t *>(v.base + v.L.geno0), surv, S, v.n, slot_length(v.n),
+                       slot_count(v.n), reinterpret_cast<uint32_t *>(v.base + v.L.alive),
                        reinterpret_cast<uint32_t *>(v.base + v.L.packed[par]),
                        reinterpret_cast<uint32_t *>(v.base + v.L.counts[par]),
                        v.L.weighted ? reinterpret_cast<uint2 *>(v.base + v.L.mate[par]) : nullptr,

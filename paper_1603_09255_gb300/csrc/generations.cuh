@@ -49,7 +49,7 @@ constexpr uint32_t kGuide = 1u << kMaxGuideBits;  // most entries of the guide
 
 template <int W, bool LINKED>
 struct GenSmem {
-    static constexpr uint32_t BLOCK = kSoloThreadsOf<W>, kSlots = 152u * (BLOCK / 32u);
+    static constexpr uint32_t BLOCK = kSoloThreads, kSlots = kMaxSlots;
     static constexpr uint32_t NW = BLOCK / 32;
     static constexpr uint32_t kPlanes = W <= 2 ? 1u : (uint32_t)W / 2u;  // 16-byte planes of a staged record
     static constexpr uint32_t kSets = W == 8 ? 2u : 1u;                  // word sets of the value fragments
@@ -614,7 +614,7 @@ __device__ __forceinline__ unsigned long long total_stats(const GenAcc *acc, uin
 template <int W, bool LINKED, bool WEIGHTED, bool GENERAL>
 __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundKeys &keys, uint32_t n_gen,
                                                  bool keep_last, uint32_t rank, uint32_t team) {
-    constexpr int BLOCK = (int)kSoloThreadsOf<W>;
+    constexpr int BLOCK = (int)kSoloThreads;
     using SM = GenSmem<W, LINKED>;
     constexpr uint32_t NW = BLOCK / 32;
     __shared__ uint32_t s_cdf[kMaxKmax];
@@ -905,7 +905,7 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
 
 // One population: every block of the grid is in its team.
 template <int W, bool LINKED, bool WEIGHTED, bool GENERAL>
-__global__ void __launch_bounds__(kSoloThreadsOf<W>, 1) k_generations(const __grid_constant__ SoloArgs a) {
+__global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_constant__ SoloArgs a) {
     form_generations<W, LINKED, WEIGHTED, GENERAL>(a, a.keys, a.n_gen, a.keep_last != 0u, blockIdx.x, gridDim.x);
 }
 
@@ -913,24 +913,32 @@ __global__ void __launch_bounds__(kSoloThreadsOf<W>, 1) k_generations(const __gr
 // blocks wait for one another, and all lists have the teams in one order, so
 // the blocks of the first unfinished team are all at it or on their way.  A
 // population stays with its team for the whole launch: its records stay in L2
-// and no other population's generation waits for it.  ONE_SEED: the members
-// share their Philox keys, which then come from the kernel's parameters.
-template <int W, bool LINKED, bool WEIGHTED, bool GENERAL, bool ONE_SEED>
-__global__ void __launch_bounds__(kSoloThreadsOf<W>, 1) k_teams(const __grid_constant__ TeamArgs t) {
-    __shared__ SoloArgs s_args;
-    const uint32_t last = t.block_places[blockIdx.x + 1u];
-    for (uint32_t p = t.block_places[blockIdx.x]; p < last; ++p) {
+// and no other population's generation waits for it.  Members of all locus
+// counts share the launch (a launch per locus count left most blocks idle for
+// batches of few members), the longest records first: a switch over the
+// locus counts spilled in every body, one after the other they do not.  A
+// member's arguments are in shared memory.
+__shared__ SoloArgs s_team_args;
+template <int W, bool LINKED, bool WEIGHTED, bool GENERAL>
+__device__ __forceinline__ void team_places(const TeamArgs &t, uint32_t &p) {
+    for (; p < t.block_places[blockIdx.x + 1u]; ++p) {
         const TeamPlace place = t.places[p];
         __syncthreads();  // the previous population's tables and arguments are no longer read
-        for (uint32_t i = threadIdx.x; i < sizeof(SoloArgs) / 4u; i += kSoloThreadsOf<W>)
-            reinterpret_cast<uint32_t *>(&s_args)[i] = reinterpret_cast<const uint32_t *>(t.members + place.member)[i];
+        for (uint32_t i = threadIdx.x; i < sizeof(SoloArgs) / 4u; i += kSoloThreads)
+            reinterpret_cast<uint32_t *>(&s_team_args)[i] = reinterpret_cast<const uint32_t *>(t.members + place.member)[i];
         __syncthreads();
-        if constexpr (ONE_SEED)
-            form_generations<W, LINKED, WEIGHTED, GENERAL>(s_args, t.keys, t.n_gen, t.keep_last != 0u, place.rank, place.team);
-        else
-            form_generations<W, LINKED, WEIGHTED, GENERAL>(s_args, s_args.keys, t.n_gen, t.keep_last != 0u, place.rank,
-                                                           place.team);
+        if (s_team_args.words != (uint32_t)W) return;
+        form_generations<W, LINKED, WEIGHTED, GENERAL>(s_team_args, s_team_args.keys, t.n_gen, t.keep_last != 0u, place.rank,
+                                                       place.team);
     }
+}
+template <bool LINKED, bool WEIGHTED, bool GENERAL>
+__global__ void __launch_bounds__(kSoloThreads, 1) k_teams(const __grid_constant__ TeamArgs t) {
+    uint32_t p = t.block_places[blockIdx.x];
+    team_places<8, LINKED, WEIGHTED, GENERAL>(t, p);
+    team_places<4, LINKED, WEIGHTED, GENERAL>(t, p);
+    team_places<2, LINKED, WEIGHTED, GENERAL>(t, p);
+    team_places<1, LINKED, WEIGHTED, GENERAL>(t, p);
 }
 
 template <int W, bool LINKED, bool WEIGHTED>
@@ -939,28 +947,14 @@ SoloKernel solo_instance(bool general) {
     k.fn = general ? (const void *)&k_generations<W, LINKED, WEIGHTED, true>
                    : (const void *)&k_generations<W, LINKED, WEIGHTED, false>;
     k.smem = GenSmem<W, LINKED>::kBytes;
-    k.threads = kSoloThreadsOf<W>;
     return k;
 }
-template <int W, bool LINKED, bool WEIGHTED, bool GENERAL, bool ONE_SEED = false>
+template <bool LINKED, bool WEIGHTED, bool GENERAL>
 SoloKernel team_instance() {
     SoloKernel k;
-    k.fn = (const void *)&k_teams<W, LINKED, WEIGHTED, GENERAL, ONE_SEED>;
-    k.smem = GenSmem<W, LINKED>::kBytes;
-    k.threads = kSoloThreadsOf<W>;
+    k.fn = (const void *)&k_teams<LINKED, WEIGHTED, GENERAL>;
+    k.smem = GenSmem<8, LINKED>::kBytes;  // the largest records' tables
     return k;
-}
-// The team kernel of one kind (team_kind).
-template <int W>
-SoloKernel team_kernel_of(uint32_t kind) {
-    switch (kind) {
-        case 0: return team_instance<W, false, false, false, true>();
-        case 1: return team_instance<W, false, false, false>();
-        case 2: return team_instance<W, false, false, true>();
-        case 3: return team_instance<W, true, false, true>();
-        case 4: return team_instance<W, false, true, true>();
-        default: return team_instance<W, true, true, true>();
-    }
 }
 
 }  // namespace

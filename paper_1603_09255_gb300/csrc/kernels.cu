@@ -1143,17 +1143,19 @@ SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted, bool general)
     }
 }
 
-SoloKernel team_kernel_w1(uint32_t kind);
-SoloKernel team_kernel_w2(uint32_t kind);
-SoloKernel team_kernel_w4(uint32_t kind);
-SoloKernel team_kernel_w8(uint32_t kind);
+SoloKernel team_kernel_plain();
+SoloKernel team_kernel_general();
+SoloKernel team_kernel_linked();
+SoloKernel team_kernel_weighted();
+SoloKernel team_kernel_both();
 
-SoloKernel team_kernel(uint32_t words, uint32_t kind) {
-    switch (words) {
-        case 1: return team_kernel_w1(kind);
-        case 2: return team_kernel_w2(kind);
-        case 4: return team_kernel_w4(kind);
-        default: return team_kernel_w8(kind);
+SoloKernel team_kernel(uint32_t kind) {
+    switch (kind) {
+        case 0: return team_kernel_plain();
+        case 1: return team_kernel_general();
+        case 2: return team_kernel_linked();
+        case 3: return team_kernel_weighted();
+        default: return team_kernel_both();
     }
 }
 
@@ -1163,7 +1165,7 @@ int prepare_solo(SoloKernel &k) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, (int)k.threads, k.smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, (int)kSoloThreads, k.smem);
     if (e != cudaSuccess || per_sm <= 0) return SPG_ERR_CUDA;
     k.resident = (uint32_t)per_sm * (uint32_t)sms;
     return SPG_OK;

@@ -78,7 +78,7 @@ int configure_solo(spg_pop *p, const Shape &shape) {
     if (rc != SPG_OK) return fail(rc, "generation kernel setup failed");
     p->solo = k;
     p->shape = shape;
-    p->solo_blocks = most_blocks(p->n, p->words, k.resident);
+    p->solo_blocks = most_blocks(p->n, k.resident);
     attach_locus(p);
     return SPG_OK;
 }
@@ -92,7 +92,7 @@ int enqueue_solo(spg_pop *p, uint32_t n_gen) {
         done += a.n_gen;
         a.keep_last = done == n_gen ? 1u : 0u;
         void *params[] = {&a};
-        const dim3 grid(p->solo_blocks), block(p->solo.threads);
+        const dim3 grid(p->solo_blocks), block(kSoloThreads);
         const cudaError_t e =
             p->solo_blocks == 1u ? cudaLaunchKernel(p->solo.fn, grid, block, params, p->solo.smem, p->stream)
                                  : cudaLaunchCooperativeKernel(p->solo.fn, grid, block, params, p->solo.smem, p->stream);

@@ -83,8 +83,7 @@ struct TeamMember {
     bool linked = false, weighted = false;
 };
 struct TeamLaunch {
-    std::vector<TeamMember> members;  // of one locus count and kind
-    uint32_t kind = 0;
+    std::vector<TeamMember> members;  // of one kind
     SoloKernel kernel;
     TeamArgs args{};
     char *table = nullptr;            // the members' arguments and the blocks' places
@@ -93,7 +92,7 @@ struct TeamLaunch {
     void release(const Allocator &alloc, cudaStream_t stream);
 };
 struct TeamSet {
-    TeamLaunch launch[4 * (kTeamKinds - 1)];  // by locus count and kind (plain members of one seed or several)
+    TeamLaunch launch[kTeamKinds];
     int build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream);  // synchronises
     int update(const SoloArgs *args);
     int step(uint32_t n_gen, bool keep_last, cudaStream_t stream);
@@ -101,7 +100,7 @@ struct TeamSet {
 };
 double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, std::vector<TeamPlace> &places,
                       std::vector<uint32_t> &block_places);
-uint32_t most_blocks(uint32_t n, uint32_t words, uint32_t resident);
+uint32_t most_blocks(uint32_t n, uint32_t resident);
 void solo_args(const PopView &v, const PopParams &prm, SoloArgs &a);
 
 int fail(int code, const char *fmt, ...);
@@ -127,8 +126,8 @@ PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap
 Segment segment_at(char *base, const PopLayout &L, uint32_t n, uint32_t ntiles, uint32_t tile_begin,
                    uint32_t nbuckets, uint32_t bucket_begin);
 uint32_t bucket_count(uint32_t n);
-uint32_t slot_length(uint32_t n, uint32_t words);
-uint32_t slot_count(uint32_t n, uint32_t words);
+uint32_t slot_length(uint32_t n);
+uint32_t slot_count(uint32_t n);
 PopLayout solo_layout_for(uint32_t n, uint32_t words, uint32_t cap, bool weighted);
 int view_pack(const PopView &v, uint32_t gen, const uint32_t *surv, uint32_t S);
 Shape default_shape(uint32_t words);

@@ -190,10 +190,8 @@ using GenKernel = void (*)(GenArgs);
 // offspring are cut into slots of slot_len groups; a generation's survivors
 // are packed slot by slot in packed[generation & 1], counts[generation & 1]
 // holding their number per slot.
-constexpr uint32_t solo_threads(uint32_t words) { return words == 0 ? 0u : 512u; }
-constexpr uint32_t max_slots(uint32_t words) { return 152u * (solo_threads(words) / 32u); }  // one per resident warp on 152 SMs
-template <int W>
-constexpr uint32_t kSoloThreadsOf = solo_threads((uint32_t)W);
+constexpr uint32_t kSoloThreads = 512;  // (768 and 1,024 threads spill: 1.1 and 1.4 times the time at L = 32)
+constexpr uint32_t kMaxSlots = 152 * (kSoloThreads / 32);  // one per resident warp on 152 SMs
 constexpr uint32_t kOneBlockGroups = 16;  // groups up to which one block is no slower than several and a grid barrier
 // The per-locus values as f16 elements, laid out as the matrix fragments of
 // the generation kernel (value_fragments): the additive values, or with
@@ -242,7 +240,7 @@ struct alignas(16) SoloArgs {
 };
 struct SoloKernel {
     const void *fn = nullptr;
-    uint32_t threads = 0, smem = 0, resident = 0;  // resident: blocks on the device at a time
+    uint32_t smem = 0, resident = 0;  // resident: blocks on the device at a time
 };
 SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted, bool general);
 int prepare_solo(SoloKernel &k);  // sets the shared-memory limit, fills `resident`
@@ -255,19 +253,18 @@ struct TeamPlace {
     uint16_t rank, team;
 };
 struct TeamArgs {
-    uint32_t keys[20];  // the members' common Philox round keys (kind 0)
     const SoloArgs *members;
     const TeamPlace *places;
     const uint32_t *block_places;
     uint32_t n_gen, keep_last;
 };
-// Kinds of members that share a launch (with their locus count): plain ones of
-// one seed, plain ones, general values, linkage map, parent weights, both.
-constexpr uint32_t kTeamKinds = 6;
+// Kinds of members that share a launch: plain ones, general values, linkage
+// map, parent weights, both.
+constexpr uint32_t kTeamKinds = 5;
 inline uint32_t team_kind(bool linked, bool weighted, bool general) {
-    return linked ? (weighted ? 5u : 3u) : weighted ? 4u : general ? 2u : 1u;
+    return linked ? (weighted ? 4u : 2u) : weighted ? 3u : general ? 1u : 0u;
 }
-SoloKernel team_kernel(uint32_t words, uint32_t kind);
+SoloKernel team_kernel(uint32_t kind);
 // Enqueue the slot layout of a generation: bitmap words and per-slot counts
 // of the survivors (surv: their ordered list of S, null for all n), their
 // records packed[slot ...] and, when mate is given, their parent thresholds;

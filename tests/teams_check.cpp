@@ -42,6 +42,8 @@ int main() {
                 team[x.member] = x.team;
                 seen[x.member].resize(x.team);
                 if (seen[x.member][x.rank]++) return fail(c, "a rank twice");
+                if (p > start[b] && members[places[p - 1].member].words < members[x.member].words)
+                    return fail(c, "locus counts not in order");
                 for (uint32_t q = start[b]; q < p; ++q)
                     if (places[q].member == x.member) return fail(c, "a block twice in a team");
             }
