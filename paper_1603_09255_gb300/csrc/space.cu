@@ -9,7 +9,7 @@
 // (age 2, then 1, then 0).  One step is eight launches, none of which waits
 // on another block:
 //   k_sp_plan      one thread per deme: interaction factor f, births B;
-//   k_sp_scan      (x2) one block: exclusive scans of births (offsets of
+//   k_sp_offsets   (x2) exclusive scans, from block sums, of births (offsets of
 //                  each deme's newborns in the step's newborn arrays) and of
 //                  the new deme sizes;
 //   k_sp_classify  one block per deme: survival, ageing and direction of
@@ -19,9 +19,11 @@
 //   k_sp_totals    one thread per destination deme: offsets of the five
 //                  source slots (stay, from N, S, E, W) per age class;
 //   k_sp_births    grid-stride over all newborns: records formed and
-//                  written with age and phenotype to their final positions;
-//   k_sp_scatter   one block per deme: surviving members' records, ages and
-//                  phenotypes to their final positions;
+//                  appended to the pool, age and phenotype written to their
+//                  final positions;
+//   k_sp_scatter   one block per deme: surviving members' record slots, ages
+//                  and phenotypes to their final positions (their records
+//                  too in the steps that move them);
 //   k_sp_finish    one thread: statistics record, step counter.
 #include <cuda_runtime.h>
 
@@ -67,16 +69,23 @@ struct alignas(16) SpState {
     int32_t status;    // SPG_OK or an error
     uint32_t total;    // individuals in the current layout
     uint32_t births;   // newborns of the step in progress
+    uint32_t pool;     // the pool that holds the records
+    uint32_t top;      // its records used so far
+    uint32_t move;     // the step in progress moves all records to the other pool
+    uint32_t pad;
 };
 
 struct SpaceArgs {
     const SpeciesParams *sp;
     uint32_t X, Y, P, ns, nd;
+    uint32_t keys[20];   // Philox round keys (word 0, word 1 of each round)
     uint32_t key0, key1, disp_q32;
     uint32_t cap, staging_cap, ring_cap;
-    uint32_t *geno[2];   // [cap][2W] by step parity
-    uint8_t *age[2];     // [cap]
-    int32_t *raw[2];     // [cap] additive phenotype of each record, set at birth
+    uint32_t *pool[2];   // [cap][2W] records (see k_sp_scatter)
+    // [cap] by step parity: the place of each individual's record in the pool,
+    // and its additive phenotype, set at birth, times 4 plus its age class (one
+    // 8-byte store moves an individual: |phenotype| <= 2^24)
+    uint2 *ind[2];
     uint32_t *off[2];    // [nd + 1]
     uint32_t *adults[2]; // [nd]
     uint32_t *f, *births, *nb_off;   // [nd], [nd], [nd + 1]
@@ -86,6 +95,7 @@ struct SpaceArgs {
     uint32_t *cnt;                   // [nd][15] per source deme and (age class, direction)
     uint32_t *slotoff;               // [nd][15] per destination deme and (age class, slot)
     uint32_t *nnew;                  // [nd]
+    uint32_t *block_sum[2];          // births and new deme sizes, summed over kSpBlock demes
     SpState *state;
     SpAcc *acc;                      // [ns]
     spg_space_stats *ring;           // [ring_cap][ns]
@@ -102,6 +112,32 @@ __device__ __forceinline__ uint4 sp_philox(uint4 c, uint32_t k0, uint32_t k1) {
         c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
         k0 += WA;
         k1 += WB;
+    }
+    return c;
+}
+// The same at counters (i, t, d, word) with t and d fixed: the round keys from
+// the kernel's parameters, and the products that the first two rounds share
+// made once per (t, d).
+struct SpRng {
+    uint32_t hx, lx, cy;
+};
+__device__ __forceinline__ SpRng sp_rng(const uint32_t (&keys)[20], uint32_t t, uint32_t d) {
+    constexpr uint32_t A = 0xD2511F53u, B = 0xCD9E8D57u;
+    const unsigned long long q = (unsigned long long)B * d;
+    const unsigned long long p = (unsigned long long)A * ((uint32_t)(q >> 32) ^ t ^ keys[0]);
+    return SpRng{(uint32_t)(p >> 32) ^ keys[3], (uint32_t)p, (uint32_t)q ^ keys[2]};
+}
+__device__ __forceinline__ uint4 sp_philox_at(const SpRng &r, const uint32_t (&keys)[20], uint32_t i, uint32_t word) {
+    constexpr uint32_t A = 0xD2511F53u, B = 0xCD9E8D57u;
+    const unsigned long long ai = (unsigned long long)A * i;
+    unsigned long long p0, p1 = (unsigned long long)B * ((uint32_t)(ai >> 32) ^ word ^ keys[1]);
+    uint4 c = make_uint4((uint32_t)(p1 >> 32) ^ r.cy, (uint32_t)p1, r.hx ^ (uint32_t)ai, r.lx);
+#pragma unroll
+    for (int k = 2; k < 10; ++k) {
+        p0 = (unsigned long long)A * c.x;
+        p1 = (unsigned long long)B * c.z;
+        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ keys[2 * k], (uint32_t)p1,
+                       (uint32_t)(p0 >> 32) ^ c.w ^ keys[2 * k + 1], (uint32_t)p0);
     }
     return c;
 }
@@ -189,6 +225,10 @@ __device__ __forceinline__ uint32_t sp_bin(const SpeciesParams *sp, int32_t raw)
     return v < 0 ? 0u : (uint32_t)min(v >> sp->shift, (long long)(kBins - 1));
 }
 
+__device__ __forceinline__ uint32_t sp_pack(int32_t raw, uint32_t age) { return ((uint32_t)raw << 2) | age; }
+__device__ __forceinline__ int32_t sp_raw(uint32_t x) { return (int32_t)x >> 2; }
+__device__ __forceinline__ uint32_t sp_age(uint32_t x) { return x & 3u; }
+
 // ------------------------------------------------------------- founders
 template <int W>
 __global__ void k_sp_founders(SpaceArgs a, const uint32_t *n0, const uint32_t *p0) {
@@ -213,13 +253,24 @@ __global__ void k_sp_founders(SpaceArgs a, const uint32_t *n0, const uint32_t *p
         rec[hw] = word;
     }
 #pragma unroll
-    for (int hw = 0; hw < 2 * W; ++hw) a.geno[0][(size_t)i * 2 * W + hw] = rec[hw];
-    a.raw[0][i] = sp_phenotype<W>(rec, a.sp + s, a.sp[s].planes);
+    for (int hw = 0; hw < 2 * W; ++hw) a.pool[0][(size_t)i * 2 * W + hw] = rec[hw];
+    const int32_t raw = sp_phenotype<W>(rec, a.sp + s, a.sp[s].planes);
     const uint32_t half = n0[s] / 2, quarter = n0[s] / 4;
-    a.age[0][i] = r < half ? 2 : (r < half + quarter ? 1 : 0);
+    a.ind[0][i] = make_uint2(i, sp_pack(raw, r < half ? 2u : r < half + quarter ? 1u : 0u));
 }
 
 // ------------------------------------------------------------- planning
+// The block's sum of x, for k_sp_offsets.
+__device__ __forceinline__ void sp_block_sum(uint32_t x, uint32_t *out) {
+    __shared__ uint32_t s_sum;
+    if (threadIdx.x == 0) s_sum = 0u;
+    __syncthreads();
+    x = __reduce_add_sync(0xFFFFFFFFu, x);
+    if ((threadIdx.x & 31u) == 0u && x) atomicAdd(&s_sum, x);
+    __syncthreads();
+    if (threadIdx.x == 0) out[blockIdx.x] = s_sum;
+}
+
 __global__ void k_sp_plan(SpaceArgs a) {
     const uint32_t par = a.state->t & 1u;
     const uint32_t d = blockIdx.x * blockDim.x + threadIdx.x;
@@ -257,6 +308,7 @@ __global__ void k_sp_plan(SpaceArgs a) {
         nad = m;
         nbirth = B;
     }
+    sp_block_sum(d < a.nd ? (uint32_t)nbirth : 0u, a.block_sum[0]);
     // per-species sums: demes of one block belong to at most two species
     for (uint32_t k = 0; k < a.ns; ++k) {
         const bool mine = d < a.nd && s == k;
@@ -271,41 +323,42 @@ __global__ void k_sp_plan(SpaceArgs a) {
     }
 }
 
-// Exclusive scan of `in` (n values) into out[0..n] (out[n] = total) by one
-// block; flags capacity overflow.  which = 0: births -> staging offsets,
-// which = 1: new deme sizes -> offsets of the next layout.
-__global__ void k_sp_scan(SpaceArgs a, int which) {
-    __shared__ uint32_t s_warp[32];
-    __shared__ uint32_t s_carry;
+// Exclusive scan of `in` (nd values) into out[0..nd] (out[nd] = total), blocks
+// of kSpBlock values: the kernel before left each block's sum, so a block adds
+// those before it (one block scanning all values took 15 us of a step at
+// 12,288 demes).  The last block flags capacity overflow.  which = 0: births
+// -> staging offsets, which = 1: new deme sizes -> offsets of the next layout.
+__global__ void __launch_bounds__(kSpBlock) k_sp_offsets(SpaceArgs a, int which) {
+    __shared__ uint32_t s_warp[kSpBlock / 32], s_before[kSpBlock / 32];
     const uint32_t *in = which == 0 ? a.births : a.nnew;
     uint32_t *out = which == 0 ? a.nb_off : a.off[(a.state->t + 1u) & 1u];
-    const uint32_t n = a.nd, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) s_carry = 0;
-    __syncthreads();
-    for (uint32_t base = 0; base < n; base += blockDim.x) {
-        const uint32_t i = base + tid;
-        const uint32_t v = i < n ? in[i] : 0u;
-        uint32_t incl = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if ((int)lane >= o) incl += y;
-        }
-        if (lane == 31) s_warp[warp] = incl;
-        __syncthreads();
-        uint32_t wbase = 0;
-        for (uint32_t q = 0; q < warp; ++q) wbase += s_warp[q];
-        const uint32_t carry = s_carry;
-        if (i < n) out[i] = carry + wbase + incl - v;
-        __syncthreads();
-        if (tid == blockDim.x - 1) s_carry = carry + wbase + incl;
-        __syncthreads();
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, i = blockIdx.x * kSpBlock + tid;
+    const uint32_t v = i < a.nd ? in[i] : 0u;
+    uint32_t before = 0;
+    for (uint32_t j = tid; j < blockIdx.x; j += kSpBlock) before += a.block_sum[which][j];
+    before = __reduce_add_sync(0xFFFFFFFFu, before);
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if ((int)lane >= o) incl += y;
     }
-    if (tid == 0) {
-        out[n] = s_carry;
+    if (lane == 31u) s_warp[warp] = incl;
+    if (lane == 0u) s_before[warp] = before;
+    __syncthreads();
+    uint32_t base = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < kSpBlock / 32; ++q) base += s_before[q] + (q < warp ? s_warp[q] : 0u);
+    if (i < a.nd) out[i] = base + incl - v;
+    if (i == a.nd - 1u) {
+        const uint32_t total = base + incl;
+        out[a.nd] = total;
         if (which == 0) {
-            a.state->births = s_carry;
-            if (s_carry > a.staging_cap) a.state->status = SPG_ERR_RANGE;
-        } else if (s_carry > a.cap) {
+            a.state->births = total;
+            if (total > a.staging_cap) a.state->status = SPG_ERR_RANGE;
+            // no room for the newborns behind the records: all move this step
+            a.state->move = (unsigned long long)a.state->top + total > a.cap ? 1u : 0u;
+        } else if (total > a.cap) {
             a.state->status = SPG_ERR_RANGE;
         }
     }
@@ -401,10 +454,10 @@ __global__ void __launch_bounds__(kSpClassBlock) k_sp_classify(SpaceArgs a) {
     const uint32_t d = blockIdx.x, s = d / a.P, tid = threadIdx.x;
     const uint32_t t = a.state->t + 1u, par = a.state->t & 1u;
     const SpeciesParams *sp = a.sp + s;
-    const uint8_t *age = a.age[par];
-    const int32_t *rawp = a.raw[par];
+    const uint2 *ind = a.ind[par];
     const uint32_t base = a.off[par][d], n = a.off[par][d + 1] - base;
     const uint32_t f = a.f[d], B = a.births[d], nb0 = a.nb_off[d];
+    const SpRng rng = sp_rng(a.keys, t, d);
     if (tid < 16) s_carry[tid] = 0;
     __syncthreads();
     long long sum_raw = 0;
@@ -417,15 +470,16 @@ __global__ void __launch_bounds__(kSpClassBlock) k_sp_classify(SpaceArgs a) {
         // a genotype is fixed for life, so its phenotype was computed once at birth
 #pragma unroll
         for (int i = 0; i < kSpIPT; ++i) {
-            ag[i] = r0 + i < n ? age[base + r0 + i] : 0u;
-            raw[i] = r0 + i < n ? rawp[base + r0 + i] : 0;
+            const uint32_t x = r0 + i < n ? ind[base + r0 + i].y : 0u;
+            ag[i] = sp_age(x);
+            raw[i] = sp_raw(x);
         }
 #pragma unroll
         for (int i = 0; i < kSpIPT; ++i) {
             const uint32_t r = r0 + (uint32_t)i;
             cls[i] = kDead;
             if (r < n) {
-                const uint4 u = sp_philox(make_uint4(r, t, d, kSpSurv << 24), a.key0, a.key1);
+                const uint4 u = sp_philox_at(rng, a.keys, r, kSpSurv << 24);
                 uint32_t thr = __ldg(&sp->table[ag[i]][sp_bin(sp, raw[i])]);
                 if (f != kCertain) thr = __umulhi(thr, f);
                 if (thr == kCertain || u.x < thr) {
@@ -455,10 +509,9 @@ __global__ void __launch_bounds__(kSpClassBlock) k_sp_classify(SpaceArgs a) {
             const uint32_t k = c0 + tid * kSpNbIPT + (uint32_t)i;
             cls[i] = kDead;
             if (k < B && nb0 + k < a.staging_cap) {
-                const uint4 u = sp_philox(make_uint4(k, t, d, kSpMate << 24), a.key0, a.key1);
+                const uint4 u = sp_philox_at(rng, a.keys, k, kSpMate << 24);
                 uint32_t dir = 0;
-                if (u.z < a.disp_q32)
-                    dir = 1u + __umulhi(sp_philox(make_uint4(k, t, d, kSpDisp << 24), a.key0, a.key1).x, 4u);
+                if (u.z < a.disp_q32) dir = 1u + __umulhi(sp_philox_at(rng, a.keys, k, kSpDisp << 24).x, 4u);
                 cls[i] = 2u * 5u + dir;
                 moved += dir != 0;
             }
@@ -502,21 +555,27 @@ __global__ void __launch_bounds__(kSpBlock) k_sp_births(SpaceArgs a) {
     for (uint32_t k = 0; k < a.ns; ++k) sp_stage_planes<W>(a.sp + k, s_planes[k]);
     __syncthreads();
     uint32_t het_s[kMaxSpecies] = {0u, 0u, 0u, 0u}, allele_s[kMaxSpecies] = {0u, 0u, 0u, 0u};
-    const uint32_t *geno = a.geno[par];
-    uint32_t *ngeno = a.geno[par ^ 1u];
+    const uint2 *ind = a.ind[par];
+    uint2 *nind = a.ind[par ^ 1u];
     const uint32_t *noff = a.off[par ^ 1u];
+    const bool move = a.state->move != 0u;
+    const uint32_t top = a.state->top;
+    const uint32_t *geno = a.pool[a.state->pool];
+    uint32_t *ngeno = a.pool[a.state->pool ^ (move ? 1u : 0u)];
     for (uint32_t i = blockIdx.x * kSpBlock + tid; i < total; i += gridDim.x * kSpBlock) {
         const uint32_t d = a.nb_deme[i], s = d / a.P, k = i - a.nb_off[d];
         const uint32_t dir = a.nb_cls[i] % 5u, rk = a.nb_rank[i];  // class 10 + dir: age 0
         const SpeciesParams *sp = a.sp + s;
         const uint32_t base = a.off[par][d], m = a.adults[par][d];
-        const uint4 u = sp_philox(make_uint4(k, t, d, kSpMate << 24), a.key0, a.key1);
+        const SpRng rng = sp_rng(a.keys, t, d);
+        const uint4 u = sp_philox_at(rng, a.keys, k, kSpMate << 24);
         uint32_t mo[2 * W], fa[2 * W], ch[2 * W];
-        sp_load_rec<W>(geno + (size_t)(base + __umulhi(u.x, m)) * 2 * W, mo);
-        sp_load_rec<W>(geno + (size_t)(base + __umulhi(u.y, m)) * 2 * W, fa);
+        const uint32_t sm = ind[base + __umulhi(u.x, m)].x, sf = ind[base + __umulhi(u.y, m)].x;
+        sp_load_rec<W>(geno + (size_t)sm * 2 * W, mo);
+        sp_load_rec<W>(geno + (size_t)sf * 2 * W, fa);
 #pragma unroll
         for (int q4 = 0; q4 < (2 * W + 3) / 4; ++q4) {
-            const uint4 dm = sp_philox(make_uint4(k, t, d, (kSpRecomb << 24) | (uint32_t)q4), a.key0, a.key1);
+            const uint4 dm = sp_philox_at(rng, a.keys, k, (kSpRecomb << 24) | (uint32_t)q4);
 #pragma unroll
             for (int l = 0; l < 4; ++l) {
                 const int q = 4 * q4 + l;
@@ -561,9 +620,9 @@ __global__ void __launch_bounds__(kSpBlock) k_sp_births(SpaceArgs a) {
         const uint32_t q = s * a.P + sp_dest(a, d % a.P, dir);
         const uint32_t pos = noff[q] + a.slotoff[(size_t)q * 15 + 2u * 5u + sp_slot(dir)] + rk;
         if (pos < a.cap) {
-            sp_store_rec<W>(ngeno + (size_t)pos * 2 * W, ch);
-            a.age[par ^ 1u][pos] = 0;
-            a.raw[par ^ 1u][pos] = sp_phenotype<W>(ch, sp, s_planes[s]);
+            const uint32_t mine = move ? pos : top + i;  // where the newborn's record goes
+            sp_store_rec<W>(ngeno + (size_t)mine * 2 * W, ch);
+            nind[pos] = make_uint2(mine, sp_pack(sp_phenotype<W>(ch, sp, s_planes[s]), 0u));
         }
         uint32_t het = 0, allele = 0;
 #pragma unroll
@@ -613,6 +672,7 @@ __global__ void k_sp_totals(SpaceArgs a) {
     } else if (q < a.nd) {
         a.nnew[q] = 0;
     }
+    sp_block_sum(total, a.block_sum[1]);
     for (uint32_t k = 0; k < a.ns; ++k) {
         const bool mine = ok && s == k;
         const uint32_t v0 = __reduce_add_sync(0xFFFFFFFFu, mine ? total : 0u);
@@ -625,32 +685,57 @@ __global__ void k_sp_totals(SpaceArgs a) {
 }
 
 // ------------------------------------------------------ new layout
+// Survivors' slots, ages and phenotypes to their places.  Records stay where
+// they are in the pool and newborns' records are appended in birth order, so a
+// deme's records remain a few contiguous pieces; when the pool has no room for
+// a step's newborns (every fifth step or so at twice the founders' capacity)
+// the step moves all records to the other pool in the new layout's order.
+// Most steps so move 8 bytes an individual instead of 8W + 5.  (A free list
+// that hands the dead's slots to newborns never moves records, but scatters a
+// deme's records over the pool: 502 us a step against 453 with every step
+// moving them, at 10^7 individuals of 64 bytes.)
 template <int W>
 __global__ void __launch_bounds__(kSpBlock) k_sp_scatter(SpaceArgs a) {
+    __shared__ uint32_t s_base[15];
     if (a.state->status != SPG_OK) return;
     const uint32_t d = blockIdx.x, s = d / a.P, p = d % a.P, tid = threadIdx.x;
     const uint32_t par = a.state->t & 1u, npar = par ^ 1u;
-    const uint32_t *geno = a.geno[par];
-    uint32_t *ngeno = a.geno[npar];
-    uint8_t *nage = a.age[npar];
-    int32_t *nraw = a.raw[npar];
-    const uint32_t *noff = a.off[npar];
+    const bool move = a.state->move != 0u;
+    const uint32_t *geno = a.pool[a.state->pool];
+    uint32_t *ngeno = a.pool[a.state->pool ^ 1u];
+    const uint2 *ind = a.ind[par];
+    uint2 *nind = a.ind[npar];
     const uint32_t base = a.off[par][d], n = a.off[par][d + 1] - base;
+    if (tid < 15u) {  // where each (age class, direction) class of the deme starts
+        const uint32_t q = s * a.P + sp_dest(a, p, tid % 5u);
+        s_base[tid] = a.off[npar][q] + a.slotoff[(size_t)q * 15 + tid / 5u * 5u + sp_slot(tid % 5u)];
+    }
+    __syncthreads();
     for (uint32_t i = tid; i < n; i += kSpBlock) {
         const uint32_t cls = a.cls[base + i], rk = a.rank[base + i];
-        const uint32_t *src = geno + (size_t)(base + i) * 2 * W;
-        const int32_t *src_raw = a.raw[par] + base + i;
+        const uint2 x = ind[base + i];
         if (cls >= kDead) continue;
-        const uint32_t ci = cls / 5u, dir = cls % 5u;
-        const uint32_t q = s * a.P + sp_dest(a, p, dir);
-        const uint32_t pos = noff[q] + a.slotoff[(size_t)q * 15 + ci * 5 + sp_slot(dir)] + rk;
+        const uint32_t pos = s_base[cls] + rk;
         if (pos >= a.cap) continue;
-        uint32_t rec[2 * W];
-        sp_load_rec<W>(src, rec);
-        sp_store_rec<W>(ngeno + (size_t)pos * 2 * W, rec);
-        nage[pos] = (uint8_t)(2u - ci);
-        nraw[pos] = *src_raw;
+        if (move) {
+            uint32_t rec[2 * W];
+            sp_load_rec<W>(geno + (size_t)x.x * 2 * W, rec);
+            sp_store_rec<W>(ngeno + (size_t)pos * 2 * W, rec);
+        }
+        nind[pos] = make_uint2(move ? pos : x.x, sp_pack(sp_raw(x.y), 2u - cls / 5u));
     }
+}
+
+// rec[i], age[i]: record and age class of individual first + i (either may be
+// null).
+__global__ void k_sp_gather(SpaceArgs a, uint32_t pool, uint32_t par, uint32_t first, uint32_t words, uint32_t count,
+                            uint32_t *rec, uint8_t *age) {
+    for (uint32_t x = blockIdx.x * blockDim.x + threadIdx.x; age && x < count; x += gridDim.x * blockDim.x)
+        age[x] = (uint8_t)sp_age(a.ind[par][first + x].y);
+    if (!rec) return;
+    const size_t total = (size_t)count * words;
+    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < total; x += (size_t)gridDim.x * blockDim.x)
+        rec[x] = a.pool[pool][(size_t)a.ind[par][first + x / words].x * words + x % words];
 }
 
 // ---------------------------------------------------------- step end
@@ -679,6 +764,8 @@ __global__ void k_sp_finish(SpaceArgs a) {
     __syncthreads();
     if (k == 0 && st->status == SPG_OK) {
         st->total = a.off[t & 1u][a.nd];
+        st->top = st->move ? st->total : st->top + st->births;
+        st->pool ^= st->move;
         st->t = t;
     }
 }
@@ -737,12 +824,12 @@ template <int W>
 int launch_step(spg_space *c) {
     const SpaceArgs &a = c->args;
     cudaStream_t s = c->stream;
-    const uint32_t g = (a.nd + 255) / 256;
-    k_sp_plan<<<g, 256, 0, s>>>(a);
-    k_sp_scan<<<1, 1024, 0, s>>>(a, 0);
+    const uint32_t g = (a.nd + kSpBlock - 1) / kSpBlock;
+    k_sp_plan<<<g, kSpBlock, 0, s>>>(a);
+    k_sp_offsets<<<g, kSpBlock, 0, s>>>(a, 0);
     k_sp_classify<<<a.nd, kSpClassBlock, 0, s>>>(a);
-    k_sp_totals<<<g, 256, 0, s>>>(a);
-    k_sp_scan<<<1, 1024, 0, s>>>(a, 1);
+    k_sp_totals<<<g, kSpBlock, 0, s>>>(a);
+    k_sp_offsets<<<g, kSpBlock, 0, s>>>(a, 1);
     // the newborns on the side stream beside the survivors' move: both only
     // read the current generation and write disjoint places of the next; the
     // newborns' kernel goes first so that its resident grid is placed before
@@ -883,8 +970,7 @@ int spg_space_create(const spg_space_desc *desc, const spg_allocator *alloc, voi
     };
     const size_t o_sp = take(sizeof(SpeciesParams) * c->ns);
     const size_t o_g0 = take((size_t)c->cap * 2 * c->W * 4), o_g1 = take((size_t)c->cap * 2 * c->W * 4);
-    const size_t o_a0 = take(c->cap), o_a1 = take(c->cap);
-    const size_t o_r0 = take((size_t)c->cap * 4), o_r1 = take((size_t)c->cap * 4);
+    const size_t o_i0 = take((size_t)c->cap * 8), o_i1 = take((size_t)c->cap * 8);
     const size_t o_nd = take((size_t)c->staging_cap * 4);
     const size_t o_off0 = take((size_t)(c->nd + 1) * 4), o_off1 = take((size_t)(c->nd + 1) * 4);
     const size_t o_ad0 = take((size_t)c->nd * 4), o_ad1 = take((size_t)c->nd * 4);
@@ -892,6 +978,7 @@ int spg_space_create(const spg_space_desc *desc, const spg_allocator *alloc, voi
     const size_t o_cls = take(c->cap), o_ncls = take(c->staging_cap);
     const size_t o_rk = take((size_t)c->cap * 4), o_nrk = take((size_t)c->staging_cap * 4);
     const size_t o_cnt = take((size_t)c->nd * 15 * 4), o_so = take((size_t)c->nd * 15 * 4), o_nn = take((size_t)c->nd * 4);
+    const size_t o_bs = take((size_t)2 * ((c->nd + kSpBlock - 1) / kSpBlock) * 4);
     const size_t o_st = take(sizeof(SpState)), o_acc = take(sizeof(SpAcc) * c->ns);
     const size_t o_ring = take((size_t)c->ring_cap * c->ns * sizeof(spg_space_stats));
     const size_t o_n0 = take(4 * c->ns), o_p0 = take(4 * c->ns);
@@ -930,12 +1017,14 @@ int spg_space_create(const spg_space_desc *desc, const spg_allocator *alloc, voi
     a.cap = c->cap;
     a.staging_cap = c->staging_cap;
     a.ring_cap = c->ring_cap;
-    a.geno[0] = reinterpret_cast<uint32_t *>(b + o_g0);
-    a.geno[1] = reinterpret_cast<uint32_t *>(b + o_g1);
-    a.age[0] = reinterpret_cast<uint8_t *>(b + o_a0);
-    a.age[1] = reinterpret_cast<uint8_t *>(b + o_a1);
-    a.raw[0] = reinterpret_cast<int32_t *>(b + o_r0);
-    a.raw[1] = reinterpret_cast<int32_t *>(b + o_r1);
+    for (uint32_t i = 0; i < 10; ++i) {
+        a.keys[2 * i] = a.key0 + i * 0x9E3779B9u;
+        a.keys[2 * i + 1] = a.key1 + i * 0xBB67AE85u;
+    }
+    a.pool[0] = reinterpret_cast<uint32_t *>(b + o_g0);
+    a.pool[1] = reinterpret_cast<uint32_t *>(b + o_g1);
+    a.ind[0] = reinterpret_cast<uint2 *>(b + o_i0);
+    a.ind[1] = reinterpret_cast<uint2 *>(b + o_i1);
     a.nb_deme = reinterpret_cast<uint32_t *>(b + o_nd);
     a.off[0] = reinterpret_cast<uint32_t *>(b + o_off0);
     a.off[1] = reinterpret_cast<uint32_t *>(b + o_off1);
@@ -951,6 +1040,8 @@ int spg_space_create(const spg_space_desc *desc, const spg_allocator *alloc, voi
     a.cnt = reinterpret_cast<uint32_t *>(b + o_cnt);
     a.slotoff = reinterpret_cast<uint32_t *>(b + o_so);
     a.nnew = reinterpret_cast<uint32_t *>(b + o_nn);
+    a.block_sum[0] = reinterpret_cast<uint32_t *>(b + o_bs);
+    a.block_sum[1] = a.block_sum[0] + (c->nd + kSpBlock - 1) / kSpBlock;
     a.state = reinterpret_cast<SpState *>(b + o_st);
     a.acc = reinterpret_cast<SpAcc *>(b + o_acc);
     a.ring = reinterpret_cast<spg_space_stats *>(b + o_ring);
@@ -964,7 +1055,7 @@ int spg_space_create(const spg_space_desc *desc, const spg_allocator *alloc, voi
             run += n0[s];
         }
     offs[c->nd] = run;
-    SpState st0{0, SPG_OK, run, 0};
+    SpState st0{0, SPG_OK, run, 0, 0, run, 0, 0};
     e = cudaMemcpy(b + o_sp, prm.data(), sizeof(SpeciesParams) * c->ns, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(a.off[0], offs.data(), offs.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(a.adults[0], adults.data(), adults.size() * 4, cudaMemcpyHostToDevice);
@@ -1074,10 +1165,20 @@ int spg_space_read_deme(spg_space *c, uint32_t species, uint32_t patch, uint32_t
     *n = o[1] - o[0];
     if (!rec && !age) return SPG_OK;
     if (capacity < *n) return fail(SPG_ERR_INVALID, "buffer holds %zu individuals, need %u", capacity, *n);
-    if (rec)
-        e = cudaMemcpy(rec, c->args.geno[par] + (size_t)o[0] * 2 * c->W, (size_t)*n * 2 * c->W * 4,
-                       cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess && age) e = cudaMemcpy(age, c->args.age[par] + o[0], *n, cudaMemcpyDeviceToHost);
+    if (*n) {  // the deme's records and ages side by side, then to the host
+        const uint32_t words = 2 * c->W;
+        const size_t rec_bytes = rec ? (size_t)*n * words * 4 : 0, bytes = rec_bytes + *n;
+        char *tmp = static_cast<char *>(c->alloc.alloc(bytes, c->stream));
+        if (!tmp) return fail(SPG_ERR_OOM, "device allocation of %zu bytes failed", bytes);
+        k_sp_gather<<<304, 256, 0, c->stream>>>(c->args, st.pool, par, o[0], words, *n,
+                                               rec ? reinterpret_cast<uint32_t *>(tmp) : nullptr,
+                                               age ? reinterpret_cast<uint8_t *>(tmp + rec_bytes) : nullptr);
+        e = cudaGetLastError();
+        if (e == cudaSuccess && rec) e = cudaMemcpyAsync(rec, tmp, rec_bytes, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess && age) e = cudaMemcpyAsync(age, tmp + rec_bytes, *n, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        c->alloc.release(tmp, c->stream);
+    }
     return e == cudaSuccess ? SPG_OK : cuda_fail(e, "read deme");
 }
 
