@@ -61,11 +61,11 @@ struct GenSmem {
     static constexpr uint32_t kSetBytes = kRegRoom * 128u, kTabBytes = kSets * kSetBytes;
     static constexpr uint32_t kStage = kFrag + 2u * kTabBytes;
     static constexpr uint32_t kRecStage = kPlanes * 512u;
-    static constexpr uint32_t kTog = LINKED ? 2u * 32u * ((uint32_t)W + 3u) * 4u : 0u;
+    static constexpr uint32_t kTog = LINKED ? 2u * 32u * (uint32_t)W * 4u : 0u;
     static constexpr uint32_t kPerWarp = kRecStage > kTog ? kRecStage : (kTog + 15u) / 16u * 16u;
     static constexpr uint32_t kLinkOff = kStage + NW * kPerWarp;
-    // linkage map: cdf, cum, guide, chrom, first, clast
-    static constexpr uint32_t kLinkBytes = LINKED ? kMaxKmax * 4u + kMaxLoci * 4u + kLinkGuide * 4u + kMaxLoci + kMaxChrom * 4u : 0u;
+    // linkage map: cdf, cum, guide, first
+    static constexpr uint32_t kLinkBytes = LINKED ? kMaxKmax * 4u + kMaxLoci * 4u + kLinkGuide * 4u + (kMaxChrom + 2u) * 2u : 0u;
     static constexpr uint32_t kThreads = BLOCK;
     static constexpr uint32_t kStats = (kLinkOff + kLinkBytes + 15u) / 16u * 16u;  // lanes' statistics, 48 bytes each
     static constexpr uint32_t kBytes = kStats + 48u * BLOCK;
@@ -308,6 +308,127 @@ __device__ __forceinline__ uint4 philox_at(const RoundKeys &keys, const GenRng &
                        (uint32_t)(p0 >> 32) ^ c.w ^ keys[2 * i + 1], (uint32_t)p0);
     }
     return c;
+}
+
+// ------------------------------------------------------- linkage map
+// A linkage map in shared memory (see LinkParams).
+struct LinkMap {
+    const uint32_t *cdf, *cum, *guide;
+    const uint16_t *first;  // first locus of each chromosome, 0xFFFF past the last
+    uint32_t kmax;
+    uint32_t *tog;          // the warp's toggle words [gamete][W][lane]
+};
+
+// Origin masks of both gametes of a warp's 32 offspring under the linkage map
+// (bit set: the locus comes from the parent's haplotype 1); all lanes take
+// part, valid = false gives a lane no crossovers.  A crossover toggles its
+// first locus; a prefix XOR over the whole genome turns the toggles into
+// flips, and a chromosome's flips are brought to its coin at its first locus
+// by one comparison with the bit before it, so neither a crossover's
+// chromosome nor its end has to be found (applying each chromosome's coin and
+// end toggles took a quarter of the kernel).  The crossovers are dealt to the
+// warp's lanes one Philox block (up to four crossovers of one gamete) at a
+// time instead of each lane looping over its own, which would run the warp to
+// its lanes' largest count; toggles go to the owner's words in shared memory
+// by atomic XOR.
+template <int W>
+__device__ __forceinline__ void linked_masks(const LinkMap &lk, const RoundKeys &keys, const GenRng &rng, uint32_t j,
+                                             bool valid, uint32_t (&mm)[W], uint32_t (&mf)[W]) {
+    constexpr uint32_t L = 32u * W;
+    const uint32_t lane = threadIdx.x & 31u;
+    const unsigned long long aj = (unsigned long long)kPhA * j;
+    uint4 d0[2];
+    uint32_t K[2];
+#pragma unroll
+    for (uint32_t pi = 0; pi < 2u; ++pi) {
+        d0[pi] = philox_at(keys, rng, aj, (kLink << 24) | (pi << 8));
+        uint32_t k = 0;
+        if (valid && lk.kmax != 0u && d0[pi].x >= lk.cdf[0]) {
+            k = 1u;
+#pragma unroll
+            for (uint32_t step = 16u; step > 0u; step >>= 1)
+                if (k + step <= lk.kmax && lk.cdf[k + step - 1u] <= d0[pi].x) k += step;
+        }
+        K[pi] = k;
+#pragma unroll
+        for (uint32_t w = 0; w < (uint32_t)W; ++w) lk.tog[(pi * W + w) * 32u + lane] = 0u;
+    }
+    // this lane's Philox blocks of crossovers, both gametes, and the warp's offsets
+    const uint32_t nb0 = (K[0] + 3u) >> 2, nb = nb0 + ((K[1] + 3u) >> 2);
+    uint32_t off = nb;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, off, o);
+        if ((int)lane >= o) off += y;
+    }
+    const uint32_t total = __shfl_sync(0xFFFFFFFFu, off, 31);
+    off -= nb;  // exclusive
+    const uint32_t mine = off | nb0 << 10 | K[0] << 14 | K[1] << 20;  // off <= 512, nb0 <= 8, K <= 32
+    __syncwarp();
+    for (uint32_t f0 = 0; f0 < total; f0 += 32u) {
+        const uint32_t f = f0 + lane;
+        uint32_t o = 0;  // the owner: the last lane whose offset is <= f
+#pragma unroll
+        for (uint32_t step = 16u; step > 0u; step >>= 1) {
+            const uint32_t v = __shfl_sync(0xFFFFFFFFu, off, (int)(o + step));
+            if (v <= f) o += step;
+        }
+        const uint32_t x = __shfl_sync(0xFFFFFFFFu, mine, (int)o), oj = __shfl_sync(0xFFFFFFFFu, j, (int)o);
+        if (f < total) {
+            const uint32_t onb0 = (x >> 10) & 15u, b = f - (x & 1023u), pi = b < onb0 ? 0u : 1u,
+                           blk = pi ? b - onb0 : b, Kp = pi ? x >> 20 : (x >> 14) & 63u;
+            const uint4 d = philox_at(keys, rng, (unsigned long long)kPhA * oj, (kLink << 24) | (pi << 8) | (1u + blk));
+            uint32_t *ot = lk.tog + pi * W * 32u + o;
+#pragma unroll
+            for (uint32_t l = 0; l < 4u; ++l) {
+                if (4u * blk + l < Kp) {
+                    const uint32_t u = lane_of(d, (int)l);
+                    const uint32_t ge = lk.guide[u >> (32 - kLinkGuideBits)], nbd = ge >> 26;
+                    uint32_t I = ge & 0xFFu;  // the bucket's first interval; with no boundary in it, cum[I] > u
+                    I = min(I + (lk.cum[I] <= u ? 1u : 0u), L - 1u);
+                    if (nbd > 1u)
+                        while (I + 1u < L && lk.cum[I] <= u) ++I;
+                    atomicXor(ot + (I >> 5) * 32u, 1u << (I & 31u));
+                }
+            }
+        }
+    }
+    __syncwarp();
+    uint32_t before[2] = {0u, 0u};  // the flip of the locus before the word
+    uint32_t fix[2] = {0u, 0u};     // all ones where the running chromosome's flips are inverted
+    uint32_t coins[2][3] = {{d0[0].y, d0[0].z, d0[0].w}, {d0[1].y, d0[1].z, d0[1].w}};  // the next chromosome's lowest
+    uint32_t c = 0, next = 0u;      // the next chromosome and its first locus
+#pragma unroll
+    for (uint32_t w = 0; w < (uint32_t)W; ++w) {
+        uint32_t x[2], shifted[2], F[2];
+#pragma unroll
+        for (uint32_t pi = 0; pi < 2u; ++pi) {
+            uint32_t y = lk.tog[(pi * W + w) * 32u + lane];
+            y ^= y << 1;
+            y ^= y << 2;
+            y ^= y << 4;
+            y ^= y << 8;
+            y ^= y << 16;
+            x[pi] = y ^ (0u - before[pi]);
+            shifted[pi] = x[pi] << 1 | before[pi];  // the flip before each locus
+            before[pi] = x[pi] >> 31;
+            F[pi] = fix[pi];
+        }
+        while (next < 32u * (w + 1u)) {  // chromosomes that start in this word (the same in all lanes)
+            const uint32_t s = next & 31u, from = 0xFFFFFFFFu << s;
+#pragma unroll
+            for (uint32_t pi = 0; pi < 2u; ++pi) {
+                fix[pi] = 0u - ((coins[pi][0] ^ (shifted[pi] >> s)) & 1u);
+                F[pi] = (F[pi] & ~from) | (fix[pi] & from);
+                coins[pi][0] = __funnelshift_r(coins[pi][0], coins[pi][1], 1);
+                coins[pi][1] = __funnelshift_r(coins[pi][1], coins[pi][2], 1);
+                coins[pi][2] >>= 1;
+            }
+            next = lk.first[++c];
+        }
+        mm[w] = x[0] ^ F[0];
+        mf[w] = x[1] ^ F[1];
+    }
 }
 
 // ------------------------------------------------------- parents
@@ -645,29 +766,21 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
     }
     cp_async_commit();
     if (tid < (uint32_t)kMaxKmax) s_cdf[tid] = tid < a.kmax ? P->cdf[tid] : 0xFFFFFFFFu;
-    LinkSmem lk{};
+    LinkMap lk{};
     if constexpr (LINKED) {
         const LinkParams *lp = P->link;
         uint32_t *cdf = reinterpret_cast<uint32_t *>(g_smem + SM::kLinkOff), *cum = cdf + kMaxKmax, *gd = cum + kMaxLoci;
-        uint16_t *first = reinterpret_cast<uint16_t *>(gd + kLinkGuide), *clast = first + kMaxChrom;
-        uint8_t *chrom = reinterpret_cast<uint8_t *>(clast + kMaxChrom);
+        uint16_t *first = reinterpret_cast<uint16_t *>(gd + kLinkGuide);
         if (tid < (uint32_t)kMaxKmax) cdf[tid] = lp->cdf[tid];
-        for (uint32_t i = tid; i < 32u * W; i += BLOCK) {
-            cum[i] = lp->cum[i];
-            chrom[i] = lp->chrom[i];
-        }
+        for (uint32_t i = tid; i < 32u * W; i += BLOCK) cum[i] = lp->cum[i];
         for (uint32_t i = tid; i < (uint32_t)kLinkGuide; i += BLOCK) gd[i] = lp->guide[i];
-        if (tid < (uint32_t)kMaxChrom) {
-            first[tid] = lp->first[tid];
-            clast[tid] = lp->clast[tid];
-        }
-        lk = LinkSmem{cdf, cum, chrom, first, clast, gd, lp->kmax, lp->nchrom, nullptr};
+        if (tid <= (uint32_t)kMaxChrom) first[tid] = tid < lp->nchrom ? lp->first[tid] : (uint16_t)0xFFFFu;
+        lk = LinkMap{cdf, cum, gd, first, lp->kmax,
+                     reinterpret_cast<uint32_t *>(g_smem + SM::kStage + warp * SM::kPerWarp)};
     }
     const uint32_t rep = a.rep, k0 = keys[0], k1 = keys[1];
     const uint32_t rec_slot = a.slot_len * 32u;
     const uint32_t stage = smem0 + SM::kStage + warp * SM::kPerWarp, my_row = stage + stage_row(lane);
-    if constexpr (LINKED) lk.tog = reinterpret_cast<uint32_t *>(g_smem + SM::kStage + warp * SM::kPerWarp) -
-                                   warp * (2u * 32u * ((uint32_t)W + 3u));  // the helper adds its warp's offset
     const uint32_t slot0 = (uint32_t)(((unsigned long long)a.nslots * rank) / team);
     const uint32_t slot1 = (uint32_t)(((unsigned long long)a.nslots * (rank + 1u)) / team);
     bool one_step = true;
@@ -720,7 +833,7 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
                 uint32_t ch[2 * W];
                 if constexpr (LINKED) {
                     uint32_t mm[W], mf[W];
-                    linked_masks_warp<W>(lk, j, valid, g, rep, k0, k1, mm, mf);
+                    linked_masks<W>(lk, keys, rng, j, valid, mm, mf);
                     __syncwarp();  // the toggles' memory holds the staged records next
 #pragma unroll
                     for (int w = 0; w < W; ++w) {
