@@ -335,6 +335,7 @@ PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap
     };
     L.params = take(sizeof(PopParams));
     L.state = take(sizeof(DevState));
+    L.ring = take((size_t)cap * sizeof(spg_stats));
     L.acc = take(sizeof(StatAcc) * kAccCopies);
     L.geno0 = take((size_t)n * 2 * words * 4);
     L.geno1 = take((size_t)n * 2 * words * 4);
@@ -343,7 +344,6 @@ PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap
     L.surv1 = take((size_t)n * 4);
     L.alive = take((size_t)nbuckets * kBucketWords * 4);
     L.buckets = take((size_t)2 * nbuckets * 4);
-    L.ring = take((size_t)cap * sizeof(spg_stats));
     L.segment = take(sizeof(Segment));
     L.link = take(sizeof(LinkParams));
     L.weighted = weighted;
@@ -380,6 +380,7 @@ PopLayout solo_layout_for(uint32_t n, uint32_t words, uint32_t cap, bool weighte
     L.solo = true;
     L.params = take(sizeof(PopParams));
     L.state = take(sizeof(DevState));
+    L.ring = take((size_t)cap * sizeof(spg_stats));
     L.acc = take(sizeof(StatAcc) * kAccCopies);
     L.geno0 = L.geno1 = take((size_t)n * 2 * words * 4);
     for (size_t &x : L.packed) x = take((size_t)n * 2 * words * 4);
@@ -388,7 +389,6 @@ PopLayout solo_layout_for(uint32_t n, uint32_t words, uint32_t cap, bool weighte
     for (size_t &x : L.counts) x = take((size_t)slot_count(n) * 4);
     L.gen_acc = take(sizeof(GenAcc) * 3 * kGenAccCopies);
     L.barrier = take(sizeof(unsigned long long));
-    L.ring = take((size_t)cap * sizeof(spg_stats));
     L.frag = take(sizeof(ValueFragments));
     L.link = take(sizeof(LinkParams));
     L.weighted = weighted;
@@ -945,12 +945,15 @@ int view_sync(const PopView &v) {
     return e == cudaSuccess ? SPG_OK : cuda_fail(e, "cudaStreamSynchronize");
 }
 
-int view_state(const PopView &v, DevState &st) {
-    int rc = view_sync(v);
-    if (rc != SPG_OK) return rc;
-    const cudaError_t e = cudaMemcpy(&st, v.base + v.L.state, sizeof st, cudaMemcpyDeviceToHost);
-    return e == cudaSuccess ? SPG_OK : cuda_fail(e, "read state");
+// One copy in stream order: it waits for what the stream has to do, so no
+// synchronisation goes before it.
+static int read_back(const PopView &v, void *host, size_t off, size_t bytes, const char *what) {
+    cudaError_t e = cudaMemcpyAsync(host, v.base + off, bytes, cudaMemcpyDeviceToHost, v.stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(v.stream);
+    return e == cudaSuccess ? SPG_OK : cuda_fail(e, what);
 }
+
+int view_state(const PopView &v, DevState &st) { return read_back(v, &st, v.L.state, sizeof st, "read state"); }
 
 int view_set_state(const PopView &v, uint32_t gen, uint32_t S, uint32_t f, double R, int32_t status,
                    uint32_t target) {
@@ -1048,10 +1051,24 @@ int view_set_ecology(const PopView &v, PopParams &prm, const spg_ecology *eco) {
     return view_sync(v);
 }
 
+// Bytes of state and ring that one copy brings at the price of a copy of the
+// state alone.
+constexpr size_t kReadTogether = 48u << 10;
+
 int view_read_stats(const PopView &v, uint32_t first_gen, uint32_t count, spg_stats *out) {
     if (!out && count) return fail(SPG_ERR_INVALID, "NULL argument");
+    // the state and, when the ring is short, the ring behind it in one copy
     DevState st;
-    int rc = view_state(v, st);
+    std::vector<char> both;
+    const size_t ring_at = v.L.ring - v.L.state, all = ring_at + (size_t)v.cap * sizeof(spg_stats);
+    int rc;
+    if (all <= kReadTogether) {
+        both.resize(all);
+        rc = read_back(v, both.data(), v.L.state, all, "read state and stats");
+        std::memcpy(&st, both.data(), sizeof st);
+    } else {
+        rc = view_state(v, st);
+    }
     if (rc != SPG_OK) return rc;
     if (count == 0) return SPG_OK;
     const uint64_t last = (uint64_t)first_gen + count - 1;
@@ -1062,8 +1079,12 @@ int view_read_stats(const PopView &v, uint32_t first_gen, uint32_t count, spg_st
     for (uint32_t i = 0; i < count;) {
         const uint32_t slot = (first_gen - 1 + i) % v.cap;
         const uint32_t run = std::min(count - i, v.cap - slot);
-        const cudaError_t e = cudaMemcpy(out + i, ring + slot, run * sizeof(spg_stats), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_fail(e, "read stats");
+        if (!both.empty()) {
+            std::memcpy(out + i, both.data() + ring_at + slot * sizeof(spg_stats), run * sizeof(spg_stats));
+        } else {
+            const cudaError_t e = cudaMemcpy(out + i, ring + slot, run * sizeof(spg_stats), cudaMemcpyDeviceToHost);
+            if (e != cudaSuccess) return cuda_fail(e, "read stats");
+        }
         i += run;
     }
     return st.status < 0 ? fail(st.status, "device status %d", st.status) : SPG_OK;
