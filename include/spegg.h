@@ -246,7 +246,7 @@ int spg_read_stats(spg_pop *pop, uint32_t first_gen, uint32_t count, spg_stats *
  * frequency of locus l is count[l] / 2N).  With enable != 0, every generation
  * formed from now on also counts, over both haplotypes of its N offspring,
  * the allele-1 copies of each locus, kept in a ring of stats_capacity rows of
- * L uint32 (one more kernel after each compaction; enable = 0 stops it).  The
+ * L uint32 (counted while they are formed; enable = 0 stops it).  The
  * first call allocates that ring through the population's allocator; the
  * call waits for the stream.  Biallelic populations only (SPG_ERR_INVALID
  * for continuous values).  Counts are not part of a checkpoint: after
@@ -283,7 +283,8 @@ int spg_restore(spg_pop *pop, const void *host, size_t bytes);
  * and lanes per offspring (1, or 2 for L >= 128: one lane per parent, each
  * loading that parent's record and forming the gamete it passes on; 0 = the
  * default, 2 for L = 256 and 1 otherwise).  A launch-shape choice only: every
- * shape gives identical results.  Populations with a linkage map or parent
+ * shape gives identical results, and the biallelic kernel, which has one
+ * shape of its own, the same speed.  Populations with a linkage map or parent
  * weights, and continuous allelic values, run 256 threads with one offspring
  * per thread.  spg_get_launch_shape reports the shape in use.
  * SPG_ERR_INVALID for an unsupported shape.  Waits for the stream. */
@@ -305,12 +306,15 @@ int spg_get_tiling(spg_pop *pop, uint32_t *items_per_thread);
  * Many independent populations advanced by shared launches: the flattened
  * loop over replicates of the paper's Fig. S5 B.  Members are grouped by
  * locus count and variant (plain; linkage map; parent weights; both;
- * continuous values); each generation is one offspring launch and one
- * compaction launch per group, groups run as independent branches of one
- * cached CUDA graph.  Members with a linkage map, parent weights or
- * continuous values run the variant shape (256 threads, one offspring per
- * thread, one lane); launch shapes and the autotuner apply to the plain
- * members of each locus count.  Every member keeps its own parameters,
+ * continuous values).  The biallelic members of a kind (plain; linkage map;
+ * parent weights; both) share cooperative launches of several generations,
+ * each member formed by a team of blocks; a group of continuous-value members
+ * takes one offspring and one compaction launch per generation, the groups
+ * as branches of one cached CUDA graph.  Members with a linkage map, parent
+ * weights or continuous values have the shape of 256 threads, one offspring
+ * per thread, one lane; other launch shapes are accepted, and reported, for
+ * the plain members of each locus count (the biallelic kernel has one shape
+ * of its own).  Every member keeps its own parameters,
  * state, buffers and statistics ring, and its results are identical to the same population
  * created with spg_create_population and stepped alone.  Member i is
  * descs[i]; the descriptions are copied.  Errors as for a population;
@@ -334,7 +338,8 @@ int spg_batch_get_tiling(spg_batch *batch, uint32_t n_loci, uint32_t *items_per_
  * times gens_per_trial real generations with each of
  * SPG_AUTOTUNE_CANDIDATES launch shapes -- threads per block (128, 256, 512)
  * x offspring per thread (1, 2) for L <= 64, x lanes per offspring (1, 2) for
- * L >= 128 -- and keeps the fastest.  Every
+ * L >= 128 -- and keeps the fastest (the biallelic kernel has one shape of
+ * its own, so the candidates differ by noise).  Every
  * member advances by the same number of generations (report->gens_run =
  * SPG_AUTOTUNE_CANDIDATES * (gens_per_trial + 1)); results do not depend on
  * the shapes chosen.  The report (may be NULL) gives each group's chosen
@@ -351,8 +356,7 @@ typedef struct {
 int spg_batch_autotune(spg_batch *batch, uint32_t gens_per_trial, spg_autotune_report *report);
 int spg_batch_read_stats(spg_batch *batch, uint32_t member, uint32_t first_gen, uint32_t count, spg_stats *out);
 /* Per-locus allele counts of every biallelic member (as
- * spg_set_locus_counts / spg_read_locus_counts for each member; a group of
- * several members counts them all in one more launch after its compaction;
+ * spg_set_locus_counts / spg_read_locus_counts for each member;
  * continuous-allele members are not counted and their reads are
  * SPG_ERR_INVALID).  The first enabling call allocates every member's ring
  * through the batch's allocator; both calls wait for the stream. */

@@ -18,7 +18,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OUT_DIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUT_DIR, "libspegg_gb300.so")
-SOURCES = ["kernels.cu", "offspring_w1.cu", "offspring_w2.cu", "offspring_w4.cu", "offspring_w8.cu", "generations_w1.cu",
+SOURCES = ["kernels.cu", "offspring.cu", "generations_w1.cu",
            "generations_w2.cu", "generations_w4.cu", "generations_w8.cu", "teams_plain.cu", "teams_general.cu", "teams_linked.cu",
            "teams_weighted.cu", "teams_both.cu", "engine.cu",
            "population.cu", "batch.cu", "server.cu", "space.cu", "noalloc.cu"]

@@ -1,14 +1,14 @@
 // Batched replicates (spg_batch): many independent populations advanced by
 // shared launches -- the flattened replicate loop of the paper's Fig. S5 B.
 //
-// Members are grouped by locus count and variant (the offspring kernel is
-// specialised on W, linkage map and parent weights, and continuous values
-// have a kernel of their own; members with a linkage map, parent weights or
-// continuous values run at the variant shape, the others' shape is tuned per
-// locus count).  A group's members are the segments of one launch: every
-// generation is one offspring launch and one compaction launch per group,
-// the groups' chains are independent branches of one CUDA graph (so groups
-// overlap on the GPU), and the graph of kGraphChunk generations is replayed.
+// The biallelic members are formed by teams of blocks (TeamSet: one
+// cooperative launch per kind -- plain, general values, linkage map, parent
+// weights, both -- and call).  Continuous members are grouped by locus count: a
+// group's members are the segments of one launch, every generation is one
+// offspring launch and one compaction launch per group, the groups' chains are
+// independent branches of one CUDA graph (so groups overlap on the GPU), and
+// the graph of kGraphChunk generations is replayed.  Groups by locus count and
+// variant also hold the launch shape that callers set and read.
 // Each member keeps its own parameters, state, buffers and statistics ring,
 // and its Philox counters carry its own replicate id, so a member's results
 // are identical to the same population stepped alone.
@@ -232,7 +232,7 @@ int spg_batch_create(const spg_pop_desc *descs, uint32_t count, const spg_alloca
         m.v.words = words;
         m.v.cap = m.prm->stats_cap;
         m.v.nbuckets = bucket_count(d.n);
-        m.v.L = continuous ? layout_for(d.n, words, m.v.nbuckets, m.v.cap, false, false)
+        m.v.L = continuous ? layout_for(d.n, words, m.v.nbuckets, m.v.cap)
                              : solo_layout_for(d.n, words, m.v.cap, weighted);
         m.group = group_index(d.n_loci, linked, weighted, continuous);
         b->groups[m.group].members.push_back(i);

@@ -1,10 +1,10 @@
 // Host engine and C ABI of libspegg_gb300 (see include/spegg.h).
 //
-// A population owns one device arena holding its parameters, two genotype
-// buffers and two survivor lists (ping-pong by generation parity, chosen on
-// the device so every generation launch has identical arguments), its
-// look-back status words, its state and its statistics ring.  Generations are
-// enqueued as a cached CUDA graph of kGraphChunk back-to-back launches.
+// A population owns one device arena.  Biallelic populations are formed by the
+// generation kernel (generations.cuh): alone, one cooperative launch per call,
+// or as members of a batch or server by teams of blocks (TeamSet).  Continuous
+// allelic values take two launches per generation, enqueued as a cached CUDA
+// graph of kGraphChunk generations.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -87,11 +87,11 @@ void effect_planes(const int16_t *effects, uint32_t n_loci, PopParams &prm) {
     offset_planes(effects, n_loci, prm.planes, prm.e_min, prm.nplanes);
 }
 
-// Byte tables of per-locus values v (effects, or dominance deviations): table
+// Byte tables of per-locus values v: table
 // k, entry b is the sum of v[8k + i] over the bits i set in b -- the value of
 // the eight loci 8k .. 8k+7 held in byte k of a haplotype (locus l is bit l % 32
 // of word l / 32).  Exact in int32 (at most 8 * 32768 in magnitude).
-static void byte_tables(const int16_t *v, uint32_t n_loci, int32_t *lut) {
+void byte_tables(const int16_t *v, uint32_t n_loci, int32_t *lut) {
     std::memset(lut, 0, sizeof(int32_t) * kMaxLutBytes * kLutWords);
     for (uint32_t k = 0; k < n_loci / 8; ++k)
         for (uint32_t b = 0; b < (uint32_t)kLutWords; ++b) {
@@ -213,13 +213,11 @@ int build_params(const spg_pop_desc *d, PopParams &prm) {
     std::memcpy(prm.table, d->surv_table, sizeof prm.table);
     effect_planes(d->effects, d->n_loci, prm);
     if (prm.nplanes > (uint32_t)kMaxPlanes) return fail(SPG_ERR_INVALID, "effects span more than 16 bits");
-    byte_tables(d->effects, d->n_loci, prm.lut);
     if (d->dominance) {
         offset_planes(d->dominance, d->n_loci, prm.dplanes, prm.d_min, prm.ndplanes);
         if (prm.ndplanes > (uint32_t)kMaxPlanes)
             return fail(SPG_ERR_INVALID, "dominance deviations span more than 16 bits");
         for (uint32_t l = 0; l < d->n_loci; ++l) prm.has_dom |= d->dominance[l] != 0 ? 1u : 0u;
-        byte_tables(d->dominance, d->n_loci, prm.dlut);
     }
     prm.kmax = mutation_cdf(d->mu, 2 * d->n_loci, prm.cdf);
     prm.bias = d->bin_bias;
@@ -257,7 +255,6 @@ int build_link(const double *map, uint32_t n_loci, LinkParams &lp) {
         const double m = map[l];
         if (!(m == m) || std::isinf(m)) return fail(SPG_ERR_INVALID, "map_morgans[%u] is not finite", l);
         if (m < 0.0) {
-            lp.clast[chrom] = (uint16_t)(l - 1);
             if (++chrom >= (uint32_t)kMaxChrom)
                 return fail(SPG_ERR_INVALID, "a linkage map holds at most %d chromosomes", kMaxChrom);
             lp.first[chrom] = (uint16_t)l;
@@ -267,11 +264,8 @@ int build_link(const double *map, uint32_t n_loci, LinkParams &lp) {
         }
         D = D + w[l];
     }
-    lp.clast[chrom] = (uint16_t)(n_loci - 1);
     lp.nchrom = chrom + 1;
     if (!(D <= kMaxMapMorgans)) return fail(SPG_ERR_INVALID, "the linkage map is longer than 16 Morgans");
-    for (uint32_t c = 0; c < lp.nchrom; ++c)
-        for (uint32_t l = lp.first[c]; l <= lp.clast[c]; ++l) lp.chrom[l] = (uint8_t)c;
     lp.kmax = mutation_cdf(D / (double)kLinkSites, kLinkSites, lp.cdf);
     double run = 0.0;
     for (uint32_t l = 0; l < n_loci; ++l) {
@@ -283,9 +277,9 @@ int build_link(const double *map, uint32_t n_loci, LinkParams &lp) {
             lp.cum[l] = 0;
         }
     }
-    // guide[h]: the interval of the bucket's first uniform, the chromosomes of
-    // it and of the next interval, and the interval boundaries inside the
-    // bucket (none for most buckets: the guide entry is the answer)
+    // guide[h]: the interval of the bucket's first uniform and the interval
+    // boundaries inside the bucket (none for most buckets: the guide entry is
+    // the answer)
     constexpr uint32_t shift = 32u - (uint32_t)kLinkGuideBits;
     auto interval = [&](uint32_t u) {
         uint32_t I = 0;
@@ -295,8 +289,7 @@ int build_link(const double *map, uint32_t n_loci, LinkParams &lp) {
     for (uint32_t h = 0; h < (uint32_t)kLinkGuide; ++h) {
         const uint32_t lo = h << shift, hi = lo | ((1u << shift) - 1u);
         const uint32_t I0 = interval(lo), nb = std::min<uint32_t>(interval(hi) - I0, 2u);
-        const uint32_t c0 = lp.chrom[I0], c1 = nb != 0u ? lp.chrom[I0 + 1u] : 0u;
-        lp.guide[h] = I0 | (c0 << 8) | (c1 << 15) | (nb << 26);
+        lp.guide[h] = I0 | (nb << 26);
     }
     return SPG_OK;
 }
@@ -325,7 +318,8 @@ int build_weights(const uint32_t *mother_w, const uint32_t *father_w, WeightPara
 // ------------------------------------------------------------ population
 uint32_t bucket_count(uint32_t n) { return (n + kBucket - 1) / kBucket; }
 
-PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap, bool weighted, bool dense) {
+// The arena of a population of continuous allelic values.
+PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap) {
     PopLayout L{};
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -339,19 +333,11 @@ PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap
     L.acc = take(sizeof(StatAcc) * kAccCopies);
     L.geno0 = take((size_t)n * 2 * words * 4);
     L.geno1 = take((size_t)n * 2 * words * 4);
-    L.dense = dense ? take((size_t)n * 2 * words * 4) : 0;
     L.surv0 = take((size_t)n * 4);
     L.surv1 = take((size_t)n * 4);
     L.alive = take((size_t)nbuckets * kBucketWords * 4);
     L.buckets = take((size_t)2 * nbuckets * 4);
     L.segment = take(sizeof(Segment));
-    L.link = take(sizeof(LinkParams));
-    L.weighted = weighted;
-    if (weighted) {
-        L.weights = take(sizeof(WeightParams));
-        L.obin = take((size_t)n * 2);
-        L.survw = take((size_t)n * 16);
-    }
     L.total = off;
     return L;
 }
@@ -624,16 +610,11 @@ Segment segment_at(char *base, const PopLayout &L, uint32_t n, uint32_t ntiles, 
     s.prm = reinterpret_cast<const PopParams *>(base + L.params);
     s.geno[0] = reinterpret_cast<uint32_t *>(base + L.geno0);
     s.geno[1] = reinterpret_cast<uint32_t *>(base + L.geno1);
-    s.dense = L.dense ? reinterpret_cast<uint32_t *>(base + L.dense) : nullptr;
     s.surv[0] = reinterpret_cast<uint32_t *>(base + L.surv0);
     s.surv[1] = reinterpret_cast<uint32_t *>(base + L.surv1);
     s.alive = reinterpret_cast<uint32_t *>(base + L.alive);
     s.bucket_sum = reinterpret_cast<uint32_t *>(base + L.buckets);
     s.state = reinterpret_cast<DevState *>(base + L.state);
-    if (L.weighted) {
-        s.obin = reinterpret_cast<uint16_t *>(base + L.obin);
-        s.survw = reinterpret_cast<unsigned long long *>(base + L.survw);
-    }
     s.ring = reinterpret_cast<spg_stats *>(base + L.ring);
     s.tile_begin = tile_begin;
     s.ntiles = ntiles;
@@ -712,33 +693,25 @@ struct KernelLaunch {
     bool programmatic;
 };
 KernelLaunch offspring_launch(const GenLaunch &gl) {
-    return {reinterpret_cast<void *>(gl.offspring.fn), dim3(gl.blocks), dim3(gl.offspring.block), gl.offspring.smem,
-            gl.offspring.persistent};
+    return {reinterpret_cast<void *>(gl.offspring.fn), dim3(gl.blocks), dim3(kBlock), gl.offspring.smem,
+            gl.offspring.programmatic};
 }
 KernelLaunch compact_launch(const GenLaunch &gl) {
-    return {reinterpret_cast<void *>(gl.compact), dim3(gl.buckets), dim3(kCompactThreads), compact_smem(), true};
-}
-// after the compaction has finished (it reads the committed state)
-KernelLaunch locus_launch(const GenLaunch &gl) {
-    return {reinterpret_cast<void *>(gl.locus), dim3(gl.la.blocks), dim3(kLocusBlock), 0u, false};
+    return {reinterpret_cast<void *>(gl.compact), dim3(gl.buckets), dim3(kCompactThreads), 0u, true};
 }
 }  // namespace
 
 int add_generation_nodes(cudaGraph_t graph, const GenLaunch &gl, void **params, uint32_t len) {
     cudaGraphNode_t prev = nullptr;
-    LocusArgs la = gl.la;
-    void *locus_params[] = {params[0], &la};  // argument values are copied into the nodes
-    const uint32_t per_gen = gl.locus ? 3u : 2u;
-    for (uint32_t i = 0; i < per_gen * len; ++i) {
-        const uint32_t step = i % per_gen;
-        const KernelLaunch k = step == 0 ? offspring_launch(gl) : step == 1 ? compact_launch(gl) : locus_launch(gl);
+    for (uint32_t i = 0; i < 2u * len; ++i) {
+        const KernelLaunch k = i % 2u == 0 ? offspring_launch(gl) : compact_launch(gl);
         cudaGraphNodeParams np{};
         np.type = cudaGraphNodeTypeKernel;
         np.kernel.func = k.fn;
         np.kernel.gridDim = k.grid;
         np.kernel.blockDim = k.block;
         np.kernel.sharedMemBytes = k.smem;
-        np.kernel.kernelParams = step == 2 ? locus_params : params;
+        np.kernel.kernelParams = params;  // argument values are copied into the nodes
         cudaGraphEdgeData edge{};
         if (k.programmatic) {
             edge.from_port = cudaGraphKernelNodePortProgrammatic;
@@ -780,11 +753,9 @@ int launch_generation(const GenLaunch &gl, cudaStream_t stream) {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
-    LocusArgs la = gl.la;
-    void *locus_params[] = {&a, &la};
     cudaError_t e = cudaSuccess;
-    for (uint32_t step = 0; step < (gl.locus ? 3u : 2u); ++step) {
-        const KernelLaunch k = step == 0 ? offspring_launch(gl) : step == 1 ? compact_launch(gl) : locus_launch(gl);
+    for (uint32_t step = 0; step < 2u; ++step) {
+        const KernelLaunch k = step == 0 ? offspring_launch(gl) : compact_launch(gl);
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = k.grid;
         cfg.blockDim = k.block;
@@ -792,7 +763,7 @@ int launch_generation(const GenLaunch &gl, cudaStream_t stream) {
         cfg.stream = stream;
         cfg.attrs = &attr;
         cfg.numAttrs = k.programmatic ? 1u : 0u;
-        e = cudaLaunchKernelExC(&cfg, k.fn, step == 2 ? locus_params : params);
+        e = cudaLaunchKernelExC(&cfg, k.fn, params);
         if (e != cudaSuccess) break;
     }
     return e == cudaSuccess ? SPG_OK : cuda_fail(e, "generation launch");
@@ -826,11 +797,6 @@ size_t group_table_bytes(uint32_t members, uint64_t offspring, uint32_t buckets)
     return align_up((size_t)members * sizeof(Segment), 256) + align_up((size_t)runs * sizeof(Run), 256) +
            align_up((size_t)(kMaxGridBlocks + 1) * 4, 256) + align_up((size_t)buckets * 4, 256) +
            align_up((size_t)(offspring / kBlock + members + 1) * 4, 256);  // tile map (continuous groups)
-}
-
-uint32_t tiles_for(uint32_t n, const Shape &shape) {
-    const uint32_t t = tile_size(shape);
-    return (n + t - 1) / t;
 }
 
 // Runs of a launch group (see GenArgs): the members' tiles, in member order,
@@ -923,7 +889,7 @@ int build_group_launch(const std::vector<const PopView *> &members, uint32_t wor
     if (e != cudaSuccess) return cuda_fail(e, "upload launch table");
     gl = GenLaunch{};
     gl.offspring = k;
-    gl.compact = compact_kernel(words);
+    gl.compact = compact_kernel();
     gl.args.segs = reinterpret_cast<const Segment *>(table);
     gl.args.bucket_seg = reinterpret_cast<const uint32_t *>(table + off_buckets);
     gl.args.tile_seg = reinterpret_cast<const uint32_t *>(table + off_tiles);
@@ -999,18 +965,9 @@ int view_init(const PopView &v, const PopParams &prm, const uint32_t *init_genot
         rc = launch_founders(v.words, geno0, surv0, v.n, prm.key0, prm.key1, prm.rep, p0_q32, v.stream);
     }
     if (rc != SPG_OK) return fail(rc, "founder launch failed");
-    if (v.L.dense) {  // every founder survives: the dense parents are the founders in index order
-        rc = launch_dense_gather(v.words, geno0, nullptr, v.n, reinterpret_cast<uint32_t *>(v.base + v.L.dense),
-                                 v.stream);
-        if (rc != SPG_OK) return fail(rc, "dense-parent launch failed");
-    }
     if (v.L.solo) {
         rc = view_pack(v, 0, nullptr, v.n);
         if (rc != SPG_OK) return fail(rc, "founder packing failed");
-    } else if (v.L.weighted) {  // every founder is a potential parent, in index order
-        rc = launch_survivor_bins(reinterpret_cast<const PopParams *>(v.base + v.L.params), v.words, geno0, nullptr,
-                                  v.n, v.n, reinterpret_cast<unsigned long long *>(v.base + v.L.survw), v.stream);
-        if (rc != SPG_OK) return fail(rc, "survivor-bin launch failed");
     }
     rc = view_set_state(v, 0, v.n, kCertain, 0.0, SPG_OK, 0xFFFFFFFFu);
     return rc == SPG_OK ? SPG_OK : fail(rc, "state launch failed");
@@ -1088,11 +1045,6 @@ int view_read_stats(const PopView &v, uint32_t first_gen, uint32_t count, spg_st
         i += run;
     }
     return st.status < 0 ? fail(st.status, "device status %d", st.status) : SPG_OK;
-}
-
-uint32_t locus_blocks(uint32_t n) {
-    const uint32_t groups = (n + 31u) / 32u, per_block = kLocusGroupsPerWarp * (kLocusBlock / 32u);
-    return std::max(1u, std::min(kLocusMaxGrid, (groups + per_block - 1u) / per_block));
 }
 
 // Rows of per-locus counts of generations first_gen .. first_gen+count-1

@@ -1,16 +1,17 @@
 // Device kernels of the per-generation update (sm_103a) other than the
-// offspring kernel (offspring.cuh): the continuous-allele generation kernel,
-// the compaction kernel that closes every generation, and the set-up kernels
-// (founders, survivor words of weighted parents, state resets).
+// biallelic generation kernel (generations.cuh) and the allocation-free
+// call's (offspring.cu): the continuous-allele generation kernel, the
+// compaction kernel that closes a generation for both of the two-launch
+// forms, and the set-up kernels (founders, the slot layout of biallelic
+// populations, state resets).
 //
-// A generation of every population in a launch group is two launches
-// (Fig. 1 A-F of the paper):
-//   k_offspring  (offspring.cuh) draws both parents of every offspring from
-//                the previous survivors (A), forms the gametes by crossover
-//                masks and mutation XOR (B), sums the genetic value (C) and
-//                decides survival from the threshold table (D); it writes the
-//                child records, the alive bitmap, per-bucket survivor counts
-//                and exact integer statistics;
+// A generation of continuous-allele populations, or of the allocation-free
+// call, is two launches (Fig. 1 A-F of the paper):
+//   offspring    draws both parents of every offspring from the previous
+//                survivors (A), forms the gametes (B), sums the genetic value
+//                (C) and decides survival from the threshold table (D); it
+//                writes the child records, the alive bitmap, per-bucket
+//                survivor counts and exact integer statistics;
 //   k_compact    one block per bucket of kBucket offspring: turns the bitmap
 //                into the ordered survivor list (E) with a two-level scan
 //                (earlier buckets' counts + a block scan), and the block that
@@ -186,7 +187,7 @@ __device__ __forceinline__ void add_step(uint4 &c, uint32_t k, int32_t step) {
 // bits, mutation counts and positions follow the biallelic model's draws;
 // mutated values take Irwin-Hall steps; the phenotype is the group sum of the
 // values plus the environmental step.  Survivors, statistics and the bitmap
-// feed the same compaction kernel as the biallelic model.
+// feed the compaction kernel.
 constexpr int kContInFlight = 1;  // offspring a group of lanes forms at a time (four blocks per SM)
 
 template <int G, int U, bool GROUP>
@@ -448,59 +449,23 @@ __global__ void k_founders_cont(const PopParams *__restrict__ P, uint32_t *__res
 // read the bucket's bitmap words and the survivor counts of all earlier
 // buckets and scan the words' popcounts; then kCompactCopyThreads threads
 // (8 warps) write every survivor's index, in offspring order, at its rank =
-// (survivors of earlier buckets) + (survivors before it in the bucket), and,
-// for populations with a dense parent buffer, its record at the same rank
-// (the parents of the next generation, read by rank without an index hop).
-// The bucket's child records reach shared memory by bulk asynchronous copies
-// of kChunkBytes each into a ring of kRingSlots slots (issued by one thread
-// before the scan, the next chunk into a slot as soon as the copy threads are
-// done with it), so the record copy is a stream of large reads instead of a
-// dependent load per survivor; the survivors are stored from shared memory
-// with whole-sector stores.  In a population's first bucket an extra warp
-// closes the generation meanwhile (finalize_warp).  The block that finishes
-// the last bucket commits the new state.  Every load that does not depend on
-// the population state is issued together with it (both parities of the
-// bucket counts are summed; the state picks one).
-// 32 KB of ring per block: rings of 64 KB and more measured up to 40%
-// slower, alone and next to other launch groups' offspring kernels
-constexpr uint32_t kChunkBytes = 16384;  // bytes of one bulk copy of child records (one ring slot)
-constexpr uint32_t kRingSlots = 2;       // chunks in flight per block
-
+// (survivors of earlier buckets) + (survivors before it in the bucket).  In a
+// population's first bucket an extra warp closes the generation meanwhile
+// (finalize_warp).  The block that finishes the last bucket commits the new
+// state.  Every load that does not depend on the population state is issued
+// together with it (both parities of the bucket counts are summed; the state
+// picks one).
 __device__ __forceinline__ void compaction_barrier() {
     asm volatile("bar.sync 1, %0;" ::"n"(kCompactCopyThreads) : "memory");  // the compaction threads
 }
 
-// A record of 2W words from shared memory (16-byte chunks, 8-byte for W = 1).
-template <int W>
-__device__ __forceinline__ void ring_record(uint32_t addr, uint32_t (&r)[2 * W]) {
-    if constexpr (W == 1) {
-        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
-    } else {
-#pragma unroll
-        for (int q = 0; q < W / 2; ++q)
-            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(r[4 * q]), "=r"(r[4 * q + 1]), "=r"(r[4 * q + 2]), "=r"(r[4 * q + 3])
-                         : "r"(addr + 16u * q)
-                         : "memory");
-    }
-}
-
-template <int W>
 __device__ __forceinline__ void compact_bucket(const Segment &sg, uint32_t b) {
-    constexpr int NW = kBucketWords / 32;          // warps that scan the bitmap words
-    constexpr uint32_t REC = 8u * W;               // bytes per record
-    constexpr uint32_t CHUNK = kChunkBytes / REC;  // offspring per ring slot
-    constexpr uint32_t SLOT = kChunkBytes;         // bytes per ring slot
-    constexpr uint32_t NCHUNK = kBucket / CHUNK;   // ring fills per bucket
-    constexpr int CW = (int)(CHUNK / 32);          // bitmap words per chunk
-    constexpr int WPW = CW / (int)(kCompactCopyThreads / 32);  // bitmap words per copying warp and chunk
-    static_assert(kBucket % CHUNK == 0 && WPW >= 1, "chunks split the bucket among the copying warps");
-    extern __shared__ __align__(128) unsigned char s_ring[];  // [kRingSlots][SLOT]
-    __shared__ alignas(8) unsigned long long s_bar[kRingSlots];
+    constexpr int NW = kBucketWords / 32;  // warps that scan the bitmap words
+    constexpr int WPW = (int)(kBucketWords / (kCompactCopyThreads / 32));  // bitmap words per writing warp
     __shared__ uint32_t s_warp[NW];
     __shared__ uint32_t s_prev[NW];
     __shared__ uint32_t s_bits[kBucketWords], s_incl[kBucketWords];
-    __shared__ uint32_t s_last, s_timeout;
+    __shared__ uint32_t s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool closer = tid >= (int)kCompactCopyThreads;  // the generation-closing warp
     const bool scanner = tid < (int)kBucketWords;
@@ -513,30 +478,9 @@ __device__ __forceinline__ void compact_bucket(const Segment &sg, uint32_t b) {
         prev1 += __ldcg(sg.bucket_sum + sg.nbuckets + i);
     }
     const PopNow now = read_state(sg.state);
-    const uint32_t g = now.gen + 1u;
-    const uint32_t first = b * kBucket, nb = min(kBucket, sg.n - first);  // the bucket's offspring
-    const uint32_t nchunks = (nb + CHUNK - 1u) / CHUNK;
-    const bool ring = sg.dense != nullptr && now.active;
-    const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(s_ring);
-    const uint32_t bar0 = (uint32_t)__cvta_generic_to_shared(&s_bar[0]);
-    const uint32_t *__restrict__ chi = sg.geno[g & 1u];
-    // chunk c of the bucket into ring slot c % kRingSlots (a partial last
-    // chunk rounded up to 16 bytes: record buffers are padded to 256 bytes)
-    auto fill = [&](uint32_t c) {
-        const uint32_t off = first + c * CHUNK, cnt = min(CHUNK, nb - c * CHUNK);
-        bulk_load(ring0 + (c % kRingSlots) * SLOT, chi + (size_t)off * (2 * W), (cnt * REC + 15u) & ~15u,
-                  bar0 + 8u * (c % kRingSlots));
-    };
-    if (tid == 0) {
-        s_timeout = 0u;
-        if (ring) {
-            for (uint32_t k = 0; k < kRingSlots; ++k) mbar_init(bar0 + 8u * k, 1u);
-            mbar_init_fence();
-            for (uint32_t c = 0; c < kRingSlots && c < nchunks; ++c) fill(c);
-        }
-    }
-    __syncthreads();  // barriers initialised
     if (!now.active) return;
+    const uint32_t g = now.gen + 1u;
+    const uint32_t first = b * kBucket;
     if (closer) {
         if (b == 0u) finalize_warp(sg, sg.prm, g, now.f);
         __threadfence();
@@ -559,57 +503,21 @@ __device__ __forceinline__ void compact_bucket(const Segment &sg, uint32_t b) {
 #pragma unroll
         for (int q = 0; q < NW; ++q) before += s_prev[q];
         uint32_t *__restrict__ sout = sg.surv[g & 1u];
-        uint32_t *__restrict__ dense = sg.dense;
         const uint32_t lt = (1u << lane) - 1u;
-        for (uint32_t c = 0; c < NCHUNK; ++c) {
-            if (c >= nchunks) break;
-            if (ring && !mbar_wait(bar0 + 8u * (c % kRingSlots), (c / kRingSlots) & 1u)) s_timeout = 1u;
-            const uint32_t slot = ring0 + (c % kRingSlots) * SLOT;
 #pragma unroll
-            for (int k = 0; k < WPW; ++k) {
-                const int q = (int)c * CW + warp * WPW + k;  // bitmap word of the bucket
-                const uint32_t word = s_bits[q];
-                uint32_t r0 = before + s_incl[q] - __popc(word);
+        for (int k = 0; k < WPW; ++k) {
+            const int q = warp * WPW + k;  // bitmap word of the bucket
+            const uint32_t word = s_bits[q];
+            uint32_t r0 = before + s_incl[q] - __popc(word);
 #pragma unroll
-                for (int v = 0; v < NW; ++v) r0 += v < q / 32 ? s_warp[v] : 0u;
-                if ((word >> lane) & 1u) {
-                    const uint32_t rank = r0 + __popc(word & lt), idx = first + (uint32_t)q * 32u + lane;
-                    sout[rank] = idx;
-                    if (ring) {
-                        uint32_t rec[2 * W];
-                        ring_record<W>(slot + ((uint32_t)(q - (int)c * CW) * 32u + lane) * REC, rec);
-                        store_record<W>(dense + (size_t)rank * (2 * W), rec);
-                    }
-                    if (sg.survw) {  // the survivor's acceptance thresholds as mother and as father
-                        const uint32_t bin = __ldcg(sg.obin + idx);
-                        const WeightParams *wt = sg.prm->weights;
-                        sg.survw[rank] = (unsigned long long)idx | ((unsigned long long)__ldg(&wt->acc[0][bin]) << 32);
-                        sg.survw[sg.n + rank] =
-                            (unsigned long long)idx | ((unsigned long long)__ldg(&wt->acc[1][bin]) << 32);
-                    }
-                }
-            }
-            if (ring && c + kRingSlots < nchunks) {  // the slot is free once every copying thread is past it
-                compaction_barrier();
-                if (tid == 0 && !s_timeout) fill(c + kRingSlots);
-            }
+            for (int v = 0; v < NW; ++v) r0 += v < q / 32 ? s_warp[v] : 0u;
+            if ((word >> lane) & 1u) sout[r0 + __popc(word & lt)] = first + (uint32_t)q * 32u + lane;
         }
     }
     // every block has read the state by now (its values fed the stores
     // above), and the closing warp of bucket 0 has published the next state
     __syncthreads();
-    if (tid == 0) {
-        if (s_timeout) {  // a copy did not land in time: the generation fails; wait (bounded) for
-                          // the last copy issued into each slot before the block's memory goes away
-            atomicExch(reinterpret_cast<int *>(&sg.state->status), SPG_ERR_TIMEOUT);
-            for (uint32_t k = 0; k < kRingSlots && k < nchunks; ++k) {
-                uint32_t lastc = k;
-                while (lastc + kRingSlots < nchunks) lastc += kRingSlots;
-                mbar_wait(bar0 + 8u * k, (lastc / kRingSlots) & 1u);
-            }
-        }
-        s_last = (atomicAdd(&sg.state->done, 1u) == sg.nbuckets - 1u) ? 1u : 0u;
-    }
+    if (tid == 0) s_last = (atomicAdd(&sg.state->done, 1u) == sg.nbuckets - 1u) ? 1u : 0u;
     __syncthreads();
     if (s_last && tid == 0) {
         __threadfence();
@@ -617,53 +525,16 @@ __device__ __forceinline__ void compact_bucket(const Segment &sg, uint32_t b) {
     }
 }
 
-template <int W>
 __global__ void __launch_bounds__(kCompactThreads, 3) k_compact(const __grid_constant__ GenArgs a) {
     griddep_release();  // the next generation's blocks may take this grid's place as its blocks finish
     griddep_wait();     // everything below reads the offspring kernel's results
     const uint32_t bkt = blockIdx.x;
     if (a.nsegs == 1u) {
-        compact_bucket<W>(a.one, bkt);
+        compact_bucket(a.one, bkt);
     } else {
         const Segment &sg = a.segs[__ldg(a.bucket_seg + bkt)];
-        compact_bucket<W>(sg, bkt - sg.bucket_begin);
+        compact_bucket(sg, bkt - sg.bucket_begin);
     }
-}
-
-// A record of 2W words read through L2 and written with whole-sector stores.
-template <int W>
-__device__ __forceinline__ void copy_record(const uint32_t *__restrict__ src, uint32_t *__restrict__ dst) {
-    uint32_t r[2 * W];
-    if constexpr (W == 1) {
-        const uint2 v = __ldcg(reinterpret_cast<const uint2 *>(src));
-        r[0] = v.x;
-        r[1] = v.y;
-    } else if constexpr (W == 2) {
-        const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(src));
-        r[0] = v.x;
-        r[1] = v.y;
-        r[2] = v.z;
-        r[3] = v.w;
-    } else {
-#pragma unroll
-        for (int q = 0; q < W / 4; ++q)
-            asm volatile("ld.global.cg.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                         : "=r"(r[8 * q]), "=r"(r[8 * q + 1]), "=r"(r[8 * q + 2]), "=r"(r[8 * q + 3]),
-                           "=r"(r[8 * q + 4]), "=r"(r[8 * q + 5]), "=r"(r[8 * q + 6]), "=r"(r[8 * q + 7])
-                         : "l"(src + 8 * q));
-    }
-    store_record<W>(dst, r);
-}
-
-// dense[r] = geno[surv[r]] (surv null: r) for r < S: the dense parent buffer
-// of founders or of a restored generation.
-template <int W>
-__global__ void k_dense_gather(const uint32_t *__restrict__ geno, const uint32_t *__restrict__ surv, uint32_t S,
-                               uint32_t *__restrict__ dense) {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= S) return;
-    const uint32_t idx = surv ? surv[r] : r;
-    copy_record<W>(geno + (size_t)idx * (2 * W), dense + (size_t)r * (2 * W));
 }
 
 // ---------------------------------------------------------- founders
@@ -721,23 +592,6 @@ __device__ __forceinline__ uint32_t record_bin(const PopParams *__restrict__ P, 
     }
     const long long v = (long long)raw + (long long)P->bias;
     return v < 0 ? 0u : (uint32_t)min(v >> P->shift, (long long)(kBins - 1));
-}
-
-// survw[pi * n + r] = surv[r] | (role pi's threshold for the survivor's bin)
-// << 32 for the current survivors, each bin from its record's genetic value
-// (planes read from the parameters).
-template <int W>
-__global__ void k_survivor_bins(const PopParams *__restrict__ P, const uint32_t *__restrict__ geno,
-                                const uint32_t *__restrict__ surv, uint32_t S, uint32_t n,
-                                unsigned long long *__restrict__ survw) {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= S) return;
-    const uint32_t idx = surv ? surv[r] : r;
-    uint32_t rec[2 * W];
-    load_record<W>(geno + (size_t)idx * (2 * W), rec);
-    const uint32_t bin = record_bin<W>(P, rec);
-    survw[r] = (unsigned long long)idx | ((unsigned long long)P->weights->acc[0][bin] << 32);
-    survw[(size_t)n + r] = (unsigned long long)idx | ((unsigned long long)P->weights->acc[1][bin] << 32);
 }
 
 // The last bitmap word of a population whose size is not a multiple of 32.
@@ -799,11 +653,6 @@ __global__ void k_set_state(DevState *st, StatAcc *acc, uint32_t gen, uint32_t S
 
 }  // namespace
 
-OffspringKernel offspring_kernel_w1(const Shape &shape, bool linked, bool weighted, bool staged);
-OffspringKernel offspring_kernel_w2(const Shape &shape, bool linked, bool weighted, bool staged);
-OffspringKernel offspring_kernel_w4(const Shape &shape, bool linked, bool weighted, bool staged);
-OffspringKernel offspring_kernel_w8(const Shape &shape, bool linked, bool weighted, bool staged);
-
 bool supported_shape(uint32_t words, const Shape &s) {
     if (!(s.block == 128 || s.block == 256 || s.block == 512)) return false;
     if (s.lanes == 2) return words >= 4 && s.items == 1;
@@ -811,208 +660,7 @@ bool supported_shape(uint32_t words, const Shape &s) {
     return words <= 2 ? (s.items == 1 || s.items == 2) : s.items == 1;
 }
 
-uint32_t tile_size(const Shape &s) { return s.block * s.items / s.lanes; }
-
-uint32_t compact_smem() { return kRingSlots * kChunkBytes; }
-
-GenKernel compact_kernel(uint32_t words) {
-    GenKernel k;
-    switch (words) {
-        case 2: k = &k_compact<2>; break;
-        case 4: k = &k_compact<4>; break;
-        case 8: k = &k_compact<8>; break;
-        default: k = &k_compact<1>; break;  // and populations without a dense buffer (no record copies)
-    }
-    // the ring of bulk-copied child records is dynamic shared memory
-    cudaFuncSetAttribute(reinterpret_cast<const void *>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)compact_smem());
-    return k;
-}
-
-// ------------------------------------------------- per-locus allele counts
-// 32 x 32 bit transpose across a warp: afterwards bit b of lane i is what bit
-// i of lane b was.  Stage s swaps the off-diagonal s x s blocks between lanes
-// i and i ^ s (masks keep the low s bits of each 2s-bit group).
-__device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, uint32_t lane) {
-    constexpr uint32_t M[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        const uint32_t s = 16u >> k;
-        const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, (int)s);
-        x = (lane & s) ? (((y >> s) & M[k]) | (x & ~M[k])) : ((x & M[k]) | ((y << s) & ~M[k]));
-    }
-    return x;
-}
-
-// Allele-1 copies of every locus over both haplotypes of the generation just
-// formed (all N offspring; S2 "Genetics": count / 2N is the locus's allele
-// frequency).  A warp takes 32 records at a time, one per lane; each lane
-// adds its record's words into bit-sliced counters (plane k holds bit k of
-// every locus's count among the lane's records), and every kLocusPlanes
-// records' worth of room (and at the end) the warp transposes each plane
-// across its lanes, so that lane b holds bit b of the 32 lanes' planes, and
-// adds 2^k times its population count to locus 32w + b; the warps of a block add theirs in
-// shared memory, blocks add theirs into the accumulator row, and the block
-// that finishes last moves the row to the generation's ring slot, clears it
-// and re-arms the counter.  A generation already counted (a launch after the
-// population has stopped forms none) is left as it is.
-template <int W, bool GROUP>
-__global__ void __launch_bounds__(kLocusBlock) k_locus_counts(const __grid_constant__ GenArgs a, const LocusArgs la_) {
-    constexpr uint32_t L = 32u * W, NW = kLocusBlock / 32u;
-    __shared__ uint32_t s_cnt[L];
-    __shared__ uint32_t s_last;
-    // the block's population, its arguments and the block's place among its
-    // blocks (GROUP: a launch group, from the block map)
-    const Segment *sgp = &a.one;
-    const LocusArgs *lap = &la_;
-    uint32_t blk = blockIdx.x, nblk = gridDim.x;
-    if constexpr (GROUP) {
-        const uint32_t m = __ldg(la_.block_member + blockIdx.x);
-        sgp = a.segs + m;
-        lap = la_.member + m;
-        blk = blockIdx.x - lap->first;
-        nblk = lap->blocks;
-    }
-    const Segment &sg = *sgp;
-    const LocusArgs &la = *lap;
-    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    const uint32_t g = ld_relaxed_u32(&sg.state->gen);  // the generation the compaction just committed
-    if (g == 0u || ld_relaxed_u32(la.last) == g) return;  // the founders, or counted already
-    for (uint32_t i = tid; i < L; i += kLocusBlock) s_cnt[i] = 0u;
-    __syncthreads();
-    const uint32_t *rec = sg.geno[g & 1u];
-    constexpr int K = kLocusPlanes;
-    uint32_t acc[W], v[2 * W][K];
-#pragma unroll
-    for (int w = 0; w < W; ++w) acc[w] = 0u;
-#pragma unroll
-    for (int c = 0; c < 2 * W; ++c)
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[c][k] = 0u;
-    auto flush = [&]() {  // the whole warp: every lane's planes into the counts
-#pragma unroll
-        for (int c = 0; c < 2 * W; ++c)
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                acc[c % W] += (uint32_t)__popc(warp_transpose32(v[c][k], lane)) << k;
-                v[c][k] = 0u;
-            }
-    };
-    const uint32_t groups = (sg.n + 31u) >> 5, stride = nblk * NW;
-    constexpr uint32_t U = kLocusBatch;  // groups whose records are loaded before any is added
-    uint32_t held = 0;  // records each lane has added since the last flush (the same in the whole warp)
-    for (uint32_t q0 = blk * NW + warp; q0 < groups; q0 += U * stride) {
-        uint32_t r[U][2 * W];
-#pragma unroll
-        for (uint32_t u = 0; u < U; ++u) {
-            const uint32_t q = q0 + u * stride, i = q * 32u + lane;
-            if (q < groups && i < sg.n) {
-                load_record<W>(rec + (size_t)i * (2 * W), r[u]);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 2 * W; ++c) r[u][c] = 0u;
-            }
-        }
-        if (held + U > (1u << K) - 1u) {  // the counters hold up to 2^K - 1
-            flush();
-            held = 0;
-        }
-#pragma unroll
-        for (uint32_t u = 0; u < U; ++u)
-#pragma unroll
-            for (int c = 0; c < 2 * W; ++c) {  // ripple-carry add of one bit per locus
-                uint32_t x = r[u][c];
-#pragma unroll
-                for (int k = 0; k < K - 1; ++k) {
-                    const uint32_t carry = v[c][k] & x;
-                    v[c][k] ^= x;
-                    x = carry;
-                }
-                v[c][K - 1] ^= x;
-            }
-        held += U;
-    }
-    if (held) flush();
-#pragma unroll
-    for (int w = 0; w < W; ++w) atomicAdd(&s_cnt[32u * w + lane], acc[w]);
-    __syncthreads();
-    for (uint32_t i = tid; i < L; i += kLocusBlock)
-        if (s_cnt[i]) atomicAdd(la.acc + i, s_cnt[i]);
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) s_last = atomicAdd(la.done, 1u) == nblk - 1u ? 1u : 0u;
-    __syncthreads();
-    if (s_last) {  // every block has added its counts
-        __threadfence();
-        uint32_t *slot = la.ring + (size_t)((g - 1u) % la.cap) * L;
-        for (uint32_t i = tid; i < L; i += kLocusBlock) {
-            slot[i] = __ldcg(la.acc + i);
-            la.acc[i] = 0u;
-        }
-        if (tid == 0) {
-            *la.done = 0u;
-            *la.last = g;
-        }
-    }
-}
-
-template <int W>
-LocusKernel locus_instance(bool group) {
-    return group ? &k_locus_counts<W, true> : &k_locus_counts<W, false>;
-}
-
-LocusKernel locus_kernel(uint32_t words, bool group) {
-    switch (words) {
-        case 1: return locus_instance<1>(group);
-        case 2: return locus_instance<2>(group);
-        case 4: return locus_instance<4>(group);
-        case 8: return locus_instance<8>(group);
-        default: return nullptr;
-    }
-}
-
-int launch_dense_gather(uint32_t words, const uint32_t *geno, const uint32_t *surv, uint32_t S, uint32_t *dense,
-                        void *stream) {
-    if (S == 0) return SPG_OK;
-    const dim3 grid((S + 255) / 256), block(256);
-    cudaStream_t s = (cudaStream_t)stream;
-    switch (words) {
-        case 1: k_dense_gather<1><<<grid, block, 0, s>>>(geno, surv, S, dense); break;
-        case 2: k_dense_gather<2><<<grid, block, 0, s>>>(geno, surv, S, dense); break;
-        case 4: k_dense_gather<4><<<grid, block, 0, s>>>(geno, surv, S, dense); break;
-        case 8: k_dense_gather<8><<<grid, block, 0, s>>>(geno, surv, S, dense); break;
-        default: return SPG_ERR_INVALID;
-    }
-    return cudaGetLastError() == cudaSuccess ? SPG_OK : SPG_ERR_CUDA;
-}
-
-OffspringKernel offspring_kernel(uint32_t words, const Shape &shape, bool linked, bool weighted, bool eco, bool dom,
-                                 bool staged) {
-    staged = staged && kStagedParents && words <= 4 && shape.lanes == 1 && !linked;
-    OffspringKernel k;
-    switch (words) {
-        case 1: k = offspring_kernel_w1(shape, linked, weighted, staged); break;
-        case 2: k = offspring_kernel_w2(shape, linked, weighted, staged); break;
-        case 4: k = offspring_kernel_w4(shape, linked, weighted, staged); break;
-        case 8: k = offspring_kernel_w8(shape, linked, weighted, staged); break;
-        default: return OffspringKernel{};
-    }
-    if (!k.fn) return k;
-    // dynamic shared memory: byte tables, thresholds (and attack rates when
-    // some population of the launch has an ecology), dominance byte tables
-    // (only when some population has dominance)
-    const uint32_t lut = words * 4u * (uint32_t)kLutWords * 4u;
-    const uint32_t tab = eco ? (uint32_t)kBins * 8u : (uint32_t)kBins * 4u;
-    k.words = words;
-    k.eco_table = eco ? 1u : 0u;
-    k.smem_dlut = dom ? lut + tab : 0u;
-    k.smem = lut + tab + (dom ? lut : 0u);
-    if (staged) {  // the ring of staged parent records
-        k.smem_parents = k.smem;
-        k.smem += kParentStages * 2u * k.block * k.items * 8u * words;
-    }
-    return k;
-}
+GenKernel compact_kernel() { return &k_compact; }
 
 template <int G>
 GenKernel cont_instance(bool group) {
@@ -1028,11 +676,7 @@ OffspringKernel continuous_kernel(uint32_t n_loci, bool group) {
         case 256: k.fn = cont_instance<32>(group); break;
         default: return OffspringKernel{};
     }
-    k.block = kBlock;
-    k.items = 1;
-    k.smem = 0;
-    k.resident = 0;
-    k.persistent = false;  // one block per 256 offspring
+    k.tile = kBlock;
     return k;
 }
 
@@ -1043,21 +687,13 @@ int prepare_offspring(OffspringKernel &k) {
     cudaGetDevice(&dev);
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return SPG_ERR_CUDA;
-    if (k.persistent) {
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
-        if (e != cudaSuccess) return SPG_ERR_CUDA;
-    }
+    if (k.smem) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+    if (e != cudaSuccess) return SPG_ERR_CUDA;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, (int)k.block, k.smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, k.smem);
     if (e != cudaSuccess || per_sm <= 0) return SPG_ERR_CUDA;
     k.resident = (uint32_t)per_sm * (uint32_t)sms;
     return SPG_OK;
-}
-
-void apply_kernel(const OffspringKernel &k, GenArgs &a) {
-    a.eco_table = k.eco_table;
-    a.smem_dlut = k.smem_dlut;
-    a.smem_parents = k.smem_parents;
 }
 
 int launch_founders_cont(const PopParams *prm, uint32_t n_loci, uint32_t *geno, uint32_t *surv, uint32_t n,
@@ -1090,21 +726,6 @@ int launch_founders(uint32_t words, uint32_t *geno, uint32_t *surv, uint32_t n, 
 
 int launch_iota(uint32_t *surv, uint32_t n, void *stream) {
     k_iota<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(surv, n);
-    return cudaGetLastError() == cudaSuccess ? SPG_OK : SPG_ERR_CUDA;
-}
-
-int launch_survivor_bins(const PopParams *prm, uint32_t words, const uint32_t *geno, const uint32_t *surv,
-                         uint32_t S, uint32_t n, unsigned long long *survw, void *stream) {
-    if (S == 0) return SPG_OK;
-    const dim3 grid((S + 255) / 256), block(256);
-    cudaStream_t s = (cudaStream_t)stream;
-    switch (words) {
-        case 1: k_survivor_bins<1><<<grid, block, 0, s>>>(prm, geno, surv, S, n, survw); break;
-        case 2: k_survivor_bins<2><<<grid, block, 0, s>>>(prm, geno, surv, S, n, survw); break;
-        case 4: k_survivor_bins<4><<<grid, block, 0, s>>>(prm, geno, surv, S, n, survw); break;
-        case 8: k_survivor_bins<8><<<grid, block, 0, s>>>(prm, geno, surv, S, n, survw); break;
-        default: return SPG_ERR_INVALID;
-    }
     return cudaGetLastError() == cudaSuccess ? SPG_OK : SPG_ERR_CUDA;
 }
 

@@ -30,10 +30,10 @@ constexpr size_t kOffAlive = kOffAcc + align256(sizeof(StatAcc) * kAccCopies);
 constexpr size_t kOffBuckets = kOffAlive + align256((size_t)kMaxBuckets * kBucketWords * 4);
 constexpr size_t kScratchBytes = kOffBuckets + align256((size_t)2 * kMaxBuckets * 4);
 static_assert(SPG_NOALLOC_MAX_N % kBucket == 0, "the maximum population must be a whole number of buckets");
-static_assert(kScratchBytes == SPG_NOALLOC_SCRATCH_BYTES, "spegg.h states the scratch size");
+static_assert(kScratchBytes <= SPG_NOALLOC_SCRATCH_BYTES, "spegg.h states the scratch size");
 
 // Shared by every call on a device; it keeps the previous call's contents.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[SPG_NOALLOC_SCRATCH_BYTES];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_scratch_mutex;
@@ -82,7 +82,6 @@ extern "C" int spg_generation_noalloc(const spg_noalloc_generation *a, void *str
     if (rc != SPG_OK) return rc;
 
     const uint32_t W = a->n_loci / 32, g = a->generation;
-    const Shape shape = default_shape(W);
     spg_pop_desc d{};
     d.n = a->n;
     d.n_loci = a->n_loci;
@@ -98,13 +97,14 @@ extern "C" int spg_generation_noalloc(const spg_noalloc_generation *a, void *str
     static thread_local PopParams prm;
     rc = build_params(&d, prm);
     if (rc != SPG_OK) return rc;
+    byte_tables(d.effects, d.n_loci, prm.lut);
     prm.stats_cap = 1;  // the caller's single statistics record
     prm.has_eco = 0;
 
-    OffspringKernel k = offspring_kernel(W, shape, false, false, false, false, false);
+    OffspringKernel k = offspring_kernel(W);
     rc = prepare_offspring(k);
     if (rc != SPG_OK) return fail(rc, "offspring kernel setup failed");
-    const uint32_t ntiles = tiles_for(a->n, shape), nbuckets = bucket_count(a->n);
+    const uint32_t ntiles = (a->n + k.tile - 1) / k.tile, nbuckets = bucket_count(a->n);
 
     Segment seg{};
     seg.prm = reinterpret_cast<const PopParams *>(scratch + kOffParams);
@@ -137,13 +137,12 @@ extern "C" int spg_generation_noalloc(const spg_noalloc_generation *a, void *str
 
     GenLaunch gl;
     gl.offspring = k;
-    gl.compact = compact_kernel(W);  // no dense buffer: parents by survivor index, no record copies
+    gl.compact = compact_kernel();
     gl.args.segs = nullptr;  // one segment: the kernels read it from their parameters
     gl.args.nsegs = 1;
     gl.args.one = seg;
     gl.args.total_tiles = ntiles;
     gl.args.total_buckets = nbuckets;
-    apply_kernel(k, gl.args);
     gl.blocks = std::min(ntiles, k.resident);
     gl.buckets = nbuckets;
     return launch_generation(gl, s);

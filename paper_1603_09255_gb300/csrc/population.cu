@@ -1,11 +1,13 @@
 // C ABI of one population (spg_pop): create, ecology, stepping, reads,
 // checkpoint/restore, tiling (see include/spegg.h).
 //
-// A population owns one device arena (parameters, state, accumulators, two
-// genotype buffers, two survivor lists, bitmap, bucket counts, statistics
-// ring).  Generations are enqueued as a cached CUDA graph of kGraphChunk
-// generations (two launches each); every launch has identical arguments
-// because buffers are chosen on the device by generation parity.
+// A population owns one device arena (parameters, state, statistics ring,
+// accumulators, genotypes, survivors).  The generations of a biallelic
+// population are formed by one cooperative launch per call (of at most
+// kSoloLaunchGens); those of continuous allelic values are enqueued as a
+// cached CUDA graph of kGraphChunk generations (two launches each), whose
+// arguments are identical because buffers are chosen on the device by
+// generation parity.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -129,7 +131,7 @@ int configure_launch(spg_pop *p, const Shape &shape) {
     if (rc != SPG_OK) return rc;
     p->gl = GenLaunch{};
     p->gl.offspring = k;
-    p->gl.compact = compact_kernel(p->words);
+    p->gl.compact = compact_kernel();
     p->gl.args.segs = reinterpret_cast<const Segment *>(p->arena + p->L.segment);
     p->gl.args.one = seg;
     p->gl.args.nsegs = 1;
@@ -198,7 +200,7 @@ int spg_create_population(const spg_pop_desc *desc, const spg_allocator *alloc, 
         }
         p->own_stream = true;
     }
-    p->L = p->host_prm->continuous ? layout_for(p->n, p->words, p->nbuckets, p->cap, false, false)
+    p->L = p->host_prm->continuous ? layout_for(p->n, p->words, p->nbuckets, p->cap)
                                    : solo_layout_for(p->n, p->words, p->cap, p->host_prm->weighted != 0u);
     p->arena = static_cast<char *>(p->alloc.alloc(p->L.total, p->stream));
     if (!p->arena) {

@@ -8,8 +8,9 @@
 //      the job's device footprint fits the memory budget,
 //   3. rebuilds the launch tables when the resident set changed, and
 //   4. advances every resident job by up to gens_per_tick generations in
-//      shared launches (one offspring + one compaction launch per locus-count
-//      group and generation; groups on their own streams, so they overlap).
+//      shared launches (biallelic jobs by teams of blocks; one offspring + one
+//      compaction launch per generation and locus count of the continuous
+//      ones, on their own streams, so they overlap).
 // A job stops at its own generation count on the device (the state's target),
 // so jobs of any length share launches; its Philox counters carry its own
 // replicate id, so its results are identical alone and in any mix.
@@ -65,7 +66,7 @@ uint32_t group_of(uint32_t n_loci) { return n_loci == 32 ? 0u : n_loci == 64 ? 1
 bool continuous_job(const spg_pop_desc &d) { return d.allele_model == 1u; }
 uint32_t job_words(const spg_pop_desc &d) { return continuous_job(d) ? d.n_loci / 2 : d.n_loci / 32; }
 PopLayout job_layout(const spg_pop_desc &d, uint32_t cap, bool weighted) {
-    return continuous_job(d) ? layout_for(d.n, job_words(d), bucket_count(d.n), cap, false, false)
+    return continuous_job(d) ? layout_for(d.n, job_words(d), bucket_count(d.n), cap)
                              : solo_layout_for(d.n, job_words(d), cap, weighted);
 }
 

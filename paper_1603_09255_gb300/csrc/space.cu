@@ -541,8 +541,8 @@ __global__ void __launch_bounds__(kSpClassBlock) k_sp_classify(SpaceArgs a) {
 }
 
 // Newborn records (A-C), one thread per newborn over all demes: parents
-// among the deme's m adults, free recombination, mutation, written with
-// their age and phenotype straight to their places in the new layout (after
+// among the deme's m adults, free recombination, mutation, appended to the
+// pool, with their age and phenotype at their places in the new layout (after
 // k_sp_totals and the second scan); heterozygosity and allele counts per
 // species.
 template <int W>

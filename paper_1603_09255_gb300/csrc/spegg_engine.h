@@ -35,11 +35,11 @@ struct Allocator {
 
 // Byte offsets of one population's buffers inside its arena.
 struct PopLayout {
-    size_t params, state, acc, geno0, geno1, dense, surv0, surv1, alive, buckets, ring, segment, link;
-    size_t weights, obin, survw;  // weighted parents only (0 otherwise)
+    size_t params, state, acc, geno0, geno1, surv0, surv1, alive, buckets, ring, segment, link;
+    size_t weights;  // weighted parents only (0 otherwise)
     bool weighted;
     // a single biallelic population (solo_layout_for): geno0 = geno1 and
-    // surv0 = surv1, no dense buffer, buckets, bins or segment
+    // surv0 = surv1, no buckets or segment
     bool solo;
     size_t packed[2], counts[2], mate[2], gen_acc, barrier, frag;
     size_t total;
@@ -60,12 +60,9 @@ struct GenLaunch {
     GenArgs args{};
     uint32_t blocks = 0;   // offspring grid: min(tiles, resident blocks)
     uint32_t buckets = 0;  // compaction grid
-    LocusKernel locus = nullptr;  // per-locus allele counts after the compaction (single populations; null: off)
-    LocusArgs la{};
 };
 
-// A cached CUDA graph of `length` generations (2 dependent launches each, 3
-// with per-locus counts).
+// A cached CUDA graph of `length` generations (2 dependent launches each).
 struct GraphChain {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -107,6 +104,7 @@ int fail(int code, const char *fmt, ...);
 int cuda_fail(cudaError_t e, const char *what);
 uint32_t mutation_cdf(double mu, uint32_t n_copies, uint32_t *cdf);
 void effect_planes(const int16_t *effects, uint32_t n_loci, PopParams &prm);
+void byte_tables(const int16_t *v, uint32_t n_loci, int32_t *lut);
 uint32_t factor_q32_host(double R, double R_half);
 size_t align_up(size_t x, size_t a);
 // Value fragments of the effects and dominance deviations (null: none);
@@ -119,10 +117,7 @@ int build_params(const spg_pop_desc *d, PopParams &prm);
 int build_link(const double *map_morgans, uint32_t n_loci, LinkParams &lp);
 // Acceptance thresholds from the mother and father weight tables (NULL: uniform).
 int build_weights(const uint32_t *mother_w, const uint32_t *father_w, WeightParams &wp);
-// dense: the population has a dense parent buffer (biallelic records; not
-// the continuous-allele model, whose generation kernel reads parents by index).
-PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap, bool weighted = false,
-                     bool dense = true);
+PopLayout layout_for(uint32_t n, uint32_t words, uint32_t nbuckets, uint32_t cap);
 Segment segment_at(char *base, const PopLayout &L, uint32_t n, uint32_t ntiles, uint32_t tile_begin,
                    uint32_t nbuckets, uint32_t bucket_begin);
 uint32_t bucket_count(uint32_t n);
@@ -143,10 +138,6 @@ int add_generation_nodes(cudaGraph_t graph, const GenLaunch &gl, void **params, 
 size_t group_table_bytes(uint32_t members, uint64_t offspring, uint32_t buckets);
 int read_locus_rows(const LocusArgs &la, uint32_t n_loci, uint32_t from, uint32_t until, const DevState &st,
                     uint32_t first_gen, uint32_t count, uint32_t *out);
-// Blocks of the per-locus count kernel for a population of n (16 groups of
-// 32 records per warp at least, at most kLocusMaxGrid).
-uint32_t locus_blocks(uint32_t n);
-uint32_t tiles_for(uint32_t n, const Shape &shape);
 void schedule_runs(const std::vector<uint32_t> &tiles, uint32_t G, uint32_t min_piece, std::vector<Run> &runs,
                    std::vector<uint32_t> &block_runs);
 // Segment table, tile and bucket maps of one group of continuous-allele
