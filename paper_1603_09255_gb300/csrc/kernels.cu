@@ -162,12 +162,38 @@ __device__ __forceinline__ void set_word(uint4 &c, uint32_t q, uint32_t v) {
 }
 // the values of b where bit k (k = 0..7, value k of the eight) of `bits` is set, of a elsewhere
 __device__ __forceinline__ uint4 pick8(const uint4 &a, const uint4 &b, uint32_t bits) {
-    auto sel = [](uint32_t x, uint32_t y, uint32_t two) {
-        const uint32_t m = ((two & 1u) ? 0x0000FFFFu : 0u) | ((two & 2u) ? 0xFFFF0000u : 0u);
-        return (x & ~m) | (y & m);
+    auto sel = [](uint32_t x, uint32_t y, uint32_t two) {  // a byte permutation of (x, y): selectors 0-3 or 4-7
+        return __byte_perm(x, y, (((two & 3u) * 0x2244u) & 0x4444u) | 0x3210u);
     };
     return make_uint4(sel(a.x, b.x, bits), sel(a.y, b.y, bits >> 2), sel(a.z, b.z, bits >> 4),
                       sel(a.w, b.w, bits >> 6));
+}
+// Sums over eight values v = 256 h + l (h signed, l unsigned): of v, and for
+// their squares 65536 h^2 + 512 hl + l^2 of h^2, hl and l^2, by byte dot
+// products.
+__device__ __forceinline__ int32_t sum8(const uint4 &c, int32_t acc) {
+    const int one = 0x0101;
+    acc = __dp2a_lo((int)c.x, one, acc);
+    acc = __dp2a_lo((int)c.y, one, acc);
+    acc = __dp2a_lo((int)c.z, one, acc);
+    return __dp2a_lo((int)c.w, one, acc);
+}
+__device__ __forceinline__ void squares8(const uint4 &c, int32_t &hh, int32_t &hl, uint32_t &ll) {
+    const uint32_t h0 = __byte_perm(c.x, c.y, 0x7531), l0 = __byte_perm(c.x, c.y, 0x6420);
+    const uint32_t h1 = __byte_perm(c.z, c.w, 0x7531), l1 = __byte_perm(c.z, c.w, 0x6420);
+    hh = __dp4a((int)h1, (int)h1, __dp4a((int)h0, (int)h0, hh));
+    ll = __dp4a(l1, l1, __dp4a(l0, l0, ll));
+    asm("dp4a.s32.u32 %0, %1, %2, %0;" : "+r"(hl) : "r"(h0), "r"(l0));
+    asm("dp4a.s32.u32 %0, %1, %2, %0;" : "+r"(hl) : "r"(h1), "r"(l1));
+}
+// How many of the eight values of a and b differ.
+__device__ __forceinline__ uint32_t differ8(const uint4 &a, const uint4 &b) {
+    auto top = [](uint32_t x) { return ((x & 0x7FFF7FFFu) + 0x7FFF7FFFu) | x; };  // a half's top bit: half != 0
+    uint32_t d = top(a.x ^ b.x) & 0x80008000u;
+    d |= (top(a.y ^ b.y) & 0x80008000u) >> 1;
+    d |= (top(a.z ^ b.z) & 0x80008000u) >> 2;
+    d |= (top(a.w ^ b.w) & 0x80008000u) >> 3;
+    return (uint32_t)__popc(d);
 }
 // value k of the eight moved by `step`, clamped to the int16 range
 __device__ __forceinline__ void add_step(uint4 &c, uint32_t k, int32_t step) {
@@ -182,24 +208,44 @@ __device__ __forceinline__ void add_step(uint4 &c, uint32_t k, int32_t step) {
 // move in coalesced 16-byte accesses; a warp holds 32/G groups, each forming
 // U offspring at a time with all their parent loads issued before any is
 // used.  The per-offspring draws (parents, survival and mutation uniforms,
-// environmental step, gamete-mask streams) are made once per warp, one
-// offspring per lane, and handed to the groups by shuffles.  Parents, gamete
-// bits, mutation counts and positions follow the biallelic model's draws;
-// mutated values take Irwin-Hall steps; the phenotype is the group sum of the
-// values plus the environmental step.  Survivors, statistics and the bitmap
+// environmental step, gamete-mask streams, mutations) are made once per warp,
+// one offspring or mutation per lane, and read by the groups from shared
+// memory.  Parents, gamete bits, mutation counts and positions follow the
+// biallelic model's draws; mutated values take Irwin-Hall steps; the phenotype
+// is the group sum of the values plus the environmental step.  Survivors, statistics and the bitmap
 // feed the compaction kernel.
+//
+// Bound by DRAM at L >= 128 (1,548 bytes an offspring at L = 128: 234 us at N =
+// 10^6, 6.6 TB/s) and by instructions below.  L = 32 / 64 / 128 at N = 10^6 and
+// L = 256 at 5 x 10^5, us per generation (mu = 10^-3): 107 / 176 / 327 / 349
+// with every mutation drawn by its group, the draws handed over by shuffles
+// and no prefetch; 93 / 145 / 255 / 254 with the list and shared memory; 92 /
+// 143 / 234 / 236 with the prefetch and the byte dot products.
 constexpr int kContInFlight = 1;  // offspring a group of lanes forms at a time (four blocks per SM)
+constexpr uint32_t kContMutations = 128;  // mutations of a warp's 32 offspring listed before the offspring are formed
+// Steps of the warp a parent's record is prefetched into L2 ahead of its use.
+// N = 10^6 (L = 256: 5 x 10^5), us per generation with 0 / 1 / 2 / 3 steps: L =
+// 128 254 / 234 / 236 / 245, L = 256 255 / 236 / 244 / 260 (further ahead, the
+// records leave L2 again before they are used); with 0 / 2 / 4: L = 64 145 /
+// 149 / 152, L = 32 93 / 106 / 106 (their steps take more records of less
+// memory each, and are bound by instructions).
+template <int G>
+constexpr uint32_t kContAhead = G >= 16 ? 1u : 0u;
 
 template <int G, int U, bool GROUP>
 __global__ void __launch_bounds__(kBlock, 4) k_offspring_cont(const __grid_constant__ GenArgs a) {
     constexpr uint32_t L = 8u * G;
     constexpr int NW = kBlock / 32, NO = 32 / G;
     constexpr int NST = G >= 8 ? G / 8 : 1;  // gamete-mask streams per offspring (2 words per parent each)
-    constexpr int PER_T = NO * NST;          // (offspring, stream) pairs one step of the warp uses
-    constexpr int T_PER_SLOT = 32 / PER_T;   // steps served by one register slot of those pairs
+    constexpr uint32_t AHEAD = kContAhead<G>;
     static_assert(G >= 4 && G <= 32 && (G & (G - 1)) == 0 && G % U == 0, "group of 4..32 lanes");
     __shared__ uint32_t s_cdf[kMaxKmax];
     __shared__ uint32_t s_mpos[NW * NO][kMaxKmax];
+    __shared__ uint4 s_draw[NW][32];        // the warp's offspring: mother, father, survival draw, mutations
+    __shared__ int32_t s_envs[NW][32];
+    __shared__ uint4 s_mask[NW][32 * NST];  // their gamete-mask streams
+    __shared__ uint16_t s_lpos[NW][kContMutations];
+    __shared__ int32_t s_lstep[NW][kContMutations];
     __shared__ long long s_ll[2][NW];
     __shared__ unsigned long long s_ull[4][NW];
     __shared__ uint32_t s_u32[2][NW];
@@ -244,32 +290,82 @@ __global__ void __launch_bounds__(kBlock, 4) k_offspring_cont(const __grid_const
     const uint4 rl = philox(make_uint4(jl, g, rep, kMate << 24), k0, k1);
     const uint32_t mom_l = jl < n ? __ldcg(sin + __umulhi(rl.x, S)) : 0u;
     const uint32_t dad_l = jl < n ? __ldcg(sin + __umulhi(rl.y, S)) : 0u;
-    const int32_t env_l = s_env != 0 ? irwin_hall_step(jl, g, rep, kEnv, 0u, s_env, k0, k1) : 0;
-    // (B) gamete-mask streams: slot q of lane k holds pair 32q + k, i.e. step
-    // (32q + k) / PER_T, group ((32q + k) % PER_T) / NST, stream (32q + k) % NST
-    uint4 dml[NST];
+    auto prefetch = [&](uint32_t rec) {
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(par + (size_t)rec * R4), "n"(16u * R4)
+                     : "memory");
+    };
+    if ((uint32_t)lane < AHEAD * NO && jl < n) {
+        prefetch(mom_l);
+        prefetch(dad_l);
+    }
+    s_envs[warp][lane] = s_env != 0 ? irwin_hall_step(jl, g, rep, kEnv, 0u, s_env, k0, k1) : 0;
+    // (B) gamete-mask streams: entry NST * o + q holds stream q of offspring o
 #pragma unroll
     for (int q = 0; q < NST; ++q) {
-        const uint32_t pr = 32u * (uint32_t)q + (uint32_t)lane, t = pr / PER_T, rem = pr % PER_T;
-        dml[q] = philox(make_uint4(wbase + t * NO + rem / NST, g, rep, (kRecomb << 24) | (rem % NST)), k0, k1);
+        const uint32_t e = 32u * (uint32_t)q + (uint32_t)lane;
+        s_mask[warp][e] = philox(make_uint4(wbase + e / NST, g, rep, (kRecomb << 24) | (e % NST)), k0, k1);
     }
 
+    // (B) mutations: each lane counts its offspring's and draws their distinct
+    // positions, then the warp's lanes draw the Irwin-Hall steps, one
+    // mutation each.  (Drawn where they are applied, a mutation in one
+    // offspring made the whole warp draw four Philox blocks.)  A warp with more
+    // than kContMutations draws them there after all.
+    uint32_t K_l = 0;
+    if (jl < n && kmax != 0u && rl.w >= s_cdf[0])
+        for (uint32_t qk = 0; qk < kmax; ++qk) K_l += rl.w >= s_cdf[qk] ? 1u : 0u;
+    uint32_t off_l = K_l;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, off_l, o);
+        if (lane >= o) off_l += y;
+    }
+    const uint32_t nmut = __shfl_sync(0xFFFFFFFFu, off_l, 31);
+    off_l -= K_l;  // the offspring's first entry in the warp's list
+    const bool listed = nmut <= kContMutations;
+    if (listed && nmut != 0u) {
+        uint16_t *lpos = s_lpos[warp] + off_l;
+        uint32_t chosen = 0;
+        uint4 dp = make_uint4(0u, 0u, 0u, 0u);
+        for (uint32_t d = 0; d < (uint32_t)kMutDraws && chosen < K_l; ++d) {
+            if ((d & 3u) == 0u) dp = philox(make_uint4(jl, g, rep, (kMutPos << 24) | (d >> 2)), k0, k1);
+            const uint32_t pos = __umulhi(lane_of(dp, (int)(d & 3u)), 2u * L);
+            bool dup = false;
+            for (uint32_t qk = 0; qk < chosen; ++qk) dup |= lpos[qk] == pos;
+            if (!dup) lpos[chosen++] = (uint16_t)pos;
+        }
+        for (uint32_t e0 = 0; e0 < nmut; e0 += 32u) {
+            const uint32_t e = e0 + (uint32_t)lane;
+            uint32_t o = 0;  // the owner: the last lane whose first entry is <= e
+#pragma unroll
+            for (uint32_t step = 16u; step > 0u; step >>= 1)
+                if (__shfl_sync(0xFFFFFFFFu, off_l, (int)(o + step)) <= e) o += step;
+            const uint32_t ooff = __shfl_sync(0xFFFFFFFFu, off_l, (int)o);
+            if (e < nmut)
+                s_lstep[warp][e] = irwin_hall_step(wbase + o, g, rep, kMutSize, 3u * (e - ooff), s_mut, k0, k1);
+        }
+        K_l = chosen;
+    }
+    s_draw[warp][lane] = make_uint4(mom_l, dad_l, rl.z, K_l | (off_l << 16));
+    __syncwarp();
+
     long long sum_raw = 0, sum_raw_s = 0;
-    unsigned long long sum_raw2 = 0, cons = 0, lane_allele = 0;
+    unsigned long long sum_raw2 = 0, cons = 0;
     uint32_t lane_het = 0, alive_bits = 0, nsurv = 0;
+    uint32_t sq_ll = 0;  // squares of at most 16 * 32 values a lane: each part below 2^25
+    int32_t sq_hh = 0, sq_hl = 0;
     int mn = INT_MAX, mx = INT_MIN;
     for (uint32_t it = 0; it < (uint32_t)(G / U); ++it) {
-        uint32_t bit[U], rz[U], rw[U];
-        int32_t env[U];
+        uint32_t bit[U], rz[U], mut[U];
         uint4 m0[U], m1[U], f0[U], f1[U];
         // the group's U offspring: parents and draws from their lanes, then all the records
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             bit[u] = (it * U + (uint32_t)u) * NO + grp;
-            const uint32_t mom = __shfl_sync(0xFFFFFFFFu, mom_l, bit[u]), dad = __shfl_sync(0xFFFFFFFFu, dad_l, bit[u]);
-            rz[u] = __shfl_sync(0xFFFFFFFFu, rl.z, bit[u]);
-            rw[u] = __shfl_sync(0xFFFFFFFFu, rl.w, bit[u]);
-            env[u] = __shfl_sync(0xFFFFFFFFu, env_l, bit[u]);
+            const uint4 dr = s_draw[warp][bit[u]];
+            const uint32_t mom = dr.x, dad = dr.y;
+            rz[u] = dr.z;
+            mut[u] = dr.w;
             const uint4 z = make_uint4(0u, 0u, 0u, 0u);
             const bool ok = wbase + bit[u] < n;
             const uint4 *pm = par + (size_t)mom * R4, *pf = par + (size_t)dad * R4;
@@ -277,28 +373,30 @@ __global__ void __launch_bounds__(kBlock, 4) k_offspring_cont(const __grid_const
             m1[u] = ok ? __ldg(pm + G + li) : z;
             f0[u] = ok ? __ldg(pf + li) : z;
             f1[u] = ok ? __ldg(pf + G + li) : z;
+            const uint32_t ahead = bit[u] + AHEAD * NO;
+            if (AHEAD != 0u && li < 2u && ahead < 32u && wbase + ahead < n)  // a parent for each of two lanes
+                prefetch(reinterpret_cast<const uint32_t *>(&s_draw[warp][ahead])[li]);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const uint32_t j = wbase + bit[u], t = it * U + (uint32_t)u;
+            const uint32_t j = wbase + bit[u];
             const bool ok = j < n;
             // (B) gametes: mask word wv of the mother (stream 2wv) and father (2wv + 1)
-            const uint32_t q = t / T_PER_SLOT;
-            uint4 dsrc = dml[0];
-#pragma unroll
-            for (int qq = 1; qq < NST; ++qq)
-                if (q == (uint32_t)qq) dsrc = dml[qq];
-            const uint32_t src = (t % T_PER_SLOT) * PER_T + grp * NST + (wv >> 1);
-            const uint32_t dx = __shfl_sync(0xFFFFFFFFu, dsrc.x, src), dy = __shfl_sync(0xFFFFFFFFu, dsrc.y, src);
-            const uint32_t dz = __shfl_sync(0xFFFFFFFFu, dsrc.z, src), dw = __shfl_sync(0xFFFFFFFFu, dsrc.w, src);
-            const uint32_t mm = (wv & 1u) ? dz : dx, mf = (wv & 1u) ? dw : dy;
+            const uint2 mk = reinterpret_cast<const uint2 *>(&s_mask[warp][NST * bit[u]])[wv];
+            const uint32_t mm = mk.x, mf = mk.y;
             uint4 c0 = pick8(m0[u], m1[u], (mm >> sh) & 0xFFu), c1 = pick8(f0[u], f1[u], (mf >> sh) & 0xFFu);
-            // (B) mutation: the biallelic count and distinct positions, each
-            // mutated value moved by an Irwin-Hall step by the lane owning it
-            const uint32_t u_mut = rw[u];
-            if (ok && kmax != 0u && u_mut >= s_cdf[0]) {  // the same in the whole group
-                uint32_t K = 0;
-                for (uint32_t qk = 0; qk < kmax; ++qk) K += u_mut >= s_cdf[qk] ? 1u : 0u;
+            // (B) mutation: the listed values moved by the lanes that own them
+            auto move = [&](uint32_t pos, int32_t step) {
+                if (pos >= L) add_step(c1, pos & 7u, step);
+                else add_step(c0, pos & 7u, step);
+            };
+            if (listed) {
+                for (uint32_t m = 0; m < (mut[u] & 0xFFFFu); ++m) {  // the same in the whole group
+                    const uint32_t e = (mut[u] >> 16) + m, pos = s_lpos[warp][e];
+                    if (((pos & (L - 1u)) >> 3) == li) move(pos, s_lstep[warp][e]);
+                }
+            } else {
+                const uint32_t K = mut[u] & 0xFFFFu;
                 uint32_t chosen = 0;
                 uint4 dp = make_uint4(0u, 0u, 0u, 0u);
                 for (uint32_t d = 0; d < (uint32_t)kMutDraws && chosen < K; ++d) {
@@ -313,12 +411,9 @@ __global__ void __launch_bounds__(kBlock, 4) k_offspring_cont(const __grid_const
                     }
                 }
                 for (uint32_t m = 0; m < chosen; ++m) {
-                    const uint32_t pos = mpos[m], locus = pos >= L ? pos - L : pos;
-                    if ((locus >> 3) == li) {
-                        const int32_t step = irwin_hall_step(j, g, rep, kMutSize, 3u * m, s_mut, k0, k1);
-                        if (pos >= L) add_step(c1, locus & 7u, step);
-                        else add_step(c0, locus & 7u, step);
-                    }
+                    const uint32_t pos = mpos[m];
+                    if (((pos & (L - 1u)) >> 3) == li)
+                        move(pos, irwin_hall_step(j, g, rep, kMutSize, 3u * m, s_mut, k0, k1));
                 }
                 __syncwarp(gmask);  // positions are rewritten by the group's next offspring
             }
@@ -326,21 +421,16 @@ __global__ void __launch_bounds__(kBlock, 4) k_offspring_cont(const __grid_const
                 chi[(size_t)j * R4 + li] = c0;
                 chi[(size_t)j * R4 + G + li] = c1;
             }
-            // this lane's part of the phenotype sum, its heterozygous loci and squares
-            int32_t part = 0;
-            uint32_t het = 0;
-            unsigned long long sq = 0;
-#pragma unroll
-            for (uint32_t k = 0; k < 8u; ++k) {
-                const int32_t x = val16(word_of(c0, k >> 1), k & 1u), y = val16(word_of(c1, k >> 1), k & 1u);
-                part += x + y;
-                het += x != y ? 1u : 0u;
-                sq += (uint32_t)(x * x) + (uint32_t)(y * y);
-            }
+            // this lane's part of the phenotype sum, its heterozygous loci and
+            // squares (no values, so zeros, past the population's end)
+            int32_t part = sum8(c0, sum8(c1, 0));
+            lane_het += differ8(c0, c1);
+            squares8(c0, sq_hh, sq_hl, sq_ll);
+            squares8(c1, sq_hh, sq_hl, sq_ll);
 #pragma unroll
             for (int o = G / 2; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
             // (C) phenotype: the sum of all values, plus the environmental step
-            const int32_t raw = part + env[u];
+            const int32_t raw = part + s_envs[warp][bit[u]];
             // (D) survival
             const long long v = (long long)raw + (long long)bias;
             const uint32_t bin = v < 0 ? 0u : (uint32_t)min(v >> shift_bin, (long long)(kBins - 1));
@@ -348,8 +438,6 @@ __global__ void __launch_bounds__(kBlock, 4) k_offspring_cont(const __grid_const
             if (f != kCertain) thr = __umulhi(thr, f);
             const bool alive = (thr == kCertain) || (rz[u] < thr);
             if (ok) {
-                lane_het += het;
-                lane_allele += sq;
                 mn = min(mn, raw);
                 mx = max(mx, raw);
                 if (alive) alive_bits |= 1u << bit[u];
@@ -365,6 +453,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_offspring_cont(const __grid_const
             }
         }
     }
+    const unsigned long long lane_allele = (unsigned long long)(65536LL * sq_hh + 512LL * sq_hl + (long long)sq_ll);
     alive_bits = __reduce_or_sync(0xFFFFFFFFu, alive_bits);
     const uint32_t w_surv = __reduce_add_sync(0xFFFFFFFFu, nsurv);
     if (lane == 0 && wbase < n) {

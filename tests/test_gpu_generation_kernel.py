@@ -1,5 +1,5 @@
-"""The generation kernel (single biallelic populations, batch members) and the
-spatial pool at the sizes and values where their own branches change, bit for
+"""The generation kernel (single biallelic populations, batch members), the
+continuous-allele kernel and the spatial pool at the sizes and values where their own branches change, bit for
 bit against the CPU oracle: one block or several, whole and ragged groups and
 slots, one- and two-digit values, 64-bit bins, calls longer than a launch,
 extinction inside a call, rare survivors, several blocks per member, stream
@@ -30,11 +30,12 @@ def spegg():
     return m
 
 
-def assert_same(orc, gpu, so, sg):
+def assert_same(orc, gpu, so, sg, continuous=False):
     assert len(so) == len(sg)
     for name in so.dtype.names:
         assert np.array_equal(so[name], sg[name]), name
-    assert np.array_equal(orc.genotypes(), gpu.genotypes())
+    read = "values" if continuous else "genotypes"
+    assert np.array_equal(getattr(orc, read)(), getattr(gpu, read)())
     assert np.array_equal(orc.survivors(), gpu.survivors())
     a, b = orc.state(), gpu.state()
     for k in ("gen", "S", "status", "f", "R"):
@@ -46,7 +47,7 @@ def check(w, n_gen):
     gpu = spegg().Population.from_workload(w, stats_capacity=n_gen + 2)
     so = orc.step(n_gen)
     gpu.step(n_gen)
-    assert_same(orc, gpu, so, gpu.read_stats(1, gpu.state()["gen"]))
+    assert_same(orc, gpu, so, gpu.read_stats(1, gpu.state()["gen"]), w.allele_model == 1)
 
 
 # groups of 32; 512 is one block's 16 groups; 77,824 = 2,432 slots of one group
@@ -134,6 +135,22 @@ def test_step_under_stream_capture(n):
     orc = oracle.OraclePopulation.from_workload(w)
     so = orc.step(7)
     assert_same(orc, gpu, so, gpu.read_stats(1, 7))
+
+
+@pytest.mark.parametrize("per_offspring", [0.5, 4.0, 7.0])
+@pytest.mark.parametrize("n_loci", [32, 64, 128, 256])
+def test_continuous_mutations_and_extreme_values(n_loci, per_offspring):
+    """Below, around and above the 128 mutations of 32 offspring that are
+    listed ahead, with values over the whole int16 range."""
+    n = 1003
+    w = S.continuous_trait(n=n, n_loci=n_loci, mu=per_offspring / (2 * n_loci), seed=n_loci)
+    rng = np.random.default_rng(n_loci)
+    v = rng.integers(-32768, 32768, (n, 2 * n_loci)).astype(np.int16)
+    v[:40] = -32768
+    v[40:80] = 32767
+    v[80:120, ::2] = 0
+    check(dataclasses.replace(w, init_values=v, bias=1 << 23, shift=12,
+                              surv_table=np.full(4096, 0xC000_0000, np.uint32)), 4)
 
 
 def test_space_pool_moves_its_records():
