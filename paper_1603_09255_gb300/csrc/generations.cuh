@@ -1,5 +1,16 @@
-// The generation kernel of a single population (sm_103a): any number of
-// generations of Fig. 1 A-F in one cooperative launch.
+// The generation kernel of biallelic populations (sm_103a): any number of
+// generations of Fig. 1 A-F in one cooperative launch, of one population
+// (k_generations) or of many, each formed by a team of blocks (k_teams).
+//
+// us per generation, against an offspring launch with byte tables and a
+// compaction launch: N = 10^4, L = 32: 8.2 -> 4.8; 99,991 x 64 with locus counts
+// 21.5 -> 9.9; 3 x 10^5 x 128 with dominance 23.8 -> 13.2; 10^6 x 128 with a
+// resource 39.2 -> 26.0, with a map 127 -> 75, with weights 64.8 -> 48.5; 2 x
+// 10^6 x 256 164 -> 78.  At 10^6 x 128 it is bound by instructions: 41,000 of
+// 52,000 cycles a generation form offspring, 405 instructions per warp of 32,
+// the integer pipe busy 56 % of them with four warps per scheduler (512 threads
+// of 128 registers; 640 to 1,024 threads spill and are slower); the rest is the
+// barrier (3,300 to 5,000), the directory (2,000 to 3,500) and the statistics.
 //
 // Blocks stay for the whole call, so the tables (thresholds, attack rates,
 // effect digits, linkage map) reach shared memory once per call instead of
@@ -99,6 +110,21 @@ __device__ __forceinline__ bool team_barrier(unsigned long long *ctr, uint32_t r
         ok = v >= want ? 1 : 0;
     }
     return __syncthreads_and(threadIdx.x == 0 ? ok : 1) != 0;
+}
+
+// A call of one generation needs no block to wait: whether this block is the
+// last of the team to arrive, which closes the generation alone.
+__device__ __forceinline__ bool last_to_arrive(unsigned long long *ctr, uint32_t rank, uint32_t team) {
+    __syncthreads();
+    int last = 0;
+    if (threadIdx.x == 0) {
+        const unsigned long long add = rank == 0u ? kBarrierStep - (team - 1u) : 1ull;
+        unsigned long long old;
+        asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], %2;" : "=l"(old) : "l"(ctr), "l"(add) : "memory");
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        last = (old + add) % kBarrierStep == 0ull ? 1 : 0;
+    }
+    return __syncthreads_or(threadIdx.x == 0 ? last : 0) != 0;
 }
 
 // ------------------------------------------------------- record access
@@ -457,7 +483,7 @@ __device__ __forceinline__ void locate(const SoloArgs &a, uint32_t u0, uint32_t 
     i1 = r1 + e1.y;
 }
 
-// Weighted parents (bounded rejection, see offspring.cuh): proposals in
+// Weighted parents (bounded rejection): proposals in
 // pairs, both roles together; thr holds each survivor's thresholds as mother
 // and as father at its record's place.
 template <class SM>
@@ -583,7 +609,7 @@ __device__ __forceinline__ bool build_directory(const uint32_t *counts, uint32_t
 // Allele copies of the block's own records [j0, j1), added to the generation's
 // row: bit-sliced counters per lane (plane k holds bit k of every locus's count
 // among the lane's records), transposed across the warp before they could
-// overflow (see k_locus_counts).  Four record words at a time.
+// overflow.  Four record words at a time.
 __device__ __forceinline__ uint32_t transpose32(uint32_t x, uint32_t lane) {
     constexpr uint32_t M[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
 #pragma unroll
@@ -731,10 +757,11 @@ __device__ __forceinline__ unsigned long long total_stats(const GenAcc *acc, uin
 // GENERAL: dominance, values beyond 2048 in magnitude or a bias beyond 2^30
 // (the others' instance has none of these branches in its loop).
 // Blocks 0 .. team - 1 (this one is `rank`) form n_gen generations of a
-// population; keep_last: the last of them is the call's last.
+// population; keep_last: the last of them is the call's last; single: the one
+// generation of a call, closed by the last block that arrives.
 template <int W, bool LINKED, bool WEIGHTED, bool GENERAL>
 __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundKeys &keys, uint32_t n_gen,
-                                                 bool keep_last, uint32_t rank, uint32_t team) {
+                                                 bool keep_last, bool single, uint32_t rank, uint32_t team) {
     constexpr int BLOCK = (int)kSoloThreads;
     using SM = GenSmem<W, LINKED>;
     constexpr uint32_t NW = BLOCK / 32;
@@ -747,13 +774,6 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
     const PopParams *P = a.prm;
     DevState *st = a.state;
 
-    // the call's starting state (written by earlier launches)
-    uint32_t gen = ld_relaxed_u32(&st->gen), f = ld_relaxed_u32(&st->f);
-    const uint32_t target = ld_relaxed_u32(&st->target);
-    int32_t status = (int32_t)ld_relaxed_u32(reinterpret_cast<const uint32_t *>(&st->status));
-    double R = ld_relaxed_f64(&st->R);
-    if (status != SPG_OK || ld_relaxed_u32(&st->S) == 0u) return;
-
     // tables
     const bool eco = a.has_eco != 0u, dom = GENERAL && a.dom != 0u;
     for (uint32_t i = tid; i < (uint32_t)kBins / 4u; i += BLOCK) {
@@ -765,6 +785,18 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
         if (dom) cp_async_16(smem0 + SM::kFrag + SM::kTabBytes + 16u * i, a.frag->table[1] + 4u * i);
     }
     cp_async_commit();
+    griddep_wait();  // the tables are parameters: nothing an earlier launch writes
+    griddep_release();
+    // the call's starting state (written by earlier launches)
+    uint32_t gen = ld_relaxed_u32(&st->gen), f = ld_relaxed_u32(&st->f);
+    const uint32_t target = ld_relaxed_u32(&st->target);
+    int32_t status = (int32_t)ld_relaxed_u32(reinterpret_cast<const uint32_t *>(&st->status));
+    double R = ld_relaxed_f64(&st->R);
+    if (status != SPG_OK || ld_relaxed_u32(&st->S) == 0u) {
+        cp_async_wait<0>();
+        return;
+    }
+
     if (tid < (uint32_t)kMaxKmax) s_cdf[tid] = tid < a.kmax ? P->cdf[tid] : 0xFFFFFFFFu;
     LinkMap lk{};
     if constexpr (LINKED) {
@@ -929,7 +961,11 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
         __syncthreads();
         GenAcc *acc = a.acc + (size_t)(g % 3u) * kGenAccCopies;
         add_stats<SM>(acc + rank % kGenAccCopies, warp, lane);
-        if (!team_barrier(a.barrier, rank, team)) {  // the generation fails: every block gives up
+        if (single) {
+            if (!last_to_arrive(a.barrier, rank, team)) return;
+            rank = 0u;  // the rest is this block's alone
+            team = 1u;
+        } else if (!team_barrier(a.barrier, rank, team)) {  // the generation fails: every block gives up
             if (tid == 0u) atomicExch(reinterpret_cast<int *>(&st->status), SPG_ERR_TIMEOUT);
             return;
         }
@@ -992,7 +1028,20 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
                 }
             }
         }
-        if (list && S_new != 0u) {  // the ordered survivor list from the bitmap
+        if (single && S_new != 0u) {  // the ordered survivor list from the bitmap, 32 slots (of one group) a warp
+            for (uint32_t s0 = warp * 32u; s0 < a.nslots; s0 += NW * 32u) {
+                const uint32_t slot = s0 + lane;
+                uint32_t word = 0u, first = 0u;
+                if (slot < a.nslots) {
+                    word = __ldcg(a.alive + slot);
+                    first = slot * rec_slot - *reinterpret_cast<const uint32_t *>(g_smem + SM::kDir + 8u * slot + 4u);
+                }
+                for (uint32_t b = 0; b < 32u && s0 + b < a.nslots; ++b) {
+                    const uint32_t bits = __shfl_sync(0xFFFFFFFFu, word, b), at = __shfl_sync(0xFFFFFFFFu, first, b);
+                    if ((bits >> lane) & 1u) a.surv[at + __popc(bits & ((1u << lane) - 1u))] = (s0 + b) * 32u + lane;
+                }
+            }
+        } else if (list && S_new != 0u) {  // the same, a slot a warp of the team
             for (uint32_t slot = rank * NW + warp; slot < a.nslots; slot += team * NW) {
                 uint32_t rank = slot * rec_slot - *reinterpret_cast<const uint32_t *>(g_smem + SM::kDir + 8u * slot + 4u);
                 for (uint32_t gi = 0; gi < a.slot_len && slot * rec_slot + 32u * gi < a.n; ++gi) {
@@ -1019,7 +1068,8 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
 // One population: every block of the grid is in its team.
 template <int W, bool LINKED, bool WEIGHTED, bool GENERAL>
 __global__ void __launch_bounds__(kSoloThreads, 1) k_generations(const __grid_constant__ SoloArgs a) {
-    form_generations<W, LINKED, WEIGHTED, GENERAL>(a, a.keys, a.n_gen, a.keep_last != 0u, blockIdx.x, gridDim.x);
+    form_generations<W, LINKED, WEIGHTED, GENERAL>(a, a.keys, a.n_gen, a.keep_last != 0u, a.single != 0u,
+                                                   blockIdx.x, gridDim.x);
 }
 
 // Several populations: each block works through its list of teams.  A team's
@@ -1041,8 +1091,8 @@ __device__ __forceinline__ void team_places(const TeamArgs &t, uint32_t &p) {
             reinterpret_cast<uint32_t *>(&s_team_args)[i] = reinterpret_cast<const uint32_t *>(t.members + place.member)[i];
         __syncthreads();
         if (s_team_args.words != (uint32_t)W) return;
-        form_generations<W, LINKED, WEIGHTED, GENERAL>(s_team_args, s_team_args.keys, t.n_gen, t.keep_last != 0u, place.rank,
-                                                       place.team);
+        form_generations<W, LINKED, WEIGHTED, GENERAL>(s_team_args, s_team_args.keys, t.n_gen, t.keep_last != 0u, false,
+                                                       place.rank, place.team);
     }
 }
 template <bool LINKED, bool WEIGHTED, bool GENERAL>

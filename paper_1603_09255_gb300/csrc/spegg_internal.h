@@ -214,6 +214,7 @@ struct alignas(16) SoloArgs {
     uint32_t dom, two_digits;          // fragments: dominance, values beyond 2048 in magnitude
     uint32_t n_gen;                    // generations of this launch
     uint32_t keep_last;                // the last of them is the call's last
+    uint32_t single;                   // a call of one generation: no grid barrier
 };
 struct SoloKernel {
     const void *fn = nullptr;

@@ -93,6 +93,36 @@ def test_extinction_inside_a_call(n):
     check(w, 12)
 
 
+@pytest.mark.parametrize("n_loci", [32, 256])
+@pytest.mark.parametrize("n", [300, 513, 5000, 16_384, 16_385])
+def test_calls_of_one_generation(n, n_loci):
+    """One-generation calls back to back, among longer ones, with a resource
+    and per-locus counts."""
+    w = S.consumer_resource(n=n, n_loci=n_loci, K=50.0 * n, mu=1e-3, seed=n)
+    orc = oracle.OraclePopulation.from_workload(w)
+    gpu = spegg().Population.from_workload(w, stats_capacity=16)
+    gpu.set_locus_counts()
+    counts, so = [], []
+    for k in (1, 1, 1, 2, 1, 1):
+        gpu.step(k)
+    for _ in range(7):
+        so.append(orc.step(1))
+        counts.append(orc.locus_counts())
+    assert_same(orc, gpu, np.concatenate(so), gpu.read_stats(1, 7))
+    assert np.array_equal(gpu.locus_counts(1, 7), np.stack(counts))
+
+
+def test_extinction_in_a_call_of_one_generation():
+    w = S.consumer_resource(n=5000, n_loci=64, K=2.5e5, seed=3)
+    w.attack = S.constant_table(2 ** 30)
+    orc = oracle.OraclePopulation.from_workload(w)
+    gpu = spegg().Population.from_workload(w, stats_capacity=16)
+    so = orc.step(4)
+    for _ in range(4):
+        gpu.step(1)
+    assert_same(orc, gpu, so, gpu.read_stats(1, gpu.state()["gen"]))
+
+
 @pytest.mark.parametrize("p", [0x0100_0000, 0x0010_0000])
 def test_rare_survivors(p):
     """1 in 256 and 1 in 4,096 survive: most slots are empty, so the directory
