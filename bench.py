@@ -45,11 +45,14 @@ def algorithmic_bytes(words: int) -> int:
     return 12 + 24 * words
 
 
-# DRAM traffic per launch of the dominant kernel (the offspring kernel of the
-# headline population) from one ncu capture, keyed by the hash of that
-# kernel's sources (null once they change).
-MEASURED_TRAFFIC = {"e961a201f358e511": 28457472}
-TRAFFIC_SOURCES = ("offspring.cuh", "device_common.cuh", "offspring_w4.cu")
+# Most generations of one launch of the generation kernel.
+LAUNCH_GENERATIONS = 512
+# DRAM traffic per generation of the headline population (a launch of four
+# generations of its kernel, caches flushed before it, divided by four) from
+# one ncu capture, keyed by the hash of that kernel's sources (null once they
+# change).
+MEASURED_TRAFFIC = {"e42f5f437614db65": 17340400}
+TRAFFIC_SOURCES = ("generations.cuh", "device_common.cuh", "ecology.cuh", "generations_w4.cu")
 
 
 def kernel_source_hash() -> str:
@@ -197,7 +200,7 @@ def timed_on(stream, torch, fn):
 
 
 def per_generation_ms(stream, torch, step_one, repeats=32, warmup=3):
-    """p50/p99 of single generations (direct launches) bracketed by events."""
+    """p50/p99 of single generations (one call each) bracketed by events."""
     for _ in range(warmup):
         step_one()
     stream.synchronize()
@@ -207,20 +210,19 @@ def per_generation_ms(stream, torch, step_one, repeats=32, warmup=3):
 
 def single_species(spegg, torch, oracle_cpu: bool):
     """The single-species workload (N = 10^4, L = 32, 100 generations): through
-    the cached graph (one step call), by direct launches (100 single-generation
-    calls), and the oracle single-threaded on the full run.  Each timed run
-    starts from the founders restored from a checkpoint, after one untimed run
-    of the same calls (which builds the cached graph)."""
+    one step call, by 100 single-generation calls, and the oracle
+    single-threaded on the full run.  Each timed run starts from the founders
+    restored from a checkpoint, after one untimed run of the same calls."""
     w = S.single_species()
     stream = torch.cuda.Stream()
     ind = w.n * w.n_gen
     times = {}
-    for mode in ("graph", "direct"):
+    for mode in ("call", "direct"):
         ms = []
         for _ in range(4):  # the first of four runs is a warm-up
             pop = spegg.Population.from_workload(w, stats_capacity=w.n_gen + 8, stream=stream)
             founders = pop.checkpoint()
-            if mode == "graph":
+            if mode == "call":
                 run = lambda: pop.step(w.n_gen)  # noqa: E731
             else:
                 run = lambda: [pop.step(1) for _ in range(w.n_gen)]  # noqa: E731
@@ -230,7 +232,7 @@ def single_species(spegg, torch, oracle_cpu: bool):
             ms.append(timed_on(stream, torch, run))
             pop.close()
         times[mode] = min(ms[1:])
-    out = {"value": ind / (times["graph"] / 1e3), "nograph": ind / (times["direct"] / 1e3)}
+    out = {"value": ind / (times["call"] / 1e3), "nograph": ind / (times["direct"] / 1e3)}
     if oracle_cpu:
         import oracle
         orc = oracle.OraclePopulation.from_workload(w)
@@ -245,10 +247,9 @@ def batched_replicates(spegg, torch, gens: int = 500, plain_members: int = 0, pl
                        oracle_cpu: bool = False, count: int = 4096):
     """Batched-replicates workload: `count` independent single-species runs (N
     log-uniform in [1e3, 2e5], L in {32, 64, 128}, s in [0, 0.5]) advanced by
-    shared, graph-captured launches with autotuned launch shapes, against the
-    plain path: every replicate (or the first `plain_members`) stepped one
-    population at a time through its own cached graph, 256 populations resident
-    at a time, each graph built before its timed run (as the batch's are)."""
+    shared launches, against the plain path: every replicate (or the first
+    `plain_members`) stepped one population at a time, 256 populations
+    resident at a time, each stepped once before its timed run."""
     ws = S.batch_replicates(count=count, n_gen=gens)
     plain_members = min(plain_members or count, count)
     stream = torch.cuda.Stream()
@@ -266,7 +267,7 @@ def batched_replicates(spegg, torch, gens: int = 500, plain_members: int = 0, pl
         idx = range(c0, min(c0 + 256, plain_members))
         pops = [spegg.Population.from_workload(ws[i], stats_capacity=2 * plain_gens + 8, stream=stream) for i in idx]
         for p in pops:
-            p.step(plain_gens)  # builds each population's cached graph
+            p.step(plain_gens)
         stream.synchronize()
         ms_plain += timed_on(stream, torch, lambda: [p.step(plain_gens) for p in pops])
         plain_work += sum(ws[i].n for i in idx) * plain_gens
@@ -509,9 +510,9 @@ def main():
     assert st["status"] == 0, f"population status {st['status']}"
     value = workload.n * GENERATIONS * args.steps * ws / (total_ms / 1000.0)
 
-    # roofline of one generation (offspring + compaction launches, timed together)
-    launches = GENERATIONS * args.steps
-    avg_gen_s = total_ms / 1000.0 / launches
+    # roofline of one generation
+    launches = -(-GENERATIONS // LAUNCH_GENERATIONS) * args.steps
+    avg_gen_s = total_ms / 1000.0 / (GENERATIONS * args.steps)
     peak, peak_kind = load_peaks()
     achieved = algorithmic_bytes(workload.words) * workload.n / avg_gen_s / 1e9
     traffic = MEASURED_TRAFFIC.get(kernel_source_hash())
@@ -567,7 +568,7 @@ def main():
                      "traffic": traffic, "peak_kind": peak_kind, "shape": list(shape)},
         "e2e": {"value": e2e_value, "unit": "individual-generations/s", "h2d_bytes_per_step": len(blob),
                 "d2h_bytes_per_step": int(stats.nbytes)},
-        "gpu_launches": 2 * launches,
+        "gpu_launches": launches,
         "clocks": clocks.summary(),
         "gen_ms": {"p50": gen_p50, "p99": gen_p99},
     }
