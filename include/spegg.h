@@ -121,7 +121,10 @@ enum spg_status_code {
     SPG_ERR_INVALID = -1,   /* bad argument or description                      */
     SPG_ERR_OOM = -2,       /* device allocation failed                         */
     SPG_ERR_CUDA = -3,      /* a CUDA runtime call failed                       */
-    SPG_ERR_TIMEOUT = -4,   /* reserved: a bounded wait gave up                 */
+    SPG_ERR_TIMEOUT = -4,   /* a block's bounded wait for the others gave up: the
+                             * population stays at its last complete generation's
+                             * number and steps no more (its records are undefined);
+                             * spg_restore starts it afresh                       */
     SPG_ERR_RANGE = -5,     /* requested generations are not in the stats ring  */
     SPG_ERR_BUDGET = -6     /* request exceeds the server's memory budget       */
 };

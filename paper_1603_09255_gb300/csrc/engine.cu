@@ -407,6 +407,7 @@ void solo_args(const PopView &v, const PopParams &prm, SoloArgs &a) {
         a.keys[2 * i] = prm.key0 + i * 0x9E3779B9u;
         a.keys[2 * i + 1] = prm.key1 + i * 0xBB67AE85u;
     }
+    a.barrier_tries = kBarrierTries;
     a.words = prm.words;
     a.rep = prm.rep;
     a.kmax = prm.kmax;

@@ -92,10 +92,16 @@ __device__ __forceinline__ uint32_t sm_u32(uint32_t off) { return *reinterpret_c
 // by kBarrierStep per barrier whatever the team's size (its first block adds
 // what the others leave).  (Every block polling a word of every other took 5 us
 // instead of 2 with 152 blocks.)
+//
+// A block whose polls run out marks the counter, in one atomic step and only
+// while the barrier is incomplete: from then on nobody passes it, however late
+// the missing blocks arrive, so the generation is closed by nobody and every
+// block of the team reports the failure.  The mark stays until the population's
+// memory is set up again (launch_pack).
 constexpr unsigned long long kBarrierStep = 1u << 16;  // more than a grid's blocks
-constexpr uint32_t kBarrierTries = 1u << 24;  // polls of about half a microsecond before a wait gives up
+constexpr unsigned long long kBarrierFailed = 1ull << 63;
 
-__device__ __forceinline__ bool team_barrier(unsigned long long *ctr, uint32_t rank, uint32_t team) {
+__device__ __forceinline__ bool team_barrier(unsigned long long *ctr, uint32_t rank, uint32_t team, uint32_t tries) {
     __syncthreads();
     if (team == 1u) return true;
     int ok = 1;
@@ -104,10 +110,14 @@ __device__ __forceinline__ bool team_barrier(unsigned long long *ctr, uint32_t r
         unsigned long long old, v = 0;
         asm volatile("atom.add.release.gpu.global.u64 %0, [%1], %2;" : "=l"(old) : "l"(ctr), "l"(add) : "memory");
         const unsigned long long want = (old / kBarrierStep + 1ull) * kBarrierStep;
-        for (uint32_t i = 0; i < kBarrierTries && v < want; ++i)
+        for (uint32_t i = 0; i < tries && v < min(want, kBarrierFailed); ++i)
             asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
+        while (v < want && old < kBarrierFailed) {  // once per arrival meanwhile, at most
+            const unsigned long long was = atomicCAS(ctr, v, v | kBarrierFailed);
+            v = was == v ? kBarrierFailed : was;
+        }
         asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        ok = v >= want ? 1 : 0;
+        ok = v >= want && v < kBarrierFailed ? 1 : 0;
     }
     return __syncthreads_and(threadIdx.x == 0 ? ok : 1) != 0;
 }
@@ -792,7 +802,9 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
     const uint32_t target = ld_relaxed_u32(&st->target);
     int32_t status = (int32_t)ld_relaxed_u32(reinterpret_cast<const uint32_t *>(&st->status));
     double R = ld_relaxed_f64(&st->R);
-    if (status != SPG_OK || ld_relaxed_u32(&st->S) == 0u) {
+    // one decision for the block: a teammate that gives up on a block this late
+    // may change the status between its threads' reads
+    if (__syncthreads_or(status != SPG_OK || ld_relaxed_u32(&st->S) == 0u)) {
         cp_async_wait<0>();
         return;
     }
@@ -965,7 +977,7 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
             if (!last_to_arrive(a.barrier, rank, team)) return;
             rank = 0u;  // the rest is this block's alone
             team = 1u;
-        } else if (!team_barrier(a.barrier, rank, team)) {  // the generation fails: every block gives up
+        } else if (!team_barrier(a.barrier, rank, team, a.barrier_tries)) {  // the generation fails: every block gives up
             if (tid == 0u) atomicExch(reinterpret_cast<int *>(&st->status), SPG_ERR_TIMEOUT);
             return;
         }

@@ -185,6 +185,7 @@ struct alignas(64) GenAcc {
 };
 constexpr uint32_t kGenAccCopies = 4;
 constexpr unsigned long long kEmptyMinMax = 0x800000007FFFFFFFull;  // mx INT_MIN over mn INT_MAX
+constexpr uint32_t kBarrierTries = 1u << 24;  // polls of about half a microsecond before a wait gives up
 constexpr int kMaxGuideBits = 13;  // the parent draw's top bits that index the directory's guide, at most
 struct alignas(16) SoloArgs {
     uint32_t keys[20];                 // Philox round keys (word 0, word 1 of each round)
@@ -198,7 +199,7 @@ struct alignas(16) SoloArgs {
     uint32_t *surv;                    // its ordered survivor list [N]
     DevState *state;
     GenAcc *acc;                       // [3][kGenAccCopies], by generation % 3
-    unsigned long long *barrier;       // grid barrier arrivals, a multiple of the grid between launches
+    unsigned long long *barrier;       // grid barrier arrivals (generations.cuh)
     spg_stats *ring;
     uint32_t *locus_row[2];            // per-locus counts of the generation being formed, by parity (null: off)
     uint32_t *locus_ring;              // [locus_cap][L]
@@ -215,6 +216,7 @@ struct alignas(16) SoloArgs {
     uint32_t n_gen;                    // generations of this launch
     uint32_t keep_last;                // the last of them is the call's last
     uint32_t single;                   // a call of one generation: no grid barrier
+    uint32_t barrier_tries;            // polls of a wait before it gives up
 };
 struct SoloKernel {
     const void *fn = nullptr;
