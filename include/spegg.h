@@ -402,7 +402,8 @@ typedef struct {
     uint64_t job;
     uint32_t state;           /* SPG_JOB_QUEUED / RESIDENT / FINISHED */
     uint32_t gen;             /* generations completed (enqueued while resident) */
-    int32_t status;           /* SPG_OK or SPG_EXTINCT once finished */
+    int32_t status;           /* once finished: SPG_OK, SPG_EXTINCT, or the error that
+                               * stopped it (SPG_ERR_TIMEOUT; gen < n_gen)        */
     uint32_t n_gen;           /* requested generations */
     double t_arrival, t_admit, t_finish;   /* -1 until reached */
     size_t footprint;         /* device bytes while resident */

@@ -112,7 +112,8 @@ int retire(spg_server *s, Job &j) {
     j.stats.resize(st.gen);
     if (st.gen) {
         rc = view_read_stats(j.v, 1, st.gen, j.stats.data());
-        if (rc != SPG_OK) return rc;
+        // a job that stopped with an error is finished with it: what it formed is kept
+        if (rc != SPG_OK && rc != st.status) return rc;
     }
     s->alloc.release(j.arena, s->stream);
     j.arena = nullptr;

@@ -1,8 +1,9 @@
 // GPU check of what a wait that runs out leaves behind (a block of a team that
-// never arrives, polls limited to a moment; nothing faults or hangs).  The
-// source of the population is part of this program, so that it reaches its
-// arguments.
+// never arrives, polls limited to a moment; nothing faults or hangs), and of a
+// served job that ends with an error.  The sources of the population and the
+// server are part of this program, so that it reaches their arguments.
 #include "population.cu"
+#include "server.cu"
 
 #include <cstdio>
 #include <cstdlib>
@@ -143,12 +144,39 @@ void barrier(uint32_t n, uint32_t missing) {
     spg_destroy(ref);
 }
 
+// A job whose device state says that a wait ran out is finished with that
+// status; the others are not held up.
+void served_job() {
+    const Inputs a(5000), b(9000), c(700);
+    spg_server_config cfg{};
+    cfg.gens_per_tick = 4;
+    spg_server *s = nullptr;
+    CHECK(spg_server_create(&cfg, nullptr, nullptr, &s) == SPG_OK);
+    uint64_t job[3];
+    const Inputs *in[3] = {&a, &b, &c};
+    for (int i = 0; i < 3; ++i) CHECK(spg_server_submit(s, &in[i]->desc, nullptr, 20, 0.0, job + i) == SPG_OK);
+    CHECK(spg_server_tick(s, nullptr, nullptr) == SPG_OK);
+    set_status(s->jobs[job[1]]->v, SPG_ERR_TIMEOUT);
+    CHECK(spg_server_drain(s) == SPG_OK);
+    std::vector<spg_stats> rec(20);
+    for (int i = 0; i < 3; ++i) {
+        spg_job_info info;
+        CHECK(spg_server_job_info(s, job[i], &info) == SPG_OK && info.state == SPG_JOB_FINISHED);
+        CHECK(info.status == (i == 1 ? SPG_ERR_TIMEOUT : SPG_OK) && info.gen == (i == 1 ? 4u : 20u));
+        CHECK(spg_server_job_stats(s, job[i], 1, info.gen, rec.data()) == SPG_OK && rec[info.gen - 1].gen == info.gen);
+    }
+    spg_server_counters n;
+    CHECK(spg_server_stats(s, &n) == SPG_OK && n.memory_used == 0 && n.resident == 0);
+    spg_server_destroy(s);
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "barrier")
         for (uint32_t missing : {0u, 2u}) barrier(20000, missing);
+    else if (what == "served") served_job();
     else return 2;
     std::printf("ok\n");
     return 0;

@@ -39,3 +39,9 @@ def test_a_wait_that_runs_out_is_kept(program):
     """Nobody passes the barrier once a block has given up: the generation is
     not closed, the status stays, and a restored checkpoint starts afresh."""
     run(program, "barrier")
+
+
+def test_a_served_job_with_an_error_is_finished(program):
+    """It gives back its memory, keeps its statistics and its status, and the
+    other jobs run to their ends."""
+    run(program, "served")
