@@ -420,6 +420,10 @@ int spg_restore(spg_pop *p, const void *host, size_t bytes) {
     }
     rc = view_set_state(p->view(), h.gen, h.S, h.f, h.R, h.status, 0xFFFFFFFFu);
     if (rc != SPG_OK) return rc;
+    if (p->locus_mem) {  // the rows of a generation that failed hold part of its counts
+        e = cudaMemsetAsync(p->locus.acc, 0, (size_t)2 * p->n_loci * 4, p->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "clear per-locus counts");
+    }
     p->locus_from = h.gen + 1u;  // counts of the restored run start with its next generation
     p->locus_until = h.gen;
     return view_sync(p->view());

@@ -106,8 +106,9 @@ spg_pop *create(const Inputs &in) {
     return p;
 }
 
-// missing: the rank that does not arrive; it comes late, in a launch of its own
-void barrier(uint32_t n, uint32_t missing) {
+// missing: the rank that does not arrive; it comes late, in a launch of its
+// own.  counts: the restored run's per-locus counts are compared too.
+void barrier(uint32_t n, uint32_t missing, bool counts) {
     const Inputs in(n);
     spg_pop *ref = create(in), *p = create(in);
     CHECK(spg_step_generations(ref, 10) == SPG_OK);
@@ -140,6 +141,7 @@ void barrier(uint32_t n, uint32_t missing) {
     CHECK(std::memcmp(got.stats.data(), want.stats.data(), want.stats.size() * sizeof(spg_stats)) == 0);
     CHECK(got.geno == want.geno && got.surv == want.surv);
     CHECK(got.state.gen == 13 && got.state.status == SPG_OK);
+    CHECK(!counts || got.counts == want.counts);
     spg_destroy(p);
     spg_destroy(ref);
 }
@@ -175,7 +177,8 @@ void served_job() {
 int main(int argc, char **argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "barrier")
-        for (uint32_t missing : {0u, 2u}) barrier(20000, missing);
+        for (uint32_t missing : {0u, 2u}) barrier(20000, missing, false);
+    else if (what == "counts") barrier(20000, 3, true);
     else if (what == "served") served_job();
     else return 2;
     std::printf("ok\n");

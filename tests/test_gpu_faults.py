@@ -41,6 +41,11 @@ def test_a_wait_that_runs_out_is_kept(program):
     run(program, "barrier")
 
 
+def test_a_failed_generation_leaves_no_locus_counts(program):
+    """The counts of the restored run hold nothing of the generation that failed."""
+    run(program, "counts")
+
+
 def test_a_served_job_with_an_error_is_finished(program):
     """It gives back its memory, keeps its statistics and its status, and the
     other jobs run to their ends."""
