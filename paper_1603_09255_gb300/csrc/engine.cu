@@ -12,6 +12,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -1016,14 +1017,14 @@ constexpr size_t kReadTogether = 48u << 10;
 int view_read_stats(const PopView &v, uint32_t first_gen, uint32_t count, spg_stats *out) {
     if (!out && count) return fail(SPG_ERR_INVALID, "NULL argument");
     // the state and, when the ring is short, the ring behind it in one copy
+    // (two copies when the host has no memory for that)
     DevState st;
-    std::vector<char> both;
     const size_t ring_at = v.L.ring - v.L.state, all = ring_at + (size_t)v.cap * sizeof(spg_stats);
+    const std::unique_ptr<char[]> both(all <= kReadTogether ? new (std::nothrow) char[all] : nullptr);
     int rc;
-    if (all <= kReadTogether) {
-        both.resize(all);
-        rc = read_back(v, both.data(), v.L.state, all, "read state and stats");
-        std::memcpy(&st, both.data(), sizeof st);
+    if (both) {
+        rc = read_back(v, both.get(), v.L.state, all, "read state and stats");
+        if (rc == SPG_OK) std::memcpy(&st, both.get(), sizeof st);
     } else {
         rc = view_state(v, st);
     }
@@ -1037,8 +1038,8 @@ int view_read_stats(const PopView &v, uint32_t first_gen, uint32_t count, spg_st
     for (uint32_t i = 0; i < count;) {
         const uint32_t slot = (first_gen - 1 + i) % v.cap;
         const uint32_t run = std::min(count - i, v.cap - slot);
-        if (!both.empty()) {
-            std::memcpy(out + i, both.data() + ring_at + slot * sizeof(spg_stats), run * sizeof(spg_stats));
+        if (both) {
+            std::memcpy(out + i, both.get() + ring_at + slot * sizeof(spg_stats), run * sizeof(spg_stats));
         } else {
             const cudaError_t e = cudaMemcpy(out + i, ring + slot, run * sizeof(spg_stats), cudaMemcpyDeviceToHost);
             if (e != cudaSuccess) return cuda_fail(e, "read stats");

@@ -1,7 +1,8 @@
 // GPU check of what a wait that runs out leaves behind (a block of a team that
-// never arrives, polls limited to a moment; nothing faults or hangs), and of a
-// served job that ends with an error.  The sources of the population and the
-// server are part of this program, so that it reaches their arguments.
+// never arrives, polls limited to a moment; nothing faults or hangs), of a
+// served job that ends with an error, and of a read without host memory.  The
+// sources of the population and the server are part of this program, so that
+// it reaches their arguments.
 #include "population.cu"
 #include "server.cu"
 
@@ -172,7 +173,31 @@ void served_job() {
     spg_server_destroy(s);
 }
 
+// Reading statistics needs no host memory that may run out unreported.
+bool g_no_memory = false;
+
+void host_memory() {
+    const Inputs in(1000);
+    spg_pop *p = nullptr;
+    CHECK(spg_create_population(&in.desc, nullptr, nullptr, &p) == SPG_OK);
+    CHECK(spg_step_generations(p, 3) == SPG_OK);
+    spg_stats rec[3];
+    g_no_memory = true;
+    const int rc = spg_read_stats(p, 1, 3, rec);
+    g_no_memory = false;
+    CHECK(rc == SPG_OK && rec[2].gen == 3);
+    spg_destroy(p);
+}
+
 }  // namespace
+
+void *operator new(size_t bytes) {
+    void *p = g_no_memory ? nullptr : std::malloc(bytes);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void operator delete(void *p) noexcept { std::free(p); }
+void operator delete(void *p, size_t) noexcept { std::free(p); }
 
 int main(int argc, char **argv) {
     const std::string what = argc > 1 ? argv[1] : "";
@@ -180,6 +205,7 @@ int main(int argc, char **argv) {
         for (uint32_t missing : {0u, 2u}) barrier(20000, missing, false);
     else if (what == "counts") barrier(20000, 3, true);
     else if (what == "served") served_job();
+    else if (what == "memory") host_memory();
     else return 2;
     std::printf("ok\n");
     return 0;

@@ -50,3 +50,8 @@ def test_a_served_job_with_an_error_is_finished(program):
     """It gives back its memory, keeps its statistics and its status, and the
     other jobs run to their ends."""
     run(program, "served")
+
+
+def test_a_read_without_host_memory(program):
+    """No exception leaves the C ABI."""
+    run(program, "memory")
