@@ -31,6 +31,7 @@
 #include <climits>
 #include <cstring>
 #include <memory>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -791,7 +792,7 @@ struct spg_space {
     Allocator alloc;
     char *arena = nullptr;
     SpaceArgs args{};
-    std::vector<spg_space_stats> host_ring;
+    std::mutex reading;  // held while a read uses the step's memory
 };
 
 namespace {
@@ -1165,19 +1166,21 @@ int spg_space_read_deme(spg_space *c, uint32_t species, uint32_t patch, uint32_t
     *n = o[1] - o[0];
     if (!rec && !age) return SPG_OK;
     if (capacity < *n) return fail(SPG_ERR_INVALID, "buffer holds %zu individuals, need %u", capacity, *n);
-    if (*n) {  // the deme's records and ages side by side, then to the host
+    if (*n) {
+        // the deme's records and ages side by side in memory that a step uses and
+        // that is free between steps (the pool that holds no records, the classes),
+        // then to the host; one reading thread at a time
+        const std::lock_guard<std::mutex> lock(c->reading);
         const uint32_t words = 2 * c->W;
-        const size_t rec_bytes = rec ? (size_t)*n * words * 4 : 0, bytes = rec_bytes + *n;
-        char *tmp = static_cast<char *>(c->alloc.alloc(bytes, c->stream));
-        if (!tmp) return fail(SPG_ERR_OOM, "device allocation of %zu bytes failed", bytes);
-        k_sp_gather<<<304, 256, 0, c->stream>>>(c->args, st.pool, par, o[0], words, *n,
-                                               rec ? reinterpret_cast<uint32_t *>(tmp) : nullptr,
-                                               age ? reinterpret_cast<uint8_t *>(tmp + rec_bytes) : nullptr);
+        uint32_t *r = c->args.pool[st.pool ^ 1u];
+        uint8_t *g = c->args.cls;
+        k_sp_gather<<<304, 256, 0, c->stream>>>(c->args, st.pool, par, o[0], words, *n, rec ? r : nullptr,
+                                               age ? g : nullptr);
         e = cudaGetLastError();
-        if (e == cudaSuccess && rec) e = cudaMemcpyAsync(rec, tmp, rec_bytes, cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess && age) e = cudaMemcpyAsync(age, tmp + rec_bytes, *n, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess && rec)
+            e = cudaMemcpyAsync(rec, r, (size_t)*n * words * 4, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess && age) e = cudaMemcpyAsync(age, g, *n, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        c->alloc.release(tmp, c->stream);
     }
     return e == cudaSuccess ? SPG_OK : cuda_fail(e, "read deme");
 }
