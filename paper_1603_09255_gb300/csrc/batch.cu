@@ -152,7 +152,7 @@ int configure_group(spg_batch *b, Group &g, const Shape &shape) {
     std::vector<const PopView *> views;
     views.reserve(g.members.size());
     for (uint32_t mi : g.members) views.push_back(&b->members[mi].v);
-    const int rc = build_group_launch(views, g.words, b->arena + g.table_off, g.table_bytes, g.gl);
+    const int rc = build_group_launch(views, g.words, b->arena + g.table_off, g.table_bytes, g.gl, b->stream);
     if (rc != SPG_OK) return rc;
     b->chains.clear();
     return SPG_OK;
@@ -321,7 +321,7 @@ int spg_batch_set_ecology(spg_batch *b, uint32_t member, const spg_ecology *eco)
     Member &m = b->members[member];
     if (m.prm->continuous) return SPG_OK;
     solo_args(m.v, *m.prm, m.sa);
-    return b->teams.update(&m.sa);
+    return b->teams.update(&m.sa, b->stream);
 }
 
 int spg_batch_step(spg_batch *b, uint32_t n_gen) {

@@ -563,12 +563,13 @@ int TeamSet::build(const std::vector<TeamMember> &all, const Allocator &alloc, c
     return SPG_OK;
 }
 
-// A member's changed arguments (its place in the tables stays).
-int TeamSet::update(const SoloArgs *args) {
+// A member's changed arguments (its place in the tables stays), in stream order.
+int TeamSet::update(const SoloArgs *args, cudaStream_t stream) {
     for (TeamLaunch &t : launch)
         for (size_t i = 0; i < t.members.size(); ++i)
             if (t.members[i].args == args) {
-                const cudaError_t e = cudaMemcpy(t.table + i * sizeof(SoloArgs), args, sizeof(SoloArgs), cudaMemcpyHostToDevice);
+                const cudaError_t e = cudaMemcpyAsync(t.table + i * sizeof(SoloArgs), args, sizeof(SoloArgs),
+                                                      cudaMemcpyHostToDevice, stream);
                 return e == cudaSuccess ? SPG_OK : cuda_fail(e, "update team table");
             }
     return SPG_OK;
@@ -855,7 +856,7 @@ void schedule_runs(const std::vector<uint32_t> &tiles, uint32_t G, uint32_t min_
 }
 
 int build_group_launch(const std::vector<const PopView *> &members, uint32_t words, char *table, size_t table_capacity,
-                       GenLaunch &gl) {
+                       GenLaunch &gl, cudaStream_t stream) {
     if (members.empty()) {
         gl = GenLaunch{};
         return SPG_OK;
@@ -883,11 +884,12 @@ int build_group_launch(const std::vector<const PopView *> &members, uint32_t wor
         return fail(SPG_ERR_INVALID, "launch table does not fit its buffer");
     const size_t off_buckets = align_up(segs.size() * sizeof(Segment), 256);
     const size_t off_tiles = off_buckets + align_up((size_t)buckets * 4, 256);
-    cudaError_t e = cudaMemcpy(table, segs.data(), segs.size() * sizeof(Segment), cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpyAsync(table, segs.data(), segs.size() * sizeof(Segment), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess)
-        e = cudaMemcpy(table + off_buckets, bucket_map.data(), bucket_map.size() * 4, cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(table + off_buckets, bucket_map.data(), bucket_map.size() * 4, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess)
-        e = cudaMemcpy(table + off_tiles, tile_map.data(), tile_map.size() * 4, cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(table + off_tiles, tile_map.data(), tile_map.size() * 4, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // the host tables go away
     if (e != cudaSuccess) return cuda_fail(e, "upload launch table");
     gl = GenLaunch{};
     gl.offspring = k;

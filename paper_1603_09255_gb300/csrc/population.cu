@@ -405,14 +405,16 @@ int spg_restore(spg_pop *p, const void *host, size_t bytes) {
     }
     rc = view_sync(p->view());
     if (rc != SPG_OK) return rc;
-    cudaError_t e = cudaMemcpy(p->arena + ((h.gen & 1u) ? p->L.geno1 : p->L.geno0), src + sizeof h, gbytes,
-                               cudaMemcpyHostToDevice);
+    // in the order of the population's stream, on which the kernels below read them
+    cudaError_t e = cudaMemcpyAsync(p->arena + ((h.gen & 1u) ? p->L.geno1 : p->L.geno0), src + sizeof h, gbytes,
+                                    cudaMemcpyHostToDevice, p->stream);
     if (e == cudaSuccess)
-        e = cudaMemcpy(p->arena + ((h.gen & 1u) ? p->L.surv1 : p->L.surv0), src + sizeof h + gbytes,
-                       (size_t)h.S * 4, cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(p->arena + ((h.gen & 1u) ? p->L.surv1 : p->L.surv0), src + sizeof h + gbytes,
+                            (size_t)h.S * 4, cudaMemcpyHostToDevice, p->stream);
     // per-bucket survivor counts of the replaced run must not leak into the
     // generations about to be replayed
-    if (e == cudaSuccess && !p->L.solo) e = cudaMemset(p->arena + p->L.buckets, 0, (size_t)2 * p->nbuckets * 4);
+    if (e == cudaSuccess && !p->L.solo)
+        e = cudaMemsetAsync(p->arena + p->L.buckets, 0, (size_t)2 * p->nbuckets * 4, p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "restore copy");
     if (p->L.solo) {  // the restored survivors in the slot layout: the next generation's parents
         rc = view_pack(p->view(), h.gen, reinterpret_cast<const uint32_t *>(p->arena + p->L.surv0), h.S);

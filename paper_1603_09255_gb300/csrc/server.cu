@@ -210,7 +210,7 @@ int rebuild(spg_server *s) {
             if (!s->table[gi]) return fail(SPG_ERR_OOM, "launch table allocation failed");
             s->table_cap[gi] = cap;
         }
-        rc = build_group_launch(views, words, s->table[gi], s->table_cap[gi], s->gl[gi]);
+        rc = build_group_launch(views, words, s->table[gi], s->table_cap[gi], s->gl[gi], s->stream);
         if (rc != SPG_OK) return rc;
     }
     s->dirty = false;

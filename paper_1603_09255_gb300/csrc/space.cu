@@ -1057,13 +1057,16 @@ int spg_space_create(const spg_space_desc *desc, const spg_allocator *alloc, voi
         }
     offs[c->nd] = run;
     SpState st0{0, SPG_OK, run, 0, 0, run, 0, 0};
-    e = cudaMemcpy(b + o_sp, prm.data(), sizeof(SpeciesParams) * c->ns, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(a.off[0], offs.data(), offs.size() * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(a.adults[0], adults.data(), adults.size() * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(a.state, &st0, sizeof st0, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(b + o_n0, n0.data(), 4 * c->ns, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(b + o_p0, p0.data(), 4 * c->ns, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(a.ring, 0, (size_t)c->ring_cap * c->ns * sizeof(spg_space_stats));
+    auto put = [&](void *dst, const void *src, size_t bytes) {  // in the order of the stream whose kernels read it
+        return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->stream);
+    };
+    e = put(b + o_sp, prm.data(), sizeof(SpeciesParams) * c->ns);
+    if (e == cudaSuccess) e = put(a.off[0], offs.data(), offs.size() * 4);
+    if (e == cudaSuccess) e = put(a.adults[0], adults.data(), adults.size() * 4);
+    if (e == cudaSuccess) e = put(a.state, &st0, sizeof st0);
+    if (e == cudaSuccess) e = put(b + o_n0, n0.data(), 4 * c->ns);
+    if (e == cudaSuccess) e = put(b + o_p0, p0.data(), 4 * c->ns);
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.ring, 0, (size_t)c->ring_cap * c->ns * sizeof(spg_space_stats), c->stream);
     if (e != cudaSuccess) {
         spg_space_destroy(c.release());
         return cuda_fail(e, "initialise community");

@@ -91,7 +91,7 @@ struct TeamLaunch {
 struct TeamSet {
     TeamLaunch launch[kTeamKinds];
     int build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream);  // synchronises
-    int update(const SoloArgs *args);
+    int update(const SoloArgs *args, cudaStream_t stream);
     int step(uint32_t n_gen, bool keep_last, cudaStream_t stream);
     void release(const Allocator &alloc, cudaStream_t stream);
 };
@@ -144,7 +144,7 @@ void schedule_runs(const std::vector<uint32_t> &tiles, uint32_t G, uint32_t min_
 // members (words = L / 2, the int16 records' words), uploaded into `table`
 // (device memory; synchronous), and the group's launch description.
 int build_group_launch(const std::vector<const PopView *> &members, uint32_t words, char *table, size_t table_capacity,
-                       GenLaunch &gl);
+                       GenLaunch &gl, cudaStream_t stream);
 int view_sync(const PopView &v);
 int view_state(const PopView &v, DevState &st);
 int view_set_state(const PopView &v, uint32_t gen, uint32_t S, uint32_t f, double R, int32_t status,
