@@ -73,8 +73,10 @@ __device__ __forceinline__ void load_record(const uint32_t *__restrict__ p, uint
 
 // Records of 32 bytes or more are written with 256-bit stores: one request
 // per whole sector (two 128-bit stores per sector would each touch the
-// sector half-written).  Nothing in a generation kernel reads the records it
-// writes, so the stores need no ordering against other memory operations.
+// sector half-written).  The generation kernel reads what it writes: packed
+// records as parents after the team's barrier (whose arrival releases them),
+// full records for the per-locus counts after a block barrier.  The stores
+// must stay ahead of those barriers, so the compiler may not move them.
 template <int W>
 __device__ __forceinline__ void store_record(uint32_t *__restrict__ p, const uint32_t (&r)[2 * W]) {
     if constexpr (W == 1) {
@@ -86,7 +88,8 @@ __device__ __forceinline__ void store_record(uint32_t *__restrict__ p, const uin
         for (int q = 0; q < W / 4; ++q)
             asm volatile("st.global.v8.u32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p + 8 * q), "r"(r[8 * q]),
                          "r"(r[8 * q + 1]), "r"(r[8 * q + 2]), "r"(r[8 * q + 3]), "r"(r[8 * q + 4]),
-                         "r"(r[8 * q + 5]), "r"(r[8 * q + 6]), "r"(r[8 * q + 7]));
+                         "r"(r[8 * q + 5]), "r"(r[8 * q + 6]), "r"(r[8 * q + 7])
+                         : "memory");
     }
 }
 
