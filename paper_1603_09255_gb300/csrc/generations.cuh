@@ -49,8 +49,7 @@
 // taken apart into f16 by this target: 2.4 times the instructions.)
 #pragma once
 
-#include "device_common.cuh"
-#include "ecology.cuh"
+#include "closing.cuh"
 
 namespace spg {
 namespace {
@@ -747,23 +746,6 @@ __device__ __forceinline__ void add_stats(GenAcc *acc, uint32_t warp, uint32_t l
     }
 }
 
-// The generation's totals over the accumulator's copies, by one warp: lane l
-// reads word l % 8 of copy l / 8 and returns the total of that word (words 0-5
-// sums, 6 the minimum below the maximum).
-__device__ __forceinline__ unsigned long long total_stats(const GenAcc *acc, uint32_t lane) {
-    static_assert(sizeof(GenAcc) == 64 && kGenAccCopies == 4, "a lane per word");
-    unsigned long long x = __ldcg(reinterpret_cast<const unsigned long long *>(acc) + lane);
-#pragma unroll
-    for (int o = 8; o <= 16; o <<= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, x, o);
-        if ((lane & 7u) == 6u)
-            x = (unsigned long long)(uint32_t)min((int)(uint32_t)x, (int)(uint32_t)y) |
-                (unsigned long long)(uint32_t)max((int)(x >> 32), (int)(y >> 32)) << 32;
-        else x += y;
-    }
-    return x;
-}
-
 // GENERAL: dominance, values beyond 2048 in magnitude or a bias beyond 2^30
 // (the others' instance has none of these branches in its loop).
 // Blocks 0 .. team - 1 (this one is `rank`) form n_gen generations of a
@@ -998,40 +980,8 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
         }
         wide = __syncthreads_and(wide) != 0;
         const uint32_t S_new = s_total, f_new = eco ? s_f[g & 1u] : f;
-        status = S_new == 0u ? SPG_EXTINCT : SPG_OK;
         if (rank == 0u) {
-            if (warp == NW - 1u) {
-                spg_stats *rec = a.ring + (g - 1u) % a.stats_cap;
-                if (lane == 0u) {
-                    rec->gen = g;
-                    rec->n = a.n;
-                    rec->s = S_new;
-                    rec->status = (uint32_t)status;
-                    rec->R = eco ? R : 0.0;
-                    rec->f = f_new;
-                    rec->pad = 0;
-                    rec->sum_raw = (long long)sum;
-                    st->gen = g;
-                    st->S = S_new;
-                    st->f = f_new;
-                    st->R = R;
-                    st->status = status;
-                } else if (lane < 7u) {
-                    if (lane == 1u) rec->sum_raw_surv = (long long)sum;
-                    if (lane == 2u) rec->sum_raw2 = sum;
-                    if (lane == 3u) rec->consumption = eco ? sum : 0ull;
-                    if (lane == 4u) rec->het = sum;
-                    if (lane == 5u) rec->allele = sum;
-                    if (lane == 6u) {
-                        rec->min_raw = (int)(uint32_t)sum;
-                        rec->max_raw = (int)(sum >> 32);
-                    }
-                }
-                // empty sums for the generation after next: every block has read
-                // what they held, and none adds before the next barrier
-                reinterpret_cast<unsigned long long *>(a.acc + (size_t)((g + 2u) % 3u) * kGenAccCopies)[lane] =
-                    (lane & 7u) == 6u ? kEmptyMinMax : 0ull;
-            }
+            if (warp == NW - 1u) write_state(a, lane, g, sum, S_new, R, f_new);
             if (a.locus_row[0]) {  // the counted row to its place; clear for the generation after next
                 uint32_t *row = a.locus_row[g & 1u], *dst = a.locus_ring + (size_t)((g - 1u) % a.locus_cap) * (32u * W);
                 for (uint32_t i = tid; i < 32u * W; i += BLOCK) {
@@ -1040,29 +990,10 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
                 }
             }
         }
-        if (single && S_new != 0u) {  // the ordered survivor list from the bitmap, 32 slots (of one group) a warp
-            for (uint32_t s0 = warp * 32u; s0 < a.nslots; s0 += NW * 32u) {
-                const uint32_t slot = s0 + lane;
-                uint32_t word = 0u, first = 0u;
-                if (slot < a.nslots) {
-                    word = __ldcg(a.alive + slot);
-                    first = slot * rec_slot - *reinterpret_cast<const uint32_t *>(g_smem + SM::kDir + 8u * slot + 4u);
-                }
-                for (uint32_t b = 0; b < 32u && s0 + b < a.nslots; ++b) {
-                    const uint32_t bits = __shfl_sync(0xFFFFFFFFu, word, b), at = __shfl_sync(0xFFFFFFFFu, first, b);
-                    if ((bits >> lane) & 1u) a.surv[at + __popc(bits & ((1u << lane) - 1u))] = (s0 + b) * 32u + lane;
-                }
-            }
-        } else if (list && S_new != 0u) {  // the same, a slot a warp of the team
-            for (uint32_t slot = rank * NW + warp; slot < a.nslots; slot += team * NW) {
-                uint32_t rank = slot * rec_slot - *reinterpret_cast<const uint32_t *>(g_smem + SM::kDir + 8u * slot + 4u);
-                for (uint32_t gi = 0; gi < a.slot_len && slot * rec_slot + 32u * gi < a.n; ++gi) {
-                    const uint32_t j = slot * rec_slot + 32u * gi, bits = __ldcg(a.alive + (j >> 5));
-                    if ((bits >> lane) & 1u) a.surv[rank + __popc(bits & ((1u << lane) - 1u))] = j + lane;
-                    rank += __popc(bits);
-                }
-            }
-        }
+        if (list && S_new != 0u)
+            list_survivors(a, 0u, a.nslots, rank * NW + warp, team * NW, lane, [&](uint32_t slot) {
+                return slot * rec_slot - *reinterpret_cast<const uint32_t *>(g_smem + SM::kDir + 8u * slot + 4u);
+            });
         gen = g;
         ++done;
         if (S_new == 0u) {

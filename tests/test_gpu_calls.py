@@ -1,0 +1,78 @@
+"""Calls of one generation and batches at the borders of their forms, bit for bit
+against the CPU oracle: the ordered survivor list for slots of any length, and
+members of every kind on one block or several."""
+import numpy as np
+import pytest
+
+import oracle
+import spegg_synth as S
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def gpu_lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1603_09255_gb300 import build
+    build.build()
+
+
+def spegg():
+    from paper_1603_09255_gb300 import spegg as m
+    return m
+
+
+def kinds(n, n_loci, seed):
+    """A workload of every kind of member: plain, dominance, map, weights, both,
+    and effects of two digits."""
+    def base(i):
+        return S.single_species(n=n, n_loci=n_loci, mu=1e-3, seed=seed, replicate=100 * n_loci + i)
+    import dataclasses
+    rng = np.random.default_rng(n_loci)
+    wide = dataclasses.replace(base(5), effects=rng.integers(-32768, 32768, n_loci).astype(np.int16), bias=1 << 23,
+                               shift=12)
+    wide.surv_table = S.stabilizing_table(wide.bias, wide.shift, 1e-5)
+    return [base(0), S.with_dominance(base(1)), S.with_linkage(base(2)), S.with_weights(base(3)),
+            S.with_weights(S.with_linkage(base(4))), wide]
+
+
+def assert_member(b, i, w, gens):
+    orc = oracle.OraclePopulation.from_workload(w)
+    so, sg = orc.step(gens), b.read_stats(i, 1, gens)
+    for name in so.dtype.names:
+        assert np.array_equal(so[name], sg[name]), (i, name)
+    if w.allele_model == 0:
+        assert np.array_equal(orc.genotypes(), b.genotypes(i)), i
+    else:
+        assert np.array_equal(orc.values(), b.values(i)), i
+    assert np.array_equal(orc.survivors(), b.survivors(i)), i
+    a, g = orc.state(), b.state(i)
+    for k in ("gen", "S", "status", "f", "R"):
+        assert a[k] == g[k], (i, k)
+
+
+# slots of 1 word, of several (31 and 32 words: one pass; 33: two), the last one ragged
+@pytest.mark.parametrize("n", [1000, 100_001, 2_412_480, 2_490_331, 2_490_400])
+def test_list_of_slots_of_any_length(n):
+    w = S.single_species(n=n, n_loci=32, mu=1e-3, seed=n)
+    orc = oracle.OraclePopulation.from_workload(w)
+    gpu = spegg().Population.from_workload(w, stats_capacity=4)
+    orc.step(1)
+    gpu.step(1)
+    assert np.array_equal(orc.survivors(), gpu.survivors())
+    assert np.array_equal(orc.genotypes(), gpu.genotypes())
+
+
+@pytest.mark.parametrize("sizes", [(33, 700), (5000, 40_000)])
+def test_batch_of_every_kind(sizes):
+    """Records, survivors and state of members of every kind, sizes and locus
+    counts mixed, after calls of one generation and of several."""
+    ws = [w for n in sizes for L in (32, 128, 256) for w in kinds(n + L, L, 7)]
+    b = spegg().Batch(ws, stats_capacity=8)
+    for k in (1, 1, 3):
+        b.step(k)
+    for i, w in enumerate(ws):
+        assert_member(b, i, w, 5)
