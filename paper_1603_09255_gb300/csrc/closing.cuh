@@ -10,12 +10,11 @@
 namespace spg {
 namespace {
 
-// The generation's totals over the accumulator's copies, by one warp: lane l
-// reads word l % 8 of copy l / 8 and returns the total of that word (words 0-5
-// sums, 6 the minimum below the maximum).
-__device__ __forceinline__ unsigned long long total_stats(const GenAcc *acc, uint32_t lane) {
+// The generation's totals over the accumulator's copies, by one warp: x is word
+// l % 8 of copy l / 8 in lane l, which returns the total of that word (words
+// 0-5 sums, 6 the minimum below the maximum).
+__device__ __forceinline__ unsigned long long total_stats(unsigned long long x, uint32_t lane) {
     static_assert(sizeof(GenAcc) == 64 && kGenAccCopies == 4, "a lane per word");
-    unsigned long long x = __ldcg(reinterpret_cast<const unsigned long long *>(acc) + lane);
 #pragma unroll
     for (int o = 8; o <= 16; o <<= 1) {
         const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, x, o);
@@ -71,19 +70,24 @@ __device__ __forceinline__ void write_state(const SoloArgs &a, uint32_t lane, ui
 // takes the bitmap words of several slots at once, a word per lane: a word and
 // its load at a time, a wait for L2 each, calls of one generation took 45.1 us
 // at N = 10^6 (43.1 now) and 4.43 ms for 4,096 members (3.83 now).
-template <class First>
+// ready() runs once, before the first rank is asked for, with the first words on
+// their way; false: nothing to list.
+template <class Ready, class First>
 __device__ __forceinline__ void list_survivors(const SoloArgs &a, uint32_t slot0, uint32_t slot1, uint32_t warp,
-                                               uint32_t warps, uint32_t lane, First first_rank) {
+                                               uint32_t warps, uint32_t lane, Ready ready, First first_rank) {
     const uint32_t len = a.slot_len, words = (a.n + 31u) >> 5, share = (slot1 - slot0 + warps - 1u) / warps;
     const uint32_t per = len > 32u ? 1u : min(32u / len, max(share, 1u));  // slots a pass
     const uint32_t seg = len > 32u ? 0u : min(lane / len, per), in = len > 32u ? lane : lane - seg * len;
-    for (uint32_t s = slot0 + warp * per; s < slot1; s += warps * per) {
+    auto load = [&](uint32_t slot, uint32_t c) {
+        const uint32_t q = slot * len + c + in;
+        return seg < per && slot < slot1 && c + in < len && q < words ? __ldcg(a.alive + q) : 0u;
+    };
+    uint32_t s = slot0 + warp * per, bits = load(s + seg, 0u);
+    if (!ready()) return;
+    for (; s < slot1; s += warps * per) {
         const uint32_t slot = s + seg;
-        const bool mine = seg < per && slot < slot1;
-        uint32_t before = mine ? first_rank(slot) : 0u;
+        uint32_t before = seg < per && slot < slot1 ? first_rank(slot) : 0u;
         for (uint32_t c = 0; c < len; c += 32u) {  // once, but for slots of more than 32 words
-            const uint32_t q = slot * len + c + in;
-            const uint32_t bits = mine && c + in < len && q < words ? __ldcg(a.alive + q) : 0u;
             const uint32_t own = __popc(bits);
             uint32_t at = own;
 #pragma unroll
@@ -95,11 +99,17 @@ __device__ __forceinline__ void list_survivors(const SoloArgs &a, uint32_t slot0
             at -= own;
             at += before - __shfl_sync(0xFFFFFFFFu, at, (int)min(lane - in, 31u));
             before += all;
-            const uint32_t q0 = s * len + c;  // the words of lanes 0, 1, ...
-            for (uint32_t b = 0; b < 32u && b < per * len && q0 + b < words; ++b) {
-                const uint32_t w = __shfl_sync(0xFFFFFFFFu, bits, (int)b), r = __shfl_sync(0xFFFFFFFFu, at, (int)b);
-                if ((w >> lane) & 1u) a.surv[r + __popc(w & ((1u << lane) - 1u))] = (q0 + b) * 32u + lane;
+            // the words of lanes 0, 1, ..., four at a time (one at a time waits for each)
+            const uint32_t q0 = s * len + c, m = q0 < words ? min(min(32u, per * len), words - q0) : 0u;
+            for (uint32_t b = 0; b < m; b += 4u) {
+#pragma unroll
+                for (uint32_t i = 0; i < 4u; ++i) {
+                    const uint32_t w = __shfl_sync(0xFFFFFFFFu, bits, (int)(b + i)),
+                                   r = __shfl_sync(0xFFFFFFFFu, at, (int)(b + i));
+                    if ((w >> lane) & 1u) a.surv[r + __popc(w & ((1u << lane) - 1u))] = (q0 + b + i) * 32u + lane;
+                }
             }
+            bits = c + 32u < len ? load(slot, c + 32u) : load(slot + warps * per, 0u);
         }
     }
 }

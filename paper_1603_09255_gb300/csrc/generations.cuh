@@ -121,21 +121,6 @@ __device__ __forceinline__ bool team_barrier(unsigned long long *ctr, uint32_t r
     return __syncthreads_and(threadIdx.x == 0 ? ok : 1) != 0;
 }
 
-// A call of one generation needs no block to wait: whether this block is the
-// last of the team to arrive, which closes the generation alone.
-__device__ __forceinline__ bool last_to_arrive(unsigned long long *ctr, uint32_t rank, uint32_t team) {
-    __syncthreads();
-    int last = 0;
-    if (threadIdx.x == 0) {
-        const unsigned long long add = rank == 0u ? kBarrierStep - (team - 1u) : 1ull;
-        unsigned long long old;
-        asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], %2;" : "=l"(old) : "l"(ctr), "l"(add) : "memory");
-        asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        last = (old + add) % kBarrierStep == 0ull ? 1 : 0;
-    }
-    return __syncthreads_or(threadIdx.x == 0 ? last : 0) != 0;
-}
-
 // ------------------------------------------------------- record access
 // Parents are read through L2: their buffers change during the launch.
 template <int W>
@@ -543,9 +528,10 @@ __device__ __forceinline__ void weighted_records(const SoloArgs &a, const RoundK
 // most slots).  Writes the total to *total; with no survivors the tables stay
 // as they are.  Returns whether every slot of the thread holds more ranks than
 // two guide entries span, so that a rank lies in its entry's slot or the next.
-// PER: runs of 32 slots a warp takes, at most.
-template <class SM, uint32_t PER>
-__device__ __forceinline__ bool directory_of(const uint32_t *counts, uint32_t nslots, uint32_t slot_records,
+// PER: runs of 32 slots a warp takes, at most; OWN: with one run, the count of
+// the thread's slot is `own` already.
+template <class SM, uint32_t PER, bool OWN>
+__device__ __forceinline__ bool directory_of(const uint32_t *counts, uint32_t first, uint32_t nslots, uint32_t slot_records,
                                                 uint32_t guide_bits, uint32_t *s_warp, uint32_t *total) {
     constexpr uint32_t T = SM::kThreads - 32u, NW = T / 32u;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
@@ -554,7 +540,7 @@ __device__ __forceinline__ bool directory_of(const uint32_t *counts, uint32_t ns
     uint32_t c[PER], own = 0;
 #pragma unroll
     for (uint32_t i = 0; i < PER; ++i) {
-        c[i] = i < per && s0 + 32u * i < nslots ? __ldcg(counts + s0 + 32u * i) : 0u;
+        c[i] = i < per && s0 + 32u * i < nslots ? OWN && PER == 1u ? first : __ldcg(counts + s0 + 32u * i) : 0u;
         own += c[i];
     }
     own = __reduce_add_sync(0xFFFFFFFFu, own);
@@ -606,12 +592,15 @@ __device__ __forceinline__ bool directory_of(const uint32_t *counts, uint32_t ns
     }
     return wide;
 }
-template <class SM>
-__device__ __forceinline__ bool build_directory(const uint32_t *counts, uint32_t nslots, uint32_t slot_records,
+// (Two runs a warp have an instance: as six, calls of one generation of N =
+// 20,000 took 11.4 us instead of 10.1.)
+template <class SM, bool OWN>
+__device__ __forceinline__ bool build_directory(const uint32_t *counts, uint32_t own, uint32_t nslots, uint32_t slot_records,
                                                 uint32_t guide_bits, uint32_t *s_warp, uint32_t *total) {
     constexpr uint32_t T = SM::kThreads - 32u;
-    if (nslots <= T) return directory_of<SM, 1>(counts, nslots, slot_records, guide_bits, s_warp, total);
-    return directory_of<SM, (SM::kSlots + T - 1) / T>(counts, nslots, slot_records, guide_bits, s_warp, total);
+    if (nslots <= T) return directory_of<SM, 1, OWN>(counts, own, nslots, slot_records, guide_bits, s_warp, total);
+    if (nslots <= 2u * T) return directory_of<SM, 2, OWN>(counts, own, nslots, slot_records, guide_bits, s_warp, total);
+    return directory_of<SM, (SM::kSlots + T - 1) / T, OWN>(counts, own, nslots, slot_records, guide_bits, s_warp, total);
 }
 
 // ------------------------------------------------------- per-locus counts
@@ -749,8 +738,8 @@ __device__ __forceinline__ void add_stats(GenAcc *acc, uint32_t warp, uint32_t l
 // GENERAL: dominance, values beyond 2048 in magnitude or a bias beyond 2^30
 // (the others' instance has none of these branches in its loop).
 // Blocks 0 .. team - 1 (this one is `rank`) form n_gen generations of a
-// population; keep_last: the last of them is the call's last; single: the one
-// generation of a call, closed by the last block that arrives.
+// population; keep_last: the last of them is the call's last; single: one
+// generation, closed by the kernel launched next (k_close).
 template <int W, bool LINKED, bool WEIGHTED, bool GENERAL>
 __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundKeys &keys, uint32_t n_gen,
                                                  bool keep_last, bool single, uint32_t rank, uint32_t team) {
@@ -760,7 +749,7 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
     __shared__ uint32_t s_cdf[kMaxKmax];
     __shared__ uint32_t s_scan[32];
     __shared__ uint32_t s_cnt[32 * W];
-    __shared__ uint32_t s_total, s_f[2];
+    __shared__ uint32_t s_total, s_f[2], s_now[8];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(g_smem);
     const PopParams *P = a.prm;
@@ -777,20 +766,6 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
         if (dom) cp_async_16(smem0 + SM::kFrag + SM::kTabBytes + 16u * i, a.frag->table[1] + 4u * i);
     }
     cp_async_commit();
-    griddep_wait();  // the tables are parameters: nothing an earlier launch writes
-    griddep_release();
-    // the call's starting state (written by earlier launches)
-    uint32_t gen = ld_relaxed_u32(&st->gen), f = ld_relaxed_u32(&st->f);
-    const uint32_t target = ld_relaxed_u32(&st->target);
-    int32_t status = (int32_t)ld_relaxed_u32(reinterpret_cast<const uint32_t *>(&st->status));
-    double R = ld_relaxed_f64(&st->R);
-    // one decision for the block: a teammate that gives up on a block this late
-    // may change the status between its threads' reads
-    if (__syncthreads_or(status != SPG_OK || ld_relaxed_u32(&st->S) == 0u)) {
-        cp_async_wait<0>();
-        return;
-    }
-
     if (tid < (uint32_t)kMaxKmax) s_cdf[tid] = tid < a.kmax ? P->cdf[tid] : 0xFFFFFFFFu;
     LinkMap lk{};
     if constexpr (LINKED) {
@@ -804,6 +779,30 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
         lk = LinkMap{cdf, cum, gd, first, lp->kmax,
                      reinterpret_cast<uint32_t *>(g_smem + SM::kStage + warp * SM::kPerWarp)};
     }
+    griddep_wait();  // the tables are parameters: nothing an earlier launch writes
+    griddep_release();
+    // the call's starting state (written by earlier launches): read once for the
+    // block -- by every thread, it kept one line of L2 busy for microseconds, and a
+    // teammate that gives up on a block this late may change the status meanwhile
+    static_assert(offsetof(DevState, S) == 4 && offsetof(DevState, f) == 8 && offsetof(DevState, status) == 12 &&
+                      offsetof(DevState, R) == 16 && offsetof(DevState, target) == 28,
+                  "the state's first eight words");
+    if (tid < 8u && tid != 6u) s_now[tid] = ld_relaxed_u32(reinterpret_cast<const uint32_t *>(st) + tid);
+    // survivors of the thread's first slot, of both parities, so that the load
+    // does not wait for the state
+    const uint32_t own0 = tid < a.nslots ? __ldcg(a.counts[0] + tid) : 0u,
+                   own1 = tid < a.nslots ? __ldcg(a.counts[1] + tid) : 0u;
+    __syncthreads();
+    uint32_t gen = s_now[0], f = s_now[2];
+    const uint32_t target = s_now[7];
+    double R = __hiloint2double((int)s_now[5], (int)s_now[4]);
+    const bool over = (int32_t)s_now[3] != SPG_OK || s_now[1] == 0u || gen >= target;
+    if (single && rank == 0u && tid == 0u) st->done = over ? 0u : gen + 1u;  // the generation to be closed
+    if (over) {
+        cp_async_wait<0>();
+        return;
+    }
+
     const uint32_t rep = a.rep, k0 = keys[0], k1 = keys[1];
     const uint32_t rec_slot = a.slot_len * 32u;
     const uint32_t stage = smem0 + SM::kStage + warp * SM::kPerWarp, my_row = stage + stage_row(lane);
@@ -811,7 +810,8 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
     const uint32_t slot1 = (uint32_t)(((unsigned long long)a.nslots * (rank + 1u)) / team);
     bool one_step = true;
     if (warp + 1u < NW)
-        one_step = build_directory<SM>(a.counts[gen & 1u], a.nslots, rec_slot, a.guide_bits, s_scan, &s_total);
+        one_step = build_directory<SM, true>(a.counts[gen & 1u], (gen & 1u) ? own1 : own0, a.nslots, rec_slot,
+                                             a.guide_bits, s_scan, &s_total);
     cp_async_wait<0>();  // the tables have landed meanwhile
     one_step = __syncthreads_and(one_step) != 0;
     uint32_t S = s_total;
@@ -955,11 +955,8 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
         __syncthreads();
         GenAcc *acc = a.acc + (size_t)(g % 3u) * kGenAccCopies;
         add_stats<SM>(acc + rank % kGenAccCopies, warp, lane);
-        if (single) {
-            if (!last_to_arrive(a.barrier, rank, team)) return;
-            rank = 0u;  // the rest is this block's alone
-            team = 1u;
-        } else if (!team_barrier(a.barrier, rank, team, a.barrier_tries)) {  // the generation fails: every block gives up
+        if (single) return;
+        if (!team_barrier(a.barrier, rank, team, a.barrier_tries)) {  // the generation fails: every block gives up
             if (tid == 0u) atomicExch(reinterpret_cast<int *>(&st->status), SPG_ERR_TIMEOUT);
             return;
         }
@@ -969,9 +966,9 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
         bool wide = true;
         unsigned long long sum = 0;
         if (warp + 1u < NW) {
-            wide = build_directory<SM>(a.counts[g & 1u], a.nslots, rec_slot, a.guide_bits, s_scan, &s_total);
+            wide = build_directory<SM, false>(a.counts[g & 1u], 0u, a.nslots, rec_slot, a.guide_bits, s_scan, &s_total);
         } else if (eco || rank == 0u) {
-            sum = total_stats(acc, lane);
+            sum = total_stats(__ldcg(reinterpret_cast<const unsigned long long *>(acc) + lane), lane);
             const unsigned long long cons = __shfl_sync(0xFFFFFFFFu, sum, 3);
             if (lane == 0u && eco) {
                 R = resource_eaten(grown, cons);
@@ -991,7 +988,7 @@ __device__ __forceinline__ void form_generations(const SoloArgs &a, const RoundK
             }
         }
         if (list && S_new != 0u)
-            list_survivors(a, 0u, a.nslots, rank * NW + warp, team * NW, lane, [&](uint32_t slot) {
+            list_survivors(a, 0u, a.nslots, rank * NW + warp, team * NW, lane, [] { return true; }, [&](uint32_t slot) {
                 return slot * rec_slot - *reinterpret_cast<const uint32_t *>(g_smem + SM::kDir + 8u * slot + 4u);
             });
         gen = g;

@@ -4,7 +4,7 @@
 // A population owns one device arena (parameters, state, statistics ring,
 // accumulators, genotypes, survivors).  The generations of a biallelic
 // population are formed by one cooperative launch per call (of at most
-// kSoloLaunchGens); those of continuous allelic values are enqueued as a
+// kSoloLaunchGens; two plain ones for a call of one generation); those of continuous allelic values are enqueued as a
 // cached CUDA graph of kGraphChunk generations (two launches each), whose
 // arguments are identical because buffers are chosen on the device by
 // generation parity.
@@ -76,7 +76,8 @@ int configure_solo(spg_pop *p, const Shape &shape) {
     SoloArgs &a = p->sa;
     solo_args(p->view(), prm, a);
     SoloKernel k = solo_kernel(p->words, prm.linked != 0u, prm.weighted != 0u, a.dom || a.two_digits || !a.narrow_bias);
-    const int rc = prepare_solo(k);
+    int rc = prepare_solo(k);
+    if (rc == SPG_OK) rc = prepare_close();
     if (rc != SPG_OK) return fail(rc, "generation kernel setup failed");
     p->solo = k;
     p->shape = shape;
@@ -85,42 +86,70 @@ int configure_solo(spg_pop *p, const Shape &shape) {
     return SPG_OK;
 }
 
-// Largest population whose calls of one generation take the form without a
-// grid barrier, closed by the last block: calls back to back, with the barrier
-// and without, us: N = 1,000 10.3 / 9.2, 3,000 10.3 / 9.2, 10,000 10.8 / 10.4,
-// 20,000 14.3 / 15.0 (one block writes the survivor list), 77,000 14.4 / 22.5.
-// (Fewer blocks for such a call gain nothing in either form.)
-constexpr uint32_t kMostSingle = 16384;
+// Blocks of a launch that forms one generation for k_close to close: four warps
+// of work each up to 32 of them (N = 1,000: 7.5 us a call with 8 blocks, 8.1 with
+// 2), then eight (N = 10,000: 8.4 us with 39 blocks, 9.4 with 78), and at most
+// half of those the device holds while each warp has one slot, so that the next
+// call's launch can load its tables beside this one (N = 30,000: 10.1 us with 76
+// blocks, 11.0 with 117).
+uint32_t single_blocks(uint32_t nslots, uint32_t resident) {
+    const uint32_t half = std::max(resident / 2u, 1u), blocks = std::max(nslots / 8u, std::min(nslots / 4u, 32u));
+    return std::max(1u, std::min(blocks, nslots <= half * (kSoloThreads / 32u) ? half : resident));
+}
 
-// n_gen generations: one cooperative launch per kSoloLaunchGens of them (the
-// blocks meet at a grid barrier, so all must be resident).  Where no block
-// waits for another, a launch may start while its predecessor finishes (N =
-// 300, calls of one generation: 8.3 -> 6.3 us).
+// Slots that a block of k_close lists: 64 bitmap words (16 and 32 are slower at
+// N = 20,000, 9.5 us a call against 8.9; 128 at most sizes), or as many as spread
+// the words over the device.
+uint32_t close_slots(const spg_pop *p) {
+    const uint32_t words = (p->n + 31u) / 32u, most = std::max(64u, (words + p->solo.resident - 1u) / p->solo.resident);
+    return std::min(256u, (most + p->sa.slot_len - 1u) / p->sa.slot_len);
+}
+
+int launch_solo(spg_pop *p, const SoloArgs &args, const void *fn, uint32_t blocks, uint32_t threads, uint32_t smem,
+                bool waits) {
+    SoloArgs a = args;
+    void *params[] = {&a};
+    cudaLaunchAttribute attr{};
+    if (waits) {  // blocks meet at a barrier, so all must be resident
+        attr.id = cudaLaunchAttributeCooperative;
+        attr.val.cooperative = 1;
+    } else {      // its tables may load while its predecessor finishes (N = 300, one generation a call: 8.3 -> 6.5 us)
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = p->stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, params);
+    return e == cudaSuccess ? SPG_OK : cuda_fail(e, "generation launch");
+}
+
+// n_gen generations: one cooperative launch per kSoloLaunchGens of them.  A call
+// of one generation is two launches without a barrier instead, which may start
+// while their predecessors finish, as a cooperative one cannot: back to back,
+// with the barrier / without, us a call: N = 3,000 10.3 / 7.8, 30,000 14.4 / 9.6,
+// 10^5 16.5 / 13.8, 10^6 43.1 / 41.1.  (Two generations are no faster in pairs:
+// N = 3,000 14.4 / 15.6, 30,000 16.5 / 19.2.)
 int enqueue_solo(spg_pop *p, uint32_t n_gen) {
+    SoloArgs a = p->sa;
+    if (n_gen == 1u && p->solo_blocks > 1u) {
+        a.n_gen = a.keep_last = a.single = 1u;
+        a.close_slots = close_slots(p);
+        const int rc = launch_solo(p, a, p->solo.fn, single_blocks(a.nslots, p->solo.resident), kSoloThreads, p->solo.smem, false);
+        if (rc != SPG_OK) return rc;
+        return launch_solo(p, a, close_kernel(), (a.nslots + a.close_slots - 1u) / a.close_slots, kCloseThreads, kCloseSmem,
+                           false);
+    }
     for (uint32_t done = 0; done < n_gen;) {
-        SoloArgs a = p->sa;
         a.n_gen = std::min(n_gen - done, kSoloLaunchGens);
         done += a.n_gen;
         a.keep_last = done == n_gen ? 1u : 0u;
-        a.single = n_gen == 1u && p->solo_blocks > 1u && p->n <= kMostSingle ? 1u : 0u;
-        void *params[] = {&a};
-        cudaLaunchAttribute attr{};
-        if (p->solo_blocks == 1u || a.single) {  // no block waits: its tables may load while its predecessor finishes
-            attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr.val.programmaticStreamSerializationAllowed = 1;
-        } else {
-            attr.id = cudaLaunchAttributeCooperative;
-            attr.val.cooperative = 1;
-        }
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(p->solo_blocks);
-        cfg.blockDim = dim3(kSoloThreads);
-        cfg.dynamicSmemBytes = p->solo.smem;
-        cfg.stream = p->stream;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        const cudaError_t e = cudaLaunchKernelExC(&cfg, p->solo.fn, params);
-        if (e != cudaSuccess) return cuda_fail(e, "generation launch");
+        const int rc = launch_solo(p, a, p->solo.fn, p->solo_blocks, kSoloThreads, p->solo.smem, p->solo_blocks > 1u);
+        if (rc != SPG_OK) return rc;
     }
     return SPG_OK;
 }

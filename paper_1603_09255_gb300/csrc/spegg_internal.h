@@ -107,7 +107,8 @@ struct alignas(16) DevState {
     uint32_t f;       // resource factor applied to the next generation
     int32_t status;   // SPG_OK or SPG_EXTINCT
     double R;         // resource density
-    uint32_t done;    // compaction buckets of the running generation that have finished
+    uint32_t done;    // compaction buckets of the running generation that have finished;
+                      // biallelic: the generation that k_close has to close, or 0
     uint32_t target;  // generations stop once gen reaches target (0xFFFFFFFF: never)
     // the generation being closed: computed while its survivors are being
     // compacted, committed by the block that finishes the last bucket
@@ -215,7 +216,8 @@ struct alignas(16) SoloArgs {
     uint32_t dom, two_digits;          // fragments: dominance, values beyond 2048 in magnitude
     uint32_t n_gen;                    // generations of this launch
     uint32_t keep_last;                // the last of them is the call's last
-    uint32_t single;                   // a call of one generation: no grid barrier
+    uint32_t single;                   // one generation without a grid barrier: k_close closes it
+    uint32_t close_slots;              // slots whose survivors a block of k_close lists, at most 256
     uint32_t barrier_tries;            // polls of a wait before it gives up
 };
 struct SoloKernel {
@@ -223,6 +225,10 @@ struct SoloKernel {
     uint32_t smem = 0, resident = 0;  // resident: blocks on the device at a time
 };
 SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted, bool general);
+const void *close_kernel();  // k_close
+int prepare_close();         // sets its shared-memory limit
+constexpr uint32_t kCloseThreads = 256 + 32;  // + one warp that closes the generation
+constexpr uint32_t kCloseSmem = 120000;  // not used: keeps its blocks on an SM each
 int prepare_solo(SoloKernel &k);  // sets the shared-memory limit, fills `resident`
 
 // Several populations in one launch (k_teams): block b works through places

@@ -66,6 +66,60 @@ def test_list_of_slots_of_any_length(n):
     assert np.array_equal(orc.genotypes(), gpu.genotypes())
 
 
+def assert_population(gpu, orc, so, gens):
+    sg = gpu.read_stats(1, gens)
+    for name in so.dtype.names:
+        assert np.array_equal(so[name], sg[name]), name
+    assert np.array_equal(orc.genotypes(), gpu.genotypes())
+    assert np.array_equal(orc.survivors(), gpu.survivors())
+    a, g = orc.state(), gpu.state()
+    for k in ("gen", "S", "status", "f", "R"):
+        assert a[k] == g[k], k
+
+
+@pytest.mark.parametrize("kind", range(6))
+@pytest.mark.parametrize("n", [513, 15_361, 30_721, 77_825])
+def test_one_generation_calls_of_every_kind(n, kind):
+    """Calls of one generation, among longer ones, of every kind of population,
+    with one, two and six runs of slots in the directory and slots of two words."""
+    L = (32, 64, 128, 256)[(kind + n) % 4]
+    w = kinds(n, L, 11)[kind]
+    orc = oracle.OraclePopulation.from_workload(w)
+    gpu = spegg().Population.from_workload(w, stats_capacity=8)
+    for k in (1, 1, 2, 1):
+        gpu.step(k)
+    assert_population(gpu, orc, orc.step(5), 5)
+
+
+@pytest.mark.parametrize("n", [700, 40_000])
+def test_one_generation_calls_with_a_drawn_growth_rate(n):
+    w = S.with_beverton_holt(S.consumer_resource(n=n, n_loci=64, K=50.0 * n, mu=1e-3, seed=n))
+    orc = oracle.OraclePopulation.from_workload(w)
+    gpu = spegg().Population.from_workload(w, stats_capacity=16)
+    for _ in range(9):
+        gpu.step(1)
+    assert_population(gpu, orc, orc.step(9), 9)
+
+
+@pytest.mark.parametrize("n", [400, 3000, 30_000])
+def test_one_generation_call_under_stream_capture(n):
+    w = S.single_species(n=n, n_loci=64, mu=1e-3, seed=8)
+    stream = torch.cuda.Stream()
+    gpu = spegg().Population.from_workload(w, stats_capacity=16, stream=stream)
+    gpu.step(1)
+    gpu.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        gpu.step(1)
+        gpu.step(1)
+    with torch.cuda.stream(stream):
+        for _ in range(3):
+            graph.replay()
+    gpu.step(1)
+    orc = oracle.OraclePopulation.from_workload(w)
+    assert_population(gpu, orc, orc.step(8), 8)
+
+
 @pytest.mark.parametrize("sizes", [(33, 700), (5000, 40_000)])
 def test_batch_of_every_kind(sizes):
     """Records, survivors and state of members of every kind, sizes and locus
