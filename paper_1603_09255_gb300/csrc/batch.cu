@@ -3,7 +3,7 @@
 //
 // The biallelic members are formed by teams of blocks (TeamSet: one
 // cooperative launch per kind -- plain, general values, linkage map, parent
-// weights, both -- and call).  Continuous members are grouped by locus count: a
+// weights, both -- and call, the kinds side by side).  Continuous members are grouped by locus count: a
 // group's members are the segments of one launch, every generation is one
 // offspring launch and one compaction launch per group, the groups' chains are
 // independent branches of one CUDA graph (so groups overlap on the GPU), and
@@ -111,6 +111,8 @@ struct spg_batch {
     bool own_stream = false;
     std::map<uint32_t, std::unique_ptr<MultiChain>> chains;  // by length
     TeamSet teams;              // the biallelic members
+    cudaStream_t side = nullptr;                     // the continuous members' launches
+    cudaEvent_t forked = nullptr, joined = nullptr;
     char *locus_mem = nullptr;  // per-locus counts: every biallelic member's ring and two rows
     bool locus_on = false;
 };
@@ -123,7 +125,7 @@ std::vector<TeamMember> team_members(spg_batch *b, const std::vector<uint32_t> &
     for (uint32_t mi : list) {
         const Member &m = b->members[mi];
         if (m.prm->continuous) continue;
-        out.push_back(TeamMember{&m.sa, m.v.n, m.v.words, m.prm->linked != 0u, m.prm->weighted != 0u});
+        out.push_back(team_member(m.sa, m.prm->linked != 0u, m.prm->weighted != 0u));
     }
     return out;
 }
@@ -131,16 +133,22 @@ std::vector<TeamMember> team_members(spg_batch *b, const std::vector<uint32_t> &
 // (Re)build the team tables of all biallelic members (synchronous upload).
 int configure_teams(spg_batch *b) {
     std::vector<uint32_t> all;
+    double beside = 0.0;  // the continuous members' work
+    uint32_t beside_blocks = 0;
     for (uint32_t i = 0; i < (uint32_t)b->members.size(); ++i) {
         Member &m = b->members[i];
-        if (m.prm->continuous) continue;
+        if (m.prm->continuous) {
+            beside += continuous_work(m.v.n, m.prm->n_loci);
+            beside_blocks += continuous_blocks(m.v.n);
+            continue;
+        }
         solo_args(m.v, *m.prm, m.sa);
         for (uint32_t k = 0; k < 2; ++k) m.sa.locus_row[k] = b->locus_on ? m.locus.acc + (size_t)k * 32u * m.v.words : nullptr;
         m.sa.locus_ring = m.locus.ring;
         m.sa.locus_cap = m.locus.cap;
         all.push_back(i);
     }
-    return b->teams.build(team_members(b, all), b->alloc, b->stream);
+    return b->teams.build(team_members(b, all), b->alloc, b->stream, beside, beside_blocks);
 }
 
 // A group's launch shape: the continuous-allele kernel's launch table
@@ -171,7 +179,7 @@ int member_view(spg_batch *b, uint32_t member, PopView &v) {
     return SPG_OK;
 }
 
-int run_chunk(spg_batch *b, uint32_t len) {
+int run_chunk(spg_batch *b, uint32_t len, cudaStream_t stream) {
     auto it = b->chains.find(len);
     if (it == b->chains.end()) {
         std::unique_ptr<MultiChain> c(new (std::nothrow) MultiChain());
@@ -180,7 +188,7 @@ int run_chunk(spg_batch *b, uint32_t len) {
         if (rc != SPG_OK) return rc;
         it = b->chains.emplace(len, std::move(c)).first;
     }
-    const cudaError_t e = cudaGraphLaunch(it->second->exec, b->stream);
+    const cudaError_t e = cudaGraphLaunch(it->second->exec, stream);
     return e == cudaSuccess ? SPG_OK : cuda_fail(e, "cudaGraphLaunch");
 }
 
@@ -260,6 +268,15 @@ int spg_batch_create(const spg_pop_desc *descs, uint32_t count, const spg_alloca
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamCreate");
         b->own_stream = true;
     }
+    if (any_continuous(b.get())) {
+        cudaError_t e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->joined, cudaEventDisableTiming);
+        if (e != cudaSuccess) {
+            spg_batch_destroy(b.release());
+            return cuda_fail(e, "continuous members' stream");
+        }
+    }
     b->arena = static_cast<char *>(b->alloc.alloc(b->arena_bytes, b->stream));
     if (!b->arena) {
         spg_batch_destroy(b.release());
@@ -327,14 +344,18 @@ int spg_batch_set_ecology(spg_batch *b, uint32_t member, const spg_ecology *eco)
 int spg_batch_step(spg_batch *b, uint32_t n_gen) {
     if (!b) return fail(SPG_ERR_INVALID, "batch is NULL");
     if (n_gen == 0) return SPG_OK;
-    const int rc = b->teams.step(n_gen, true, b->stream);
-    if (rc != SPG_OK || !any_continuous(b)) return rc;
-    for (uint32_t i = 0; i + kGraphChunk <= n_gen; i += kGraphChunk) {
-        const int rc2 = run_chunk(b, kGraphChunk);
-        if (rc2 != SPG_OK) return rc2;
-    }
-    if (n_gen % kGraphChunk) return run_chunk(b, n_gen % kGraphChunk);
-    return SPG_OK;
+    if (!any_continuous(b)) return b->teams.step(n_gen, true, b->stream);
+    // the continuous members beside the others, on a stream of their own
+    cudaError_t e = cudaEventRecord(b->forked, b->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->forked, 0);
+    if (e != cudaSuccess) return cuda_fail(e, "fork continuous members");
+    int rc = b->teams.step(n_gen, true, b->stream);
+    for (uint32_t i = 0; i + kGraphChunk <= n_gen && rc == SPG_OK; i += kGraphChunk) rc = run_chunk(b, kGraphChunk, b->side);
+    if (rc == SPG_OK && n_gen % kGraphChunk) rc = run_chunk(b, n_gen % kGraphChunk, b->side);
+    e = cudaEventRecord(b->joined, b->side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->joined, 0);
+    if (rc == SPG_OK && e != cudaSuccess) return cuda_fail(e, "join continuous members");
+    return rc;
 }
 
 int spg_batch_set_tiling(spg_batch *b, uint32_t n_loci, uint32_t items) {
@@ -541,12 +562,16 @@ uint32_t spg_batch_size(const spg_batch *b) { return b ? (uint32_t)b->members.si
 void spg_batch_destroy(spg_batch *b) {
     if (!b) return;
     if (b->stream) cudaStreamSynchronize(b->stream);
+    if (b->side) cudaStreamSynchronize(b->side);
     b->chains.clear();
     b->teams.release(b->alloc, b->stream);
     if (b->locus_mem) b->alloc.release(b->locus_mem, b->stream);
     if (b->arena) b->alloc.release(b->arena, b->stream);
     if (b->stream) cudaStreamSynchronize(b->stream);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
+    if (b->side) cudaStreamDestroy(b->side);
+    if (b->forked) cudaEventDestroy(b->forked);
+    if (b->joined) cudaEventDestroy(b->joined);
     delete b;
 }
 

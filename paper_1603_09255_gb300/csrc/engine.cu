@@ -442,11 +442,23 @@ uint32_t most_blocks(uint32_t n, uint32_t resident) {
 // ------------------------------------------------------------ teams
 // Cycles of a generation on k blocks of 16 warps: closing it alone or with a
 // barrier, and rounds of the warps' groups (measured, L = 32 .. 256; a linkage
-// map or parent weights make a round longer).
+// map, parent weights and general values make a round longer: 10^6 x 128 takes
+// 75, 48 and 31 us a generation, plain 26).
 static double round_cycles(const TeamMember &m) {
     const double plain = m.words == 1 ? 2000.0 : m.words == 2 ? 2300.0 : m.words == 4 ? 3100.0 : 5400.0;
-    return plain * (m.linked ? 4.0 : 1.0) * (m.weighted ? 1.9 : 1.0);
+    return plain * (m.linked ? 3.0 : 1.0) * (m.weighted ? 1.9 : 1.0) * (m.general ? 1.2 : 1.0);
 }
+TeamMember team_member(const SoloArgs &a, bool linked, bool weighted) {
+    TeamMember m;
+    m.args = &a;
+    m.n = a.n;
+    m.words = a.words;
+    m.linked = linked;
+    m.weighted = weighted;
+    m.general = a.dom || a.two_digits || !a.narrow_bias;
+    return m;
+}
+static double block_work(const TeamMember &m) { return ((double)m.n + 31.0) / 32.0 / 16.0 * round_cycles(m); }
 static double team_cycles(const TeamMember &m, uint32_t k) {
     const double groups = ((double)m.n + 31.0) / 32.0;
     return (k == 1 ? 6000.0 : 11000.0) + std::max(1.0, groups / (16.0 * k)) * round_cycles(m);
@@ -475,7 +487,7 @@ double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, s
     double total = 0.0;
     for (uint32_t m = 0; m < M; ++m) {
         order[m] = m;
-        work[m] = ((double)members[m].n + 31.0) / 32.0 / 16.0 * round_cycles(members[m]);
+        work[m] = block_work(members[m]);
         total += work[m];
     }
     std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
@@ -517,27 +529,99 @@ double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, s
     return std::max(best, 0.0);
 }
 
-int TeamSet::build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream) {
+// SM cycles of a generation of continuous values (92, 143, 234 and 472 us at N =
+// 10^6 for L = 32 .. 256), and the SMs it fills: four blocks of 256 each.
+double continuous_work(uint32_t n, uint32_t n_loci) {
+    return (double)n * (n_loci == 32 ? 29.0 : n_loci == 64 ? 45.0 : n_loci == 128 ? 74.0 : 148.0);
+}
+uint32_t continuous_blocks(uint32_t n) { return (uint32_t)(((uint64_t)n + 1023u) / 1024u); }
+
+// `blocks` blocks dealt to several kinds by their work, each at least one and at
+// most as many as it can use.
+std::vector<uint32_t> deal_blocks(const std::vector<double> &work, const std::vector<uint32_t> &most, uint32_t blocks) {
+    std::vector<uint32_t> got(work.size(), 0u);
+    uint32_t left = blocks;
+    for (size_t k = 0; k < work.size(); ++k)
+        if (work[k] > 0.0 && left) {
+            got[k] = 1u;
+            --left;
+        }
+    for (; left; --left) {  // the next block to the kind with the most work per block
+        size_t next = work.size();
+        for (size_t k = 0; k < work.size(); ++k)
+            if (got[k] && got[k] < most[k] && (next == work.size() || work[k] * got[next] > work[next] * got[k])) next = k;
+        if (next == work.size()) break;
+        ++got[next];
+    }
+    return got;
+}
+
+// Kinds need kernels of their own (bodies of all kinds in one kernel take minutes
+// to compile and spill), and a launch of a kind with few members leaves most
+// blocks idle.  So the blocks are dealt to the kinds and their launches run side
+// by side, unless the kinds one after the other, each on all blocks, are
+// estimated to be faster.
+int TeamSet::build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream, double kept,
+                   uint32_t kept_blocks) {
+    std::vector<double> work(kTeamKinds + 1u, 0.0);
+    std::vector<uint32_t> most(kTeamKinds + 1u, 0u);
+    uint32_t kinds = 0, resident = 0;
+    for (TeamLaunch &t : launch) t.members.clear();
+    for (const TeamMember &m : all) launch[team_kind(m.linked, m.weighted, m.general)].members.push_back(m);
     for (uint32_t kind = 0; kind < kTeamKinds; ++kind) {
         TeamLaunch &t = launch[kind];
-        t.members.clear();
-        for (const TeamMember &m : all)
-            if (team_kind(m.linked, m.weighted, m.args->dom || m.args->two_digits || !m.args->narrow_bias) == kind)
-                t.members.push_back(m);
         if (t.members.empty()) continue;
         if (!t.kernel.fn) {
             t.kernel = team_kernel(kind);
             const int rc = prepare_solo(t.kernel);
             if (rc != SPG_OK) return fail(rc, "team kernel setup failed");
         }
-        std::vector<TeamPlace> places;
-        std::vector<uint32_t> block_places;
-        t.cycles = schedule_teams(t.members, t.kernel.resident, places, block_places);
+        ++kinds;
+        resident = resident ? std::min(resident, t.kernel.resident) : t.kernel.resident;
+        for (const TeamMember &m : t.members) {
+            work[kind] += block_work(m);
+            most[kind] = std::min(t.kernel.resident, most[kind] + most_blocks(m.n, t.kernel.resident));
+        }
+    }
+    work[kTeamKinds] = kept;
+    most[kTeamKinds] = kept_blocks;
+    const std::vector<uint32_t> dealt = deal_blocks(work, most, resident);
+    const uint32_t mine = resident - (kinds ? std::min(dealt[kTeamKinds], resident - 1u) : 0u);
+    std::vector<TeamPlace> places[2][kTeamKinds];
+    std::vector<uint32_t> starts[2][kTeamKinds];
+    double cycles[2][kTeamKinds] = {}, total[2] = {0.0, 0.0};  // one after the other, side by side
+    for (uint32_t kind = 0; kind < kTeamKinds; ++kind) {
+        const TeamLaunch &t = launch[kind];
+        if (t.members.empty()) continue;
+        cycles[0][kind] = schedule_teams(t.members, mine, places[0][kind], starts[0][kind]);
+        total[0] += cycles[0][kind];
+        if (kinds > 1u && kinds <= mine) {
+            cycles[1][kind] = schedule_teams(t.members, dealt[kind], places[1][kind], starts[1][kind]);
+            total[1] = std::max(total[1], cycles[1][kind]);
+        }
+    }
+    beside = kinds > 1u && kinds <= mine && total[1] < total[0];
+    if (beside && !forked && cudaEventCreateWithFlags(&forked, cudaEventDisableTiming) != cudaSuccess)
+        return fail(SPG_ERR_CUDA, "cudaEventCreate");
+    uint32_t first = kTeamKinds;  // stays on the caller's stream
+    for (uint32_t kind = 0; kind < kTeamKinds; ++kind) {
+        TeamLaunch &t = launch[kind];
+        if (t.members.empty()) continue;
+        first = std::min(first, kind);
+        const std::vector<TeamPlace> &place = places[beside ? 1 : 0][kind];
+        const std::vector<uint32_t> &start = starts[beside ? 1 : 0][kind];
+        t.blocks = beside ? dealt[kind] : mine;
+        t.cycles = cycles[beside ? 1 : 0][kind];
+        if (beside && first != kind && !t.side) {
+            cudaError_t e = cudaStreamCreateWithFlags(&t.side, cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t.joined, cudaEventDisableTiming);
+            if (e != cudaSuccess) return cuda_fail(e, "team streams");
+        }
         const size_t o_places = align_up(t.members.size() * sizeof(SoloArgs), 256),
-                     o_blocks = align_up(o_places + places.size() * sizeof(TeamPlace), 256),
-                     need = o_blocks + block_places.size() * 4;
+                     o_blocks = align_up(o_places + place.size() * sizeof(TeamPlace), 256),
+                     need = o_blocks + start.size() * 4;
         if (need > t.capacity) {
-            t.release(alloc, stream);
+            if (t.table) alloc.release(t.table, stream);
             t.capacity = 2 * need;  // (a server's set changes)
             t.table = static_cast<char *>(alloc.alloc(t.capacity, stream));
             if (!t.table) {
@@ -549,11 +633,10 @@ int TeamSet::build(const std::vector<TeamMember> &all, const Allocator &alloc, c
         for (const TeamMember &m : t.members) args.push_back(*m.args);
         cudaError_t e = cudaMemcpyAsync(t.table, args.data(), args.size() * sizeof(SoloArgs), cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(t.table + o_places, places.data(), places.size() * sizeof(TeamPlace),
-                                cudaMemcpyHostToDevice, stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(t.table + o_blocks, block_places.data(), block_places.size() * 4, cudaMemcpyHostToDevice,
+            e = cudaMemcpyAsync(t.table + o_places, place.data(), place.size() * sizeof(TeamPlace), cudaMemcpyHostToDevice,
                                 stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(t.table + o_blocks, start.data(), start.size() * 4, cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // the host tables go away
         if (e != cudaSuccess) return cuda_fail(e, "upload team table");
         t.args.members = reinterpret_cast<const SoloArgs *>(t.table);
@@ -578,31 +661,51 @@ int TeamSet::update(const SoloArgs *args, cudaStream_t stream) {
 // n_gen generations of every member.  A launch is cut at about a quarter of a
 // second, so that a team's blocks never wait long for one another.
 int TeamSet::step(uint32_t n_gen, bool keep_last, cudaStream_t stream) {
+    cudaError_t e = beside ? cudaEventRecord(forked, stream) : cudaSuccess;
+    bool first = true;  // the first kind stays on the caller's stream
     for (TeamLaunch &t : launch) {
         if (t.members.empty()) continue;
+        cudaStream_t s = beside && !first ? t.side : stream;
+        if (e == cudaSuccess && s != stream) e = cudaStreamWaitEvent(s, forked, 0);
         const uint32_t most = (uint32_t)std::max(1.0, std::min<double>(kSoloLaunchGens, 5e8 / std::max(1.0, t.cycles)));
-        for (uint32_t done = 0; done < n_gen;) {
+        for (uint32_t done = 0; done < n_gen && e == cudaSuccess;) {
             TeamArgs a = t.args;
             a.n_gen = std::min(n_gen - done, most);
             done += a.n_gen;
             a.keep_last = keep_last && done == n_gen ? 1u : 0u;
             void *params[] = {&a};
-            const cudaError_t e = cudaLaunchCooperativeKernel(t.kernel.fn, dim3(t.kernel.resident), dim3(kSoloThreads),
-                                                              params, t.kernel.smem, stream);
-            if (e != cudaSuccess) return cuda_fail(e, "team launch");
+            e = cudaLaunchCooperativeKernel(t.kernel.fn, dim3(t.blocks), dim3(kSoloThreads), params, t.kernel.smem, s);
         }
+        if (e == cudaSuccess && s != stream) e = cudaEventRecord(t.joined, s);
+        if (e != cudaSuccess) return cuda_fail(e, "team launch");
+        first = false;
+    }
+    first = true;
+    for (TeamLaunch &t : launch) {
+        if (!beside || t.members.empty()) continue;
+        if (!first && (e = cudaStreamWaitEvent(stream, t.joined, 0)) != cudaSuccess) return cuda_fail(e, "join teams");
+        first = false;
     }
     return SPG_OK;
 }
 
 void TeamLaunch::release(const Allocator &alloc, cudaStream_t stream) {
     if (table) alloc.release(table, stream);
+    if (side) {
+        cudaStreamSynchronize(side);  // (a launch that an error left unjoined)
+        cudaStreamDestroy(side);
+    }
+    if (joined) cudaEventDestroy(joined);
     table = nullptr;
     capacity = 0;
+    side = nullptr;
+    joined = nullptr;
 }
 
 void TeamSet::release(const Allocator &alloc, cudaStream_t stream) {
     for (TeamLaunch &t : launch) t.release(alloc, stream);
+    if (forked) cudaEventDestroy(forked);
+    forked = nullptr;
 }
 
 Segment segment_at(char *base, const PopLayout &L, uint32_t n, uint32_t ntiles, uint32_t tile_begin,

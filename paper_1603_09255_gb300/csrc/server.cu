@@ -181,12 +181,18 @@ int rebuild(spg_server *s) {
     int rc = server_sync(s);
     if (rc != SPG_OK) return rc;
     std::vector<TeamMember> members;
+    double beside = 0.0;  // the continuous jobs' work
+    uint32_t beside_blocks = 0;
     for (uint64_t id : s->resident) {
         const Job &j = *s->jobs[id];
-        if (j.v.L.solo)
-            members.push_back(TeamMember{&j.sa, j.v.n, j.v.words, j.link != nullptr, j.weights != nullptr});
+        if (j.v.L.solo) {
+            members.push_back(team_member(j.sa, j.link != nullptr, j.weights != nullptr));
+        } else {
+            beside += continuous_work(j.v.n, j.desc.n_loci);
+            beside_blocks += continuous_blocks(j.v.n);
+        }
     }
-    rc = s->teams.build(members, s->alloc, s->stream);
+    rc = s->teams.build(members, s->alloc, s->stream, beside, beside_blocks);
     if (rc != SPG_OK) return rc;
     for (int gi = 0; gi < kGroups; ++gi) {
         std::vector<const PopView *> views;
@@ -465,9 +471,9 @@ double spg_server_clock(spg_server *s) { return s ? s->now() : 0.0; }
 void spg_server_destroy(spg_server *s) {
     if (!s) return;
     if (s->stream) cudaStreamSynchronize(s->stream);
+    s->teams.release(s->alloc, s->stream);  // (waits for launches of its own streams)
     for (auto &jp : s->jobs)
         if (jp && jp->arena) s->alloc.release(jp->arena, s->stream);
-    s->teams.release(s->alloc, s->stream);
     for (int gi = 0; gi < kGroups; ++gi) {
         if (s->table[gi]) s->alloc.release(s->table[gi], s->stream);
         if (s->group_stream[gi]) cudaStreamDestroy(s->group_stream[gi]);

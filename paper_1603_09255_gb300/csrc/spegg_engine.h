@@ -77,7 +77,7 @@ constexpr uint32_t kSoloLaunchGens = 512;  // generations of one launch of the g
 struct TeamMember {
     const SoloArgs *args = nullptr;  // (read when the tables are built)
     uint32_t n = 0, words = 0;
-    bool linked = false, weighted = false;
+    bool linked = false, weighted = false, general = false;  // (the kind: team_kind)
 };
 struct TeamLaunch {
     std::vector<TeamMember> members;  // of one kind
@@ -85,16 +85,28 @@ struct TeamLaunch {
     TeamArgs args{};
     char *table = nullptr;            // the members' arguments and the blocks' places
     size_t capacity = 0;
+    uint32_t blocks = 0;              // of its launches
     double cycles = 0.0;              // estimated cycles of a generation of all members
+    cudaStream_t side = nullptr;      // its launches' stream, beside the other kinds'
+    cudaEvent_t joined = nullptr;
     void release(const Allocator &alloc, cudaStream_t stream);
 };
 struct TeamSet {
     TeamLaunch launch[kTeamKinds];
-    int build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream);  // synchronises
+    bool beside = false;              // the kinds' launches run side by side
+    cudaEvent_t forked = nullptr;
+    // `kept`: work of other launches that run beside these, in SM cycles a
+    // generation, and the most SMs it fills (0: none)
+    int build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream, double kept = 0.0,
+              uint32_t kept_blocks = 0);  // synchronises
     int update(const SoloArgs *args, cudaStream_t stream);
     int step(uint32_t n_gen, bool keep_last, cudaStream_t stream);
     void release(const Allocator &alloc, cudaStream_t stream);
 };
+TeamMember team_member(const SoloArgs &a, bool linked, bool weighted);
+double continuous_work(uint32_t n, uint32_t n_loci);
+uint32_t continuous_blocks(uint32_t n);
+std::vector<uint32_t> deal_blocks(const std::vector<double> &work, const std::vector<uint32_t> &most, uint32_t blocks);
 double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, std::vector<TeamPlace> &places,
                       std::vector<uint32_t> &block_places);
 uint32_t most_blocks(uint32_t n, uint32_t resident);

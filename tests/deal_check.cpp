@@ -1,0 +1,47 @@
+// Host-side check of dealing blocks to kinds of members (spg::deal_blocks):
+// every kind with work has a block while there are enough, none more than it can
+// use, all blocks are dealt while a kind can use one, and no kind with room has
+// more work per block left than the one that got the last block.
+#include <cstdint>
+#include <cstdio>
+#include <random>
+#include <vector>
+
+#include "spegg_engine.h"
+
+static int fail(int c, const char *what) {
+    std::printf("FAIL case %d: %s\n", c, what);
+    return 1;
+}
+
+int main() {
+    std::mt19937 rng(7u);
+    for (int c = 0; c < 2000; ++c) {
+        const size_t K = 1 + rng() % 6;
+        const uint32_t blocks = c % 3 ? 152u : rng() % 153u;
+        std::vector<double> work(K);
+        std::vector<uint32_t> most(K);
+        uint32_t kinds = 0;
+        for (size_t k = 0; k < K; ++k) {
+            work[k] = rng() % 4 == 0 ? 0.0 : (double)(1u + rng() % 1000000u);
+            most[k] = work[k] > 0.0 ? 1u + rng() % 152u : 0u;
+            kinds += work[k] > 0.0;
+        }
+        const std::vector<uint32_t> got = spg::deal_blocks(work, most, blocks);
+        uint32_t sum = 0, room = 0;
+        for (size_t k = 0; k < K; ++k) {
+            sum += got[k];
+            if (got[k] > most[k]) return fail(c, "more than a kind can use");
+            if (work[k] > 0.0 && !got[k] && kinds <= blocks) return fail(c, "a kind without a block");
+            if (work[k] == 0.0 && got[k]) return fail(c, "a block without work");
+            if (got[k] && got[k] < most[k]) ++room;
+        }
+        if (sum > blocks || (sum < blocks && room && kinds <= blocks)) return fail(c, "blocks left over or invented");
+        for (size_t k = 0; k < K; ++k)  // taking one block back would not have been better
+            for (size_t j = 0; j < K; ++j)
+                if (got[k] > 1u && got[j] && got[j] < most[j] && work[j] / got[j] > work[k] / (got[k] - 1u) * (1.0 + 1e-12))
+                    return fail(c, "not by work");
+    }
+    std::printf("ok\n");
+    return 0;
+}

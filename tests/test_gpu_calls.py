@@ -120,13 +120,59 @@ def test_one_generation_call_under_stream_capture(n):
     assert_population(gpu, orc, orc.step(8), 8)
 
 
+def continuous(n, n_loci, seed):
+    return S.continuous_trait(n=n, n_loci=n_loci, seed=seed, replicate=7)
+
+
 @pytest.mark.parametrize("sizes", [(33, 700), (5000, 40_000)])
 def test_batch_of_every_kind(sizes):
     """Records, survivors and state of members of every kind, sizes and locus
     counts mixed, after calls of one generation and of several."""
-    ws = [w for n in sizes for L in (32, 128, 256) for w in kinds(n + L, L, 7)]
+    ws = [w for n in sizes for L in (32, 128, 256) for w in kinds(n + L, L, 7)] + [continuous(sizes[0], 64, 3)]
     b = spegg().Batch(ws, stats_capacity=8)
     for k in (1, 1, 3):
         b.step(k)
     for i, w in enumerate(ws):
         assert_member(b, i, w, 5)
+
+
+def test_batch_of_every_kind_longer_than_a_launch():
+    """One member of each kind, over more generations than a launch holds."""
+    ws = kinds(300, 32, 5) + [continuous(200, 32, 5)]
+    b = spegg().Batch(ws, stats_capacity=600)
+    b.step(530)
+    b.step(7)
+    for i, w in enumerate(ws):
+        assert_member(b, i, w, 537)
+
+
+def test_batch_of_every_kind_under_stream_capture():
+    """The kinds' launches fork from the captured stream and join it."""
+    ws = kinds(2000, 64, 6)
+    stream = torch.cuda.Stream()
+    b = spegg().Batch(ws, stats_capacity=16, stream=stream)
+    b.step(1)
+    b.step(3)
+    b.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        b.step(3)
+        b.step(1)
+    with torch.cuda.stream(stream):
+        graph.replay()
+        graph.replay()
+    b.step(1)
+    for i, w in enumerate(ws):
+        assert_member(b, i, w, 13)
+
+
+def test_served_jobs_of_every_kind():
+    ws = kinds(3000, 64, 8) + kinds(200, 256, 9) + [continuous(1000, 64, 8)]
+    gens = [20 + 5 * (i % 4) for i in range(len(ws))]
+    sv = spegg().Server(gens_per_tick=8, max_resident=9)
+    jobs = [sv.submit(w, g, 0.0) for w, g in zip(ws, gens)]
+    sv.drain()
+    for w, g, j in zip(ws, gens, jobs):
+        so, sg = oracle.OraclePopulation.from_workload(w).step(g), sv.job_stats(j, 1, g)
+        for name in so.dtype.names:
+            assert np.array_equal(so[name], sg[name]), (w.name, name)
