@@ -1,7 +1,9 @@
 // Host-side check of dealing blocks to kinds of members (spg::deal_blocks):
 // every kind with work has a block while there are enough, none more than it can
 // use, all blocks are dealt while a kind can use one, and no kind with room has
-// more work per block left than the one that got the last block.
+// more work per block left than the one that got the last block.  And members
+// of about the same work are scheduled side by side.
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 #include <random>
@@ -41,6 +43,26 @@ int main() {
             for (size_t j = 0; j < K; ++j)
                 if (got[k] > 1u && got[j] && got[j] < most[j] && work[j] / got[j] > work[k] / (got[k] - 1u) * (1.0 + 1e-12))
                     return fail(c, "not by work");
+    }
+    // members of about the same work, no more of them than blocks, are formed side
+    // by side: no block has two, and the schedule takes little longer than one of
+    // them on its part of the blocks
+    for (int c = 0; c < 200; ++c) {
+        const uint32_t M = 2 + rng() % 15;
+        std::vector<spg::TeamMember> members(M);
+        double alone = 0.0;
+        for (auto &m : members) {
+            m.n = 150000u + rng() % 100000u;
+            m.words = 1u;
+            m.general = rng() % 2 == 0;
+        }
+        std::vector<spg::TeamPlace> places;
+        std::vector<uint32_t> start;
+        for (auto &m : members) alone = std::max(alone, spg::schedule_teams({m}, 152u / M, places, start));
+        const double cycles = spg::schedule_teams(members, 152u, places, start);
+        for (uint32_t b = 0; b < 152u; ++b)
+            if (start[b + 1] - start[b] > 1u) return fail(c, "two members on a block");
+        if (cycles > 1.25 * alone) return fail(c, "members one after the other");
     }
     std::printf("ok\n");
     return 0;
