@@ -148,7 +148,7 @@ int configure_teams(spg_batch *b) {
         m.sa.locus_cap = m.locus.cap;
         all.push_back(i);
     }
-    return b->teams.build(team_members(b, all), b->alloc, b->stream, beside, beside_blocks);
+    return b->teams.build(team_members(b, all), b->alloc, b->stream, true, beside, beside_blocks);
 }
 
 // A group's launch shape: the continuous-allele kernel's launch table
@@ -415,7 +415,7 @@ int spg_batch_autotune(spg_batch *b, uint32_t gens_per_trial, spg_autotune_repor
             continue;
         }
         TeamSet set;
-        rc = set.build(team_members(b, g.members), b->alloc, b->stream);
+        rc = set.build(team_members(b, g.members), b->alloc, b->stream, true);
         float best_ms = 0.f, worst_ms = 0.f;
         Shape best = g.shape;
         for (uint32_t c = 0; c < kAutotuneCandidates && rc == SPG_OK; ++c) {
@@ -447,7 +447,7 @@ int spg_batch_autotune(spg_batch *b, uint32_t gens_per_trial, spg_autotune_repor
     const uint32_t gens = kAutotuneCandidates * (gens_per_trial + 1u);
     if (!variants.empty() && rc == SPG_OK) {
         TeamSet set;
-        rc = set.build(team_members(b, variants), b->alloc, b->stream);
+        rc = set.build(team_members(b, variants), b->alloc, b->stream, true);
         if (rc == SPG_OK) rc = set.step(gens, true, b->stream);
         if (rc == SPG_OK) rc = view_sync(b->members[0].v);
         set.release(b->alloc, b->stream);

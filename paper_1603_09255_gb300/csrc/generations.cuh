@@ -1031,8 +1031,8 @@ __device__ __forceinline__ void team_places(const TeamArgs &t, uint32_t &p) {
             reinterpret_cast<uint32_t *>(&s_team_args)[i] = reinterpret_cast<const uint32_t *>(t.members + place.member)[i];
         __syncthreads();
         if (s_team_args.words != (uint32_t)W) return;
-        form_generations<W, LINKED, WEIGHTED, GENERAL>(s_team_args, s_team_args.keys, t.n_gen, t.keep_last != 0u, false,
-                                                       place.rank, place.team);
+        form_generations<W, LINKED, WEIGHTED, GENERAL>(s_team_args, s_team_args.keys, t.n_gen, t.keep_last != 0u,
+                                                       t.single != 0u, place.rank, place.team);
     }
 }
 template <bool LINKED, bool WEIGHTED, bool GENERAL>

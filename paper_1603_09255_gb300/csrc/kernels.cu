@@ -635,14 +635,12 @@ __global__ void __launch_bounds__(kCompactThreads, 3) k_compact(const __grid_con
 // picks one.  The blocks start as the previous kernel's leave; kCloseSmem bytes
 // of shared memory keep them from crowding onto the first SMs that are free (N =
 // 10^6: 45.7 us a call without, 41.1 with).
-__global__ void __launch_bounds__(kCloseThreads) k_close(const __grid_constant__ SoloArgs a) {
+__device__ __forceinline__ void close_part(const SoloArgs &a, uint32_t part) {
     constexpr uint32_t NW = (kCloseThreads - 32u) / 32u;
     __shared__ uint32_t s_gen, s_sum[2][NW], s_own[2][NW], s_first[2][32u * NW];
-    griddep_release();
-    griddep_wait();
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    const bool close = blockIdx.x == 0u;
-    const uint32_t slot0 = blockIdx.x * a.close_slots, slot1 = min(slot0 + a.close_slots, a.nslots);
+    const bool close = part == 0u;
+    const uint32_t slot0 = part * a.close_slots, slot1 = min(slot0 + a.close_slots, a.nslots);
     DevState *st = a.state;
     if (warp == NW) {
         if (!close) {
@@ -726,6 +724,22 @@ __global__ void __launch_bounds__(kCloseThreads) k_close(const __grid_constant__
             row[i] = 0u;
         }
     }
+}
+__global__ void __launch_bounds__(kCloseThreads) k_close(const __grid_constant__ SoloArgs a) {
+    griddep_release();
+    griddep_wait();
+    close_part(a, blockIdx.x);
+}
+// The same of the members of a batch.
+__global__ void __launch_bounds__(kCloseThreads) k_close_members(const ClosePart *__restrict__ parts) {
+    __shared__ SoloArgs s_args;
+    const ClosePart part = parts[blockIdx.x];
+    for (uint32_t i = threadIdx.x; i < sizeof(SoloArgs) / 4u; i += kCloseThreads)
+        reinterpret_cast<uint32_t *>(&s_args)[i] = reinterpret_cast<const uint32_t *>(part.member)[i];
+    griddep_release();
+    griddep_wait();
+    __syncthreads();
+    close_part(s_args, part.part);
 }
 
 // ---------------------------------------------------------- founders
@@ -853,6 +867,7 @@ bool supported_shape(uint32_t words, const Shape &s) {
 
 GenKernel compact_kernel() { return &k_compact; }
 const void *close_kernel() { return (const void *)&k_close; }
+const void *close_members_kernel() { return (const void *)&k_close_members; }
 int prepare_close() {
     return cudaFuncSetAttribute(close_kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCloseSmem) == cudaSuccess
                ? SPG_OK

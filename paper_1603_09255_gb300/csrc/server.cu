@@ -192,7 +192,7 @@ int rebuild(spg_server *s) {
             beside_blocks += continuous_blocks(j.v.n);
         }
     }
-    rc = s->teams.build(members, s->alloc, s->stream, beside, beside_blocks);
+    rc = s->teams.build(members, s->alloc, s->stream, false, beside, beside_blocks);
     if (rc != SPG_OK) return rc;
     for (int gi = 0; gi < kGroups; ++gi) {
         std::vector<const PopView *> views;

@@ -95,10 +95,14 @@ struct TeamSet {
     TeamLaunch launch[kTeamKinds];
     bool beside = false;              // the kinds' launches run side by side
     cudaEvent_t forked = nullptr;
-    // `kept`: work of other launches that run beside these, in SM cycles a
-    // generation, and the most SMs it fills (0: none)
-    int build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream, double kept = 0.0,
-              uint32_t kept_blocks = 0);  // synchronises
+    ClosePart *parts = nullptr;       // calls of one generation: k_close_members' blocks
+    uint32_t nparts = 0;
+    size_t parts_capacity = 0;
+    // singles: calls of one generation are formed without barriers; `kept`: work of
+    // other launches that run beside these, in SM cycles a generation, and the most
+    // SMs it fills (0: none).  Synchronises.
+    int build(const std::vector<TeamMember> &all, const Allocator &alloc, cudaStream_t stream, bool singles,
+              double kept = 0.0, uint32_t kept_blocks = 0);
     int update(const SoloArgs *args, cudaStream_t stream);
     int step(uint32_t n_gen, bool keep_last, cudaStream_t stream);
     void release(const Allocator &alloc, cudaStream_t stream);

@@ -217,15 +217,16 @@ struct alignas(16) SoloArgs {
     uint32_t n_gen;                    // generations of this launch
     uint32_t keep_last;                // the last of them is the call's last
     uint32_t single;                   // one generation without a grid barrier: k_close closes it
-    uint32_t close_slots;              // slots whose survivors a block of k_close lists, at most 256
     uint32_t barrier_tries;            // polls of a wait before it gives up
+    uint32_t close_slots;              // slots whose survivors a block of k_close lists, at most 256
 };
 struct SoloKernel {
     const void *fn = nullptr;
     uint32_t smem = 0, resident = 0;  // resident: blocks on the device at a time
 };
 SoloKernel solo_kernel(uint32_t words, bool linked, bool weighted, bool general);
-const void *close_kernel();  // k_close
+const void *close_kernel();          // k_close
+const void *close_members_kernel();  // k_close_members
 int prepare_close();         // sets its shared-memory limit
 constexpr uint32_t kCloseThreads = 256 + 32;  // + one warp that closes the generation
 constexpr uint32_t kCloseSmem = 120000;  // not used: keeps its blocks on an SM each
@@ -243,6 +244,12 @@ struct TeamArgs {
     const TeamPlace *places;
     const uint32_t *block_places;
     uint32_t n_gen, keep_last;
+    uint32_t single;  // one generation without barriers: k_close_members closes it
+};
+// Block b of k_close_members closes slots from part * close_slots of a member.
+struct ClosePart {
+    const SoloArgs *member;
+    uint32_t part, pad;
 };
 // Kinds of members that share a launch: plain ones, general values, linkage
 // map, parent weights, both.
