@@ -439,6 +439,19 @@ uint32_t most_blocks(uint32_t n, uint32_t resident) {
     return n <= 32u * kOneBlockGroups ? 1u : std::max(1u, std::min(resident, slot_count(n) / kSoloMinWarps));
 }
 
+// Blocks of a population alone: a block fills an SM, so populations on streams of
+// their own run at the same time only when their blocks fit together.  A small
+// one therefore takes half of what the device holds at most while that is ten
+// slots a block or less: 200 generations of one, two and four populations of 10^4,
+// ms: 0.95 / 1.88 / 3.75 with 78 blocks, 0.95 / 0.96 / 1.90 with 76 (a quarter:
+// 0.99 / 0.99 / 1.00), of 2 x 10^4 1.04 / 2.07 / 4.10 and 1.06 / 1.07 / 2.11; before
+// the generation kernel 1.66 / 1.64 / 1.78 and 1.80 / 1.93 / 2.20.  With 16 slots a
+// block one alone takes a fifth longer.
+uint32_t solo_grid(uint32_t n, uint32_t resident) {
+    const uint32_t blocks = most_blocks(n, resident), half = std::max(resident / 2u, 1u);
+    return slot_count(n) <= 10u * half ? std::min(blocks, half) : blocks;
+}
+
 // ------------------------------------------------------------ teams
 // Cycles of a generation on k blocks of 16 warps: closing it alone or with a
 // barrier, and rounds of the warps' groups (measured, L = 32 .. 256; a linkage

@@ -176,3 +176,16 @@ def test_served_jobs_of_every_kind():
         so, sg = oracle.OraclePopulation.from_workload(w).step(g), sv.job_stats(j, 1, g)
         for name in so.dtype.names:
             assert np.array_equal(so[name], sg[name]), (w.name, name)
+
+
+def test_populations_on_streams_of_their_own():
+    """Small and large populations stepped at the same time, with calls of one
+    generation and of several, equal to the oracle's."""
+    ws = [S.single_species(n=n, n_loci=32, mu=1e-3, seed=20 + i) for i, n in enumerate((10_000, 24_321, 300, 120_000, 10_000))]
+    pops = [spegg().Population.from_workload(w, stats_capacity=32) for w in ws]
+    for k in (5, 1, 1, 7):
+        for p in pops:
+            p.step(k)
+    for w, p in zip(ws, pops):
+        orc = oracle.OraclePopulation.from_workload(w)
+        assert_population(p, orc, orc.step(14), 14)
