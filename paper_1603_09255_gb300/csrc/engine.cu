@@ -477,6 +477,16 @@ static double team_cycles(const TeamMember &m, uint32_t k) {
     return (k == 1 ? 6000.0 : 11000.0) + std::max(1.0, groups / (16.0 * k)) * round_cycles(m);
 }
 
+// Generations of one launch of a population on `blocks` blocks: other streams'
+// work waits for the launch, so it is cut at about 1.5 ms (at eight generations at
+// least; a launch costs about 6 us more than its generations, 26.0 -> 26.1 us a
+// generation at 10^6 x 128).  A call of one generation of 1,000 offspring beside
+// 1,000 generations of 10^6 x 128 waited 13.5 ms with launches of 512, and 1.5 now.
+constexpr double kLaunchCycles = 3.0e6;
+uint32_t launch_generations(const TeamMember &m, uint32_t blocks) {
+    return (uint32_t)std::min<double>(kSoloLaunchGens, std::max(8.0, kLaunchCycles / team_cycles(m, blocks)));
+}
+
 // Blocks below which all teams' records together would not stay in L2: with
 // every block at its share of such a member, parents and survivors (16 W bytes
 // an individual) come to kTeamL2Bytes (152 members of 60,000 x 128 loci on a

@@ -3,11 +3,11 @@
 //
 // A population owns one device arena (parameters, state, statistics ring,
 // accumulators, genotypes, survivors).  The generations of a biallelic
-// population are formed by one cooperative launch per call (of at most
-// kSoloLaunchGens; two plain ones for a call of one generation); those of continuous allelic values are enqueued as a
-// cached CUDA graph of kGraphChunk generations (two launches each), whose
-// arguments are identical because buffers are chosen on the device by
-// generation parity.
+// population are formed by cooperative launches of many (launch_generations; a
+// call of one generation takes two plain ones); those of continuous allelic
+// values are enqueued as a cached CUDA graph of kGraphChunk generations (two
+// launches each), whose arguments are identical because buffers are chosen on
+// the device by generation parity.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -36,7 +36,7 @@ struct spg_pop {
     WeightParams *weights = nullptr;  // parent acceptance thresholds (when host_prm->weighted)
     SoloKernel solo;   // biallelic records: the generation kernel, its grid and arguments
     SoloArgs sa{};
-    uint32_t solo_blocks = 0;
+    uint32_t solo_blocks = 0, launch_gens = 0;
     GenLaunch gl;      // continuous allelic values: generation and compaction launches
     GraphChain chain;
     // per-locus allele counts (off until spg_set_locus_counts): ring, partial
@@ -82,6 +82,7 @@ int configure_solo(spg_pop *p, const Shape &shape) {
     p->solo = k;
     p->shape = shape;
     p->solo_blocks = solo_grid(p->n, k.resident);
+    p->launch_gens = launch_generations(team_member(a, prm.linked != 0u, prm.weighted != 0u), p->solo_blocks);
     attach_locus(p);
     return SPG_OK;
 }
@@ -128,7 +129,7 @@ int launch_solo(spg_pop *p, const SoloArgs &args, const void *fn, uint32_t block
     return e == cudaSuccess ? SPG_OK : cuda_fail(e, "generation launch");
 }
 
-// n_gen generations: one cooperative launch per kSoloLaunchGens of them.  A call
+// n_gen generations: one cooperative launch per launch_gens of them.  A call
 // of one generation is two launches without a barrier instead, which may start
 // while their predecessors finish, as a cooperative one cannot: back to back,
 // with the barrier / without, us a call: N = 3,000 10.3 / 7.8, 30,000 14.4 / 9.6,
@@ -145,7 +146,7 @@ int enqueue_solo(spg_pop *p, uint32_t n_gen) {
                            false);
     }
     for (uint32_t done = 0; done < n_gen;) {
-        a.n_gen = std::min(n_gen - done, kSoloLaunchGens);
+        a.n_gen = std::min(n_gen - done, p->launch_gens);
         done += a.n_gen;
         a.keep_last = done == n_gen ? 1u : 0u;
         const int rc = launch_solo(p, a, p->solo.fn, p->solo_blocks, kSoloThreads, p->solo.smem, p->solo_blocks > 1u);

@@ -2,7 +2,8 @@
 // every kind with work has a block while there are enough, none more than it can
 // use, all blocks are dealt while a kind can use one, and no kind with room has
 // more work per block left than the one that got the last block.  And members
-// of about the same work are scheduled side by side.
+// of about the same work are scheduled side by side, and a population's launches
+// are cut.
 #include <algorithm>
 #include <cstdint>
 #include <cstdio>
@@ -63,6 +64,17 @@ int main() {
         for (uint32_t b = 0; b < 152u; ++b)
             if (start[b + 1] - start[b] > 1u) return fail(c, "two members on a block");
         if (cycles > 1.25 * alone) return fail(c, "members one after the other");
+    }
+    // a population's launches: whole for small ones, short for large ones
+    uint32_t last = 512u;
+    for (uint32_t n = 100u; n < 100000000u; n *= 2u) {
+        spg::TeamMember m;
+        m.n = n;
+        m.words = 4u;
+        const uint32_t gens = spg::launch_generations(m, spg::solo_grid(n, 152u));
+        if (gens > last + 16u || gens < 8u || gens > 512u) return fail((int)n, "launch length");
+        if (n > 900000u && n < 4000000u && gens > 80u) return fail((int)n, "a launch of several milliseconds");
+        last = gens;
     }
     std::printf("ok\n");
     return 0;
