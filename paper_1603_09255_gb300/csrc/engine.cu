@@ -526,8 +526,10 @@ double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, s
     std::vector<double> free_at;
     std::vector<uint32_t> by_time;
     // (a little above one: members that divide the blocks without rounding up to
-    // one block too many, which would put them one after the other)
+    // one block too many, which would put them one after the other; the same for
+    // more members than blocks)
     for (const double share : {0.1, 0.15, 0.25, 0.4, 0.6, 1.0, 1.06, 1.25, 1.6}) {
+        if (share > 1.0 && M > blocks) break;
         free_at.assign(blocks, 0.0);
         by_time.resize(blocks);
         for (uint32_t b = 0; b < blocks; ++b) by_time[b] = b;
@@ -536,6 +538,13 @@ double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, s
         for (const uint32_t m : order) {
             const double want = std::max(std::ceil(work[m] / (share * total / blocks)), resident_blocks(members[m], blocks));
             const uint32_t k = (uint32_t)std::max(1.0, std::min<double>(want, most_blocks(members[m].n, blocks)));
+            if (k == 1u) {  // (most members of a large batch: a plain search is quicker)
+                const size_t b = (size_t)(std::min_element(free_at.begin(), free_at.end()) - free_at.begin());
+                free_at[b] += team_cycles(members[m], 1u);
+                dealt.push_back(Dealt{(uint32_t)b, TeamPlace{m, 0u, 1u}});
+                end = std::max(end, free_at[b]);
+                continue;
+            }
             std::nth_element(by_time.begin(), by_time.begin() + (k - 1), by_time.end(),
                              [&](uint32_t x, uint32_t y) { return free_at[x] != free_at[y] ? free_at[x] < free_at[y] : x < y; });
             double start = 0.0;
