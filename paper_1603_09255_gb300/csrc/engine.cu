@@ -999,14 +999,10 @@ int enqueue_generations(const GenLaunch &gl, uint32_t n_gen, GraphChain &chain, 
 }
 
 // ------------------------------------------------- launch groups
-// Bytes of a launch group's table: segments, runs (at most one per member plus
-// one per piece: one round of blocks, or pieces of kPieceOffspring offspring
-// or more), the blocks' run offsets, the bucket map and the tile map.
+// Bytes of a launch group's table: segments, the bucket map and the tile map.
 size_t group_table_bytes(uint32_t members, uint64_t offspring, uint32_t buckets) {
-    const uint64_t runs = 2ull * members + offspring / kPieceOffspring + kMaxGridBlocks + 1ull;
-    return align_up((size_t)members * sizeof(Segment), 256) + align_up((size_t)runs * sizeof(Run), 256) +
-           align_up((size_t)(kMaxGridBlocks + 1) * 4, 256) + align_up((size_t)buckets * 4, 256) +
-           align_up((size_t)(offspring / kBlock + members + 1) * 4, 256);  // tile map (continuous groups)
+    return align_up((size_t)members * sizeof(Segment), 256) + align_up((size_t)buckets * 4, 256) +
+           align_up((size_t)(offspring / kBlock + members + 1) * 4, 256);
 }
 
 // Runs of a launch group (see GenArgs): the members' tiles, in member order,
@@ -1017,7 +1013,8 @@ size_t group_table_bytes(uint32_t members, uint64_t offspring, uint32_t buckets)
 // formed at any moment are few and their parent records stay in L2 -- the
 // flattened replicate loop of Fig. S5 B, scheduled for locality).  A piece is
 // one run per member it touches, so every block's work is within a set-up or
-// two of the others'.
+// two of the others'.  (Only its test reaches it: teams and tile maps took its
+// place.)
 void schedule_runs(const std::vector<uint32_t> &tiles, uint32_t G, uint32_t min_piece, std::vector<Run> &runs,
                    std::vector<uint32_t> &block_runs) {
     const uint32_t M = (uint32_t)tiles.size();

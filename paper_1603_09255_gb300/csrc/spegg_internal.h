@@ -95,7 +95,8 @@ struct alignas(16) PopParams {
     const WeightParams *weights;
 };
 
-// the offspring kernel copies these tables with 16-byte cp.async
+// the generation kernel and the allocation-free call's offspring kernel copy
+// these tables with 16-byte cp.async
 static_assert(offsetof(PopParams, table) % 16 == 0 && offsetof(PopParams, attack) % 16 == 0 &&
                   offsetof(PopParams, lut) % 16 == 0,
               "tables copied in 16-byte chunks");
