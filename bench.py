@@ -45,14 +45,16 @@ def algorithmic_bytes(words: int) -> int:
     return 12 + 24 * words
 
 
-# Most generations of one launch of the generation kernel.
-LAUNCH_GENERATIONS = 512
-# DRAM traffic per generation of the headline population (a launch of four
-# generations of its kernel, caches flushed before it, divided by four) from
-# one ncu capture, keyed by the hash of that kernel's sources (null once they
-# change).
-MEASURED_TRAFFIC = {"cdd82d88b1f571eb": 17248640}
-TRAFFIC_SOURCES = ("generations.cuh", "device_common.cuh", "ecology.cuh", "generations_w4.cu")
+# Generations of one launch of the headline population's kernel (cut at about a
+# millisecond and a half).
+LAUNCH_GENERATIONS = 59
+# DRAM traffic of the headline population: bytes per launch (its parents read,
+# the records of the call's last generation written) and per generation, from
+# ncu captures of launches of 4 and of 36 generations (69.0 and 139.4 MB, caches
+# flushed before them), keyed by the hash of that kernel's sources (null once
+# they change).
+MEASURED_TRAFFIC = {"c7d5174255116a3a": (60_260_000, 2_198_000)}
+TRAFFIC_SOURCES = ("generations.cuh", "closing.cuh", "device_common.cuh", "ecology.cuh", "generations_w4.cu")
 
 
 def kernel_source_hash() -> str:
@@ -259,7 +261,6 @@ def batched_replicates(spegg, torch, gens: int = 500, plain_members: int = 0, pl
     batch.synchronize()
     ms = timed_on(stream, torch, lambda: batch.step(gens))
     sum_n = sum(w.n for w in ws)
-    tuned = getattr(batch, "autotune_report", {})
     p50, p99 = per_generation_ms(stream, torch, lambda: batch.step(1))
     batch.close()
     ms_plain, plain_work = 0.0, 0
@@ -279,9 +280,7 @@ def batched_replicates(spegg, torch, gens: int = 500, plain_members: int = 0, pl
     algo = sum(w.n * algorithmic_bytes(w.words) for w in ws) * gens
     peak, _ = load_peaks()
     out = {"value": value, "vs_plain": value / plain, "frac": algo / (ms / 1e3) / 1e9 / peak,
-           "p50_ms": p50, "p99_ms": p99,
-           "shapes": {str(L): list(r["shape"]) for L, r in tuned.items()},
-           "spread": {str(L): round(r["worst_ms"] / r["best_ms"], 3) for L, r in tuned.items() if r["best_ms"] > 0}}
+           "p50_ms": p50, "p99_ms": p99}
     if oracle_cpu:
         out["cpu"] = oracle_batched_baseline(ws)["value"]
     return out
@@ -355,10 +354,19 @@ def spatial_community(spegg, torch, steps: int = 200, oracle_cpu: bool = False):
     ind = int(st["n_before"].sum())
     births = int(st["births"].sum())
     words = c.n_loci // 32
-    # algorithmic bytes: every member's record (8W B) and age read once and
-    # written once at its new place; every newborn reads two parent records
-    # and is written once with its age
-    algo = ind * (16 * words + 2) + births * (24 * words + 1)
+    # algorithmic bytes: every member's 8-byte entry (record slot, phenotype and
+    # age) read and written; every newborn's two parent records and entries read,
+    # its record and entry written; the survivors' records read and written in the
+    # steps that move them, because the next newborns do not fit behind
+    founders = sum(sp.n0 for sp in c.species) * c.patches
+    moved, top, capacity = 0, founders, 2 * founders
+    history = g.read_stats(1, steps + 3)
+    for k in range(steps + 3):
+        b, after, alive = (int(history[f][k].sum()) for f in ("births", "n_after", "survivors"))
+        move = top + b > capacity
+        top = after if move else top + b
+        moved += alive if move and k >= 3 else 0
+    algo = ind * 16 + births * (24 * words + 24) + moved * 16 * words
     peak, _ = load_peaks()
     out = {"value": ind / (ms / 1e3), "ms": ms / steps, "frac": algo / (ms / 1e3) / 1e9 / peak}
     if oracle_cpu:
@@ -515,7 +523,9 @@ def main():
     avg_gen_s = total_ms / 1000.0 / (GENERATIONS * args.steps)
     peak, peak_kind = load_peaks()
     achieved = algorithmic_bytes(workload.words) * workload.n / avg_gen_s / 1e9
-    traffic = MEASURED_TRAFFIC.get(kernel_source_hash())
+    traffic = MEASURED_TRAFFIC.get(kernel_source_hash())  # bytes per generation
+    if traffic:
+        traffic = traffic[0] // LAUNCH_GENERATIONS + traffic[1]
     gen_p50, gen_p99 = per_generation_ms(stream, torch, lambda: pop.step(1), repeats=50)
 
     # end to end through the C ABI with host buffers: restore the population

@@ -1,16 +1,18 @@
 // The generation kernel of biallelic populations (sm_103a): any number of
 // generations of Fig. 1 A-F in one cooperative launch, of one population
-// (k_generations) or of many, each formed by a team of blocks (k_teams).
+// (k_generations) or of many of a kind, each formed by a team of blocks (k_teams).
 //
 // us per generation, against an offspring launch with byte tables and a
 // compaction launch: N = 10^4, L = 32: 8.2 -> 4.8; 99,991 x 64 with locus counts
 // 21.5 -> 9.9; 3 x 10^5 x 128 with dominance 23.8 -> 13.2; 10^6 x 128 with a
-// resource 39.2 -> 26.0, with a map 127 -> 75, with weights 64.8 -> 48.5; 2 x
-// 10^6 x 256 164 -> 78.  At 10^6 x 128 it is bound by instructions: 41,000 of
-// 52,000 cycles a generation form offspring, 405 instructions per warp of 32,
-// the integer pipe busy 56 % of them with four warps per scheduler (512 threads
-// of 128 registers; 640 to 1,024 threads spill and are slower); the rest is the
-// barrier (3,300 to 5,000), the directory (2,000 to 3,500) and the statistics.
+// resource 39.2 -> 26.1, with a map 127 -> 74, with weights 64.8 -> 48.5; 2 x
+// 10^6 x 256 164 -> 78.  At 10^6 x 128 it is bound by instructions: 479 per warp
+// of 32 offspring in a launch of four generations, of which some 400 form the
+// offspring (41,000 of 52,000 cycles of a generation); the ALU pipe is busy 46 %
+// of the cycles and an instruction issues in 44 % of them, with four warps per
+// scheduler (512 threads of 128 registers; 640 to 1,024 threads spill and are
+// slower).  The rest is the barrier (3,300 to 5,000 cycles), the directory (2,000
+// to 3,500) and the statistics.
 //
 // Blocks stay for the whole call, so the tables (thresholds, attack rates,
 // effect digits, linkage map) reach shared memory once per call instead of
@@ -31,7 +33,8 @@
 // visible between calls, so they are written in a call's last generation
 // (and in one that leaves no survivors: it is formed a second time for them).
 // The per-locus counts read full records, so those are written every
-// generation while counting.
+// generation while counting.  A call of one generation has no barrier: k_close
+// (kernels.cu) closes what this kernel has formed.
 //
 // Genetic value.  A child's value is a counts x effects product: the warp's 32
 // records go through shared memory into mma.m16n8k16 fragments, each locus as
