@@ -237,7 +237,12 @@ int spg_set_ecology(spg_pop *pop, const spg_ecology *eco);
 
 /* Enqueue n_gen generations (Fig. 1 A-F each) on the population's stream and
  * return without waiting.  Generations after an extinction do nothing;
- * extinction is reported by spg_get_state and spg_read_stats. */
+ * extinction is reported by spg_get_state and spg_read_stats.  A biallelic
+ * population's launches are cooperative and fill the SMs that they take: about
+ * N / 128 SMs, half of the device from about 10,000 and all of it from about
+ * 25,000 individuals.  Other streams' work takes the SMs that are left or waits
+ * for the launch: one that fills the device takes about 1.5 ms or eight
+ * generations, whichever is longer. */
 int spg_step_generations(spg_pop *pop, uint32_t n_gen);
 
 /* Copy statistics of generations first_gen .. first_gen+count-1 to out
@@ -311,13 +316,16 @@ int spg_get_tiling(spg_pop *pop, uint32_t *items_per_thread);
  * locus count and variant (plain; linkage map; parent weights; both;
  * continuous values).  The biallelic members of a kind (plain; linkage map;
  * parent weights; both) share cooperative launches of several generations,
- * each member formed by a team of blocks; a group of continuous-value members
- * takes one offspring and one compaction launch per generation, the groups
- * as branches of one cached CUDA graph.  Members with a linkage map, parent
- * weights or continuous values have the shape of 256 threads, one offspring
- * per thread, one lane; other launch shapes are accepted, and reported, for
- * the plain members of each locus count (the biallelic kernel has one shape
- * of its own).  Every member keeps its own parameters,
+ * each member formed by a team of blocks, the kinds side by side; other
+ * streams' work waits for such a launch, of up to about a quarter of a second.
+ * A group of continuous-value members takes one offspring and one compaction
+ * launch per generation, the groups as branches of one cached CUDA graph beside
+ * the other members (a batch that holds some cannot be stepped while its stream
+ * is being captured).  Members with a linkage map, parent weights or continuous
+ * values have the shape of 256 threads, one offspring per thread, one lane;
+ * other launch shapes are accepted, and reported, for the plain members of each
+ * locus count (the biallelic kernel has one shape of its own).  Every member
+ * keeps its own parameters,
  * state, buffers and statistics ring, and its results are identical to the same population
  * created with spg_create_population and stepped alone.  Member i is
  * descs[i]; the descriptions are copied.  Errors as for a population;

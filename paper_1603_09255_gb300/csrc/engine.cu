@@ -477,13 +477,16 @@ static double team_cycles(const TeamMember &m, uint32_t k) {
     return (k == 1 ? 6000.0 : 11000.0) + std::max(1.0, groups / (16.0 * k)) * round_cycles(m);
 }
 
-// Generations of one launch of a population on `blocks` blocks: other streams'
-// work waits for the launch, so it is cut at about 1.5 ms (at eight generations at
-// least; a launch costs about 6 us more than its generations, 26.0 -> 26.1 us a
-// generation at 10^6 x 128).  A call of one generation of 1,000 offspring beside
-// 1,000 generations of 10^6 x 128 waited 13.5 ms with launches of 512, and 1.5 now.
+// Generations of one launch of a population on `blocks` of the device's blocks:
+// other streams' work waits for a launch that fills the device, so it is cut at
+// about 1.5 ms (at eight generations at least; a launch costs about 6 us more than
+// its generations, 26.0 -> 26.1 us a generation at 10^6 x 128).  A call of one
+// generation of 1,000 offspring beside 1,000 generations of 10^6 x 128 waited 13.5
+// ms with launches of 512, and 1.5 now.  Beside a launch of half the device or
+// less there is room (512 generations of it are some 2.5 ms).
 constexpr double kLaunchCycles = 3.0e6;
-uint32_t launch_generations(const TeamMember &m, uint32_t blocks) {
+uint32_t launch_generations(const TeamMember &m, uint32_t blocks, uint32_t resident) {
+    if (2u * blocks <= resident) return kSoloLaunchGens;
     return (uint32_t)std::min<double>(kSoloLaunchGens, std::max(8.0, kLaunchCycles / team_cycles(m, blocks)));
 }
 

@@ -106,7 +106,7 @@ struct TeamSet {
     void release(const Allocator &alloc, cudaStream_t stream);
 };
 TeamMember team_member(const SoloArgs &a, bool linked, bool weighted);
-uint32_t launch_generations(const TeamMember &m, uint32_t blocks);
+uint32_t launch_generations(const TeamMember &m, uint32_t blocks, uint32_t resident);
 double continuous_work(uint32_t n, uint32_t n_loci);
 uint32_t continuous_blocks(uint32_t n);
 std::vector<uint32_t> deal_blocks(const std::vector<double> &work, const std::vector<uint32_t> &most, uint32_t blocks);
