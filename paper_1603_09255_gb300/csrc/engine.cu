@@ -446,10 +446,11 @@ uint32_t most_blocks(uint32_t n, uint32_t resident) {
 // ms: 0.95 / 1.88 / 3.75 with 78 blocks, 0.95 / 0.96 / 1.90 with 76 (a quarter:
 // 0.99 / 0.99 / 1.00), of 2 x 10^4 1.04 / 2.07 / 4.10 and 1.06 / 1.07 / 2.11; before
 // the generation kernel 1.66 / 1.64 / 1.78 and 1.80 / 1.93 / 2.20.  With 16 slots a
-// block one alone takes a fifth longer.
-uint32_t solo_grid(uint32_t n, uint32_t resident) {
+// block one alone takes a fifth longer.  At L = 256 the line is at five slots (2 x
+// 10^4 alone: 6.9 us a generation on all blocks, 7.2 on half).
+uint32_t solo_grid(uint32_t n, uint32_t words, uint32_t resident) {
     const uint32_t blocks = most_blocks(n, resident), half = std::max(resident / 2u, 1u);
-    return slot_count(n) <= 10u * half ? std::min(blocks, half) : blocks;
+    return slot_count(n) <= (words == 8u ? 5u : 10u) * half ? std::min(blocks, half) : blocks;
 }
 
 // ------------------------------------------------------------ teams

@@ -103,23 +103,30 @@ __device__ __forceinline__ uint32_t sm_u32(uint32_t off) { return *reinterpret_c
 constexpr unsigned long long kBarrierStep = 1u << 16;  // more than a grid's blocks
 constexpr unsigned long long kBarrierFailed = 1ull << 63;
 
+// The end of a wait whose polls ran out, or that met the mark: whether the
+// barrier was complete after all.
+__device__ __noinline__ int barrier_given_up(unsigned long long *ctr, unsigned long long v, unsigned long long want) {
+    while (v < want && v < kBarrierFailed) {  // once per arrival meanwhile, at most
+        const unsigned long long was = atomicCAS(ctr, v, v | kBarrierFailed);
+        v = was == v ? kBarrierFailed : was;
+    }
+    return v < kBarrierFailed ? 1 : 0;
+}
+
 __device__ __forceinline__ bool team_barrier(unsigned long long *ctr, uint32_t rank, uint32_t team, uint32_t tries) {
     __syncthreads();
     if (team == 1u) return true;
     int ok = 1;
     if (threadIdx.x == 0) {
         const unsigned long long add = rank == 0u ? kBarrierStep - (team - 1u) : 1ull;
-        unsigned long long old, v = 0;
+        unsigned long long old;
         asm volatile("atom.add.release.gpu.global.u64 %0, [%1], %2;" : "=l"(old) : "l"(ctr), "l"(add) : "memory");
         const unsigned long long want = (old / kBarrierStep + 1ull) * kBarrierStep;
-        for (uint32_t i = 0; i < tries && v < min(want, kBarrierFailed); ++i)
+        unsigned long long v = old < kBarrierFailed ? 0ull : ~0ull;  // (a marked barrier is not waited for)
+        for (uint32_t i = 0; i < tries && v < want; ++i)
             asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
-        while (v < want && old < kBarrierFailed) {  // once per arrival meanwhile, at most
-            const unsigned long long was = atomicCAS(ctr, v, v | kBarrierFailed);
-            v = was == v ? kBarrierFailed : was;
-        }
         asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        ok = v >= want && v < kBarrierFailed ? 1 : 0;
+        if (v < want || v >= kBarrierFailed) ok = barrier_given_up(ctr, v, want);
     }
     return __syncthreads_and(threadIdx.x == 0 ? ok : 1) != 0;
 }
@@ -595,14 +602,15 @@ __device__ __forceinline__ bool directory_of(const uint32_t *counts, uint32_t fi
     }
     return wide;
 }
-// (Two runs a warp have an instance: as six, calls of one generation of N =
-// 20,000 took 11.4 us instead of 10.1.)
+// (Two runs a warp have an instance but at L = 256: as six, calls of one generation
+// of N = 20,000 x 32 took 11.4 us instead of 10.1; at L = 256 the instance cost the
+// kernel one percent at every size.)
 template <class SM, bool OWN>
 __device__ __forceinline__ bool build_directory(const uint32_t *counts, uint32_t own, uint32_t nslots, uint32_t slot_records,
                                                 uint32_t guide_bits, uint32_t *s_warp, uint32_t *total) {
     constexpr uint32_t T = SM::kThreads - 32u;
     if (nslots <= T) return directory_of<SM, 1, OWN>(counts, own, nslots, slot_records, guide_bits, s_warp, total);
-    if (nslots <= 2u * T) return directory_of<SM, 2, OWN>(counts, own, nslots, slot_records, guide_bits, s_warp, total);
+    if (SM::kPlanes < 4u && nslots <= 2u * T) return directory_of<SM, 2, OWN>(counts, own, nslots, slot_records, guide_bits, s_warp, total);
     return directory_of<SM, (SM::kSlots + T - 1) / T, OWN>(counts, own, nslots, slot_records, guide_bits, s_warp, total);
 }
 

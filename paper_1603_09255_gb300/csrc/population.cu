@@ -81,7 +81,7 @@ int configure_solo(spg_pop *p, const Shape &shape) {
     if (rc != SPG_OK) return fail(rc, "generation kernel setup failed");
     p->solo = k;
     p->shape = shape;
-    p->solo_blocks = solo_grid(p->n, k.resident);
+    p->solo_blocks = solo_grid(p->n, p->words, k.resident);
     p->launch_gens = launch_generations(team_member(a, prm.linked != 0u, prm.weighted != 0u), p->solo_blocks, k.resident);
     attach_locus(p);
     return SPG_OK;

@@ -113,7 +113,7 @@ std::vector<uint32_t> deal_blocks(const std::vector<double> &work, const std::ve
 double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, std::vector<TeamPlace> &places,
                       std::vector<uint32_t> &block_places);
 uint32_t most_blocks(uint32_t n, uint32_t resident);
-uint32_t solo_grid(uint32_t n, uint32_t resident);
+uint32_t solo_grid(uint32_t n, uint32_t words, uint32_t resident);
 void solo_args(const PopView &v, const PopParams &prm, SoloArgs &a);
 
 int fail(int code, const char *fmt, ...);

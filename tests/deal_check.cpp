@@ -71,7 +71,7 @@ int main() {
         spg::TeamMember m;
         m.n = n;
         m.words = 4u;
-        const uint32_t gens = spg::launch_generations(m, spg::solo_grid(n, 152u), 152u);
+        const uint32_t gens = spg::launch_generations(m, spg::solo_grid(n, m.words, 152u), 152u);
         if (gens > last + 16u || gens < 8u || gens > 512u) return fail((int)n, "launch length");
         if (n > 900000u && n < 4000000u && gens > 80u) return fail((int)n, "a launch of several milliseconds");
         last = gens;
