@@ -350,8 +350,22 @@ int spg_batch_step(spg_batch *b, uint32_t n_gen) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->forked, 0);
     if (e != cudaSuccess) return cuda_fail(e, "fork continuous members");
     int rc = b->teams.step(n_gen, true, b->stream);
-    for (uint32_t i = 0; i + kGraphChunk <= n_gen && rc == SPG_OK; i += kGraphChunk) rc = run_chunk(b, kGraphChunk, b->side);
-    if (rc == SPG_OK && n_gen % kGraphChunk) rc = run_chunk(b, n_gen % kGraphChunk, b->side);
+    // one generation of one small group: its two launches are quicker than a graph
+    // (two members of 1,000, one of them continuous, 15.7 us a call against 18.6; of
+    // 2 x 10^5 43.6 against 35.5)
+    const Group *only = nullptr;
+    uint32_t groups = 0;
+    for (const Group &g : b->groups)
+        if (g.continuous && !g.members.empty()) {
+            only = &g;
+            ++groups;
+        }
+    if (rc == SPG_OK && n_gen == 1u && groups == 1u && only->gl.blocks <= 128u) {
+        rc = launch_generation(only->gl, b->side);
+    } else {
+        for (uint32_t i = 0; i + kGraphChunk <= n_gen && rc == SPG_OK; i += kGraphChunk) rc = run_chunk(b, kGraphChunk, b->side);
+        if (rc == SPG_OK && n_gen % kGraphChunk) rc = run_chunk(b, n_gen % kGraphChunk, b->side);
+    }
     e = cudaEventRecord(b->joined, b->side);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->joined, 0);
     if (rc == SPG_OK && e != cudaSuccess) return cuda_fail(e, "join continuous members");

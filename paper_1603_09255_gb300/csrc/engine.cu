@@ -575,10 +575,13 @@ double schedule_teams(const std::vector<TeamMember> &members, uint32_t blocks, s
     return std::max(best, 0.0);
 }
 
-// SM cycles of a generation of continuous values (92, 143, 234 and 472 us at N =
-// 10^6 for L = 32 .. 256), and the SMs it fills: four blocks of 256 each.
+// SM cycles of a generation of continuous values beside teams, and the SMs it
+// fills: four blocks of 256 each.  Half of what it takes alone (92, 143, 234 and 472
+// us at N = 10^6 for L = 32 .. 256): much of that waits for memory, which more SMs
+// do not shorten (two members of 2 x 10^5, one of them continuous, 36.4 us a
+// generation with all of it, 29.7 with half).
 double continuous_work(uint32_t n, uint32_t n_loci) {
-    return (double)n * (n_loci == 32 ? 29.0 : n_loci == 64 ? 45.0 : n_loci == 128 ? 74.0 : 148.0);
+    return (double)n * (n_loci == 32 ? 14.5 : n_loci == 64 ? 22.5 : n_loci == 128 ? 37.0 : 74.0);
 }
 uint32_t continuous_blocks(uint32_t n) { return (uint32_t)(((uint64_t)n + 1023u) / 1024u); }
 
