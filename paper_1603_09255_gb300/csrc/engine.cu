@@ -1,14 +1,13 @@
 // Host engine and C ABI of libspegg_gb300 (see include/spegg.h).
 //
 // A population owns one device arena.  Biallelic populations are formed by the
-// generation kernel (generations.cuh): alone, one cooperative launch per call,
-// or as members of a batch or server by teams of blocks (TeamSet).  Continuous
-// allelic values take two launches per generation, enqueued as a cached CUDA
-// graph of kGraphChunk generations.
+// generation kernel (generations.cuh): alone, in cooperative launches of many
+// generations, or as members of a batch or server by teams of blocks (TeamSet).
+// Continuous allelic values take two launches per generation, enqueued as a
+// cached CUDA graph of kGraphChunk generations.
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <queue>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
