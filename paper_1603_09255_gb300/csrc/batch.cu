@@ -345,8 +345,14 @@ int spg_batch_step(spg_batch *b, uint32_t n_gen) {
     if (!b) return fail(SPG_ERR_INVALID, "batch is NULL");
     if (n_gen == 0) return SPG_OK;
     if (!any_continuous(b)) return b->teams.step(n_gen, true, b->stream);
+    // a graph launch cannot be captured: refused before anything is enqueued
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(b->stream, &capturing);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamIsCapturing");
+    if (capturing != cudaStreamCaptureStatusNone)
+        return fail(SPG_ERR_CUDA, "continuous members cannot be stepped while the stream is being captured");
     // the continuous members beside the others, on a stream of their own
-    cudaError_t e = cudaEventRecord(b->forked, b->stream);
+    e = cudaEventRecord(b->forked, b->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->forked, 0);
     if (e != cudaSuccess) return cuda_fail(e, "fork continuous members");
     int rc = b->teams.step(n_gen, true, b->stream);

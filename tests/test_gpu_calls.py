@@ -189,3 +189,21 @@ def test_populations_on_streams_of_their_own():
     for w, p in zip(ws, pops):
         orc = oracle.OraclePopulation.from_workload(w)
         assert_population(p, orc, orc.step(14), 14)
+
+
+@pytest.mark.parametrize("gens", [1, 3, 40])
+def test_continuous_members_under_stream_capture_are_refused(gens):
+    """Before anything is enqueued: the batch goes on afterwards."""
+    m = spegg()
+    ws = kinds(600, 32, 6)[:2] + [continuous(500, 32, 6)]
+    stream = torch.cuda.Stream()
+    b = m.Batch(ws, stats_capacity=64, stream=stream)
+    b.step(gens)
+    b.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        with pytest.raises(m.SpeggError):
+            b.step(gens)
+    b.step(2)
+    for i, w in enumerate(ws):
+        assert_member(b, i, w, gens + 2)
